@@ -297,9 +297,127 @@ __device__ __forceinline__ int64_t row_own(const Row& r, int deg, int32_t p) {
   return s;
 }
 
-// Sub-warp work queue of a staged tile: the lanes in `work` (vertices with a
-// neighbour outside their own PE) are served four at a time by 8-lane
-// sub-warps; each sub-warp evaluates T(q) for every distinct neighbouring PE
+// The neighbourhood of one vertex summed by PE, in the registers of one lane:
+// the weight inside P(v) and the (at most kPeSlots) distinct PEs outside it
+// with their summed weights.  On a mapping that is being refined nearly every
+// vertex touches one to three foreign PEs, so one pass over the row and a sum
+// over the few PEs replace a distance sum over the row per entry: a warp rates
+// its 32 vertices side by side.  Vertices with more foreign PEs (n > kPeSlots)
+// go to the sub-warp queue, which takes any row.  Four slots: with six or
+// eight the passes over meshes were 2-4 % slower (a slot costs every entry two
+// instructions), and only random mappings gained (3 %).
+constexpr int kPeSlots = 4;
+struct PeSums {
+  int32_t q[kPeSlots], w[kPeSlots];
+  int32_t own;
+  int32_t n;  // distinct foreign PEs; above kPeSlots: the slots are not complete
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int k = 0; k < kPeSlots; k++) {
+      q[k] = -1;
+      w[k] = 0;
+    }
+    own = 0;
+    n = 0;
+  }
+  __device__ __forceinline__ void add(int32_t c, int32_t x, int32_t p) {
+    if (c == p) {
+      own += x;
+      return;
+    }
+    bool hit = false;
+#pragma unroll
+    for (int k = 0; k < kPeSlots; k++) {
+      const bool m = q[k] == c;
+      w[k] += m ? x : 0;
+      hit |= m;
+    }
+    if (!hit) {
+#pragma unroll
+      for (int k = 0; k < kPeSlots; k++)
+        if (k == n) {
+          q[k] = c;
+          w[k] = x;
+        }
+      n++;
+    }
+  }
+  // sum_u w(v, u) D(b, P(u)); an unused slot has weight 0 and q = -1, whose
+  // distance reads the zero entry of the table
+  __device__ __forceinline__ int64_t cost(const int32_t* sdist, int32_t b, int32_t p) const {
+    int64_t T = (int64_t)own * dcode(sdist, b, p);
+#pragma unroll
+    for (int k = 0; k < kPeSlots; k++) T += (int64_t)w[k] * dcode(sdist, b, q[k]);
+    return T;
+  }
+};
+
+// Sums the row at adj / adjw (deg entries) of a vertex on PE p, up to the
+// entry that no slot is left for; the loads and gathers of four entries are in
+// flight together.
+template <class Pi>
+__device__ __forceinline__ void pe_sums_global(PeSums& ps, const int32_t* __restrict__ adj,
+                                               const int32_t* __restrict__ adjw, Pi pi, int deg, int32_t p) {
+  ps.clear();
+  for (int j = 0; j < deg && ps.n <= kPeSlots; j += 4) {
+    int32_t c[4], w[4];
+#pragma unroll
+    for (int b = 0; b < 4; b++) {
+      c[b] = j + b < deg ? adj[j + b] : -1;
+      w[b] = j + b < deg ? adjw[j + b] : 0;
+    }
+#pragma unroll
+    for (int b = 0; b < 4; b++) c[b] = c[b] >= 0 ? pi[c[b]] : p;
+#pragma unroll
+    for (int b = 0; b < 4; b++) ps.add(c[b], w[b], p);
+  }
+}
+__device__ __forceinline__ void pe_sums_staged(PeSums& ps, const int32_t* c, const int32_t* w, int deg, int32_t p) {
+  ps.clear();
+  for (int j = 0; j < deg && ps.n <= kPeSlots; j++) ps.add(c[j], w[j], p);
+}
+
+// Alg. 4 step 1 from complete sums (0 < n <= kPeSlots): the foreign PE of
+// smallest T (lowest code on ties) and the gain G = T(P(v)) - T(q).
+__device__ __forceinline__ int64_t pe_best_gain(const PeSums& ps, const int32_t* sdist, int32_t p, int32_t& bc) {
+  int64_t bt = INT64_MAX;
+  bc = INT32_MAX;
+#pragma unroll
+  for (int k = 0; k < kPeSlots; k++) {
+    if (k >= ps.n) continue;
+    const int64_t T = ps.cost(sdist, ps.q[k], p);
+    if (T < bt || (T == bt && ps.q[k] < bc)) {
+      bt = T;
+      bc = ps.q[k];
+    }
+  }
+  return ps.cost(sdist, p, p) - bt;
+}
+
+// Alg. 5 destination from complete sums: the foreign PE with W <= sigma of
+// largest score (conn, or -T with kJ), lowest code on ties; false if none.
+template <bool kJ>
+__device__ __forceinline__ bool pe_best_dest(const PeSums& ps, const int32_t* sdist, const int64_t* W, int64_t sigma,
+                                             int32_t p, int32_t& bc, int64_t& score) {
+  bool found = false;
+  bc = INT32_MAX;
+  score = 0;
+#pragma unroll
+  for (int k = 0; k < kPeSlots; k++) {
+    if (k >= ps.n || W[ps.q[k]] > sigma) continue;
+    const int64_t sc = kJ ? -ps.cost(sdist, ps.q[k], p) : (int64_t)ps.w[k];
+    if (!found || sc > score || (sc == score && ps.q[k] < bc)) {
+      score = sc;
+      bc = ps.q[k];
+      found = true;
+    }
+  }
+  return found;
+}
+
+// Sub-warp work queue of a staged tile: the lanes in `work` (vertices with
+// too many foreign PEs for one lane's slots) are served four at a time by
+// 8-lane sub-warps; each sub-warp evaluates T(q) for every distinct neighbouring PE
 // q != p of its vertex from the staged entries and keeps the minimum (lowest
 // code on ties).  out(lane, G = T(p) - T(q*), q*, p, conn(v, p)) runs on the
 // sub-warp's first lane; conn(v, p) is summed only when `own` is set (else 0).
@@ -317,13 +435,20 @@ struct RowLoader {
     }
   }
 };
-struct NoRowLoader {  // callers that never queue a vertex of an unstaged tile
-  __device__ __forceinline__ void operator()(int64_t, int, int, int32_t*, int32_t*) const {}
+struct PlainRowLoader {  // neighbour PEs through plain loads (the mapping changes inside the launch)
+  const int32_t* __restrict__ adj;
+  const int32_t* __restrict__ adjw;
+  const int32_t* pi;
+  __device__ __forceinline__ void operator()(int64_t vb, int dg, int sl, int32_t* c, int32_t* w) const {
+    for (int j = sl; j < dg; j += kSubWarp) {
+      c[j] = pi[adj[vb + j]];
+      w[j] = adjw[vb + j];
+    }
+  }
 };
 
 template <class Load, class Out>
-__device__ __forceinline__ void tile_gain_queue(unsigned work, const TileLane& t, int32_t p, int64_t Tp,
-                                                int32_t* sc, int32_t* sw, int cap, Load load,
+__device__ __forceinline__ void tile_gain_queue(unsigned work, const TileLane& t, int32_t p, int32_t* sc, int32_t* sw, int cap, Load load,
                                                 const int32_t* sdist, int lane, bool own, Out out) {
   const int sub = lane >> 3, sl = lane & 7;
   const int rounds = (__popc(work) + 3) / 4;
@@ -333,7 +458,6 @@ __device__ __forceinline__ void tile_gain_queue(unsigned work, const TileLane& t
     const int64_t vb = __shfl_sync(0xffffffffu, t.b, s2);
     const int dg = (int)(__shfl_sync(0xffffffffu, t.e, s2) - vb);
     const int32_t pv = __shfl_sync(0xffffffffu, p, s2);
-    const int64_t tp = __shfl_sync(0xffffffffu, Tp, s2);
     int64_t off = vb - t.E0;
     if (!t.staged) {  // warp-uniform
       off = sub * (cap / 4);
@@ -343,7 +467,7 @@ __device__ __forceinline__ void tile_gain_queue(unsigned work, const TileLane& t
     }
     const int32_t* c = sc + off;
     const int32_t* w = sw + off;
-    int64_t bt = INT64_MAX, ow = 0;
+    int64_t bt = INT64_MAX, tp = 0, ow = 0;
     int32_t bc = INT32_MAX;
     if (src >= 0) {
       for (int j = sl; j < dg; j += kSubWarp) {
@@ -352,6 +476,7 @@ __device__ __forceinline__ void tile_gain_queue(unsigned work, const TileLane& t
           ow += w[j];
           continue;
         }
+        tp += (int64_t)w[j] * dcode(sdist, pv, q);
         int64_t T = 0;
         for (int l = 0; l < dg; l++) T += (int64_t)w[l] * dcode(sdist, q, c[l]);
         if (T < bt || (T == bt && q < bc)) {
@@ -368,17 +493,22 @@ __device__ __forceinline__ void tile_gain_queue(unsigned work, const TileLane& t
         bt = ot;
         bc = oc;
       }
+      tp += __shfl_xor_sync(0xffffffffu, tp, o);
       if (own) ow += __shfl_xor_sync(0xffffffffu, ow, o);
     }
     if (src >= 0 && sl == 0) out(src, tp - bt, bc, pv, ow);
   }
 }
 
-// Alg. 4 step 1 for the low-degree vertices.  Warp tiles stage the
-// neighbour PEs; each lane checks its own vertex (T(P(v)), any neighbour
-// outside P(v)); the vertices with candidates are then evaluated four at a
-// time by 8-lane sub-warps from the staged entries (in a tile too long to
-// stage, from the row each sub-warp copies into shared memory first).
+// Alg. 4 step 1 for the low-degree vertices.  Warp tiles stage the neighbour
+// PEs; each lane sums its own row by PE (PeSums) and decides its vertex from
+// the sums; the vertices with more than kPeSlots foreign PEs are evaluated
+// four at a time by 8-lane sub-warps from the staged entries (in a tile too
+// long to stage, from the row each sub-warp copies into shared memory first).
+// What bounds it is the instructions per vertex, so the lane sums come first:
+// with every vertex that has a foreign neighbour in the queue it took 170 us
+// on a 3D grid of 2^21 vertices (12.5 M entries) and 82 us on a random
+// geometric graph of 2^20 (12.6 M entries), with the sums 78 and 41 us.
 __global__ void __launch_bounds__(kTileThreads, kTileMinBlocks) k_lp_gain_tile(GraphView g, const int32_t* __restrict__ pi,
                                                                uint8_t* __restrict__ lock, int32_t* __restrict__ pp,
                                                                int64_t* __restrict__ gain, uint8_t* __restrict__ inx,
@@ -395,38 +525,35 @@ __global__ void __launch_bounds__(kTileThreads, kTileMinBlocks) k_lp_gain_tile(G
   for (int64_t tile = (int64_t)blockIdx.x * kTileWarps + warp; tile < ntiles; tile += (int64_t)gridDim.x * kTileWarps) {
     const TileLane t = stage_tile(tg, tile * kTileV, lane, sc[warp], sw[warp], GatherPi{pi});
     const int deg = (int)(t.e - t.b);
-    const bool low = t.v < g.n && deg <= kLowDeg;
     int32_t p = -1;
-    int64_t Tp = 0;
-    bool cand = false;
-    if (low) {
+    bool over = false;
+    if (t.v < g.n && deg <= kLowDeg) {
       p = pi[t.v];
-      if (lock[t.v]) {
+      PeSums ps;
+      if (lock[t.v]) {  // stays this step
         lock[t.v] = 0;
+        ps.clear();
       } else if (t.staged) {
-        // T(P(v)) only for vertices with a neighbour outside P(v): interior
-        // vertices (most of them on a refined level) skip the distance sum
-        const int32_t* c = sc[warp] + (t.b - t.E0);
-        const int32_t* w = sw[warp] + (t.b - t.E0);
-        for (int j = 0; j < deg; j++) cand |= c[j] != p;
-        if (cand)
-          for (int j = 0; j < deg; j++) Tp += (int64_t)w[j] * dcode(sdist, p, c[j]);
-      } else {  // oversized tile: the lane check from global memory; a sub-warp stages the row below
-        for (int j = 0; j < deg; j++) {
-          const int32_t q = pi[g.adj[t.b + j]];
-          cand |= q != p;
-          Tp += (int64_t)g.adjw[t.b + j] * dcode(sdist, p, q);
-        }
+        pe_sums_staged(ps, sc[warp] + (t.b - t.E0), sw[warp] + (t.b - t.E0), deg, p);
+      } else {
+        pe_sums_global(ps, g.adj + t.b, g.adjw + t.b, pi, deg, p);
       }
-      if (!cand) {  // locked, or no neighbour outside P(v)
-        inx[t.v] = 0;
-        pp[t.v] = p;
-        gain[t.v] = 0;
+      over = ps.n > kPeSlots;
+      if (!over) {
+        int32_t bc = p;
+        int64_t G = 0;
+        bool in = ps.n > 0;
+        if (in) {
+          G = pe_best_gain(ps, sdist, p, bc);
+          in = flt.admit(G, ps.own);
+        }
+        inx[t.v] = in ? 1 : 0;
+        pp[t.v] = in ? bc : p;
+        gain[t.v] = in ? G : 0;
       }
     }
-    const unsigned work = __ballot_sync(0xffffffffu, cand);
-    tile_gain_queue(work, t, p, Tp, sc[warp], sw[warp], kTileE, RowLoader{g.adj, g.adjw, pi}, sdist, lane,
-                    flt.num > 0,
+    const unsigned work = __ballot_sync(0xffffffffu, over);
+    tile_gain_queue(work, t, p, sc[warp], sw[warp], kTileE, RowLoader{g.adj, g.adjw, pi}, sdist, lane, flt.num > 0,
                     [&](int src, int64_t G, int32_t bc, int32_t pv, int64_t own) {
                       const int64_t v = tile * kTileV + src;
                       const bool in = flt.admit(G, own);
@@ -728,22 +855,36 @@ __global__ void __launch_bounds__(kThreads) k_lp_after_low(GraphView g, const in
   if (!kind_is(st, 1 << KIND_LP)) return;
   load_sdist(sdist, topo);
   __syncthreads();
-  auto tile = cg::tiled_partition<kSubWarp>(cg::this_thread_block());
-  const int lane = tile.thread_rank();
-  const int64_t nsw = ((int64_t)gridDim.x * blockDim.x) / kSubWarp;
-  for (int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kSubWarp; v < g.n; v += nsw) {
-    if (!inx[v]) continue;
-    const int64_t beg = g.xadj[v], end = g.xadj[v + 1];
-    if (end - beg > kLowDeg) continue;
-    const int32_t p = pi[v], q = pp[v];
-    const int64_t gv = gain[v];
-    int64_t s = 0;
-    for (int64_t e = beg + lane; e < end; e += kSubWarp) {
-      const int32_t b = future_block(g.adj[e], (int32_t)v, gv, pi, pp, gain, inx);
-      s += (int64_t)g.adjw[e] * (dcode(sdist, p, b) - dcode(sdist, q, b));
+  // 32 vertices per warp: one lane reads a vertex's flag, then the candidates
+  // are served four at a time by 8-lane sub-warps (most vertices are none; a
+  // sub-warp per vertex spent its time on their flags: 28 us on a 3D grid of
+  // 2^21 vertices, 17 us so)
+  const int lane = threadIdx.x & 31, sub = lane / kSubWarp, sl = lane & (kSubWarp - 1);
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t base = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; base < g.n; base += nwarps * 32) {
+    const int64_t vl = base + lane;
+    const unsigned work = __ballot_sync(0xffffffffu, vl < g.n && inx[vl]);
+    const int rounds = (__popc(work) + 3) / 4;
+    for (int r = 0; r < rounds; r++) {
+      const int src = tile_worker(work, r, sub);
+      const int64_t v = base + (src < 0 ? 0 : src);
+      int64_t s = -1;
+      if (src >= 0) {
+        const int64_t beg = g.xadj[v], end = g.xadj[v + 1];
+        if (end - beg <= kLowDeg) {
+          const int32_t p = pi[v], q = pp[v];
+          const int64_t gv = gain[v];
+          s = 0;
+          for (int64_t e = beg + sl; e < end; e += kSubWarp) {
+            const int32_t b = future_block(g.adj[e], (int32_t)v, gv, pi, pp, gain, inx);
+            s += (int64_t)g.adjw[e] * (dcode(sdist, p, b) - dcode(sdist, q, b));
+          }
+        }
+      }
+#pragma unroll
+      for (int o = kSubWarp / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (src >= 0 && sl == 0 && s >= 0) lock[v] = 1;
     }
-    s = tile_sum64(tile, s);
-    if (lane == 0 && s >= 0) lock[v] = 1;
   }
 }
 
@@ -882,7 +1023,8 @@ __device__ __forceinline__ int64_t delta_entry(const Mv& mv, const int32_t* pi, 
   return um ? d : 2 * d;
 }
 
-// movers of degree <= kLowDeg: one 8-lane sub-warp per vertex
+// movers of degree <= kLowDeg: found by one lane per vertex, served four at a
+// time by the 8-lane sub-warps of the warp (as k_lp_after_low)
 template <class Mv>
 __global__ void __launch_bounds__(kThreads) k_delta_low(GraphView g, const int32_t* __restrict__ pi, Mv mv, Topo topo,
                                                         int64_t* Jacc, const RefineState* st, int kind) {
@@ -891,15 +1033,22 @@ __global__ void __launch_bounds__(kThreads) k_delta_low(GraphView g, const int32
   if (st->kind != kind) return;
   load_sdist(sdist, topo);
   __syncthreads();
-  const int lane = threadIdx.x & (kSubWarp - 1);
-  const int64_t nsw = ((int64_t)gridDim.x * blockDim.x) / kSubWarp;
+  const int lane = threadIdx.x & 31, sub = lane / kSubWarp, sl = lane & (kSubWarp - 1);
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   int64_t acc = 0;
-  for (int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kSubWarp; v < g.n; v += nsw) {
-    if (!mv.moved(v)) continue;
-    const int64_t b = g.xadj[v], e = g.xadj[v + 1];
-    if (e - b > kLowDeg) continue;
-    const int32_t ov = pi[v], nv = mv.target(v);
-    for (int64_t x = b + lane; x < e; x += kSubWarp) acc += delta_entry(mv, pi, sdist, ov, nv, g.adj[x], g.adjw[x]);
+  for (int64_t base = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; base < g.n; base += nwarps * 32) {
+    const int64_t vl = base + lane;
+    const unsigned work = __ballot_sync(0xffffffffu, vl < g.n && mv.moved(vl));
+    const int rounds = (__popc(work) + 3) / 4;
+    for (int r = 0; r < rounds; r++) {
+      const int src = tile_worker(work, r, sub);
+      if (src < 0) continue;
+      const int64_t v = base + src;
+      const int64_t b = g.xadj[v], e = g.xadj[v + 1];
+      if (e - b > kLowDeg) continue;
+      const int32_t ov = pi[v], nv = mv.target(v);
+      for (int64_t x = b + sl; x < e; x += kSubWarp) acc += delta_entry(mv, pi, sdist, ov, nv, g.adj[x], g.adjw[x]);
+    }
   }
   acc = block_sum(acc, sm);
   if (threadIdx.x == 0 && acc) atomicAdd((unsigned long long*)Jacc, (unsigned long long)acc);
@@ -1142,24 +1291,59 @@ __global__ void __launch_bounds__(kThreads) k_reb_select_low(GraphView g, const 
   const int64_t sigma = a.cnt[CNT_SIGMA];
   const int64_t nU = a.cnt[CNT_NU];
   const int32_t level = st->level, t = st->t;
-  // 32 vertices per warp: each lane checks its vertex's eligibility (most
-  // are not: their blocks are not overloaded), then the eligible ones are
-  // served four at a time by the 8-lane sub-warps
+  // 32 vertices per warp: each lane checks its vertex's eligibility (most are
+  // not: their blocks are not overloaded), sums its row by PE and picks the
+  // destination; the vertices with more than kPeSlots foreign PEs are served
+  // four at a time by the 8-lane sub-warps.  3D grid of 2^21 vertices: 175 us
+  // with every eligible vertex in the queue, 55 us so
   for (int64_t base = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; base < g.n; base += nwarps * 32) {
     const int64_t vl = base + wl;
     bool want = false;
     int64_t beg_l = 0;
     int deg_l = 0;
-    int32_t A_l = 0;
+    int32_t A_l = 0, cv_l = 0;
     if (vl < g.n) {
       beg_l = g.xadj[vl];
       deg_l = (int)(g.xadj[vl + 1] - beg_l);
       if (deg_l <= kLowDeg) {
         A_l = pi[vl];
-        want = reb_eligible(a, A_l, g.vw[vl]);
+        cv_l = g.vw[vl];
+        want = reb_eligible(a, A_l, cv_l);
         if (!want) elig[vl] = 0;
       }
     }
+    if (!__any_sync(0xffffffffu, want)) continue;
+    int32_t slot = -1;  // (block, bucket) of a vertex decided by its own lane
+    if (want) {
+      PeSums ps;
+      pe_sums_global(ps, g.adj + beg_l, g.adjw + beg_l, pi, deg_l, A_l);
+      if (ps.n <= kPeSlots) {
+        want = false;
+        int32_t bc;
+        int64_t sc;
+        const bool found = a.obj ? pe_best_dest<true>(ps, sdist, a.W, sigma, A_l, bc, sc)
+                                 : pe_best_dest<false>(ps, sdist, a.W, sigma, A_l, bc, sc);
+        if (found || nU > 0) {
+          if (!found) {
+            bc = a.U[h_rebalance(a.seed, level, t, (int32_t)vl) % (uint64_t)nU];
+            sc = a.obj ? -ps.cost(sdist, bc, A_l) : 0;
+          }
+          const int32_t bk = loss_bucket(sc - (a.obj ? -ps.cost(sdist, A_l, A_l) : (int64_t)ps.own));
+          dest[vl] = bc;
+          bkt[vl] = (uint8_t)bk;
+          elig[vl] = 1;
+          slot = A_l * kBuckets + bk;
+        } else {
+          elig[vl] = 0;
+        }
+      }
+    }
+    // one update per (block, bucket) of the tile: neighbours sit in the same
+    // few blocks, and their single updates would queue on the same words
+    const unsigned same = __match_any_sync(0xffffffffu, slot);
+    const int32_t cw = (int32_t)__reduce_add_sync(same, (unsigned)cv_l);
+    if (slot >= 0 && wl == __ffs(same) - 1)
+      atomicAdd((unsigned long long*)&a.tab[slot], (unsigned long long)(int64_t)cw);
     const unsigned work = __ballot_sync(0xffffffffu, want);
     const int rounds = (__popc(work) + 3) / 4;
     for (int rnd = 0; rnd < rounds; rnd++) {
@@ -2132,7 +2316,7 @@ void launch_eval(Ctx& c, int lvl, const EvalCtl* ec = nullptr, bool full = true)
 template <class Mv>
 void launch_delta(Ctx& c, int lvl, Mv mv, int kind) {
   Level& L = c.lv[lvl];
-  k_delta_low<Mv><<<grid_for(c, kThreads / kSubWarp, L.n), kThreads, 0, c.st>>>(view(L), L.pi, mv, c.topo, c.Jacc,
+  k_delta_low<Mv><<<grid_for(c, kThreads, L.n), kThreads, 0, c.st>>>(view(L), L.pi, mv, c.topo, c.Jacc,
                                                                                  c.state, kind); count_launch();
   if (L.n_hi > L.n_huge) {
     k_delta_mid<Mv><<<mid_grid(c, (const void*)k_delta_mid<Mv>, 0, L.n_hi), kMidThreads, 0, c.st>>>(
@@ -2147,7 +2331,7 @@ void launch_delta(Ctx& c, int lvl, Mv mv, int kind) {
 
 void launch_lp(Ctx& c, int lvl) {
   Level& L = c.lv[lvl];
-  const unsigned gl = grid_for(c, kThreads / kSubWarp, L.n);
+  const unsigned gl = grid_for(c, kThreads, L.n);
   const bool mid_tab = mid_tables(c);
   const GroupLayout glay = group_layout(c.topo);
   // vertices of degree > kLowDeg left to the CTA-per-vertex kernels
@@ -2215,7 +2399,7 @@ void launch_rebalance(Ctx& c, int lvl, bool prep_done = false) {
     k_reb_prep<<<1, 1024, 0, c.st>>>(reb_prep_args(c), c.state); count_launch();
   }
   RebArgs a{c.W, c.U, c.counters, c.tab, c.lmax, c.cV, c.k, c.cfg.seed, c.cfg.reb_objective, c.topo};
-  k_reb_select_low<<<grid_for(c, kThreads / kSubWarp, n), kThreads, 0, c.st>>>(view(L), L.pi, a, c.dest, bucket,
+  k_reb_select_low<<<grid_for(c, kThreads, n), kThreads, 0, c.st>>>(view(L), L.pi, a, c.dest, bucket,
                                                                                  c.elig, c.state); count_launch();
   if (L.n_hi) {
     const GroupLayout gl = group_layout(c.topo);
@@ -2660,28 +2844,17 @@ struct PlainGather {  // neighbour PEs through plain loads (the mapping changes 
 };
 
 // Stages one tile of neighbour PEs and returns T(P(v)) = sum_j w_j D(P(v), c_j)
-// of the lane's vertex; `cand` tells whether a staged row has a neighbour
-// outside P(v) (oversized tiles are left to the global path: cand false).
-// A row of more than kEngLaneDeg entries gives 0 and no candidate here.
+// of the lane's vertex (0 for a row of more than kEngLaneDeg entries).
 template <int kTE>
 __device__ __forceinline__ TileLane eng_stage(const EngineJob& J, const TileGraph& tg, int64_t tile, int lane,
-                                              int32_t* sc, int32_t* sw, const int32_t* sdist, int64_t& Tp,
-                                              bool& cand, bool all_tp) {
+                                              int32_t* sc, int32_t* sw, const int32_t* sdist, int64_t& Tp) {
   const TileLane t = stage_tile<kTE>(tg, tile * kTileV, lane, sc, sw, PlainGather{J.pi});
   Tp = 0;
-  cand = false;
   if (t.v < tg.n && !eng_heavy(J, t.e - t.b)) {
     const int deg = (int)(t.e - t.b);
     const int32_t p = J.pi[t.v];
-    if (t.staged) {
-      const int32_t* c = sc + (t.b - t.E0);
-      const int32_t* w = sw + (t.b - t.E0);
-      for (int j = 0; j < deg; j++) cand |= c[j] != p;
-      if (cand || all_tp)
-        for (int j = 0; j < deg; j++) Tp += (int64_t)w[j] * dcode(sdist, p, c[j]);
-    } else {
-      Tp = row_cost(PlainRow{tg.adj + t.b, tg.adjw + t.b, J.pi}, deg, sdist, p);
-    }
+    if (t.staged) Tp = row_cost(StagedRow{sc + (t.b - t.E0), sw + (t.b - t.E0)}, deg, sdist, p);
+    else Tp = row_cost(PlainRow{tg.adj + t.b, tg.adjw + t.b, J.pi}, deg, sdist, p);
   }
   return t;
 }
@@ -2693,9 +2866,11 @@ __device__ __forceinline__ TileLane eng_stage(const EngineJob& J, const TileGrap
 // -T(q) = -sum_u w D(q, P(u)) for the J gains (kJ).  out(lane, A, found, q,
 // score of A, score of q, staged codes, staged weights, degree) runs on the
 // sub-warp's first lane; the gain is the difference of the two scores.
-template <bool kJ, class Out>
-__device__ __forceinline__ void reb_tile_queue(unsigned work, const TileLane& tl, int32_t A, const int32_t* sc,
-                                               const int32_t* sw, const int64_t* W, int64_t sigma,
+// In a tile that was not staged each sub-warp first copies its vertex's row
+// into its quarter of the buffer (capacity `cap`) with `load`.
+template <bool kJ, class Load, class Out>
+__device__ __forceinline__ void reb_tile_queue(unsigned work, const TileLane& tl, int32_t A, int32_t* sc,
+                                               int32_t* sw, int cap, Load load, const int64_t* W, int64_t sigma,
                                                const int32_t* sdist, int lane, Out out) {
   const int sub = lane >> 3, sl = lane & 7;
   const int rounds = (__popc(work) + 3) / 4;
@@ -2705,8 +2880,15 @@ __device__ __forceinline__ void reb_tile_queue(unsigned work, const TileLane& tl
     const int64_t vb = __shfl_sync(0xffffffffu, tl.b, s2);
     const int dg = (int)(__shfl_sync(0xffffffffu, tl.e, s2) - vb);
     const int32_t a = __shfl_sync(0xffffffffu, A, s2);
-    const int32_t* c = sc + (vb - tl.E0);
-    const int32_t* w = sw + (vb - tl.E0);
+    int64_t off = vb - tl.E0;
+    if (!tl.staged) {  // warp-uniform
+      off = sub * (cap / 4);
+      __syncwarp();  // the previous round has read this quarter
+      if (src >= 0) load(vb, dg, sl, sc + off, sw + off);
+      __syncwarp();
+    }
+    const int32_t* c = sc + off;
+    const int32_t* w = sw + off;
     if constexpr (!kJ) {
       int32_t ca = 0, bconn = -1, bc = INT32_MAX;
       if (src >= 0) {
@@ -2935,8 +3117,6 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
   int phase = 0;
   int32_t prev_kind = KIND_NONE;
   TileLane t0{};
-  int64_t Tp0 = 0;
-  bool cand0 = false;
   while (true) {
     // J of the current mapping (after an LP or weak step the accumulator
     // already holds it: old J plus the step's exact change), then the Alg. 6
@@ -2947,14 +3127,9 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
       int64_t acc = 0;
       for (int64_t tile = eg.gw; tile < ntiles; tile += eg.GW) {
         int64_t Tp;
-        bool cand;
-        const TileLane t = eng_stage<kTE>(J, tg, tile, lane, sc, sw, S.sdist, Tp, cand, true);
+        const TileLane t = eng_stage<kTE>(J, tg, tile, lane, sc, sw, S.sdist, Tp);
         acc += Tp;
-        if (single) {
-          t0 = t;
-          Tp0 = Tp;
-          cand0 = cand;
-        }
+        if (single) t0 = t;
         __syncwarp();
       }
       eng_heavy_rows(J, eg, [&](int32_t v, int64_t b, int64_t e) {
@@ -2992,41 +3167,52 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
     phase = 1;
     prev_kind = kind;
     if (kind == KIND_LP) {
-      // Alg. 4 step 1: staged tiles, lane check, sub-warp work queue
+      // Alg. 4 step 1: staged tiles, each lane decides its vertex from its
+      // row's sums by PE; the others through the sub-warp work queue
       for (int64_t tile = eg.gw; tile < ntiles; tile += eg.GW) {
         TileLane t = t0;
-        int64_t Tp = Tp0;
-        bool cand = cand0;
-        if (!reuse) t = eng_stage<kTE>(J, tg, tile, lane, sc, sw, S.sdist, Tp, cand, false);
+        if (!reuse) t = stage_tile<kTE>(tg, tile * kTileV, lane, sc, sw, PlainGather{J.pi});
         int32_t p = -1;
+        bool over = false;
         if (t.v < n && !eng_heavy(J, t.e - t.b)) {
+          const int deg = (int)(t.e - t.b);
           p = J.pi[t.v];
-          bool written = false;
-          if (J.lock[t.v]) {
+          PeSums ps;
+          if (J.lock[t.v]) {  // stays this step
             J.lock[t.v] = 0;
-            cand = false;
-          } else if (!t.staged) {  // oversized tile: this lane alone, from global memory
-            const PlainRow r{g.adj + t.b, g.adjw + t.b, J.pi};
-            int32_t bc;
-            int64_t bt;
-            if (best_target(r, (int)(t.e - t.b), p, S.sdist, bc, bt) &&
-                (kVar ? J.flt.admit(Tp - bt, J.flt.num > 0 ? row_own(r, (int)(t.e - t.b), p) : 0)
-                      : Tp - bt >= 0)) {
-              J.inx[t.v] = 1;
-              J.pp[t.v] = bc;
-              J.gain[t.v] = Tp - bt;
-              written = true;
-            }
+            ps.clear();
+          } else if (t.staged) {
+            pe_sums_staged(ps, sc + (t.b - t.E0), sw + (t.b - t.E0), deg, p);
+          } else {
+            pe_sums_global(ps, g.adj + t.b, g.adjw + t.b, J.pi, deg, p);
           }
-          if (!cand && !written) {
-            J.inx[t.v] = 0;
-            J.pp[t.v] = p;
-            J.gain[t.v] = 0;
+          over = ps.n > kPeSlots;
+          int32_t bc = p;
+          int64_t G = 0;
+          bool in = false;
+          if (!over) {
+            in = ps.n > 0;
+            if (in) {
+              G = pe_best_gain(ps, S.sdist, p, bc);
+              in = kVar ? J.flt.admit(G, ps.own) : G >= 0;
+            }
+          } else if (!t.staged && deg > kTE / 4) {  // longer than a sub-warp's quarter of the staging area
+            over = false;
+            const PlainRow r{g.adj + t.b, g.adjw + t.b, J.pi};
+            int64_t bt;
+            best_target(r, deg, p, S.sdist, bc, bt);
+            G = row_cost(r, deg, S.sdist, p) - bt;
+            in = kVar ? J.flt.admit(G, row_own(r, deg, p)) : G >= 0;
+          }
+          if (!over) {
+            J.inx[t.v] = in ? 1 : 0;
+            J.pp[t.v] = in ? bc : p;
+            J.gain[t.v] = in ? G : 0;
           }
         }
-        const unsigned work = __ballot_sync(0xffffffffu, cand);
-        tile_gain_queue(work, t, p, Tp, sc, sw, kTE, NoRowLoader{}, S.sdist, lane, kVar && J.flt.num > 0,
-                        [&](int src, int64_t Gv, int32_t bc, int32_t pv, int64_t own) {
+        const unsigned work = __ballot_sync(0xffffffffu, over);
+        tile_gain_queue(work, t, p, sc, sw, kTE, PlainRowLoader{g.adj, g.adjw, J.pi}, S.sdist, lane,
+                        kVar && J.flt.num > 0, [&](int src, int64_t Gv, int32_t bc, int32_t pv, int64_t own) {
           const int64_t v = tile * kTileV + src;
           const bool in = kVar ? J.flt.admit(Gv, own) : Gv >= 0;
           J.inx[v] = in ? 1 : 0;
@@ -3123,20 +3309,63 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
     const int32_t t = *(volatile int32_t*)&s->t;
     const int64_t sigma = *(volatile int64_t*)&J.cnt[CNT_SIGMA];
     const int64_t nU = *(volatile int64_t*)&J.cnt[CNT_NU];
-    // eligible vertices and their destinations: lane check, then staged rows
+    // eligible vertices and their destinations: each lane from its row's sums
+    // by PE, the vertices with more foreign PEs from staged rows
+    const bool obj = kVar && J.reb_obj != 0;
+    auto drawn = [&](int64_t v) { return J.U[h_rebalance(J.seed, J.level, t, (int32_t)v) % (uint64_t)nU]; };
+    auto reb_write = [&](int64_t v, int32_t A, int32_t dst, int64_t gcut) {
+      const int bk = loss_bucket(gcut);
+      J.elig[v] = 1;
+      J.dest[v] = dst;
+      J.bkt[v] = (uint8_t)bk;
+      return A * kBuckets + bk;
+    };
     for (int64_t tile = eg.gw; tile < ntiles; tile += eg.GW) {
       const int64_t v = tile * kTileV + lane;
-      int32_t A = -1;
+      int32_t A = -1, cv = 0;
       bool cand = false;
+      int64_t vb = 0;
+      int deg = 0;
       if (v < n && !eng_heavy_row(J, v)) {
         A = J.pi[v];
+        cv = g.vw[v];
+        vb = g.xadj[v];
+        deg = (int)(g.xadj[v + 1] - vb);
         const int64_t WA = J.W[A];
-        cand = WA > J.lmax && 2 * (int64_t)J.k * g.vw[v] <= 3 * ((int64_t)J.k * WA - J.cV);
+        cand = WA > J.lmax && 2 * (int64_t)J.k * cv <= 3 * ((int64_t)J.k * WA - J.cV);
         if (!cand) J.elig[v] = 0;
       }
       if (__ballot_sync(0xffffffffu, cand) == 0) continue;
+      int32_t slot = -1;  // (block, bucket) of a vertex decided by its own lane
+      if (cand) {
+        PeSums ps;
+        pe_sums_global(ps, g.adj + vb, g.adjw + vb, J.pi, deg, A);
+        if (ps.n <= kPeSlots) {
+          cand = false;
+          int32_t dst;
+          int64_t sc2;
+          const bool found = obj ? pe_best_dest<true>(ps, S.sdist, J.W, sigma, A, dst, sc2)
+                                 : pe_best_dest<false>(ps, S.sdist, J.W, sigma, A, dst, sc2);
+          if (found || nU > 0) {
+            if (!found) {
+              dst = drawn(v);
+              sc2 = obj ? -ps.cost(S.sdist, dst, A) : 0;
+            }
+            slot = reb_write(v, A, dst, sc2 - (obj ? -ps.cost(S.sdist, A, A) : (int64_t)ps.own));
+          } else {
+            J.elig[v] = 0;
+          }
+        }
+      }
+      if (__any_sync(0xffffffffu, slot >= 0)) {  // one update per (block, bucket) of the tile
+        const unsigned same = __match_any_sync(0xffffffffu, slot);
+        const int32_t cw = (int32_t)__reduce_add_sync(same, (unsigned)cv);
+        if (slot >= 0 && lane == __ffs(same) - 1)
+          atomicAdd((unsigned long long*)&J.tab[slot], (unsigned long long)(int64_t)cw);
+      }
+      if (__ballot_sync(0xffffffffu, cand) == 0) continue;
       const TileLane tl = stage_tile<kTE>(tg, tile * kTileV, lane, sc, sw, PlainGather{J.pi});
-      if (cand && !tl.staged) {  // oversized tile: this lane alone, from global memory
+      if (cand && !tl.staged && deg > kTE / 4) {  // longer than a sub-warp's quarter: this lane alone
         int32_t dst, bk;
         bool ok;
         if constexpr (kVar)
@@ -3148,40 +3377,32 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
         if (ok) {
           J.dest[v] = dst;
           J.bkt[v] = (uint8_t)bk;
-          atomicAdd((unsigned long long*)&J.tab[(int64_t)A * kBuckets + bk], (unsigned long long)(int64_t)g.vw[v]);
+          atomicAdd((unsigned long long*)&J.tab[(int64_t)A * kBuckets + bk], (unsigned long long)(int64_t)cv);
         }
         cand = false;
       }
       const unsigned work = __ballot_sync(0xffffffffu, cand);
       auto reb_out = [&](int src, int32_t a, bool found, int32_t bc, int64_t sa, int64_t sb, const int32_t* rc,
                          const int32_t* rw, int dg) {
-                       const int64_t u = tile * kTileV + src;
-                       int64_t gcut;
-                       int32_t dst;
-                       if (found) {
-                         gcut = sb - sa;
-                         dst = bc;
-                       } else if (nU > 0) {
-                         dst = J.U[h_rebalance(J.seed, J.level, t, u) % (uint64_t)nU];
-                         int64_t sr = 0;  // the drawn block is not a neighbour: conn 0, or -T(q)
-                         if (kVar && J.reb_obj)
-                           for (int l = 0; l < dg; l++) sr -= (int64_t)rw[l] * dcode(S.sdist, dst, rc[l]);
-                         gcut = sr - sa;
-                       } else {
-                         J.elig[u] = 0;
-                         return;
-                       }
-                       const int bk = loss_bucket(gcut);
-                       J.elig[u] = 1;
-                       J.dest[u] = dst;
-                       J.bkt[u] = (uint8_t)bk;
-                       atomicAdd((unsigned long long*)&J.tab[(int64_t)a * kBuckets + bk],
-                                 (unsigned long long)(int64_t)g.vw[u]);
-                     };
-      if (kVar && J.reb_obj != 0)
-        reb_tile_queue<true>(work, tl, A, sc, sw, J.W, sigma, S.sdist, lane, reb_out);
+        const int64_t u = tile * kTileV + src;
+        if (!found && nU <= 0) {
+          J.elig[u] = 0;
+          return;
+        }
+        if (!found) {
+          bc = drawn(u);
+          sb = 0;  // the drawn block is not a neighbour: conn 0, or -T(q)
+          if (obj)
+            for (int l = 0; l < dg; l++) sb -= (int64_t)rw[l] * dcode(S.sdist, bc, rc[l]);
+        }
+        const int32_t at = reb_write(u, a, bc, sb - sa);
+        atomicAdd((unsigned long long*)&J.tab[at], (unsigned long long)(int64_t)g.vw[u]);
+      };
+      const PlainRowLoader load{g.adj, g.adjw, J.pi};
+      if (obj)
+        reb_tile_queue<true>(work, tl, A, sc, sw, kTE, load, J.W, sigma, S.sdist, lane, reb_out);
       else
-        reb_tile_queue<false>(work, tl, A, sc, sw, J.W, sigma, S.sdist, lane, reb_out);
+        reb_tile_queue<false>(work, tl, A, sc, sw, kTE, load, J.W, sigma, S.sdist, lane, reb_out);
       __syncwarp();
     }
     if (J.has_heavy) {
