@@ -4015,9 +4015,22 @@ static bool engine_rows_fit(const Ctx& c, const Level& L) {
   return L.max_deg <= kEngLaneDeg || (size_t)group_layout(c.topo).total * sizeof(int32_t) <= engine_smem(256);
 }
 
+// Whether a level that a size limit gives to the engine is better refined by
+// the graph of kernels: the engine takes a row of 33..128 entries with one
+// sub-warp and a larger one with a whole CTA, one after the other, where the
+// graph has a warp per vertex and the hub chunks.
+// Per Alg. 6 iteration, engine against graph (us), by the share of the
+// level's entries in rows above 32: meshes and their coarse levels with at
+// most 4 %: 24-81 against 43-97; random geometric graph of degree 40, 90 %:
+// 134 against 104; R-MAT with 770 to 200 k vertices, 67-98 %: 370-1900
+// against 109-284.  Hence one entry in 16.
+// A limit set in the config (`asked`) is followed as it stands.
+static bool engine_slower(const Level& L, int32_t asked) { return asked == 0 && L.m_hi * 16 > L.m; }
+
 // Cluster size of the fused engine for a level (0: not used).
 static int engine_cluster(Ctx& c, const Level& L) {
   const int64_t lim = c.cfg.engine_max_n > 0 ? c.cfg.engine_max_n : (c.cfg.engine_max_n < 0 ? -1 : kEngMaxN);
+  if (engine_slower(L, c.cfg.engine_max_n)) return 0;
   if (!c.use_graphs || c.prof || L.n > lim || !engine_rows_fit(c, L)) return 0;
   int C = (L.n + 1023) / 1024;  // about one vertex per thread
   if (C < 1) C = 1;
@@ -4189,6 +4202,7 @@ static void refine_engine(Ctx& c, int lvl, int32_t rounds, int C, int64_t* J, in
 static bool engine_grid_ok(Ctx& c, const Level& L) {
   const int64_t lim =
       c.cfg.grid_engine_max_n > 0 ? c.cfg.grid_engine_max_n : (c.cfg.grid_engine_max_n < 0 ? -1 : (1 << 18));
+  if (engine_slower(L, c.cfg.grid_engine_max_n)) return false;
   if (!c.use_graphs || c.prof || L.n > lim || !engine_rows_fit(c, L)) return false;
   static std::atomic<int> cached[64];  // a property of the device: once per process
   if (c.eng_grid_blocks == 0) c.eng_grid_blocks = cached[c.dev & 63].load();
