@@ -15,7 +15,9 @@
 // Contraction (Section 2.1 semantics, replacing the CAS hashing of Alg. 3):
 // keys (M(u), M(v)) of the non-self-loop edges are radix-sorted, equal keys
 // are reduced by a prefix sum of the weights, and the coarse CSR rows follow
-// from the sorted unique keys, so adjacency order is deterministic.
+// from the sorted unique keys, so adjacency order is deterministic.  That is
+// the path of levels of at most kCtMinEntries entries (one CTA sorts them) and
+// of weights too wide for contract.cu, which takes the other levels.
 #include <algorithm>
 #include <atomic>
 #include <chrono>
@@ -1622,14 +1624,37 @@ void contract_level(Ctx& c, int lvl, int32_t nc, Level* spare) {
   const unsigned gv = grid_for(c, kThreads, F.n);
   if (!reuse_n) C.vw = c.mem.make<int32_t>((size_t)std::max(1, nc));
   GM_CUDA(cudaMemsetAsync(C.vw, 0, (size_t)std::max(1, nc) * sizeof(int32_t), c.st));
-  k_coarse_vw<<<gv, kThreads, 0, c.st>>>(F.n, F.M, F.vw, C.vw); count_launch();
   const int bits = bits_for(nc);  // ids < 2^bits - 1, so the all-ones key is free
+  const int wbits = bits_for(F.max_w);
+  const bool by_target = contract_fits(F, bits, wbits);
+  if (!by_target) {
+    k_coarse_vw<<<gv, kThreads, 0, c.st>>>(F.n, F.M, F.vw, C.vw); count_launch();
+  }
   int64_t* d_valid = c.counters + 7;
   GM_CUDA(cudaMemsetAsync(d_valid, 0, sizeof(int64_t), c.st));
   int64_t mc = 0;
   if (!reuse_n) C.xadj = c.mem.make<int64_t>((size_t)nc + 1);
   const int64_t old_m = reuse_n ? C.m : -1;
-  if (m > 0) {
+  auto entries = [&] {  // the coarse entry arrays, kept when their size is the same
+    if (old_m == mc) return;
+    if (C.adj) c.mem.put(C.adj);
+    if (C.adjw) c.mem.put(C.adjw);
+    drop_graph(C);
+    C.adj = c.mem.make<int32_t>((size_t)std::max<int64_t>(1, mc));
+    C.adjw = c.mem.make<int32_t>((size_t)std::max<int64_t>(1, mc));
+  };
+  c.prof_level = lvl;
+  if (by_target) {
+    cudaEvent_t ev = c.prof_begin();
+    const ContractSort s = contract_sort(c, F, nc, bits, wbits, C.vw);
+    // per entry: adjacency, weight and M 4 each, the word 8; then per pass the word read and written, and read
+    // again to count the next digit
+    const int64_t passes = (bits + 9) / 10;
+    c.prof_end(ev, PK_SORT, m * (20 + 16 * passes + 8 * (passes - 1)));
+    mc = s.mc;
+    entries();
+    contract_rows(c, s, nc, C.xadj, C.adj, C.adjw);
+  } else if (m > 0) {
     k_contract_keys<<<grid_for(c, kThreads, F.n), kThreads, 0, c.st>>>(view(F), F.M, bits, c.sort.key[0],
                                                                        c.sort.val[0], d_valid); count_launch();
     if (F.n_huge) {
@@ -1637,7 +1662,6 @@ void contract_level(Ctx& c, int lvl, int32_t nc, Level* spare) {
                             kThreads, 0, c.st>>>(view(F), hub_rows(F), F.M, bits, c.sort.key[0], c.sort.val[0],
                                                  d_valid); count_launch();
     }
-    c.prof_level = lvl;
     cudaEvent_t ev = c.prof_begin();
     const int cur = radix_sort_pairs(c.sort, m, d_valid, 2 * bits, c.st);  // the valid keys only
     // per 8-bit pass: keys read twice (histogram, scatter), key + value read and written once
@@ -1650,13 +1674,7 @@ void contract_level(Ctx& c, int lvl, int32_t nc, Level* spare) {
     scan(LoadValid32{sval, d_valid}, StoreExcl{c.P64}, m, nullptr, c.scan, c.st);
     // P64[valid] = total weight of the valid entries
     k_put_total<<<1, 1, 0, c.st>>>(c.scan.tile_sums + std::max<int64_t>(1, scan_tiles(m)), d_valid, c.P64); count_launch();
-    if (old_m != mc) {
-      if (C.adj) c.mem.put(C.adj);
-      if (C.adjw) c.mem.put(C.adjw);
-      drop_graph(C);
-      C.adj = c.mem.make<int32_t>((size_t)std::max<int64_t>(1, mc));
-      C.adjw = c.mem.make<int32_t>((size_t)std::max<int64_t>(1, mc));
-    }
+    entries();
     if (mc > 0)
       k_contract_fill<<<grid_for(c, kThreads, mc), kThreads, 0, c.st>>>(mc, ukey, c.P64b, c.P64, d_valid, bits, C.adj,
                                                                        C.adjw); count_launch();
@@ -1668,6 +1686,7 @@ void contract_level(Ctx& c, int lvl, int32_t nc, Level* spare) {
     GM_CUDA(cudaMemsetAsync(C.xadj, 0, ((size_t)nc + 1) * sizeof(int64_t), c.st));
   }
   C.m = mc;
+  C.max_w = 0;
   if (!reuse_n) C.pi = c.mem.make<int32_t>((size_t)std::max(1, nc));
   GM_CUDA(cudaMemsetAsync(C.pi, 0, (size_t)std::max(1, nc) * sizeof(int32_t), c.st));
   GM_CUDA(cudaGetLastError());

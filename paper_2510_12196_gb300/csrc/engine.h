@@ -115,6 +115,7 @@ struct Level {
   int64_t hub_chunk_cap = 0;
   int64_t n_hub_chunks = 0;
   int32_t max_vw = 0;
+  int32_t max_w = 0;  // largest edge weight (0: not known yet)
   // instantiated Alg. 6 graph of this level and what it was captured for
   cudaGraphExec_t gexec = nullptr;
   int32_t g_rounds = -2;
@@ -234,7 +235,7 @@ struct Ctx {
   RefineState* h_state = nullptr;  // pinned mirror
   int64_t* h_small = nullptr;      // pinned, a few values read back together
   void* h_tables = nullptr;        // pinned staging of small PE code tables
-  int64_t* d_stats = nullptr;      // device, per-level statistics
+  int64_t* d_stats = nullptr;      // device, per-level statistics (5 values)
   int32_t* trace_kind = nullptr;
   int64_t* trace_J = nullptr;
   int64_t* trace_maxw = nullptr;
@@ -352,6 +353,22 @@ inline void cap_streams(Ctx& c) {
 // initial.cu: breadth-first initial mapping of a large coarsest graph over the whole GPU; false when
 // its component labelling did not settle within its round limit (the caller then runs the one-CTA kernel)
 bool initial_map_large(Ctx& c);
+
+// contract.cu: contraction by one sort over the coarse targets
+constexpr int64_t kCtMinEntries = 4096;  // smaller levels: the single-CTA sort by (source, target)
+struct ContractSort {
+  const uint64_t* key = nullptr;  // sorted words (target, source, weight)
+  const int64_t* d_n = nullptr;   // their number (device)
+  int64_t mc = 0;                 // distinct (target, source): entries of the coarse graph
+  int64_t tiles = 0;
+  int bits = 0, wbits = 0;
+};
+// whether a level takes this path: target, source and weight share a 64-bit word
+bool contract_fits(const Level& F, int bits, int wbits);
+// sorts F's entries between different coarse vertices and adds the coarse vertex weights into vwc (zeroed)
+ContractSort contract_sort(Ctx& c, const Level& F, int32_t nc, int bits, int wbits, int32_t* vwc);
+// writes the coarse CSR (xadj nc + 1, adj and adjw s.mc entries)
+void contract_rows(Ctx& c, const ContractSort& s, int32_t nc, int64_t* xadj, int32_t* adj, int32_t* adjw);
 
 // match.cu
 int32_t match_level(Ctx& c, int lvl);  // two-hop matching of level lvl into its M; returns n_c

@@ -3785,7 +3785,7 @@ void refine_alloc(Ctx& c) {
   if (!c.h_small) c.h_small = static_cast<int64_t*>(pinned_get(8 * sizeof(int64_t)));
   c.gbar = c.mem.make<GridBar>(1);
   GM_CUDA(cudaMemsetAsync(c.gbar, 0, sizeof(GridBar), c.st));
-  c.d_stats = c.mem.make<int64_t>(4);
+  c.d_stats = c.mem.make<int64_t>(5);
   const size_t smem = conn_smem(c);
   if (smem > 48 * 1024) raise_smem((const void*)k_lp_gain_high, smem);
   static std::atomic<unsigned long long> resolve_done{0};  // one bit per device
@@ -4024,13 +4024,14 @@ static bool engine_rows_fit(const Ctx& c, const Level& L) {
 // most 4 %: 24-81 against 43-97; random geometric graph of degree 40, 90 %:
 // 134 against 104; R-MAT with 770 to 200 k vertices, 67-98 %: 370-1900
 // against 109-284.  Hence one entry in 16.
-// A limit set in the config (`asked`) is followed as it stands.
+// A limit set in the config (`asked`) is followed as it stands, and a server's
+// jobs keep the cluster engine, in which its batcher runs them together.
 static bool engine_slower(const Level& L, int32_t asked) { return asked == 0 && L.m_hi * 16 > L.m; }
 
 // Cluster size of the fused engine for a level (0: not used).
 static int engine_cluster(Ctx& c, const Level& L) {
   const int64_t lim = c.cfg.engine_max_n > 0 ? c.cfg.engine_max_n : (c.cfg.engine_max_n < 0 ? -1 : kEngMaxN);
-  if (engine_slower(L, c.cfg.engine_max_n)) return 0;
+  if (!c.sink && engine_slower(L, c.cfg.engine_max_n)) return 0;
   if (!c.use_graphs || c.prof || L.n > lim || !engine_rows_fit(c, L)) return 0;
   int C = (L.n + 1023) / 1024;  // about one vertex per thread
   if (C < 1) C = 1;
@@ -4355,6 +4356,13 @@ __global__ void k_level_stats(int32_t n, const int64_t* __restrict__ xadj, const
     if (mhuge) atomicAdd(&out[3], mhuge);
   }
 }
+__global__ void k_max_weight(int64_t m, const int32_t* __restrict__ w, int* out) {
+  int x = 0;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x)
+    x = max(x, w[i]);
+  x = __reduce_max_sync(0xffffffffu, x);
+  if ((threadIdx.x & 31) == 0 && x) atomicMax(out, x);
+}
 }  // namespace
 
 namespace {
@@ -4471,11 +4479,18 @@ void classify_with(Ctx& c, Level& L, int32_t mid_deg, int64_t split_deg) {
   const int64_t blocks = std::min<int64_t>(((int64_t)L.n + 255) / 256, (int64_t)c.num_sms * 8);
   k_level_stats<<<(unsigned)std::max<int64_t>(1, blocks), 256, 0, c.st>>>(L.n, L.xadj, L.vw, mid_deg, st);
   count_launch();
-  // count of high-degree vertices and the four statistics, one synchronisation
+  GM_CUDA(cudaMemsetAsync(c.d_stats + 4, 0, sizeof(int64_t), c.st));
+  const bool new_level = L.max_w == 0 && L.m > 0;  // the largest edge weight, once per level
+  if (new_level) {
+    k_max_weight<<<grid_for(c, 256 * 8, L.m), 256, 0, c.st>>>(L.m, L.adjw, reinterpret_cast<int*>(c.d_stats + 4));
+    count_launch();
+  }
+  // count of high-degree vertices and the statistics, one synchronisation
   GM_CUDA(cudaMemcpyAsync(c.h_small, c.scan.tile_sums + std::max<int64_t>(1, scan_tiles(L.n)), sizeof(int64_t),
                           cudaMemcpyDeviceToHost, c.st));
-  GM_CUDA(cudaMemcpyAsync(c.h_small + 1, st, 4 * sizeof(int64_t), cudaMemcpyDeviceToHost, c.st));
+  GM_CUDA(cudaMemcpyAsync(c.h_small + 1, st, 5 * sizeof(int64_t), cudaMemcpyDeviceToHost, c.st));
   GM_CUDA(cudaStreamSynchronize(c.st));
+  if (new_level) L.max_w = (int32_t)c.h_small[5];
   L.n_hi = (int32_t)(c.h_small[0] & 0xffffffffLL);
   L.n_huge = (int32_t)(c.h_small[0] >> 32);
   L.m_hi = c.h_small[1];
