@@ -1837,31 +1837,55 @@ __global__ void k_copy_count(const int64_t* src, int64_t* dst) { *dst = *src; }
 // buckets with C_b >= E not at all, and in the one bucket with
 // C_b < E < C_b + T_b a vertex moves iff the weight of the lower ids of that
 // bucket is < rem = E - C_b.  Only that bucket needs an id order.
-__global__ void __launch_bounds__(1024) k_reb_cut(const int64_t* __restrict__ W, int32_t kc, int64_t lmax,
-                                                  int64_t* tab, int32_t* bcut, int64_t* rem, int64_t* cnt,
-                                                  const RefineState* st) {
-  if (!kind_is(st, (1 << KIND_WEAK) | (1 << KIND_STRONG))) return;
-  for (int32_t A = threadIdx.x; A < kc; A += blockDim.x) {
-    if (W[A] <= lmax) continue;  // only overloaded blocks have eligible vertices
-    const int64_t E = W[A] - lmax;
-    int64_t cum = 0, r = 0;
-    int32_t cut = kBuckets;
-    for (int b = 0; b < kBuckets; b++) {
-      const int64_t t = tab[(int64_t)A * kBuckets + b];
-      tab[(int64_t)A * kBuckets + b] = 0;  // the table is zero between steps
-      if (cut == kBuckets) {
-        if (cum + t <= E) {
-          cum += t;
-        } else {
-          cut = b;
-          r = E - cum;
-        }
-      }
-    }
-    bcut[A] = cut;
-    rem[A] = r;
+// Inclusive prefix sum over the 32 lanes of a warp.
+__device__ __forceinline__ int64_t warp_incl_scan(int64_t x, int lane) {
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
   }
-  if (threadIdx.x == 0) cnt[CNT_ELIG] = 0;
+  return x;
+}
+
+// The first of 64 totals t whose inclusive prefix exceeds E (64: none), by one
+// warp; `before` receives the prefix before it.  The totals are put back to
+// zero when `zero` is set.
+__device__ __forceinline__ int warp_first_above(int64_t* t, bool zero, int64_t E, int lane, int64_t& before) {
+  static_assert(kBuckets == 64, "two totals per lane");
+  const int64_t x0 = t[lane], x1 = t[32 + lane];
+  if (zero) {
+    t[lane] = 0;
+    t[32 + lane] = 0;
+  }
+  const int64_t p0 = warp_incl_scan(x0, lane);
+  const int64_t p1 = warp_incl_scan(x1, lane) + __shfl_sync(0xffffffffu, p0, 31);
+  const unsigned m0 = __ballot_sync(0xffffffffu, p0 > E), m1 = __ballot_sync(0xffffffffu, p1 > E);
+  const int cut = m0 ? __ffs(m0) - 1 : (m1 ? 32 + __ffs(m1) - 1 : kBuckets);
+  const int pl = cut - 1;
+  const int64_t q0 = __shfl_sync(0xffffffffu, p0, pl < 0 ? 0 : (pl & 31));
+  const int64_t q1 = __shfl_sync(0xffffffffu, p1, pl < 32 ? 0 : (pl & 31));
+  before = pl < 0 ? 0 : (pl < 32 ? q0 : q1);
+  return cut;
+}
+
+// One warp per block (PE): at 1024 codes 3.4 us, where one thread per block
+// with 64 dependent steps took 21 us.
+constexpr int kCutThreads = 256;
+__global__ void __launch_bounds__(kCutThreads) k_reb_cut(const int64_t* __restrict__ W, int32_t kc, int64_t lmax,
+                                                         int64_t* tab, int32_t* bcut, int64_t* rem, int64_t* cnt,
+                                                         const RefineState* st) {
+  if (!kind_is(st, (1 << KIND_WEAK) | (1 << KIND_STRONG))) return;
+  if (blockIdx.x == 0 && threadIdx.x == 0) cnt[CNT_ELIG] = 0;
+  const int32_t A = (int32_t)(blockIdx.x * (kCutThreads / 32) + (threadIdx.x >> 5));
+  const int lane = threadIdx.x & 31;
+  if (A >= kc || W[A] <= lmax) return;  // only overloaded blocks have eligible vertices
+  const int64_t E = W[A] - lmax;
+  int64_t before;
+  const int cut = warp_first_above(tab + (int64_t)A * kBuckets, true, E, lane, before);  // the table is zero between steps
+  if (lane == 0) {
+    bcut[A] = cut;
+    rem[A] = cut < kBuckets ? E - before : 0;
+  }
 }
 
 // Buckets below the cut move, above it stay; the cut bucket's vertices go to
@@ -1943,26 +1967,57 @@ __global__ void __launch_bounds__(kSmallThreads) k_reb_resolve(const uint64_t* _
   }
 }
 
-// Larger cut-bucket lists: after a multi-CTA sort by (block, id).
-__global__ void k_heads_shift(const uint64_t* __restrict__ key, const int64_t* __restrict__ P,
-                              const int64_t* __restrict__ cnt, int shift, int64_t* headP) {
+// Larger cut-bucket lists, without sorting them: a block's vertices move while
+// the weight of the lower ids in the list is below its remainder, so all that
+// is wanted is the id where that weight reaches it.  It is found digit by
+// digit from the top (kCutDigit bits each): the weights of the list by (block,
+// digit) among the ids that share the digits found so far (k_cut_sums), then
+// per block the digit where the sum passes the remainder, which is lowered by
+// the weight of the digits below (k_cut_digit).  The totals use the (block,
+// bucket) table, which is zero between steps.  Nine small launches (25 us on a
+// 3D grid of 2^21 vertices, where the sort of the list by (block, id) and the
+// prefix over it took 100 us); the single-CTA sort (k_reb_resolve) stays for
+// lists of at most 4096.
+constexpr int kCutDigit = 6;
+static_assert((1 << kCutDigit) == kBuckets, "the digit totals use the bucket table");
+__global__ void k_cut_sums(const uint64_t* __restrict__ key, const int32_t* __restrict__ val,
+                           const int64_t* __restrict__ cnt, int idbits, int shift, int first,
+                           const int64_t* __restrict__ prefix, const int32_t* __restrict__ vw, int64_t* tab) {
   const int64_t n = cnt[CNT_ELIG];
   if (n <= kSmallSort) return;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const uint64_t grp = key[i] >> shift;
-    if (i == 0 || (key[i - 1] >> shift) != grp) headP[grp] = P[i];
+    const int32_t A = (int32_t)(key[i] >> idbits), v = val[i];
+    if (!first && (v >> (shift + kCutDigit)) != prefix[A]) continue;
+    atomicAdd((unsigned long long*)&tab[(int64_t)A * kBuckets + ((v >> shift) & (kBuckets - 1))],
+              (unsigned long long)(int64_t)vw[v]);
+  }
+}
+__global__ void __launch_bounds__(kCutThreads) k_cut_digit(const int64_t* __restrict__ W, int32_t kc, int64_t lmax,
+                                                           const int64_t* __restrict__ cnt, int first, int64_t* tab,
+                                                           int64_t* rem, int64_t* prefix) {
+  if (cnt[CNT_ELIG] <= kSmallSort) return;
+  const int32_t A = (int32_t)(blockIdx.x * (kCutThreads / 32) + (threadIdx.x >> 5));
+  const int lane = threadIdx.x & 31;
+  if (A >= kc || W[A] <= lmax) return;
+  const int64_t E = rem[A];
+  if (first && E <= 0) return;  // no vertex of the block is in the list (later digits may start at 0)
+  int64_t before;
+  const int d = warp_first_above(tab + (int64_t)A * kBuckets, true, E, lane, before);
+  if (lane == 0) {  // (the list's weight of the block exceeds its remainder: d is a digit)
+    prefix[A] = (first ? 0 : prefix[A] << kCutDigit) + d;
+    rem[A] = E - before;
   }
 }
 __global__ void k_reb_mark_cut(const uint64_t* __restrict__ key, const int32_t* __restrict__ val,
-                               const int64_t* __restrict__ P, const int64_t* __restrict__ headP,
-                               const int64_t* __restrict__ cnt, int shift, const int64_t* __restrict__ rem,
-                               uint8_t* sel, unsigned long long* kcount, unsigned long long body) {
+                               const int64_t* __restrict__ prefix, const int64_t* __restrict__ cnt, int idbits,
+                               const int64_t* __restrict__ rem, uint8_t* sel, unsigned long long* kcount,
+                               unsigned long long body) {
   const int64_t n = cnt[CNT_ELIG];
   if (kcount && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(kcount, body);
   if (n <= kSmallSort) return;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t A = (int32_t)(key[i] >> shift);
-    sel[val[i]] = (P[i] - headP[A] < rem[A]) ? 1 : 0;
+    const int32_t A = (int32_t)(key[i] >> idbits), v = val[i];
+    sel[v] = (v < prefix[A] || (v == prefix[A] && rem[A] > 0)) ? 1 : 0;
   }
 }
 
@@ -2421,7 +2476,9 @@ void launch_rebalance(Ctx& c, int lvl, bool prep_done = false) {
       count_launch();
     }
   }
-  k_reb_cut<<<1, 1024, 0, c.st>>>(c.W, c.topo.kc, c.lmax, c.tab, c.bcut, c.rem, c.counters, c.state); count_launch();
+  const unsigned gcut = (unsigned)((c.topo.kc + kCutThreads / 32 - 1) / (kCutThreads / 32));
+  k_reb_cut<<<gcut, kCutThreads, 0, c.st>>>(c.W, c.topo.kc, c.lmax, c.tab, c.bcut, c.rem, c.counters, c.state);
+  count_launch();
   const int idbits = bits_for_n(n);
   const int bits = c.topo.code_bits + idbits;
   const unsigned g = grid_for(c, kThreads, n);
@@ -2431,17 +2488,18 @@ void launch_rebalance(Ctx& c, int lvl, bool prep_done = false) {
   k_reb_resolve<<<1, kSmallThreads, small_sort_smem(), c.st>>>(c.sort.key[0], c.sort.val[0], c.counters, bits, idbits,
                                                                L.vw, c.rem, c.headP, selected, c.state, h,
                                                                c.cap.on() ? 1 : 0); count_launch();
-  int64_t* d_list = c.counters + CNT_ELIG;
   auto big = [&](cudaStream_t bs, unsigned long long* kcount, long long* body) {
-    cudaStream_t saved = c.st;
-    c.st = bs;
-    const int cur = radix_sort_pairs(c.sort, n, d_list, bits, bs);
-    scan(LoadSortedWeight{c.sort.val[cur], L.vw}, StoreExcl{c.P64}, n, d_list, c.scan, bs);
-    k_heads_shift<<<g, kThreads, 0, bs>>>(c.sort.key[cur], c.P64, c.counters, idbits, c.headP); count_launch();
+    const int digits = std::max(1, (idbits + kCutDigit - 1) / kCutDigit);
+    for (int d = digits - 1; d >= 0; d--) {
+      const int first = d == digits - 1;
+      k_cut_sums<<<g, kThreads, 0, bs>>>(c.sort.key[0], c.sort.val[0], c.counters, idbits, d * kCutDigit, first,
+                                         c.headP, L.vw, c.tab); count_launch();
+      k_cut_digit<<<gcut, kCutThreads, 0, bs>>>(c.W, c.topo.kc, c.lmax, c.counters, first, c.tab, c.rem, c.headP);
+      count_launch();
+    }
     const unsigned long long bk = body ? (unsigned long long)(*body + 1) : 0ULL;
-    k_reb_mark_cut<<<g, kThreads, 0, bs>>>(c.sort.key[cur], c.sort.val[cur], c.P64, c.headP, c.counters, idbits, c.rem,
-                                          selected, kcount, bk); count_launch();
-    c.st = saved;
+    k_reb_mark_cut<<<g, kThreads, 0, bs>>>(c.sort.key[0], c.sort.val[0], c.headP, c.counters, idbits, c.rem, selected,
+                                          kcount, bk); count_launch();
   };
   if (c.cap.on()) {
     long long body = 0;
@@ -2622,6 +2680,7 @@ struct EngSmem {
   int64_t smax[32];
   int64_t hb[32];  // per-warp best scores of a CTA-wide row decision
   int32_t hc[32];  // and their codes
+  int32_t count;   // a list being built by the CTA
 };
 
 // Stable LSD radix sort (8-bit digits) of n pairs by one CTA through global
@@ -2967,16 +3026,6 @@ __device__ __forceinline__ void reb_tile_queue(unsigned work, const TileLane& tl
   }
 }
 
-// Inclusive prefix sum over the 32 lanes of a warp.
-__device__ __forceinline__ int64_t warp_incl_scan(int64_t x, int lane) {
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
-  }
-  return x;
-}
-
 // Exact change of J by the moves of an LP or weak step, added to the J
 // accumulator (the mapping still holds the old values): the movers of each
 // warp tile are served four at a time by 8-lane sub-warps, the movers with
@@ -3014,11 +3063,13 @@ __device__ void eng_delta(const EngineJob& J, const Mv& mv, EngSmem& S, const En
 
 // Shared-memory layout of the rebalancing steps in the engine's dynamic
 // shared memory: the cut bucket and remainder of every block (code spaces up
-// to kEngCutSmem) and the short-list resolution behind them; the sorts of the
+// to kEngCutSmem), the short-list resolution behind them and the list of the
+// overloaded blocks; the sorts of the
 // first CTA reuse the area once the cuts are no longer read from it.
 constexpr int kEngCutSmem = 4096;
-static_assert(kEngCutSmem * 12 + kEngThreads * (8 + 8 + 4 + 8 + 1) <= 2 * kSmallSort * 12,
-              "cut tables and short-list resolution fit in the engine's smallest dynamic shared memory");
+constexpr int kEngOverAt = kEngCutSmem * 12 + kEngThreads * (8 + 8 + 4 + 8 + 1);  // list of the overloaded blocks
+static_assert(kEngOverAt + kEngCutSmem * 4 <= 2 * kSmallSort * 12,
+              "cut tables, short-list resolution and block list fit in the engine's smallest dynamic shared memory");
 
 // weak step, short list: movers are the selected vertices below the cut
 // bucket and those of the cut bucket that the CTA's own resolution selected
@@ -3148,6 +3199,7 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
         control_step(s, mx, Jv, J.ctl, phase, 0, 0);
         *J.Jacc = next_j_base(s, Jv);
         J.cnt[CNT_ELIG] = 0;  // the cut-bucket list of a rebalancing step
+        J.cnt[CNT_SEL] = 0;   // and the movers of a strong one
       }
       __syncthreads();
       // a rebalancing step: its threshold sigma and destination list U now
@@ -3422,43 +3474,38 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
     // the cut bucket of each overloaded block A: the first bucket whose
     // inclusive prefix of eligible weight exceeds W(A) - L_max (one warp per
     // block, buckets lane and 32 + lane)
-    static_assert(kBuckets == 64, "two buckets per lane");
     const int idbits = bits_for_n(n);
     const int32_t kc = J.topo.kc;
     auto warp_cut = [&](int64_t A, bool zero, int32_t* bcut_out, int64_t* rem_out) {
-      const int64_t WA = J.W[A];
-      if (WA <= J.lmax) return;
-      const int64_t E = WA - J.lmax;
-      int64_t* row = J.tab + A * kBuckets;
-      const int64_t x0 = row[lane], x1 = row[32 + lane];
-      if (zero) {
-        row[lane] = 0;
-        row[32 + lane] = 0;
-      }
-      const int64_t p0 = warp_incl_scan(x0, lane);
-      const int64_t p1 = warp_incl_scan(x1, lane) + __shfl_sync(0xffffffffu, p0, 31);
-      const unsigned m0 = __ballot_sync(0xffffffffu, p0 > E), m1 = __ballot_sync(0xffffffffu, p1 > E);
-      const int cut = m0 ? __ffs(m0) - 1 : (m1 ? 32 + __ffs(m1) - 1 : kBuckets);
-      const int pl = cut - 1;  // exclusive prefix of the cut bucket
-      const int64_t q0 = __shfl_sync(0xffffffffu, p0, pl < 0 ? 0 : (pl & 31));
-      const int64_t q1 = __shfl_sync(0xffffffffu, p1, pl < 32 ? 0 : (pl & 31));
-      const int64_t excl = pl < 0 ? 0 : (pl < 32 ? q0 : q1);
+      const int64_t E = J.W[A] - J.lmax;
+      int64_t before;
+      const int cut = warp_first_above(J.tab + A * kBuckets, zero, E, lane, before);
       if (lane == 0) {
         bcut_out[A] = cut;
-        rem_out[A] = cut < kBuckets ? E - excl : 0;
+        rem_out[A] = cut < kBuckets ? E - before : 0;
       }
     };
-    // With a small code space every CTA computes the cuts itself into shared
-    // memory (no barrier before the classification; the bucket totals are
-    // cleared after the next barrier); else one warp per block, cluster-wide.
+    // With a small code space every CTA lists the overloaded blocks and
+    // computes their cuts itself into shared memory (no barrier before the
+    // classification; the bucket totals are cleared after the next barrier);
+    // else one warp per block, cluster-wide.
     const bool cut_local = kc <= kEngCutSmem;
     int64_t* s_rem = reinterpret_cast<int64_t*>(dyn);
     int32_t* s_bcut = reinterpret_cast<int32_t*>(s_rem + kEngCutSmem);
+    int32_t* s_over = reinterpret_cast<int32_t*>(reinterpret_cast<char*>(dyn) + kEngOverAt);
+    int n_over = 0;
     if (cut_local) {
-      for (int64_t A = threadIdx.x >> 5; A < kc; A += blockDim.x >> 5) warp_cut(A, false, s_bcut, s_rem);
+      if (threadIdx.x == 0) S.count = 0;
+      __syncthreads();
+      for (int32_t A = threadIdx.x; A < kc; A += blockDim.x)
+        if (J.W[A] > J.lmax) s_over[atomicAdd(&S.count, 1)] = A;
+      __syncthreads();
+      n_over = S.count;
+      for (int i = threadIdx.x >> 5; i < n_over; i += blockDim.x >> 5) warp_cut(s_over[i], false, s_bcut, s_rem);
       __syncthreads();
     } else {
-      for (int64_t A = eg.gw; A < kc; A += eg.GW) warp_cut(A, true, J.bcut, J.rem);
+      for (int64_t A = eg.gw; A < kc; A += eg.GW)
+        if (J.W[A] > J.lmax) warp_cut(A, true, J.bcut, J.rem);
       sy.sync();
     }
     const int32_t* bcut = cut_local ? s_bcut : J.bcut;
@@ -3486,7 +3533,8 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
     }
     sy.sync();
     if (cut_local && lead)  // the bucket totals for the next step
-      for (int64_t i = threadIdx.x; i < (int64_t)kc * kBuckets; i += blockDim.x) J.tab[i] = 0;
+      for (int i = threadIdx.x; i < n_over * kBuckets; i += blockDim.x)
+        J.tab[(int64_t)s_over[i / kBuckets] * kBuckets + i % kBuckets] = 0;
     const int ln = (int)*(volatile int64_t*)&J.cnt[CNT_ELIG];
     if (!strong && cut_local && ln <= (int)blockDim.x) {
       // every CTA orders the short cut-bucket list by (block, id) itself and
@@ -3510,7 +3558,7 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
     if (lead) {  // the cut-bucket list by (block, id), per-block prefix
       if (ln > 0) {
         if (cut_local) {  // the sort below reuses the shared memory of the cuts
-          for (int64_t A = threadIdx.x; A < kc; A += blockDim.x) J.rem[A] = s_rem[A];
+          for (int i = threadIdx.x; i < n_over; i += blockDim.x) J.rem[s_over[i]] = s_rem[s_over[i]];
           __syncthreads();
         }
         rem = J.rem;
@@ -3546,45 +3594,88 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
       sy.sync();
       continue;
     }
-    if (lead) {  // strong: destinations in (bucket, id) order, acceptance, water-filling
-      const int64_t ns = cta_scan(
-          n, [&](int64_t v) { return (int64_t)((J.elig[v] && J.sel[v]) ? 1 : 0); },
-          [&](int64_t v, int64_t e, int64_t x) {
-            if (x) {
-              J.key0[e] = ((uint64_t)(uint32_t)J.dest[v] << kBucketBits) | J.bkt[v];
-              J.val0[e] = (int32_t)v;
-            }
-          },
-          S.sm);
-      __syncthreads();
+    // strong: the movers, listed by all CTAs in any order under the complete
+    // key (destination, bucket, id); the first CTA orders them, accepts and
+    // lays out the rejected ones (its own scans of all n vertices for the two
+    // lists were the longest phase of an iteration on the larger levels: 97 k
+    // vertices, 1024 codes, 13 of 62 iterations strong: 129 us per iteration
+    // with them, 73 us so)
+    for (int64_t v = gt; v < n; v += GT) {
+      if (!J.elig[v] || !J.sel[v]) continue;
+      const unsigned m = __activemask();
+      const int leader = __ffs(m) - 1;
+      unsigned long long at = 0;
+      if (lane == leader) at = atomicAdd((unsigned long long*)&J.cnt[CNT_SEL], (unsigned long long)__popc(m));
+      at = __shfl_sync(m, at, leader) + __popc(m & ((1u << lane) - 1u));
+      J.key0[at] = ((((uint64_t)(uint32_t)J.dest[v]) << kBucketBits | J.bkt[v]) << idbits) | (uint64_t)v;
+      J.val0[at] = (int32_t)v;
+    }
+    sy.sync();
+    if (lead) {  // destinations in (bucket, id) order, acceptance, water-filling
+      int64_t ns = *(volatile int64_t*)&J.cnt[CNT_SEL];
+      const bool listed = ns <= kSmallSort;  // longer lists: compacted in id order, then sorted by the short key
+      if (!listed) {
+        ns = cta_scan(
+            n, [&](int64_t v) { return (int64_t)((J.elig[v] && J.sel[v]) ? 1 : 0); },
+            [&](int64_t v, int64_t e, int64_t x) {
+              if (x) {
+                J.key0[e] = ((uint64_t)(uint32_t)J.dest[v] << kBucketBits) | J.bkt[v];
+                J.val0[e] = (int32_t)v;
+              }
+            },
+            S.sm);
+        __syncthreads();
+      }
+      const int dshift = listed ? idbits + kBucketBits : kBucketBits;  // key bits below the destination
       const uint64_t* K = J.key0;
       const int32_t* V = J.val0;
-      if (ns) eng_sort(J, S, dyn, (int)ns, J.topo.code_bits + kBucketBits, K, V);
+      if (ns) eng_sort(J, S, dyn, (int)ns, J.topo.code_bits + dshift, K, V);
       cta_scan(
           ns, [&](int64_t i) { return (int64_t)g.vw[V[i]]; },
           [&](int64_t i, int64_t e, int64_t) {
             J.P[i] = e;
-            if (i == 0 || (K[i] >> kBucketBits) != (K[i - 1] >> kBucketBits)) J.headP[K[i] >> kBucketBits] = e;
+            if (i == 0 || (K[i] >> dshift) != (K[i - 1] >> dshift)) J.headP[K[i] >> dshift] = e;
           },
           S.sm);
+      if (threadIdx.x == 0) S.count = 0;
       __syncthreads();
       for (int64_t i = threadIdx.x; i < ns; i += blockDim.x) {
-        const int32_t d = (int32_t)(K[i] >> kBucketBits);
+        const int32_t d = (int32_t)(K[i] >> dshift);
         const int32_t v = V[i];
         const int64_t inc = J.P[i] + g.vw[v] - J.headP[d];
         const bool ok = J.W[d] + inc <= J.lmax;
         J.acc[v] = ok ? 1 : 0;
         if (ok) atomicAdd((unsigned long long*)&J.accepted[d], (unsigned long long)(int64_t)g.vw[v]);
+        if (listed) {
+          J.val1[i] = v;  // (K and V lie in the shared memory that the next sort uses)
+          if (!ok) {
+            const int j = atomicAdd(&S.count, 1);
+            J.key0[j] = (uint64_t)v;
+            J.val0[j] = v;
+          }
+        }
       }
       __syncthreads();
-      cta_scan(
-          n,
-          [&](int64_t v) { return (J.elig[v] && J.sel[v] && !J.acc[v]) ? (int64_t)g.vw[v] : (int64_t)0; },
-          [&](int64_t v, int64_t e, int64_t x) {
-            if (x) J.sarr[v] = e;
-          },
-          S.sm);
-      const int32_t kc = J.topo.kc;
+      if (listed) {
+        V = J.val1;
+        const int nr = S.count;
+        const uint64_t* KR;
+        const int32_t* VR;
+        if (nr) {
+          eng_sort(J, S, dyn, nr, idbits, KR, VR);
+          cta_scan(
+              nr, [&](int64_t i) { return (int64_t)g.vw[VR[i]]; },
+              [&](int64_t i, int64_t e, int64_t) { J.sarr[VR[i]] = e; }, S.sm);
+        }
+      } else {
+        cta_scan(
+            n,
+            [&](int64_t v) { return (J.elig[v] && J.sel[v] && !J.acc[v]) ? (int64_t)g.vw[v] : (int64_t)0; },
+            [&](int64_t v, int64_t e, int64_t x) {
+              if (x) J.sarr[v] = e;
+            },
+            S.sm);
+      }
       const int64_t tot = cta_scan(
           kc,
           [&](int64_t b) {
@@ -3603,7 +3694,7 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
         const int64_t c = g.vw[v];
         int32_t q = -1;
         if (J.acc[v]) {
-          q = (int32_t)(K[i] >> kBucketBits);
+          q = J.dest[v];
         } else {
           const int64_t sv = J.sarr[v];
           int32_t lo = 0, hi = kc + 1;
