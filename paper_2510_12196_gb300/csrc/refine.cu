@@ -1229,7 +1229,8 @@ __device__ void reb_prep_body(const RebPrepArgs& p, bool strong) {
     if (ok) p.U[carry + e] = b;
     carry += tot;
   }
-  for (int32_t b = threadIdx.x; b < p.topo.kc; b += blockDim.x) p.accepted[b] = 0;
+  if (p.accepted)
+    for (int32_t b = threadIdx.x; b < p.topo.kc; b += blockDim.x) p.accepted[b] = 0;
   if (threadIdx.x == 0) {
     p.cnt[CNT_NU] = carry;
     p.cnt[CNT_SIGMA] = sigma;
@@ -2539,6 +2540,7 @@ static_assert(kEngThreads == kSmallThreads, "the engine's CTA sorts with the sin
 struct EngineJob {
   GraphView g;
   int32_t* pi;
+  int32_t* pi2;  // scratch: the mapping after a step that moves vertices while others still read the old one
   int32_t* pp;
   int64_t* gain;
   uint8_t* inx;
@@ -2564,7 +2566,7 @@ struct EngineJob {
   uint64_t* key1;
   int32_t* val1;
   int64_t* cnt;
-  int64_t* Jacc;
+  int64_t* Jacc;  // [2], used in turn
   RefineState* s;
   const int32_t* pe_of_code;
   Topo topo;
@@ -2670,6 +2672,7 @@ __device__ int64_t cta_scan(int64_t n, F f, O out, int64_t* sm) {
   return carry;
 }
 
+constexpr int kEngListPes = 1024;
 struct EngSmem {
   int32_t hist[256];
   int32_t ctot[256];
@@ -2681,6 +2684,9 @@ struct EngSmem {
   int64_t hb[32];  // per-warp best scores of a CTA-wide row decision
   int32_t hc[32];  // and their codes
   int32_t count;   // a list being built by the CTA
+  RefineState st;  // Alg. 6 state, the same in every CTA
+  int64_t cnt[CNT_N];  // sigma and the number of destinations of a rebalancing step
+  int32_t U[kEngListPes];  // and the destinations (code spaces up to kEngListPes)
 };
 
 // Stable LSD radix sort (8-bit digits) of n pairs by one CTA through global
@@ -2795,15 +2801,15 @@ __device__ void eng_sort(const EngineJob& J, EngSmem& S, int32_t* dyn, int n, in
 // Alg. 5 destination of one vertex (thread level): edge-cut gain, lowest id
 // on ties, the random-block fallback; returns false if the vertex cannot move.
 template <bool kJ>
-__device__ bool eng_reb_select(const EngineJob& J, int32_t v, int64_t sigma, int64_t nU, int32_t t,
-                               const int32_t* sdist, int32_t& dst, int32_t& bucket) {
+__device__ bool eng_reb_select(const EngineJob& J, const int32_t* pi, const int32_t* U, int32_t v, int64_t sigma,
+                               int64_t nU, int32_t t, const int32_t* sdist, int32_t& dst, int32_t& bucket) {
   const GraphView& g = J.g;
-  const int32_t A = J.pi[v];
+  const int32_t A = pi[v];
   const int64_t WA = J.W[A];
   if (WA <= J.lmax) return false;
   if (2 * (int64_t)J.k * g.vw[v] > 3 * ((int64_t)J.k * WA - J.cV)) return false;
   const int64_t b = g.xadj[v], e = g.xadj[v + 1];
-  const PlainRow row{g.adj + b, g.adjw + b, J.pi};
+  const PlainRow row{g.adj + b, g.adjw + b, pi};
   const int deg = (int)(e - b);
   // score: conn(v, q), or -T(q) for the J gains (kJ)
   using Score = typename std::conditional<kJ, int64_t, int32_t>::type;
@@ -2812,7 +2818,7 @@ __device__ bool eng_reb_select(const EngineJob& J, int32_t v, int64_t sigma, int
   int32_t bc = INT32_MAX;
   bool found = false;
   for (int64_t x = b; x < e; x++) {
-    const int32_t c = J.pi[g.adj[x]];
+    const int32_t c = pi[g.adj[x]];
     if (c == A) {
       if constexpr (!kJ) connA += g.adjw[x];
       continue;
@@ -2820,7 +2826,7 @@ __device__ bool eng_reb_select(const EngineJob& J, int32_t v, int64_t sigma, int
     if (J.W[c] > sigma) continue;
     bool seen = false;
     for (int64_t y = b; y < x; y++)
-      if (J.pi[g.adj[y]] == c) {
+      if (pi[g.adj[y]] == c) {
         seen = true;
         break;
       }
@@ -2829,7 +2835,7 @@ __device__ bool eng_reb_select(const EngineJob& J, int32_t v, int64_t sigma, int
     if constexpr (kJ) {
       cc = -row_cost(row, deg, sdist, c);
     } else {
-      for (int64_t y = x; y < e; y++) cc += (J.pi[g.adj[y]] == c) ? g.adjw[y] : 0;
+      for (int64_t y = x; y < e; y++) cc += (pi[g.adj[y]] == c) ? g.adjw[y] : 0;
     }
     if (!found || cc > bconn || (cc == bconn && c < bc)) {
       bconn = cc;
@@ -2841,7 +2847,7 @@ __device__ bool eng_reb_select(const EngineJob& J, int32_t v, int64_t sigma, int
   if (found) {
     gcut = (int64_t)bconn - connA;
   } else if (nU > 0) {
-    bc = J.U[h_rebalance(J.seed, J.level, t, v) % (uint64_t)nU];
+    bc = U[h_rebalance(J.seed, J.level, t, v) % (uint64_t)nU];
     int64_t sr = 0;  // the drawn block is not a neighbour
     if constexpr (kJ) sr = -row_cost(row, deg, sdist, bc);
     gcut = sr - connA;
@@ -2888,11 +2894,11 @@ __device__ __forceinline__ void eng_heavy_rows(const EngineJob& J, const EngGeom
 // zeroed first): conn per PE code, and with `groups` the level group sums
 // (the layout of GroupLayout).  The mapping is read through plain loads.
 // All threads of the CTA call it; ends with a barrier.
-__device__ __forceinline__ void eng_row_table(const EngineJob& J, int64_t b, int64_t e, int32_t* tab, int32_t total,
-                                              bool groups) {
+__device__ __forceinline__ void eng_row_table(const EngineJob& J, const int32_t* pi, int64_t b, int64_t e,
+                                              int32_t* tab, int32_t total, bool groups) {
   for (int32_t i = threadIdx.x; i < total; i += blockDim.x) tab[i] = 0;
   __syncthreads();
-  for (int64_t x = b + threadIdx.x; x < e; x += blockDim.x) atomicAdd(&tab[J.pi[J.g.adj[x]]], J.g.adjw[x]);
+  for (int64_t x = b + threadIdx.x; x < e; x += blockDim.x) atomicAdd(&tab[pi[J.g.adj[x]]], J.g.adjw[x]);
   __syncthreads();
   if (groups) conn_groups(J.topo, J.gl, tab);
 }
@@ -2905,15 +2911,15 @@ struct PlainGather {  // neighbour PEs through plain loads (the mapping changes 
 // Stages one tile of neighbour PEs and returns T(P(v)) = sum_j w_j D(P(v), c_j)
 // of the lane's vertex (0 for a row of more than kEngLaneDeg entries).
 template <int kTE>
-__device__ __forceinline__ TileLane eng_stage(const EngineJob& J, const TileGraph& tg, int64_t tile, int lane,
-                                              int32_t* sc, int32_t* sw, const int32_t* sdist, int64_t& Tp) {
-  const TileLane t = stage_tile<kTE>(tg, tile * kTileV, lane, sc, sw, PlainGather{J.pi});
+__device__ __forceinline__ TileLane eng_stage(const EngineJob& J, const int32_t* pi, const TileGraph& tg,
+                                              int64_t tile, int lane, int32_t* sc, int32_t* sw, const int32_t* sdist, int64_t& Tp) {
+  const TileLane t = stage_tile<kTE>(tg, tile * kTileV, lane, sc, sw, PlainGather{pi});
   Tp = 0;
   if (t.v < tg.n && !eng_heavy(J, t.e - t.b)) {
     const int deg = (int)(t.e - t.b);
-    const int32_t p = J.pi[t.v];
+    const int32_t p = pi[t.v];
     if (t.staged) Tp = row_cost(StagedRow{sc + (t.b - t.E0), sw + (t.b - t.E0)}, deg, sdist, p);
-    else Tp = row_cost(PlainRow{tg.adj + t.b, tg.adjw + t.b, J.pi}, deg, sdist, p);
+    else Tp = row_cost(PlainRow{tg.adj + t.b, tg.adjw + t.b, pi}, deg, sdist, p);
   }
   return t;
 }
@@ -3026,39 +3032,56 @@ __device__ __forceinline__ void reb_tile_queue(unsigned work, const TileLane& tl
   }
 }
 
-// Exact change of J by the moves of an LP or weak step, added to the J
-// accumulator (the mapping still holds the old values): the movers of each
-// warp tile are served four at a time by 8-lane sub-warps, the movers with
-// more than kEngLaneDeg entries by whole CTAs.
+// The moves of an LP or weak step and the exact change of J by them, in one
+// phase: the new mapping goes to `pn` (every vertex), so that the rows still
+// see the old one in `pi`.  The movers of each warp tile are served four at a
+// time by 8-lane sub-warps, the movers with more than kEngLaneDeg entries by
+// whole CTAs.
 template <class Mv>
-__device__ void eng_delta(const EngineJob& J, const Mv& mv, EngSmem& S, const EngGeom& eg, int64_t ntiles) {
+__device__ void eng_move(const EngineJob& J, const Mv& mv, const int32_t* pi, int32_t* pn, int64_t* Jacc, EngSmem& S,
+                         const EngGeom& eg, int64_t ntiles) {
   const GraphView& g = J.g;
   const int lane = eg.lane, sub = lane >> 3, sl = lane & 7;
   int64_t acc = 0;
   for (int64_t tile = eg.gw; tile < ntiles; tile += eg.GW) {
     const int64_t v = tile * kTileV + lane;
-    const unsigned work =
-        __ballot_sync(0xffffffffu, v < g.n && mv.moved(v) && !eng_heavy_row(J, v));
+    int32_t ol = 0, nl = 0;
+    int64_t bl = 0, el = 0;
+    bool move = false;
+    if (v < g.n) {
+      ol = nl = pi[v];
+      move = mv.moved(v);
+      if (move) {
+        nl = mv.target(v);
+        bl = g.xadj[v];
+        el = g.xadj[v + 1];
+        const int64_t c = g.vw[v];
+        atomicAdd((unsigned long long*)&J.W[ol], (unsigned long long)(-c));
+        atomicAdd((unsigned long long*)&J.W[nl], (unsigned long long)c);
+      }
+      pn[v] = nl;
+    }
+    const unsigned work = __ballot_sync(0xffffffffu, move && !eng_heavy(J, el - bl));
     const int rounds = (__popc(work) + 3) / 4;
     for (int r = 0; r < rounds; r++) {
       const int src = tile_worker(work, r, sub);
+      const int s2 = src < 0 ? 0 : src;
+      const int32_t ov = __shfl_sync(0xffffffffu, ol, s2), nv = __shfl_sync(0xffffffffu, nl, s2);
+      const int64_t xb = __shfl_sync(0xffffffffu, bl, s2), xe = __shfl_sync(0xffffffffu, el, s2);
       if (src < 0) continue;
-      const int64_t vv = tile * kTileV + src;
-      const int32_t ov = J.pi[vv], nv = mv.target(vv);
-      const int64_t xe = g.xadj[vv + 1];
-      for (int64_t x = g.xadj[vv] + sl; x < xe; x += kSubWarp)
-        acc += delta_entry(mv, J.pi, S.sdist, ov, nv, g.adj[x], g.adjw[x]);
+      for (int64_t x = xb + sl; x < xe; x += kSubWarp)
+        acc += delta_entry(mv, pi, S.sdist, ov, nv, g.adj[x], g.adjw[x]);
     }
     __syncwarp();
   }
   eng_heavy_rows(J, eg, [&](int32_t v, int64_t b, int64_t e) {
     if (!mv.moved(v)) return;
-    const int32_t ov = J.pi[v], nv = mv.target(v);
+    const int32_t ov = pi[v], nv = mv.target(v);
     for (int64_t x = b + threadIdx.x; x < e; x += blockDim.x)
-      acc += delta_entry(mv, J.pi, S.sdist, ov, nv, g.adj[x], g.adjw[x]);
+      acc += delta_entry(mv, pi, S.sdist, ov, nv, g.adj[x], g.adjw[x]);
   });
   acc = block_sum(acc, S.sm);
-  if (threadIdx.x == 0 && acc) atomicAdd((unsigned long long*)J.Jacc, (unsigned long long)acc);
+  if (threadIdx.x == 0 && acc) atomicAdd((unsigned long long*)Jacc, (unsigned long long)acc);
 }
 
 // Shared-memory layout of the rebalancing steps in the engine's dynamic
@@ -3131,6 +3154,17 @@ __device__ uint8_t* eng_resolve_local(const EngineJob& J, EngSmem& S, int32_t* a
 // Alg. 6 on one job by the calling cluster (all its threads call it).
 // kVar: the job may use the refinement variants (relaxed filter, J gains in
 // rebalancing); the plain instantiation leaves their code out.
+//
+// What bounds a small level is the chain of phases, each a barrier and a few
+// L2 round trips, so every phase that can do without a barrier does: every
+// CTA takes the Alg. 6 decision itself (its own copy of the state, from the
+// same W and J), prepares a rebalancing step itself, and the moves are made in
+// the phase that sums their change of J, into a second mapping.  An LP step
+// has three barriers (gains | recomputed gains | moves) and a weak one three
+// (destinations | cuts and lists | moves); with the decision and the moves in
+// phases of their own they had six and five.  Per iteration, before and now
+// (us): 4 k vertices on one cluster 23 -> 17, 17 k 31 -> 24, 76 k over all SMs
+// 38 -> 27, 97 k with 1024 PEs 73 -> 63.
 template <int kTE, bool kVar, class Sync>
 __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int32_t* sc, int32_t* sw,
                                const EngGeom& eg, const Sync& sy) {
@@ -3144,7 +3178,14 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
   // with at most one tile per warp, the entries staged for J stay valid for
   // the gain pass of the same iteration (the mapping does not change between)
   const bool single = ntiles <= eg.GW;
-  RefineState* s = J.s;
+  RefineState* s = &S.st;
+  int32_t* pi = J.pi;   // the mapping
+  int32_t* pn = J.pi2;  // where the next LP or weak step puts it
+  int par = 0;          // the J accumulator in use
+  // with a larger code space, or rows for whole CTAs (which take the lists from
+  // global memory), the first CTA prepares the rebalancing steps
+  const bool own_prep = J.topo.kc <= kEngListPes && !J.has_heavy;
+  const int32_t* U = own_prep ? S.U : J.U;
   __syncthreads();
   load_sdist(S.sdist, J.topo);
   __syncthreads();
@@ -3152,69 +3193,75 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
   // --- initial state: block weights, locks, best copy, J, controller ---
   if (lead)
     for (int32_t b = threadIdx.x; b < J.topo.kc; b += blockDim.x) J.W[b] = 0;
-  if (lead && threadIdx.x == 0) {
+  if (threadIdx.x == 0) {
     RefineState z{};
     z.rounds = J.rounds;
     z.level = J.level;
     *s = z;
-    *J.Jacc = 0;
+    if (lead) J.Jacc[0] = 0;
   }
   sy.sync();
   for (int64_t v = gt; v < n; v += GT) {
-    atomicAdd((unsigned long long*)&J.W[J.pi[v]], (unsigned long long)(int64_t)g.vw[v]);
+    atomicAdd((unsigned long long*)&J.W[pi[v]], (unsigned long long)(int64_t)g.vw[v]);
     J.lock[v] = 0;
-    J.best[v] = J.pi[v];
+    J.best[v] = pi[v];
   }
   int phase = 0;
   int32_t prev_kind = KIND_NONE;
   TileLane t0{};
   while (true) {
-    // J of the current mapping (after an LP or weak step the accumulator
-    // already holds it: old J plus the step's exact change), then the Alg. 6
-    // decision
+    // J of the current mapping (after an LP or weak step the accumulator holds
+    // the step's exact change), then the Alg. 6 decision
     const bool full = phase == 0 || !(prev_kind == KIND_LP || prev_kind == KIND_WEAK);
     const bool reuse = single && full;  // the gain pass may use this pass's staged tiles
     if (full) {  // (uniform: the previous step's kind is known to every thread)
       int64_t acc = 0;
       for (int64_t tile = eg.gw; tile < ntiles; tile += eg.GW) {
         int64_t Tp;
-        const TileLane t = eng_stage<kTE>(J, tg, tile, lane, sc, sw, S.sdist, Tp);
+        const TileLane t = eng_stage<kTE>(J, pi, tg, tile, lane, sc, sw, S.sdist, Tp);
         acc += Tp;
         if (single) t0 = t;
         __syncwarp();
       }
       eng_heavy_rows(J, eg, [&](int32_t v, int64_t b, int64_t e) {
-        const int32_t p = J.pi[v];
+        const int32_t p = pi[v];
         for (int64_t x = b + threadIdx.x; x < e; x += blockDim.x)
-          acc += (int64_t)g.adjw[x] * dcode(S.sdist, p, J.pi[g.adj[x]]);
+          acc += (int64_t)g.adjw[x] * dcode(S.sdist, p, pi[g.adj[x]]);
       });
       acc = block_sum(acc, S.sm);
-      if (threadIdx.x == 0 && acc) atomicAdd((unsigned long long*)J.Jacc, (unsigned long long)acc);
+      if (threadIdx.x == 0 && acc) atomicAdd((unsigned long long*)&J.Jacc[par], (unsigned long long)acc);
       sy.sync();
     }
-    if (lead) {
+    {
       const int64_t mx = block_max_w(J.W, J.topo.kc, S.smax);
       if (threadIdx.x == 0) {
-        const int64_t Jv = *(volatile int64_t*)J.Jacc;
-        control_step(s, mx, Jv, J.ctl, phase, 0, 0);
-        *J.Jacc = next_j_base(s, Jv);
-        J.cnt[CNT_ELIG] = 0;  // the cut-bucket list of a rebalancing step
-        J.cnt[CNT_SEL] = 0;   // and the movers of a strong one
+        const int64_t acc = *(volatile int64_t*)&J.Jacc[par];
+        CtlArgs ctl = J.ctl;
+        if (!lead) ctl.tcap = 0;  // one CTA writes the trace
+        control_step(s, mx, full ? acc : s->J + acc, ctl, phase, 0, 0);
+        if (lead) {
+          J.Jacc[par ^ 1] = 0;  // every CTA has read it an iteration ago
+          J.cnt[CNT_ELIG] = 0;  // the cut-bucket list of a rebalancing step
+          J.cnt[CNT_SEL] = 0;   // and the movers of a strong one
+        }
       }
+      par ^= 1;
       __syncthreads();
       // a rebalancing step: its threshold sigma and destination list U now
-      const int32_t next = *(volatile int32_t*)&s->kind;
-      if (next == KIND_WEAK || next == KIND_STRONG) {
-        const RebPrepArgs pa{J.W, J.pe_of_code, J.topo, J.lmax, J.cV, J.sigma_gap, J.U, J.cnt, J.accepted};
-        reb_prep_body(pa, next == KIND_STRONG);
+      if (s->kind == KIND_WEAK || s->kind == KIND_STRONG) {
+        const bool strong = s->kind == KIND_STRONG;
+        if (own_prep || lead) {
+          const RebPrepArgs pa{J.W, J.pe_of_code, J.topo, J.lmax, J.cV, J.sigma_gap, own_prep ? S.U : J.U,
+                               own_prep ? S.cnt : J.cnt, lead ? J.accepted : nullptr};
+          reb_prep_body(pa, strong);
+        }
+        if (!own_prep) sy.sync();
+        else __syncthreads();
       }
     }
-    sy.sync();
-    const int32_t done = *(volatile int32_t*)&s->done;
-    const int32_t kind = *(volatile int32_t*)&s->kind;
-    const int32_t copy = *(volatile int32_t*)&s->copy_best;
+    const int32_t done = s->done, kind = s->kind, copy = s->copy_best;
     if (copy)
-      for (int64_t v = gt; v < n; v += GT) J.best[v] = J.pi[v];
+      for (int64_t v = gt; v < n; v += GT) J.best[v] = pi[v];
     if (done) break;
     phase = 1;
     prev_kind = kind;
@@ -3223,12 +3270,12 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
       // row's sums by PE; the others through the sub-warp work queue
       for (int64_t tile = eg.gw; tile < ntiles; tile += eg.GW) {
         TileLane t = t0;
-        if (!reuse) t = stage_tile<kTE>(tg, tile * kTileV, lane, sc, sw, PlainGather{J.pi});
+        if (!reuse) t = stage_tile<kTE>(tg, tile * kTileV, lane, sc, sw, PlainGather{pi});
         int32_t p = -1;
         bool over = false;
         if (t.v < n && !eng_heavy(J, t.e - t.b)) {
           const int deg = (int)(t.e - t.b);
-          p = J.pi[t.v];
+          p = pi[t.v];
           PeSums ps;
           if (J.lock[t.v]) {  // stays this step
             J.lock[t.v] = 0;
@@ -3236,7 +3283,7 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
           } else if (t.staged) {
             pe_sums_staged(ps, sc + (t.b - t.E0), sw + (t.b - t.E0), deg, p);
           } else {
-            pe_sums_global(ps, g.adj + t.b, g.adjw + t.b, J.pi, deg, p);
+            pe_sums_global(ps, g.adj + t.b, g.adjw + t.b, pi, deg, p);
           }
           over = ps.n > kPeSlots;
           int32_t bc = p;
@@ -3250,7 +3297,7 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
             }
           } else if (!t.staged && deg > kTE / 4) {  // longer than a sub-warp's quarter of the staging area
             over = false;
-            const PlainRow r{g.adj + t.b, g.adjw + t.b, J.pi};
+            const PlainRow r{g.adj + t.b, g.adjw + t.b, pi};
             int64_t bt;
             best_target(r, deg, p, S.sdist, bc, bt);
             G = row_cost(r, deg, S.sdist, p) - bt;
@@ -3263,7 +3310,7 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
           }
         }
         const unsigned work = __ballot_sync(0xffffffffu, over);
-        tile_gain_queue(work, t, p, sc, sw, kTE, PlainRowLoader{g.adj, g.adjw, J.pi}, S.sdist, lane,
+        tile_gain_queue(work, t, p, sc, sw, kTE, PlainRowLoader{g.adj, g.adjw, pi}, S.sdist, lane,
                         kVar && J.flt.num > 0, [&](int src, int64_t Gv, int32_t bc, int32_t pv, int64_t own) {
           const int64_t v = tile * kTileV + src;
           const bool in = kVar ? J.flt.admit(Gv, own) : Gv >= 0;
@@ -3277,7 +3324,7 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
         __syncthreads();  // the warps' staging areas are free for the row tables
         const LpFilter flt = kVar ? J.flt : LpFilter{0, 1};
         eng_heavy_rows(J, eg, [&](int32_t v, int64_t b, int64_t e) {
-          const int32_t p = J.pi[v];
+          const int32_t p = pi[v];
           if (J.lock[v]) {
             __syncthreads();  // every thread has read the lock
             if (threadIdx.x == 0) {
@@ -3288,7 +3335,7 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
             }
             return;
           }
-          eng_row_table(J, b, e, dyn, J.gl.total, true);
+          eng_row_table(J, pi, b, e, dyn, J.gl.total, true);
           lp_hub_decide(dyn, J.topo, J.gl, flt, v, p, J.pp, J.gain, J.inx, S.hb, S.hc);
         });
       }
@@ -3305,12 +3352,12 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
           const int64_t vv = tile * kTileV + (src < 0 ? 0 : src);
           int64_t sum = 0;
           if (src >= 0) {
-            const int32_t p = J.pi[vv], q = J.pp[vv];
+            const int32_t p = pi[vv], q = J.pp[vv];
             const int64_t gv = J.gain[vv];
             const int64_t xe = g.xadj[vv + 1];
             for (int64_t x = g.xadj[vv] + sl; x < xe; x += kSubWarp) {
               const int32_t u = g.adj[x];
-              int32_t bu = J.pi[u];
+              int32_t bu = pi[u];
               if (J.inx[u]) {
                 const int64_t gu = J.gain[u];
                 if (gu > gv || (gu == gv && u < vv)) bu = J.pp[u];
@@ -3326,12 +3373,12 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
       }
       eng_heavy_rows(J, eg, [&](int32_t v, int64_t b, int64_t e) {
         if (!J.inx[v]) return;
-        const int32_t p = J.pi[v], q = J.pp[v];
+        const int32_t p = pi[v], q = J.pp[v];
         const int64_t gv = J.gain[v];
         int64_t sum = 0;
         for (int64_t x = b + threadIdx.x; x < e; x += blockDim.x) {
           const int32_t u = g.adj[x];
-          int32_t bu = J.pi[u];
+          int32_t bu = pi[u];
           if (J.inx[u]) {
             const int64_t gu = J.gain[u];
             if (gu > gv || (gu == gv && u < v)) bu = J.pp[u];
@@ -3342,29 +3389,23 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
         if (threadIdx.x == 0 && sum >= 0) J.lock[v] = 1;
       });
       sy.sync();
-      eng_delta(J, LpMoves{J.lock, J.pp}, S, eg, ntiles);
+      // step 3: simultaneous move of M, and its change of J
+      eng_move(J, LpMoves{J.lock, J.pp}, pi, pn, &J.Jacc[par], S, eg, ntiles);
       sy.sync();
-      // step 3: simultaneous move of M
-      for (int64_t v = gt; v < n; v += GT) {
-        if (!J.lock[v]) continue;
-        const int32_t p = J.pi[v], q = J.pp[v];
-        const int64_t c = g.vw[v];
-        J.pi[v] = q;
-        atomicAdd((unsigned long long*)&J.W[p], (unsigned long long)(-c));
-        atomicAdd((unsigned long long*)&J.W[q], (unsigned long long)c);
-      }
-      sy.sync();
+      int32_t* const old = pi;
+      pi = pn;
+      pn = old;
       continue;
     }
     // --- weak / strong rebalancing ---
     const bool strong = kind == KIND_STRONG;
-    const int32_t t = *(volatile int32_t*)&s->t;
-    const int64_t sigma = *(volatile int64_t*)&J.cnt[CNT_SIGMA];
-    const int64_t nU = *(volatile int64_t*)&J.cnt[CNT_NU];
+    const int32_t t = s->t;
+    const int64_t sigma = own_prep ? S.cnt[CNT_SIGMA] : *(volatile int64_t*)&J.cnt[CNT_SIGMA];
+    const int64_t nU = own_prep ? S.cnt[CNT_NU] : *(volatile int64_t*)&J.cnt[CNT_NU];
     // eligible vertices and their destinations: each lane from its row's sums
     // by PE, the vertices with more foreign PEs from staged rows
     const bool obj = kVar && J.reb_obj != 0;
-    auto drawn = [&](int64_t v) { return J.U[h_rebalance(J.seed, J.level, t, (int32_t)v) % (uint64_t)nU]; };
+    auto drawn = [&](int64_t v) { return U[h_rebalance(J.seed, J.level, t, (int32_t)v) % (uint64_t)nU]; };
     auto reb_write = [&](int64_t v, int32_t A, int32_t dst, int64_t gcut) {
       const int bk = loss_bucket(gcut);
       J.elig[v] = 1;
@@ -3379,7 +3420,7 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
       int64_t vb = 0;
       int deg = 0;
       if (v < n && !eng_heavy_row(J, v)) {
-        A = J.pi[v];
+        A = pi[v];
         cv = g.vw[v];
         vb = g.xadj[v];
         deg = (int)(g.xadj[v + 1] - vb);
@@ -3391,7 +3432,7 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
       int32_t slot = -1;  // (block, bucket) of a vertex decided by its own lane
       if (cand) {
         PeSums ps;
-        pe_sums_global(ps, g.adj + vb, g.adjw + vb, J.pi, deg, A);
+        pe_sums_global(ps, g.adj + vb, g.adjw + vb, pi, deg, A);
         if (ps.n <= kPeSlots) {
           cand = false;
           int32_t dst;
@@ -3416,15 +3457,15 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
           atomicAdd((unsigned long long*)&J.tab[slot], (unsigned long long)(int64_t)cw);
       }
       if (__ballot_sync(0xffffffffu, cand) == 0) continue;
-      const TileLane tl = stage_tile<kTE>(tg, tile * kTileV, lane, sc, sw, PlainGather{J.pi});
+      const TileLane tl = stage_tile<kTE>(tg, tile * kTileV, lane, sc, sw, PlainGather{pi});
       if (cand && !tl.staged && deg > kTE / 4) {  // longer than a sub-warp's quarter: this lane alone
         int32_t dst, bk;
         bool ok;
         if constexpr (kVar)
-          ok = J.reb_obj != 0 ? eng_reb_select<true>(J, (int32_t)v, sigma, nU, t, S.sdist, dst, bk)
-                              : eng_reb_select<false>(J, (int32_t)v, sigma, nU, t, S.sdist, dst, bk);
+          ok = J.reb_obj != 0 ? eng_reb_select<true>(J, pi, U, (int32_t)v, sigma, nU, t, S.sdist, dst, bk)
+                              : eng_reb_select<false>(J, pi, U, (int32_t)v, sigma, nU, t, S.sdist, dst, bk);
         else
-          ok = eng_reb_select<false>(J, (int32_t)v, sigma, nU, t, S.sdist, dst, bk);
+          ok = eng_reb_select<false>(J, pi, U, (int32_t)v, sigma, nU, t, S.sdist, dst, bk);
         J.elig[v] = ok ? 1 : 0;
         if (ok) {
           J.dest[v] = dst;
@@ -3450,7 +3491,7 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
         const int32_t at = reb_write(u, a, bc, sb - sa);
         atomicAdd((unsigned long long*)&J.tab[at], (unsigned long long)(int64_t)g.vw[u]);
       };
-      const PlainRowLoader load{g.adj, g.adjw, J.pi};
+      const PlainRowLoader load{g.adj, g.adjw, pi};
       if (obj)
         reb_tile_queue<true>(work, tl, A, sc, sw, kTE, load, J.W, sigma, S.sdist, lane, reb_out);
       else
@@ -3461,12 +3502,12 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
       __syncthreads();  // the warps' staging areas are free for the row tables
       const RebArgs ra{J.W, J.U, J.cnt, J.tab, J.lmax, J.cV, J.k, J.seed, kVar ? J.reb_obj : 0, J.topo};
       eng_heavy_rows(J, eg, [&](int32_t v, int64_t b, int64_t e) {
-        const int32_t A = J.pi[v];
+        const int32_t A = pi[v];
         if (!reb_eligible(ra, A, g.vw[v])) {
           if (threadIdx.x == 0) J.elig[v] = 0;
           return;
         }
-        eng_row_table(J, b, e, dyn, ra.obj ? J.gl.total : J.topo.kc, ra.obj != 0);
+        eng_row_table(J, pi, b, e, dyn, ra.obj ? J.gl.total : J.topo.kc, ra.obj != 0);
         reb_hub_decide(dyn, ra, J.topo.kc, J.gl, v, A, g.vw[v], J.dest, J.bkt, J.elig, s, S.hb, S.hc);
       });
     }
@@ -3514,7 +3555,7 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
     // (in a weak step marked 2, with its list slot)
     for (int64_t v = gt; v < n; v += GT) {
       if (!J.elig[v]) continue;
-      const int32_t A = J.pi[v];
+      const int32_t A = pi[v];
       const int32_t bb = J.bkt[v], cut = bcut[A];
       if (bb != cut) {
         J.sel[v] = bb < cut ? 1 : 0;
@@ -3542,17 +3583,11 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
       // change of J
       uint8_t* s_sel = eng_resolve_local(J, S, s_bcut + kEngCutSmem, ln, idbits, rem);
       const WeakMovesShared mv{J.elig, J.sel, J.dest, J.sarr, s_sel};
-      eng_delta(J, mv, S, eg, ntiles);
+      eng_move(J, mv, pi, pn, &J.Jacc[par], S, eg, ntiles);
       sy.sync();
-      for (int64_t v = gt; v < n; v += GT) {
-        if (!mv.moved(v)) continue;
-        const int32_t p = J.pi[v], q = J.dest[v];
-        const int64_t c = g.vw[v];
-        J.pi[v] = q;
-        atomicAdd((unsigned long long*)&J.W[p], (unsigned long long)(-c));
-        atomicAdd((unsigned long long*)&J.W[q], (unsigned long long)c);
-      }
-      sy.sync();
+      int32_t* const old = pi;
+      pi = pn;
+      pn = old;
       continue;
     }
     if (lead) {  // the cut-bucket list by (block, id), per-block prefix
@@ -3581,17 +3616,11 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
     }
     sy.sync();
     if (!strong) {
-      eng_delta(J, WeakMoves{J.elig, J.sel, J.dest}, S, eg, ntiles);
+      eng_move(J, WeakMoves{J.elig, J.sel, J.dest}, pi, pn, &J.Jacc[par], S, eg, ntiles);
       sy.sync();
-      for (int64_t v = gt; v < n; v += GT) {
-        if (!J.elig[v] || !J.sel[v]) continue;
-        const int32_t p = J.pi[v], q = J.dest[v];
-        const int64_t c = g.vw[v];
-        J.pi[v] = q;
-        atomicAdd((unsigned long long*)&J.W[p], (unsigned long long)(-c));
-        atomicAdd((unsigned long long*)&J.W[q], (unsigned long long)c);
-      }
-      sy.sync();
+      int32_t* const old = pi;
+      pi = pn;
+      pn = old;
       continue;
     }
     // strong: the movers, listed by all CTAs in any order under the complete
@@ -3707,21 +3736,31 @@ __device__ void engine_run_job(const EngineJob& J, EngSmem& S, int32_t* dyn, int
           if (bb >= 0 && bb < kc && sv + c <= J.Rb[bb + 1]) q = bb;
         }
         if (q < 0) continue;
-        const int32_t p = J.pi[v];
-        J.pi[v] = q;
+        const int32_t p = pi[v];
+        pi[v] = q;
         atomicAdd((unsigned long long*)&J.W[p], (unsigned long long)(-c));
         atomicAdd((unsigned long long*)&J.W[q], (unsigned long long)c);
       }
     }
     sy.sync();
   }
+  if (lead && threadIdx.x == 0) *J.s = *s;
   for (int64_t v = gt; v < n; v += GT) J.pi[v] = J.best[v];
+}
+
+// The job descriptor on chip: its fields are read all along the run.
+static_assert(sizeof(EngineJob) % sizeof(int32_t) == 0, "copied in words");
+__device__ __forceinline__ void eng_load_job(EngineJob& J, const EngineJob* src) {
+  for (int i = threadIdx.x; i < (int)(sizeof(EngineJob) / sizeof(int32_t)); i += blockDim.x)
+    reinterpret_cast<int32_t*>(&J)[i] = reinterpret_cast<const int32_t*>(src)[i];
+  __syncthreads();
 }
 
 template <int kTE, bool kVar>
 __global__ void __launch_bounds__(kEngThreads, 1) k_engine(const EngineJob* __restrict__ jobs, int32_t njobs,
                                                           unsigned int* queue) {
   __shared__ EngSmem S;
+  __shared__ EngineJob J;
   __shared__ int32_t job_slot;
   extern __shared__ __align__(16) int32_t eng_dyn[];
   cg::cluster_group cl = cg::this_cluster();
@@ -3741,7 +3780,10 @@ __global__ void __launch_bounds__(kEngThreads, 1) k_engine(const EngineJob* __re
   int32_t* sw = sc + kTE;
   if (!queue) {  // one job per cluster
     const int32_t jid = (int32_t)(blockIdx.x / csize);
-    if (jid < njobs) engine_run_job<kTE, kVar>(jobs[jid], S, eng_dyn, sc, sw, eg, ClusterSync{});
+    if (jid < njobs) {
+      eng_load_job(J, jobs + jid);
+      engine_run_job<kTE, kVar>(J, S, eng_dyn, sc, sw, eg, ClusterSync{});
+    }
     return;
   }
   // persistent clusters: the next job from the queue (jobs in the order given)
@@ -3751,7 +3793,8 @@ __global__ void __launch_bounds__(kEngThreads, 1) k_engine(const EngineJob* __re
     const int32_t jid = *cl.map_shared_rank(&job_slot, 0);
     eng_sync();
     if (jid >= njobs) break;
-    engine_run_job<kTE, kVar>(jobs[jid], S, eng_dyn, sc, sw, eg, ClusterSync{});
+    eng_load_job(J, jobs + jid);
+    engine_run_job<kTE, kVar>(J, S, eng_dyn, sc, sw, eg, ClusterSync{});
   }
 }
 
@@ -3761,6 +3804,7 @@ __global__ void __launch_bounds__(kEngThreads, 1) k_engine(const EngineJob* __re
 template <int kTE, bool kVar>
 __global__ void __launch_bounds__(kEngThreads, 1) k_engine_grid(const EngineJob* __restrict__ job, GridBar* bar) {
   __shared__ EngSmem S;
+  __shared__ EngineJob J;
   __shared__ unsigned int bar_flag;
   extern __shared__ __align__(16) int32_t eng_dyn[];
   const int warp = threadIdx.x >> 5;
@@ -3775,7 +3819,8 @@ __global__ void __launch_bounds__(kEngThreads, 1) k_engine_grid(const EngineJob*
   eg.ncta = (int)gridDim.x;
   int32_t* sc = eng_dyn + warp * 2 * kTE;
   int32_t* sw = sc + kTE;
-  engine_run_job<kTE, kVar>(*job, S, eng_dyn, sc, sw, eg, GridSync{bar, &bar_flag, gridDim.x});
+  eng_load_job(J, job);
+  engine_run_job<kTE, kVar>(J, S, eng_dyn, sc, sw, eg, GridSync{bar, &bar_flag, gridDim.x});
 }
 
 // Self-test of the bounded grid barrier: a barrier that waits for one more
@@ -3858,7 +3903,7 @@ void refine_alloc(Ctx& c) {
   c.rem = c.mem.make<int64_t>(kc);
   GM_CUDA(cudaMemsetAsync(c.tab, 0, kc * kBuckets * sizeof(int64_t), c.st));
   c.counters = c.mem.make<int64_t>(CNT_N);
-  c.Jacc = c.mem.make<int64_t>(1);
+  c.Jacc = c.mem.make<int64_t>(2);
   c.evctr = reinterpret_cast<unsigned int*>(c.mem.make<int64_t>(1));
   GM_CUDA(cudaMemsetAsync(c.evctr, 0, sizeof(int64_t), c.st));
   c.state = c.mem.make<RefineState>(1);
@@ -4112,17 +4157,22 @@ static bool engine_rows_fit(const Ctx& c, const Level& L) {
 // graph has a warp per vertex and the hub chunks.
 // Per Alg. 6 iteration, engine against graph (us), by the share of the
 // level's entries in rows above 32: meshes and their coarse levels with at
-// most 4 %: 24-81 against 43-97; random geometric graph of degree 40, 90 %:
-// 134 against 104; R-MAT with 770 to 200 k vertices, 67-98 %: 370-1900
+// most 4 %: 17-63 against 43-94; random geometric graph of degree 40, 90 %:
+// 107 against 101; R-MAT with 770 to 200 k vertices, 67-98 %: 370-1900
 // against 109-284.  Hence one entry in 16.
 // A limit set in the config (`asked`) is followed as it stands, and a server's
-// jobs keep the cluster engine, in which its batcher runs them together.
-static bool engine_slower(const Level& L, int32_t asked) { return asked == 0 && L.m_hi * 16 > L.m; }
+// jobs keep the cluster engine, in which its batcher runs them together, for
+// levels of up to kEngServedEntries entries (14 R-MAT requests of 2000 to 50000
+// vertices at once: 276 ms with all of them in the batcher, 130 ms with none).
+constexpr int64_t kEngServedEntries = 1 << 17;
+static bool engine_slower(const Ctx& c, const Level& L, int32_t asked) {
+  return asked == 0 && L.m_hi * 16 > L.m && (!c.sink || L.m > kEngServedEntries);
+}
 
 // Cluster size of the fused engine for a level (0: not used).
 static int engine_cluster(Ctx& c, const Level& L) {
   const int64_t lim = c.cfg.engine_max_n > 0 ? c.cfg.engine_max_n : (c.cfg.engine_max_n < 0 ? -1 : kEngMaxN);
-  if (!c.sink && engine_slower(L, c.cfg.engine_max_n)) return 0;
+  if (engine_slower(c, L, c.cfg.engine_max_n)) return 0;
   if (!c.use_graphs || c.prof || L.n > lim || !engine_rows_fit(c, L)) return 0;
   int C = (L.n + 1023) / 1024;  // about one vertex per thread
   if (C < 1) C = 1;
@@ -4208,6 +4258,7 @@ static EngineJob engine_job(Ctx& c, int lvl, int32_t rounds) {
   EngineJob j{};
   j.g = view(L);
   j.pi = L.pi;
+  j.pi2 = c.req;  // (coarsening scratch)
   j.pp = c.pp;
   j.gain = c.gain;
   j.inx = c.inx;
@@ -4294,7 +4345,7 @@ static void refine_engine(Ctx& c, int lvl, int32_t rounds, int C, int64_t* J, in
 static bool engine_grid_ok(Ctx& c, const Level& L) {
   const int64_t lim =
       c.cfg.grid_engine_max_n > 0 ? c.cfg.grid_engine_max_n : (c.cfg.grid_engine_max_n < 0 ? -1 : (1 << 18));
-  if (engine_slower(L, c.cfg.grid_engine_max_n)) return false;
+  if (engine_slower(c, L, c.cfg.grid_engine_max_n)) return false;
   if (!c.use_graphs || c.prof || L.n > lim || !engine_rows_fit(c, L)) return false;
   static std::atomic<int> cached[64];  // a property of the device: once per process
   if (c.eng_grid_blocks == 0) c.eng_grid_blocks = cached[c.dev & 63].load();
