@@ -319,17 +319,31 @@ __device__ __forceinline__ uint32_t slot_hash(int32_t t) {
 // it never carries into the label).  The own cluster is inserted with weight
 // 0.  The decision takes the largest weight, then the smaller tie-hash, then
 // the smaller label, and puts every slot back to empty.
-//  * rows of at most kSmemRowDeg entries: the whole row on one CTA, its
-//    table in shared memory (no global atomics);
+//  * rows of at most kBigRowDeg entries: the whole row on one CTA (or a part
+//    of one), its table in shared memory.  Every thread keeps the slots of its
+//    entries (at most kRowPer) in registers, so that the decision and the
+//    reset touch those slots only, not the table: k_cluster_high takes the
+//    rows up to kSmemRowDeg, k_cluster_big the others.  Scanning the tables
+//    instead, with the rows above 2047 entries in global tables, took 1.13 ms a
+//    sub-round of R-MAT 2^22 (k_cluster_high 0.83, k_cluster_giant 0.29), this
+//    0.82 (0.53 + k_cluster_big 0.17 + k_cluster_giant 0.12).
 //  * larger rows: their entries, flattened in huge[] order, are cut into
 //    chunks of kHubChunk entries that the CTAs of one wave take in turn, the
 //    table in global memory.  A second launch reads the table back in the
 //    same chunks (each chunk takes the slots in proportion to its share of
 //    the row's entries) and stores each slice's best label; a third combines
 //    the slices of every row and files its request.
+//  * the first sub-round of a level: every vertex is its own cluster, so the
+//    labels of a row are distinct, no table is needed, and the entries are
+//    rated as they stream past.
 constexpr unsigned long long kEmptySlot = ~0ULL;
-constexpr int64_t kSmemRowDeg = 2047;
 constexpr uint32_t kSmemSlots = 4096;  // >= 2 (kSmemRowDeg + 1)
+constexpr int kRowPer = 8;             // entries per thread of a row rated in shared memory
+static_assert(kRowPer * kHiThreads >= kSmemRowDeg, "a CTA holds a row's slots in registers");
+// k_cluster_big<T>: rows of at most kRowPer T - 1 entries, twice the slots
+constexpr uint32_t big_slots(int threads) { return 2u * kRowPer * (uint32_t)threads; }
+static_assert(kRowPer * 512 > kSmemRowDeg && kRowPer * 1024 - 1 == kBigRowDeg, "k_cluster_big's rows");
+static_assert(big_slots(1024) < 0xffff, "slots are kept in 16 bits");
 static_assert(kSmemSlots >= 2 * (kSmemRowDeg + 1), "shared-memory row table at most half full");
 // rows of one chunk at most: every row there has more than kLowDeg + 1 >= 33 entries
 constexpr int kChunkRows = 64;
@@ -338,25 +352,26 @@ constexpr int kChunkRows = 64;
 constexpr int kRowGroups = 2;
 constexpr int64_t kGroupRowDeg = kSmemSlots / kRowGroups / 2 - 1;
 static_assert(kSmemSlots / kRowGroups >= 2 * (kGroupRowDeg + 1), "a group's table at most half full");
+static_assert(kRowPer * (kHiThreads / kRowGroups) >= kGroupRowDeg, "a group holds a row's slots in registers");
 static_assert(kRowGroups <= 2, "named barriers 1 and 2 serve the row groups");
 static_assert(kHubChunk / 34 + 2 <= kChunkRows, "a chunk's rows fit the per-chunk row table");
 
-// Inserts from slot h on (`probes` already made).
-__device__ __forceinline__ bool hub_insert_from(unsigned long long* T, uint32_t mask, int32_t t, int32_t w, uint32_t h,
-                                                uint32_t probes) {
+// Inserts from slot h on (`probes` already made); the slot, or -1 if the table is full.
+__device__ __forceinline__ int32_t hub_insert_from(unsigned long long* T, uint32_t mask, int32_t t, int32_t w,
+                                                   uint32_t h, uint32_t probes) {
   const unsigned long long key = (unsigned long long)(uint32_t)t << 32;
   for (uint32_t probe = probes; probe <= mask; probe++) {
     const unsigned long long prev = atomicCAS(&T[h], kEmptySlot, key | (uint32_t)w);
-    if (prev == kEmptySlot) return true;
+    if (prev == kEmptySlot) return (int32_t)h;
     if ((prev >> 32) == (uint32_t)t) {
       if (w) atomicAdd(&T[h], (unsigned long long)(uint32_t)w);
-      return true;
+      return (int32_t)h;
     }
     h = (h + 1) & mask;
   }
-  return false;
+  return -1;
 }
-__device__ __forceinline__ bool hub_insert(unsigned long long* T, uint32_t mask, int32_t t, int32_t w) {
+__device__ __forceinline__ int32_t hub_insert(unsigned long long* T, uint32_t mask, int32_t t, int32_t w) {
   return hub_insert_from(T, mask, t, w, slot_hash(t) & mask, 0);
 }
 
@@ -413,78 +428,198 @@ __device__ __forceinline__ bool hub_insert_range(const GraphView& g, const int32
       if ((prev[b] >> 32) == (uint32_t)t[b]) {
         if (w[b]) atomicAdd(&T[h[b]], (unsigned long long)(uint32_t)w[b]);
       } else {
-        ok &= hub_insert_from(T, mask, t[b], w[b], (h[b] + 1) & mask, 1);
+        ok &= hub_insert_from(T, mask, t[b], w[b], (h[b] + 1) & mask, 1) >= 0;
       }
     }
   }
   return ok;
 }
 
-struct HubScratch {
-  int32_t bs[kHiThreads / 32];
-  uint64_t bh[kHiThreads / 32];
-  int32_t bt[kHiThreads / 32];
+template <int kWarps>
+struct BestScratch {
+  int32_t bs[kWarps];
+  uint64_t bh[kWarps];
+  int32_t bt[kWarps];
 };
+using HubScratch = BestScratch<kHiThreads / 32>;
 
-// The best label of the slots T[s0, s1) of a row table (kGlobal: read from
-// L2, where other CTAs' atomics were performed): the largest weight, then
-// the smaller tie-hash, then the smaller label, in two passes so that only
-// labels of the largest weight are hashed; every slot is put back to empty.
-// All threads of group gr call it; the group's thread 0 receives the result
-// (bs = -1 for no label); ends with the group's barrier.
-template <bool kGlobal>
-__device__ __forceinline__ void table_best(unsigned long long* T, uint32_t s0, uint32_t s1, const ClusterArgs& a,
-                                           HubScratch& sx, const RowGroup& gr, int32_t& out_bs, uint64_t& out_bh,
-                                           int32_t& out_bt) {
+// Whether the labels are still the vertices themselves (the first sub-round of a level).
+__device__ __forceinline__ bool cluster_single(const ClusterArgs& a) { return a.cs->it == 0 && a.round == 0; }
+
+__device__ __forceinline__ bool label_before(uint64_t h, int32_t t, uint64_t bh, int32_t bt) {
+  return h < bh || (h == bh && t < bt);
+}
+
+// The smallest (tie-hash, label) of a warp in every lane.
+__device__ __forceinline__ void warp_first_label(uint64_t& bh, int32_t& bt) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const uint64_t oh = __shfl_xor_sync(0xffffffffu, bh, o);
+    const int32_t ot = __shfl_xor_sync(0xffffffffu, bt, o);
+    if (label_before(oh, ot, bh, bt)) {
+      bh = oh;
+      bt = ot;
+    }
+  }
+}
+
+// Rates one row of deg <= kRowPer * gr.size entries from CSR position e0 in
+// the shared-memory table T (empty before and after) and returns the best
+// label to the group's thread 0; all threads of group gr call it, ends with
+// the group's barrier.
+template <int kWarps>
+__device__ __forceinline__ int32_t rate_row(const GraphView& g, const ClusterArgs& a, int64_t e0, int32_t deg,
+                                            int32_t own, unsigned long long* T, uint32_t mask,
+                                            BestScratch<kWarps>& sx, const RowGroup& gr, uint32_t* err) {
   const int warp = (int)(threadIdx.x >> 5);
-  int32_t bs = -1;
-#pragma unroll 4
-  for (uint32_t s = s0 + gr.tid; s < s1; s += gr.size) {
-    const unsigned long long x = kGlobal ? __ldcg(T + s) : T[s];
-    if (x != kEmptySlot) bs = max(bs, (int32_t)(uint32_t)x);
+  uint32_t slot2[kRowPer / 2];  // two 16-bit slots per word, 0xffff: none
+  int32_t own_slot = -1;
+  bool ok = true;
+  if (gr.tid == 0) {
+    own_slot = hub_insert(T, mask, own, 0);
+    ok = own_slot >= 0;
   }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) bs = max(bs, __shfl_xor_sync(0xffffffffu, bs, o));
+  for (int half = 0; half < kRowPer / kHubBatch; half++) {
+    slot2[2 * half] = slot2[2 * half + 1] = 0xffffffffu;
+    if (half * kHubBatch * gr.size >= deg) continue;  // (uniform)
+    int32_t t[kHubBatch], w[kHubBatch];
+    uint32_t h[kHubBatch];
+    unsigned long long prev[kHubBatch];
+    const int64_t f = e0 + half * kHubBatch * gr.size + gr.tid;
+    const int32_t left = deg - half * kHubBatch * gr.size - gr.tid;
+#pragma unroll
+    for (int b = 0; b < kHubBatch; b++) {
+      t[b] = b * gr.size < left ? g.adj[f + b * gr.size] : -1;
+      w[b] = b * gr.size < left ? g.adjw[f + b * gr.size] : 0;
+    }
+#pragma unroll
+    for (int b = 0; b < kHubBatch; b++) t[b] = t[b] >= 0 ? a.C[t[b]] : -1;
+#pragma unroll
+    for (int b = 0; b < kHubBatch; b++) {
+      h[b] = slot_hash(t[b]) & mask;
+      prev[b] = t[b] >= 0 ? atomicCAS(&T[h[b]], kEmptySlot, ((unsigned long long)(uint32_t)t[b] << 32) | (uint32_t)w[b])
+                          : kEmptySlot;
+    }
+#pragma unroll
+    for (int b = 0; b < kHubBatch; b++) {
+      int32_t at = -1;
+      if (t[b] >= 0) {
+        at = (int32_t)h[b];
+        if (prev[b] != kEmptySlot) {
+          if ((prev[b] >> 32) == (uint32_t)t[b]) atomicAdd(&T[h[b]], (unsigned long long)(uint32_t)w[b]);
+          else at = hub_insert_from(T, mask, t[b], w[b], (h[b] + 1) & mask, 1);
+        }
+        ok &= at >= 0;
+      }
+      const uint32_t at16 = (uint32_t)at & 0xffffu;
+      uint32_t& word = slot2[2 * half + b / 2];
+      word = (b & 1) ? (word & 0x0000ffffu) | (at16 << 16) : (word & 0xffff0000u) | at16;
+    }
+  }
+  if (!ok) atomicOr(err, ERR_CAPACITY);
+  gr.sync();
+  auto slot_of = [&](int i) { return (i & 1) ? slot2[i / 2] >> 16 : slot2[i / 2] & 0xffffu; };
+  int32_t bs = own_slot >= 0 ? (int32_t)(uint32_t)T[own_slot] : -1;
+#pragma unroll
+  for (int i = 0; i < kRowPer; i++) {
+    const uint32_t at = slot_of(i);
+    if (at != 0xffffu) bs = max(bs, (int32_t)(uint32_t)T[at]);
+  }
+  bs = __reduce_max_sync(0xffffffffu, bs);
   if ((threadIdx.x & 31) == 0) sx.bs[warp] = bs;
   gr.sync();
   bs = sx.bs[gr.warp0];
   for (int w = 1; w < gr.warps; w++) bs = max(bs, sx.bs[gr.warp0 + w]);
   uint64_t bh = ~0ULL;
   int32_t bt = INT32_MAX;
-#pragma unroll 4
-  for (uint32_t s = s0 + gr.tid; s < s1; s += gr.size) {
-    const unsigned long long x = kGlobal ? __ldcg(T + s) : T[s];
-    if (x == kEmptySlot) continue;
-    T[s] = kEmptySlot;
-    if ((int32_t)(uint32_t)x != bs) continue;
+  auto consider = [&](unsigned long long x) {
+    if ((int32_t)(uint32_t)x != bs) return;
     const int32_t t = (int32_t)(x >> 32);
     const uint64_t h = h_tie(a.seed, a.level, t);
-    if (h < bh || (h == bh && t < bt)) {
+    if (label_before(h, t, bh, bt)) {
       bh = h;
       bt = t;
     }
-  }
+  };
+  if (own_slot >= 0) consider(T[own_slot]);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const uint64_t oh = __shfl_xor_sync(0xffffffffu, bh, o);
-    const int32_t ot = __shfl_xor_sync(0xffffffffu, bt, o);
-    if (oh < bh || (oh == bh && ot < bt)) {
-      bh = oh;
-      bt = ot;
+  for (int i = 0; i < kRowPer; i++) {
+    const uint32_t at = slot_of(i);
+    if (at != 0xffffu) consider(T[at]);
+  }
+  warp_first_label(bh, bt);
+  if ((threadIdx.x & 31) == 0) {
+    sx.bh[warp] = bh;
+    sx.bt[warp] = bt;
+  }
+  gr.sync();
+  // every slot has been read: back to empty
+  if (own_slot >= 0) T[own_slot] = kEmptySlot;
+#pragma unroll
+  for (int i = 0; i < kRowPer; i++) {
+    const uint32_t at = slot_of(i);
+    if (at != 0xffffu) T[at] = kEmptySlot;
+  }
+  if (gr.tid == 0)
+    for (int w = 1; w < gr.warps; w++)
+      if (label_before(sx.bh[gr.warp0 + w], sx.bt[gr.warp0 + w], bh, bt)) {
+        bh = sx.bh[gr.warp0 + w];
+        bt = sx.bt[gr.warp0 + w];
+      }
+  gr.sync();
+  return bt;
+}
+
+// The best of the distinct neighbours at CSR positions [e0, e1) (first
+// sub-round: the label of a neighbour is the neighbour): the largest weight,
+// then the smaller tie-hash, then the smaller id.  All threads of group gr call
+// it; the group's thread 0 receives the result; ends with the group's barrier.
+__device__ __forceinline__ void rate_single(const GraphView& g, const ClusterArgs& a, int64_t e0, int64_t e1,
+                                            HubScratch& sx, const RowGroup& gr, int32_t& out_bs, uint64_t& out_bh,
+                                            int32_t& out_bt) {
+  const int warp = (int)(threadIdx.x >> 5);
+  int32_t bs = -1, bt = INT32_MAX;
+  uint64_t bh = ~0ULL;
+  for (int64_t f = e0; f < e1; f += (int64_t)gr.size * kHubBatch) {
+    int32_t t[kHubBatch], w[kHubBatch];
+#pragma unroll
+    for (int b = 0; b < kHubBatch; b++) {
+      const int64_t e = f + (int64_t)b * gr.size + gr.tid;
+      t[b] = e < e1 ? g.adj[e] : -1;
+      w[b] = e < e1 ? g.adjw[e] : -1;
+    }
+#pragma unroll
+    for (int b = 0; b < kHubBatch; b++) {
+      if (t[b] < 0 || w[b] < bs) continue;
+      const uint64_t h = h_tie(a.seed, a.level, t[b]);
+      if (w[b] > bs || label_before(h, t[b], bh, bt)) {
+        bs = w[b];
+        bh = h;
+        bt = t[b];
+      }
     }
   }
+  const int32_t wmax = __reduce_max_sync(0xffffffffu, bs);
+  if (bs != wmax) {
+    bh = ~0ULL;
+    bt = INT32_MAX;
+  }
+  bs = wmax;
+  warp_first_label(bh, bt);
   if ((threadIdx.x & 31) == 0) {
+    sx.bs[warp] = bs;
     sx.bh[warp] = bh;
     sx.bt[warp] = bt;
   }
   gr.sync();
   if (gr.tid == 0) {
     for (int w = 1; w < gr.warps; w++) {
-      const uint64_t h = sx.bh[gr.warp0 + w];
-      const int32_t t = sx.bt[gr.warp0 + w];
-      if (h < bh || (h == bh && t < bt)) {
-        bh = h;
-        bt = t;
+      const int32_t s = sx.bs[gr.warp0 + w];
+      if (s > bs || (s == bs && label_before(sx.bh[gr.warp0 + w], sx.bt[gr.warp0 + w], bh, bt))) {
+        bs = s;
+        bh = sx.bh[gr.warp0 + w];
+        bt = sx.bt[gr.warp0 + w];
       }
     }
     out_bs = bs;
@@ -494,9 +629,63 @@ __device__ __forceinline__ void table_best(unsigned long long* T, uint32_t s0, u
   gr.sync();
 }
 
+// The best label of the slots T[s0, s1) of a row table in global memory (read
+// from L2, where other CTAs' atomics were performed): the largest weight,
+// then the smaller tie-hash, then the smaller label, in two passes so that
+// only labels of the largest weight are hashed; every slot is put back to
+// empty.  All threads of the CTA call it; thread 0 receives the result (bs =
+// -1 for no label); ends with a barrier.
+__device__ __forceinline__ void table_best(unsigned long long* T, uint32_t s0, uint32_t s1, const ClusterArgs& a,
+                                           HubScratch& sx, int32_t& out_bs, uint64_t& out_bh, int32_t& out_bt) {
+  const int warp = (int)(threadIdx.x >> 5);
+  int32_t bs = -1;
+#pragma unroll 4
+  for (uint32_t s = s0 + threadIdx.x; s < s1; s += kHiThreads) {
+    const unsigned long long x = __ldcg(T + s);
+    if (x != kEmptySlot) bs = max(bs, (int32_t)(uint32_t)x);
+  }
+  bs = __reduce_max_sync(0xffffffffu, bs);
+  if ((threadIdx.x & 31) == 0) sx.bs[warp] = bs;
+  __syncthreads();
+  bs = sx.bs[0];
+  for (int w = 1; w < kHiThreads / 32; w++) bs = max(bs, sx.bs[w]);
+  uint64_t bh = ~0ULL;
+  int32_t bt = INT32_MAX;
+#pragma unroll 4
+  for (uint32_t s = s0 + threadIdx.x; s < s1; s += kHiThreads) {
+    const unsigned long long x = __ldcg(T + s);
+    if (x == kEmptySlot) continue;
+    T[s] = kEmptySlot;
+    if ((int32_t)(uint32_t)x != bs) continue;
+    const int32_t t = (int32_t)(x >> 32);
+    const uint64_t h = h_tie(a.seed, a.level, t);
+    if (label_before(h, t, bh, bt)) {
+      bh = h;
+      bt = t;
+    }
+  }
+  warp_first_label(bh, bt);
+  if ((threadIdx.x & 31) == 0) {
+    sx.bh[warp] = bh;
+    sx.bt[warp] = bt;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kHiThreads / 32; w++)
+      if (label_before(sx.bh[w], sx.bt[w], bh, bt)) {
+        bh = sx.bh[w];
+        bt = sx.bt[w];
+      }
+    out_bs = bs;
+    out_bh = bh;
+    out_bt = bt;
+  }
+  __syncthreads();
+}
+
 // The larger rows' slice results: per chunk two slots (0: the large row
 // holding the chunk's first entry, 1: a large row starting inside the chunk;
-// a row of at least kSmemRowDeg + 1 >= kHubChunk entries leaves room for no
+// a row of more than kBigRowDeg >= kHubChunk entries leaves room for no
 // other), each ((weight << 32) | label, tie-hash).
 __device__ __forceinline__ int64_t part_slot(int64_t ch, int64_t rb) {
   return 4 * ch + (rb >= ch * kHubChunk ? 2 : 0);
@@ -506,8 +695,8 @@ __device__ __forceinline__ int64_t part_slot(int64_t ch, int64_t rb) {
 // shared-memory path are rated and decided here; the larger rows only insert.
 __global__ void __launch_bounds__(kHiThreads, 5) k_cluster_high(GraphView g, HubRows hr,
                                                              const int64_t* __restrict__ hoff,
-                                                             unsigned long long* htab, ClusterArgs a,
-                                                             unsigned long long* ctr, uint32_t* err) {
+                                                             unsigned long long* htab, unsigned long long* part,
+                                                             ClusterArgs a, unsigned long long* ctr, uint32_t* err) {
   static_assert(kHiThreads >= kChunkRows, "one thread per row of a chunk");
   static_assert(kHiThreads % (32 * kRowGroups) == 0, "whole warps per row group");
   __shared__ unsigned long long stab[kSmemSlots];  // the groups' tables side by side, or one CTA table
@@ -523,6 +712,7 @@ __global__ void __launch_bounds__(kHiThreads, 5) k_cluster_high(GraphView g, Hub
   __shared__ int64_t s_rb[kChunkRows], s_re[kChunkRows], s_x0[kChunkRows];
   for (uint32_t s = threadIdx.x; s < kSmemSlots; s += blockDim.x) stab[s] = kEmptySlot;
   __syncthreads();
+  const bool single = cluster_single(a);
   const int64_t m_hub = hr.pre[hr.n_huge];
   for (int64_t ch = next_chunk(ctr, &s_ch); ch < hr.nchunks; ch = next_chunk(ctr, &s_ch)) {
     const int64_t cb = ch * kHubChunk, ce = min(cb + kHubChunk, m_hub);
@@ -538,12 +728,12 @@ __global__ void __launch_bounds__(kHiThreads, 5) k_cluster_high(GraphView g, Hub
       }
       const int64_t deg = re - rb;
       const bool first = rb >= cb;  // this chunk holds the row's first entry
-      // a row on the shared-memory path belongs to the chunk of its first entry
-      if (row && (deg > kSmemRowDeg || first)) {
+      // a row rated whole belongs to the chunk of its first entry
+      if (row && (deg > kBigRowDeg || first)) {
         const int32_t idx = hr.huge[r];
         const int32_t u = hr.hi[idx];
         if (cluster_active(a, u, deg)) {
-          v = u;
+          if (deg <= kSmemRowDeg || deg > kBigRowDeg || single) v = u;  // (else k_cluster_big)
           s_idx[threadIdx.x] = idx;
           s_own[threadIdx.x] = a.C[u];
           s_x0[threadIdx.x] = g.xadj[u] - rb;  // CSR position of flat entry f: x0 + f
@@ -568,15 +758,17 @@ __global__ void __launch_bounds__(kHiThreads, 5) k_cluster_high(GraphView g, Hub
         const int64_t deg = s_re[i] - s_rb[i];
         if (v < 0 || deg > kGroupRowDeg) continue;
         const int32_t own = s_own[i];
-        uint32_t size = 64;
-        while (size < 2 * (uint32_t)(deg + 1)) size <<= 1;
-        bool ok = true;
-        if (gr.tid == 0) ok = hub_insert(gtab, size - 1, own, 0);
-        ok &= hub_insert_range(g, a.C, s_x0[i] + s_rb[i], s_x0[i] + s_re[i], gtab, size - 1, gr);
-        if (!ok) atomicOr(err, ERR_CAPACITY);
-        gr.sync();
-        table_best<false>(gtab, 0, size, a, sx, gr, s_bs[gi], s_bh[gi], s_bt[gi]);
-        if (gr.tid == 0) cluster_request(a, v, own, s_bt[gi], g.vw[v]);
+        const int64_t e0 = s_x0[i] + s_rb[i];
+        int32_t best;
+        if (single) {
+          rate_single(g, a, e0, e0 + deg, sx, gr, s_bs[gi], s_bh[gi], s_bt[gi]);
+          best = s_bt[gi];
+        } else {
+          uint32_t size = 64;
+          while (size < 2 * (uint32_t)(deg + 1)) size <<= 1;
+          best = rate_row(g, a, e0, (int32_t)deg, own, gtab, size - 1, sx, gr, err);
+        }
+        if (gr.tid == 0) cluster_request(a, v, own, best, g.vw[v]);
       }
     }
     __syncthreads();  // the groups' tables are empty again: the whole table is the CTA's
@@ -587,26 +779,66 @@ __global__ void __launch_bounds__(kHiThreads, 5) k_cluster_high(GraphView g, Hub
       const int64_t rb = s_rb[i], re = s_re[i], deg = re - rb, x0 = s_x0[i];
       if (deg <= kGroupRowDeg) continue;  // rated by a row group above
       const int32_t own = s_own[i];
+      if (single) {
+        const int64_t fb = deg <= kBigRowDeg ? rb : max(rb, cb), fe = deg <= kBigRowDeg ? re : min(re, ce);
+        rate_single(g, a, x0 + fb, x0 + fe, sx, cta, s_bs[0], s_bh[0], s_bt[0]);
+        if (threadIdx.x == 0) {
+          if (deg <= kBigRowDeg) {
+            cluster_request(a, v, own, s_bt[0], g.vw[v]);
+          } else {  // this chunk's part; k_cluster_giant_finish combines them
+            const int64_t p = part_slot(ch, rb);
+            part[p] = ((unsigned long long)(uint32_t)s_bs[0] << 32) | (uint32_t)s_bt[0];
+            part[p + 1] = s_bh[0];
+          }
+        }
+        continue;
+      }
       bool ok = true;
       if (deg <= kSmemRowDeg) {
         uint32_t size = 64;
         while (size < 2 * (uint32_t)(deg + 1)) size <<= 1;
-        if (threadIdx.x == 0) ok = hub_insert(stab, size - 1, own, 0);
-        ok &= hub_insert_range(g, a.C, x0 + rb, x0 + re, stab, size - 1, cta);
-        if (!ok) atomicOr(err, ERR_CAPACITY);
-        __syncthreads();
-        table_best<false>(stab, 0, size, a, sx, cta, s_bs[0], s_bh[0], s_bt[0]);
-        if (threadIdx.x == 0) cluster_request(a, v, own, s_bt[0], g.vw[v]);
+        const int32_t best = rate_row(g, a, x0 + rb, (int32_t)deg, own, stab, size - 1, sx, cta, err);
+        if (threadIdx.x == 0) cluster_request(a, v, own, best, g.vw[v]);
         continue;
       }
       const int32_t idx = s_idx[i];
       const int64_t base = hoff[idx];
       const uint32_t mask = (uint32_t)(hoff[idx + 1] - base) - 1u;
       unsigned long long* T = htab + base;
-      if (rb >= cb && threadIdx.x == 0) ok = hub_insert(T, mask, own, 0);
+      if (rb >= cb && threadIdx.x == 0) ok = hub_insert(T, mask, own, 0) >= 0;
       ok &= hub_insert_range(g, a.C, x0 + max(rb, cb), x0 + min(re, ce), T, mask, cta);
       if (!ok) atomicOr(err, ERR_CAPACITY);
     }
+  }
+  leave_chunks(ctr);
+}
+
+// The rows of kSmemRowDeg + 1 .. kBigRowDeg entries, one CTA each (tickets over
+// their list `big` of huge[] positions): 512 threads and a 64 KB table (three
+// CTAs per SM) for the rows up to 4095 entries, 1024 threads and 128 KB for
+// the others; a row's phases wait on memory and barriers, so several rows per
+// SM run beside each other where the tables allow it.
+template <int kT>
+__global__ void __launch_bounds__(kT) k_cluster_big(GraphView g, HubRows hr, const int32_t* __restrict__ big,
+                                                    int32_t n_big, ClusterArgs a, unsigned long long* ctr,
+                                                    uint32_t* err) {
+  extern __shared__ __align__(16) unsigned long long btab[];  // [big_slots(kT)]
+  __shared__ BestScratch<kT / 32> sx;
+  __shared__ int64_t s_j;
+  if (cluster_single(a)) return;  // k_cluster_high rated them
+  for (uint32_t s = threadIdx.x; s < big_slots(kT); s += kT) btab[s] = kEmptySlot;
+  const RowGroup cta = cta_group();
+  for (int64_t j = next_chunk(ctr, &s_j); j < n_big; j = next_chunk(ctr, &s_j)) {
+    const int32_t r = big[j];
+    const int32_t deg = (int32_t)(hr.pre[r + 1] - hr.pre[r]);
+    if ((deg < kRowPer * 512) != (kT == 512)) continue;  // the other build's
+    const int32_t v = hr.hi[hr.huge[r]];
+    if (!cluster_active(a, v, deg)) continue;  // (k_cluster_high cleared its request)
+    uint32_t size = 64;
+    while (size < 2 * (uint32_t)(deg + 1)) size <<= 1;
+    const int32_t own = a.C[v];
+    const int32_t best = rate_row(g, a, g.xadj[v], deg, own, btab, size - 1, sx, cta, err);
+    if (threadIdx.x == 0) cluster_request(a, v, own, best, g.vw[v]);
   }
   leave_chunks(ctr);
 }
@@ -623,6 +855,7 @@ __global__ void __launch_bounds__(kHiThreads) k_cluster_giant(HubRows hr, const 
   __shared__ int64_t s_ch;
   __shared__ int32_t s_idx[kChunkRows];  // the chunk's active larger rows (-1: none)
   __shared__ int64_t s_rb[kChunkRows], s_re[kChunkRows];
+  if (cluster_single(a)) return;  // no tables: k_cluster_high stored the parts
   const int64_t m_hub = hr.pre[hr.n_huge];
   for (int64_t ch = next_chunk(ctr, &s_ch); ch < hr.nchunks; ch = next_chunk(ctr, &s_ch)) {
     const int64_t cb = ch * kHubChunk, ce = min(cb + kHubChunk, m_hub);
@@ -636,7 +869,7 @@ __global__ void __launch_bounds__(kHiThreads) k_cluster_giant(HubRows hr, const 
         re = hr.pre[r + 1];
         row = rb < ce;
       }
-      if (row && re - rb > kSmemRowDeg) {
+      if (row && re - rb > kBigRowDeg) {
         const int32_t j = hr.huge[r];
         if (cluster_active(a, hr.hi[j], re - rb)) idx = j;
       }
@@ -652,7 +885,7 @@ __global__ void __launch_bounds__(kHiThreads) k_cluster_giant(HubRows hr, const 
       const int64_t base = hoff[idx];
       const int64_t S = hoff[idx + 1] - base;
       const uint32_t s0 = (uint32_t)(S * (max(rb, cb) - rb) / deg), s1 = (uint32_t)(S * (min(re, ce) - rb) / deg);
-      table_best<true>(htab + base, s0, s1, a, sx, cta_group(), s_bs, s_bh, s_bt);
+      table_best(htab + base, s0, s1, a, sx, s_bs, s_bh, s_bt);
       if (threadIdx.x == 0) {
         const int64_t p = part_slot(ch, rb);
         part[p] = ((unsigned long long)(uint32_t)s_bs << 32) | (uint32_t)s_bt;
@@ -669,7 +902,7 @@ __global__ void k_cluster_giant_finish(HubRows hr, const unsigned long long* __r
                                        ClusterArgs a) {
   for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < hr.n_huge; r += (int64_t)gridDim.x * blockDim.x) {
     const int64_t rb = hr.pre[r], re = hr.pre[r + 1];
-    if (re - rb <= kSmemRowDeg) continue;
+    if (re - rb <= kBigRowDeg) continue;
     const int32_t v = hr.hi[hr.huge[r]];
     if (!cluster_active(a, v, re - rb)) continue;
     int32_t bs = -1, bt = INT32_MAX;
@@ -1411,14 +1644,25 @@ void launch_subround(Ctx& c, int lvl, int32_t r, int64_t wcap) {
     // one wave of resident CTAs over the chunks
     const int64_t res = (int64_t)c.num_sms * c.resident_blocks((const void*)k_cluster_high, kHiThreads, 0);
     const unsigned gh = (unsigned)std::max<int64_t>(1, std::min<int64_t>(L.n_hub_chunks, res));
-    k_cluster_high<<<gh, kHiThreads, 0, c.st>>>(view(L), hr, L.hi_off, c.htab, a, c.hub_ctr, c.errword);
+    k_cluster_high<<<gh, kHiThreads, 0, c.st>>>(view(L), hr, L.hi_off, c.htab, L.hub_part, a, c.hub_ctr, c.errword);
     count_launch();
-    const int64_t res2 = (int64_t)c.num_sms * c.resident_blocks((const void*)k_cluster_giant, kHiThreads, 0);
-    k_cluster_giant<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(L.n_hub_chunks, res2)), kHiThreads, 0, c.st>>>(
-        hr, L.hi_off, c.htab, L.hub_part, a, c.hub_ctr); count_launch();
-    k_cluster_giant_finish<<<grid_for(c, kThreads, L.n_huge), kThreads, 0, c.st>>>(hr, L.hub_part, L.vw, a);
-    count_launch();
-    // the three launches of the class together
+    if (L.n_big) {
+      k_cluster_big<512><<<(unsigned)std::min(L.n_big, 3 * c.num_sms), 512, big_slots(512) * sizeof(unsigned long long),
+                           c.st>>>(view(L), hr, L.hub_big, L.n_big, a, c.hub_ctr, c.errword); count_launch();
+      if (L.max_deg >= kRowPer * 512) {
+        k_cluster_big<1024><<<(unsigned)std::min(L.n_big, c.num_sms), 1024,
+                              big_slots(1024) * sizeof(unsigned long long), c.st>>>(
+            view(L), hr, L.hub_big, L.n_big, a, c.hub_ctr, c.errword); count_launch();
+      }
+    }
+    if (L.max_deg > kBigRowDeg) {
+      const int64_t res2 = (int64_t)c.num_sms * c.resident_blocks((const void*)k_cluster_giant, kHiThreads, 0);
+      k_cluster_giant<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(L.n_hub_chunks, res2)), kHiThreads, 0, c.st>>>(
+          hr, L.hi_off, c.htab, L.hub_part, a, c.hub_ctr); count_launch();
+      k_cluster_giant_finish<<<grid_for(c, kThreads, L.n_huge), kThreads, 0, c.st>>>(hr, L.hub_part, L.vw, a);
+      count_launch();
+    }
+    // the launches of the class together
     c.prof_end(ev, PK_CLUSTER_HIGH, 8 * (int64_t)L.n_huge + (8 * (int64_t)L.n_huge + 12 * L.m_huge) / 2);
   }
   k_cluster_classify<<<gv, kThreads, 0, c.st>>>(n, c.req, c.Wc, c.ReqW, wcap, flag, c.cfg.seed, lvl, c.sort.key[0],
@@ -1542,7 +1786,7 @@ int32_t cluster_level(Ctx& c, int lvl) {
   ClusterState* cs = c.cstate;
   bool graph_ran = false;
   if (c.use_graphs && !c.prof) {
-    const int64_t key[8] = {(int64_t)L.n, L.m, (int64_t)L.n_hi | ((int64_t)L.n_huge << 32), L.hi_slots, wcap,
+    const int64_t key[8] = {(int64_t)L.n | ((int64_t)L.n_big << 32), L.m, (int64_t)L.n_hi | ((int64_t)L.n_huge << 32), L.hi_slots, wcap,
                             (int64_t)(intptr_t)c.htab, (int64_t)(intptr_t)L.hub_chunk, L.n_hub_chunks};
     bool same = L.cgexec != nullptr;
     for (int i = 0; i < 8 && same; i++) same = L.cg_key[i] == key[i];
@@ -1601,7 +1845,7 @@ void free_level(Ctx& c, Level& L) {
   for (void* p : {(void*)L.xadj, (void*)L.adj, (void*)L.adjw, (void*)L.vw, (void*)L.pi, (void*)L.hi,
                   (void*)L.huge, (void*)L.hi_off, (void*)L.M, (void*)L.hub_pre, (void*)L.hub_chunk,
                   (void*)L.hub_part, (void*)L.hub_sidx, (void*)L.hub_split, (void*)L.hub_gtab,
-                  (void*)L.hub_acc})
+                  (void*)L.hub_acc, (void*)L.hub_big})
     if (p) c.mem.put(p);
   L = Level{};
 }
@@ -1720,6 +1964,15 @@ void coarsen_alloc(Ctx& c) {
   c.req = c.mem.make<int32_t>(n);
   c.rank = c.mem.make<int32_t>(2 * n + 2);
   c.hub_ctr = c.mem.make<unsigned long long>(2);
+  static std::atomic<unsigned long long> attr_done{0};  // one bit per device
+  const unsigned long long bit = 1ULL << (c.dev & 63);
+  if (!(attr_done.load() & bit)) {
+    GM_CUDA(cudaFuncSetAttribute(k_cluster_big<512>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(big_slots(512) * sizeof(unsigned long long))));
+    GM_CUDA(cudaFuncSetAttribute(k_cluster_big<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(big_slots(1024) * sizeof(unsigned long long))));
+    attr_done.fetch_or(bit);
+  }
   GM_CUDA(cudaMemsetAsync(c.hub_ctr, 0, 2 * sizeof(unsigned long long), c.st));
 }
 

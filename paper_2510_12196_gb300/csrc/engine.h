@@ -110,6 +110,9 @@ struct Level {
   int32_t* hub_split = nullptr;
   int32_t* hub_gtab = nullptr;
   int32_t n_split = 0;
+  int32_t* hub_big = nullptr;  // huge[] positions of the rows of kSmemRowDeg + 1 .. kBigRowDeg entries (clustering)
+  int32_t n_big = 0;
+  int64_t hub_big_cap = 0;
   int64_t hub_gtab_cap = 0;
   int64_t hub_split_deg = 0;
   int64_t hub_chunk_cap = 0;

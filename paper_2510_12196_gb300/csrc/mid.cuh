@@ -26,6 +26,11 @@ constexpr int64_t kHubChunk = 2048;
 constexpr int64_t kSpanChunks = 4;
 constexpr int kSpanRows = 256;  // rows of one span at most (rows there have more than kLowDeg + 1 entries)
 static_assert(kSpanChunks * kHubChunk / 34 + 2 <= kSpanRows, "a span's rows fit the per-span row table");
+// clustering: rows of at most kSmemRowDeg entries are rated by a CTA of the hub
+// kernel in shared memory, those up to kBigRowDeg by a CTA of their own kernel,
+// larger ones in global tables
+constexpr int64_t kSmemRowDeg = 2047;
+constexpr int64_t kBigRowDeg = 8191;
 // rows rated by one CTA whole (PE-code tables); larger rows sum chunk tables
 constexpr int64_t kSplitDeg = 4096;
 // bound of the per-level partial tables of the larger rows (else rated whole)

@@ -4536,6 +4536,24 @@ struct StoreSplit {
   }
 };
 
+// rows that the clustering rates in k_cluster_big
+struct LoadBig {
+  const int32_t* hi;
+  const int32_t* huge;
+  const int64_t* xadj;
+  __device__ int64_t operator()(int64_t j) const {
+    const int32_t v = hi[huge[j]];
+    const int64_t d = xadj[v + 1] - xadj[v];
+    return d > kSmemRowDeg && d <= kBigRowDeg ? 1 : 0;
+  }
+};
+struct StoreBig {
+  int32_t* list;
+  __device__ void operator()(int64_t j, int64_t e, int64_t x) const {
+    if (x) list[e] = (int32_t)j;
+  }
+};
+
 struct LoadHubDeg {
   const int32_t* hi;
   const int32_t* huge;
@@ -4559,6 +4577,7 @@ int64_t read_i64_at(Ctx& c, const int64_t* d) {
 void prepare_hubs(Ctx& c, Level& L, int64_t split_deg) {
   if (!L.n_huge) {
     L.n_hub_chunks = 0;
+    L.n_big = 0;
     return;
   }
   if (!L.hub_pre) L.hub_pre = c.mem.make<int64_t>((size_t)L.n + 1);
@@ -4585,12 +4604,24 @@ void prepare_hubs(Ctx& c, Level& L, int64_t split_deg) {
     L.hub_acc = c.mem.make<int64_t>((size_t)std::max(1, L.n));
     GM_CUDA(cudaMemsetAsync(L.hub_acc, 0, (size_t)std::max(1, L.n) * sizeof(int64_t), c.st));
   }
+  const int64_t big_cap = L.m / kSmemRowDeg + 1;
+  if (L.hub_big_cap < big_cap) {
+    if (L.cgexec) cudaGraphExecDestroy(L.cgexec);  // holds the old pointer
+    L.cgexec = nullptr;
+    if (L.hub_big) c.mem.put(L.hub_big);
+    L.hub_big = c.mem.make<int32_t>((size_t)big_cap);
+    L.hub_big_cap = big_cap;
+  }
+  scan(LoadBig{L.hi, L.huge, L.xadj}, StoreBig{L.hub_big}, L.n_huge, nullptr, c.scan, c.st);
+  GM_CUDA(cudaMemcpyAsync(c.h_small + 4, c.scan.tile_sums + std::max<int64_t>(1, scan_tiles(L.n_huge)), sizeof(int64_t),
+                          cudaMemcpyDeviceToHost, c.st));  // read with the next count
   // the rows whose PE-code tables are summed over chunks
   if (!L.hub_sidx) L.hub_sidx = c.mem.make<int32_t>((size_t)std::max(1, L.n));
   if (!L.hub_split) L.hub_split = c.mem.make<int32_t>((size_t)std::max(1, L.n));
   scan(LoadSplit{L.hi, L.huge, L.xadj, split_deg}, StoreSplit{L.hub_sidx, L.hub_split}, L.n_huge, nullptr, c.scan,
        c.st);
   int64_t ns = read_i64_at(c, c.scan.tile_sums + std::max<int64_t>(1, scan_tiles(L.n_huge)));
+  L.n_big = (int32_t)c.h_small[4];
   const int64_t need = ns * c.topo.kc;
   if (need * (int64_t)sizeof(int32_t) > kSplitTableBytes) {
     ns = 0;  // too many: every row is rated whole
