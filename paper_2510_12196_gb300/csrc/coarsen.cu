@@ -1623,48 +1623,55 @@ void launch_subround(Ctx& c, int lvl, int32_t r, int64_t wcap) {
   const int kbits = bits_for(n) + 32;
   ClusterArgs a{c.C, c.Wc, c.ReqW, c.req, wcap, c.cfg.seed, c.cstate, lvl, r};
   c.prof_level = lvl;
-  cudaEvent_t ev = c.prof_begin();
-  k_cluster_tile<<<tile_grid(c, (const void*)k_cluster_tile, n), kTileThreads, 0, c.st>>>(view(L), a); count_launch();
-  // per vertex: xadj 8, C 4, request 4 (+ hash, no memory); per entry: adjacency 4, weight 4, C(u) 4
-  c.prof_end(ev, PK_CLUSTER, 16 * (int64_t)(L.n - L.n_hi) + 12 * (L.m - L.m_hi));
+  cudaEvent_t ev = nullptr;
+  Branches br(c, L.n_hi > 0);
   // mid / high classes: xadj (8) of every listed vertex; the active half (the
   // sub-round's hash bit) also reads C and writes its request (8) and
   // streams its row (12 per entry): expected bytes
-  if (L.n_hi > L.n_huge) {
-    const int64_t nv = L.n_hi - L.n_huge, me = L.m_hi - L.m_huge;
-    ev = c.prof_begin();
-    k_cluster_mid<<<mid_grid(c, (const void*)k_cluster_mid, 0, L.n_hi), kMidThreads, 0, c.st>>>(view(L), L.hi,
-                                                                                                L.n_hi, a, c.errword);
-    count_launch();
-    c.prof_end(ev, PK_CLUSTER_MID, 8 * nv + (8 * nv + 12 * me) / 2);
-  }
-  if (L.n_huge) {
-    ev = c.prof_begin();
-    const HubRows hr = hub_rows(L);
-    // one wave of resident CTAs over the chunks
-    const int64_t res = (int64_t)c.num_sms * c.resident_blocks((const void*)k_cluster_high, kHiThreads, 0);
-    const unsigned gh = (unsigned)std::max<int64_t>(1, std::min<int64_t>(L.n_hub_chunks, res));
-    k_cluster_high<<<gh, kHiThreads, 0, c.st>>>(view(L), hr, L.hi_off, c.htab, L.hub_part, a, c.hub_ctr, c.errword);
-    count_launch();
-    if (L.n_big) {
-      k_cluster_big<512><<<(unsigned)std::min(L.n_big, 3 * c.num_sms), 512, big_slots(512) * sizeof(unsigned long long),
-                           c.st>>>(view(L), hr, L.hub_big, L.n_big, a, c.hub_ctr, c.errword); count_launch();
-      if (L.max_deg >= kRowPer * 512) {
-        k_cluster_big<1024><<<(unsigned)std::min(L.n_big, c.num_sms), 1024,
-                              big_slots(1024) * sizeof(unsigned long long), c.st>>>(
-            view(L), hr, L.hub_big, L.n_big, a, c.hub_ctr, c.errword); count_launch();
-      }
-    }
-    if (L.max_deg > kBigRowDeg) {
-      const int64_t res2 = (int64_t)c.num_sms * c.resident_blocks((const void*)k_cluster_giant, kHiThreads, 0);
-      k_cluster_giant<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(L.n_hub_chunks, res2)), kHiThreads, 0, c.st>>>(
-          hr, L.hi_off, c.htab, L.hub_part, a, c.hub_ctr); count_launch();
-      k_cluster_giant_finish<<<grid_for(c, kThreads, L.n_huge), kThreads, 0, c.st>>>(hr, L.hub_part, L.vw, a);
+  br.side([&] {
+    if (L.n_huge) {
+      ev = c.prof_begin();
+      const HubRows hr = hub_rows(L);
+      // one wave of resident CTAs over the chunks
+      const int64_t res = (int64_t)c.num_sms * c.resident_blocks((const void*)k_cluster_high, kHiThreads, 0);
+      const unsigned gh = (unsigned)std::max<int64_t>(1, std::min<int64_t>(L.n_hub_chunks, res));
+      k_cluster_high<<<gh, kHiThreads, 0, c.st>>>(view(L), hr, L.hi_off, c.htab, L.hub_part, a, c.hub_ctr, c.errword);
       count_launch();
+      if (L.n_big) {
+        k_cluster_big<512><<<(unsigned)std::min(L.n_big, 3 * c.num_sms), 512, big_slots(512) * sizeof(unsigned long long),
+                             c.st>>>(view(L), hr, L.hub_big, L.n_big, a, c.hub_ctr, c.errword); count_launch();
+        if (L.max_deg >= kRowPer * 512) {
+          k_cluster_big<1024><<<(unsigned)std::min(L.n_big, c.num_sms), 1024,
+                                big_slots(1024) * sizeof(unsigned long long), c.st>>>(
+              view(L), hr, L.hub_big, L.n_big, a, c.hub_ctr, c.errword); count_launch();
+        }
+      }
+      if (L.max_deg > kBigRowDeg) {
+        const int64_t res2 = (int64_t)c.num_sms * c.resident_blocks((const void*)k_cluster_giant, kHiThreads, 0);
+        k_cluster_giant<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(L.n_hub_chunks, res2)), kHiThreads, 0, c.st>>>(
+            hr, L.hi_off, c.htab, L.hub_part, a, c.hub_ctr); count_launch();
+        k_cluster_giant_finish<<<grid_for(c, kThreads, L.n_huge), kThreads, 0, c.st>>>(hr, L.hub_part, L.vw, a);
+        count_launch();
+      }
+      // the launches of the class together
+      c.prof_end(ev, PK_CLUSTER_HIGH, 8 * (int64_t)L.n_huge + (8 * (int64_t)L.n_huge + 12 * L.m_huge) / 2);
     }
-    // the launches of the class together
-    c.prof_end(ev, PK_CLUSTER_HIGH, 8 * (int64_t)L.n_huge + (8 * (int64_t)L.n_huge + 12 * L.m_huge) / 2);
-  }
+  });
+  br.side([&] {
+    if (L.n_hi > L.n_huge) {
+      const int64_t nv = L.n_hi - L.n_huge, me = L.m_hi - L.m_huge;
+      ev = c.prof_begin();
+      k_cluster_mid<<<mid_grid(c, (const void*)k_cluster_mid, 0, L.n_hi), kMidThreads, 0, c.st>>>(view(L), L.hi,
+                                                                                                  L.n_hi, a, c.errword);
+      count_launch();
+      c.prof_end(ev, PK_CLUSTER_MID, 8 * nv + (8 * nv + 12 * me) / 2);
+    }
+  });
+  ev = c.prof_begin();
+  k_cluster_tile<<<tile_grid(c, (const void*)k_cluster_tile, n), kTileThreads, 0, c.st>>>(view(L), a); count_launch();
+  // per vertex: xadj 8, C 4, request 4 (+ hash, no memory); per entry: adjacency 4, weight 4, C(u) 4
+  c.prof_end(ev, PK_CLUSTER, 16 * (int64_t)(L.n - L.n_hi) + 12 * (L.m - L.m_hi));
+  br.join();
   k_cluster_classify<<<gv, kThreads, 0, c.st>>>(n, c.req, c.Wc, c.ReqW, wcap, flag, c.cfg.seed, lvl, c.sort.key[0],
                                                 c.sort.val[0], c.cstate); count_launch();
   // contested requests: compaction in id order, stable sort by (target,

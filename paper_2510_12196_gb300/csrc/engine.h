@@ -2,6 +2,7 @@
 // hierarchy) and the entry points of the refinement and coarsening engines.
 #pragma once
 
+#include <algorithm>
 #include <stdexcept>
 #include <string>
 #include <unordered_map>
@@ -233,7 +234,6 @@ struct Ctx {
   int64_t* rem = nullptr;       // [kc] weight still to move inside the cut bucket
   int64_t* counters = nullptr;  // small device counters
   int64_t* Jacc = nullptr;
-  unsigned int* evctr = nullptr;  // blocks finished in a fused J evaluation
   RefineState* state = nullptr;
   RefineState* h_state = nullptr;  // pinned mirror
   int64_t* h_small = nullptr;      // pinned, a few values read back together
@@ -352,6 +352,52 @@ inline void cap_streams(Ctx& c) {
   for (auto& cs : c.cap.s)
     if (!cs) GM_CUDA(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
 }
+
+// Parallel branches of a captured graph: kernels of one step that write
+// disjoint data (the degree classes of a pass) all depend on the nodes before
+// the step and not on each other, so that one class's last wave does not hold
+// up the next class.  The launches stay on one stream; only the capture's
+// dependency set is moved.  Outside a capture (stream launches) the branches
+// run one after the other.
+class Branches {
+  using Nodes = std::vector<cudaGraphNode_t>;
+  cudaStream_t st;
+  bool on;
+  Nodes fork, tails;
+  Nodes deps() const {
+    cudaStreamCaptureStatus status;
+    const cudaGraphNode_t* d = nullptr;
+    const cudaGraphEdgeData* ed = nullptr;
+    size_t n = 0;
+    GM_CUDA(cudaStreamGetCaptureInfo(st, &status, nullptr, nullptr, &d, &ed, &n));
+    return Nodes(d, d + n);
+  }
+  void set(Nodes& n) const {
+    GM_CUDA(cudaStreamUpdateCaptureDependencies(st, n.data(), nullptr, n.size(), cudaStreamSetCaptureDependencies));
+  }
+  void add_tails() {  // the nodes the branch ended with (none of its own: nothing was launched)
+    for (cudaGraphNode_t x : deps())
+      if (std::find(fork.begin(), fork.end(), x) == fork.end()) tails.push_back(x);
+  }
+
+ public:
+  Branches(Ctx& c, bool want) : st(c.st), on(want && c.cap.on()) {
+    if (on) fork = deps();
+  }
+  // a branch beside the others; the launches after the last of these are one more
+  template <class F>
+  void side(F&& f) {
+    f();
+    if (!on) return;
+    add_tails();
+    set(fork);
+  }
+  void join() {
+    if (!on) return;
+    add_tails();
+    if (!tails.empty()) set(tails);
+  }
+};
 
 // initial.cu: breadth-first initial mapping of a large coarsest graph over the whole GPU; false when
 // its component labelling did not settle within its round limit (the caller then runs the one-CTA kernel)

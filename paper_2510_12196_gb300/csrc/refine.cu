@@ -120,30 +120,9 @@ struct CtlArgs {
   int32_t tcap;
 };
 
-// Controller attached to a J evaluation (s == nullptr: J only).
-struct EvalCtl {
-  RefineState* s;
-  unsigned int* ctr;  // blocks finished (zero between launches)
-  const int64_t* W;
-  CtlArgs a;
-  int phase;
-  cudaGraphConditionalHandle h;
-  int use_h;
-};
-__device__ void eval_finish(int64_t* Jacc, const EvalCtl& ec);
-
-// True when the J evaluation closing an Alg. 6 iteration has nothing to do:
-// after an LP or weak step the step itself added its exact change of J to the
-// accumulator, which the previous decision had set to the old J.
-__device__ __forceinline__ bool incremental_j(const RefineState* st, int phase) {
-  return st && phase == 1 && (st->kind == KIND_LP || st->kind == KIND_WEAK);
-}
-
 // J contribution of the low-degree vertices (warp tiles, one lane per vertex).
-// With a controller attached, the last block to finish runs the Alg. 6
-// decision on the complete J (the high-degree part is added before).
 __global__ void __launch_bounds__(kTileThreads, kTileMinBlocks) k_eval_tile(GraphView g, const int32_t* __restrict__ pi, Topo topo,
-                                                            int64_t* Jacc, EvalCtl ec) {
+                                                            int64_t* Jacc) {
   __shared__ int32_t sdist[32];
   __shared__ int64_t sm[33];
   __shared__ int32_t sc[kTileWarps][kTileE];
@@ -152,16 +131,6 @@ __global__ void __launch_bounds__(kTileThreads, kTileMinBlocks) k_eval_tile(Grap
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const TileGraph tg{g.n, g.xadj, g.adj, g.adjw};
-  if (incremental_j(ec.s, ec.phase)) {
-    // after an LP or weak step Jacc already holds J (old J + the exact
-    // change): the blocks only arrive, and the last one runs the decision.
-    // The decision rewrites the step kind that every block reads on entry,
-    // so it must wait for all of them: a block scheduled late (the SMs
-    // shared with other streams' kernels) would otherwise read the next
-    // step's kind and stream its tiles into the accumulator.
-    eval_finish(Jacc, ec);
-    return;
-  }
   const int64_t ntiles = ((int64_t)g.n + kTileV - 1) / kTileV;
   int64_t acc = 0;
   for (int64_t tile = (int64_t)blockIdx.x * kTileWarps + warp; tile < ntiles; tile += (int64_t)gridDim.x * kTileWarps) {
@@ -176,7 +145,6 @@ __global__ void __launch_bounds__(kTileThreads, kTileMinBlocks) k_eval_tile(Grap
   }
   acc = block_sum(acc, sm);
   if (threadIdx.x == 0 && acc) atomicAdd((unsigned long long*)Jacc, (unsigned long long)acc);
-  eval_finish(Jacc, ec);
 }
 
 // The high-degree kernels below come in two forms: one warp per vertex of
@@ -189,11 +157,9 @@ __device__ __forceinline__ int32_t hi_vertex(const int32_t* hi, const int32_t* s
 
 // J contribution of the vertices of degree in (kLowDeg, kMidDeg], one warp per vertex.
 __global__ void __launch_bounds__(kMidThreads) k_eval_mid(GraphView g, const int32_t* __restrict__ hi, int32_t n_hi,
-                                                          const int32_t* __restrict__ pi, Topo topo, int64_t* Jacc,
-                                                          const RefineState* st, int phase) {
+                                                          const int32_t* __restrict__ pi, Topo topo, int64_t* Jacc) {
   __shared__ int32_t sdist[32];
   __shared__ int64_t sm[33];
-  if (incremental_j(st, phase)) return;
   load_sdist(sdist, topo);
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -214,10 +180,9 @@ __global__ void __launch_bounds__(kMidThreads) k_eval_mid(GraphView g, const int
 // one wave (every entry's term is independent), so no CTA waits on a hub's
 // whole row; each thread follows the row of its own entries.
 __global__ void __launch_bounds__(kHiThreads) k_eval_high(GraphView g, HubRows hr, const int32_t* __restrict__ pi,
-                                                          Topo topo, int64_t* Jacc, const RefineState* st, int phase) {
+                                                          Topo topo, int64_t* Jacc) {
   __shared__ int32_t sdist[32];
   __shared__ int64_t sm[33];
-  if (incremental_j(st, phase)) return;
   load_sdist(sdist, topo);
   __syncthreads();
   const int64_t m_hub = hr.pre[hr.n_huge];
@@ -2239,31 +2204,22 @@ __device__ __forceinline__ int64_t next_j_base(const RefineState* s, int64_t J) 
   return (s->kind == KIND_LP || s->kind == KIND_WEAK) ? J : 0;
 }
 
-// Every block of a J evaluation arrives here once its part of J is in the
-// accumulator; the last one to arrive takes the Alg. 6 decision on the
-// complete J (all blocks have read the step kind by then).
-__device__ void eval_finish(int64_t* Jacc, const EvalCtl& ec) {
-  __shared__ unsigned int last;
+// The Alg. 6 decision that closes an iteration (phase 1) or the first J
+// evaluation (phase 0), once J is complete in the accumulator: after an LP or
+// weak step it holds the old J plus the step's exact change, after a strong
+// step and at the start a full evaluation.  A launch of its own: attached to
+// the last block of a J evaluation it cost every LP and weak iteration the
+// arrival of all that kernel's blocks (7-9 us; 2-3 us so).
+__global__ void __launch_bounds__(1024) k_control(RefineState* s, int64_t* Jacc, const int64_t* __restrict__ W,
+                                                  CtlArgs a, int phase, cudaGraphConditionalHandle h, int use_h) {
   __shared__ int64_t smax[32];
-  if (!ec.s) return;
-  __syncthreads();
+  const int64_t mx = block_max_w(W, a.kc, smax);
   if (threadIdx.x == 0) {
-    __threadfence();
-    last = atomicAdd(ec.ctr, 1u) == gridDim.x - 1 ? 1u : 0u;
-  }
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  const int64_t mx = block_max_w(ec.W, ec.a.kc, smax);
-  if (threadIdx.x == 0) {
-    const int64_t J = (int64_t)atomicAdd((unsigned long long*)Jacc, 0ULL);
-    *ec.ctr = 0;
-    control_step(ec.s, mx, J, ec.a, ec.phase, ec.h, ec.use_h);
-    *Jacc = next_j_base(ec.s, J);
+    const int64_t J = *Jacc;
+    control_step(s, mx, J, a, phase, h, use_h);
+    *Jacc = next_j_base(s, J);
   }
 }
-
-
 
 // Kernels run by one graph iteration: the fixed nodes plus the body of the
 // step that ran (the kind is recorded by k_control before it moves on).
@@ -2337,52 +2293,54 @@ void launch_hub_tab(Ctx& c, Level& L, const P& pol, size_t smem) {
   }
 }
 
-// J of the current mapping of a level; with `ec`, the last block of the
-// low-degree pass also takes the Alg. 6 decision (the high-degree pass runs
-// first so that J is complete then).
-// full: the launch streams the whole CSR (false when it only closes an LP or
-// weak step whose exact change of J is already accumulated)
-void launch_eval(Ctx& c, int lvl, const EvalCtl* ec = nullptr, bool full = true) {
+// Adds J of the current mapping of a level to the accumulator.
+void launch_eval(Ctx& c, int lvl) {
   Level& L = c.lv[lvl];
   c.prof_level = lvl;
   cudaEvent_t ev = nullptr;
   // per vertex xadj (8) + P(v) (4), per entry adjacency (4) + weight (4) + P(u) (4), per degree class
-  if (L.n_hi > L.n_huge) {
-    if (full) ev = c.prof_begin();
-    k_eval_mid<<<mid_grid(c, (const void*)k_eval_mid, 0, L.n_hi), kMidThreads, 0, c.st>>>(
-        view(L), L.hi, L.n_hi, L.pi, c.topo, c.Jacc, ec ? ec->s : nullptr, ec ? ec->phase : 0); count_launch();
-    if (full) c.prof_end(ev, PK_EVAL_MID, 12 * (int64_t)(L.n_hi - L.n_huge) + 12 * (L.m_hi - L.m_huge));
-  }
-  if (L.n_huge) {
-    if (full) ev = c.prof_begin();
+  Branches br(c, L.n_hi > 0);
+  br.side([&] {
+    if (!L.n_huge) return;
+    ev = c.prof_begin();
     k_eval_high<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(L.n_hub_chunks, (int64_t)c.num_sms * 8)), kHiThreads,
-                  0, c.st>>>(view(L), hub_rows(L), L.pi, c.topo, c.Jacc, ec ? ec->s : nullptr, ec ? ec->phase : 0);
-    count_launch();
-    if (full) c.prof_end(ev, PK_EVAL_HIGH, 12 * (int64_t)L.n_huge + 12 * L.m_huge);
-  }
+                  0, c.st>>>(view(L), hub_rows(L), L.pi, c.topo, c.Jacc); count_launch();
+    c.prof_end(ev, PK_EVAL_HIGH, 12 * (int64_t)L.n_huge + 12 * L.m_huge);
+  });
+  br.side([&] {
+    if (L.n_hi <= L.n_huge) return;
+    ev = c.prof_begin();
+    k_eval_mid<<<mid_grid(c, (const void*)k_eval_mid, 0, L.n_hi), kMidThreads, 0, c.st>>>(
+        view(L), L.hi, L.n_hi, L.pi, c.topo, c.Jacc); count_launch();
+    c.prof_end(ev, PK_EVAL_MID, 12 * (int64_t)(L.n_hi - L.n_huge) + 12 * (L.m_hi - L.m_huge));
+  });
   ev = c.prof_begin();
-  const EvalCtl none{nullptr, nullptr, nullptr, CtlArgs{}, 0, 0, 0};
-  k_eval_tile<<<tile_grid(c, (const void*)k_eval_tile, L.n), kTileThreads, 0, c.st>>>(view(L), L.pi, c.topo, c.Jacc,
-                                                                                       ec ? *ec : none); count_launch();
+  k_eval_tile<<<tile_grid(c, (const void*)k_eval_tile, L.n), kTileThreads, 0, c.st>>>(view(L), L.pi, c.topo, c.Jacc);
+  count_launch();
   // xadj (8) + P(v) (4) per vertex; adjacency (4) + weight (4) + gathered P(u) (4) per entry
-  if (full) c.prof_end(ev, PK_EVAL, 12 * (int64_t)(L.n - L.n_hi) + 12 * (L.m - L.m_hi));
-  else c.prof_end(ev, PK_EVAL_CTL, 0);
+  c.prof_end(ev, PK_EVAL, 12 * (int64_t)(L.n - L.n_hi) + 12 * (L.m - L.m_hi));
+  br.join();
 }
 
 template <class Mv>
 void launch_delta(Ctx& c, int lvl, Mv mv, int kind) {
   Level& L = c.lv[lvl];
-  k_delta_low<Mv><<<grid_for(c, kThreads, L.n), kThreads, 0, c.st>>>(view(L), L.pi, mv, c.topo, c.Jacc,
-                                                                                 c.state, kind); count_launch();
-  if (L.n_hi > L.n_huge) {
-    k_delta_mid<Mv><<<mid_grid(c, (const void*)k_delta_mid<Mv>, 0, L.n_hi), kMidThreads, 0, c.st>>>(
-        view(L), L.hi, L.n_hi, L.pi, mv, c.topo, c.Jacc, c.state, kind); count_launch();
-  }
+  Branches br(c, L.n_hi > 0);
   if (L.n_huge)
-    k_delta_high<Mv><<<(unsigned)std::max<int64_t>(
-                           1, std::min<int64_t>((L.n_hub_chunks + kSpanChunks - 1) / kSpanChunks, (int64_t)c.num_sms * 8)),
-                       kHiThreads, 0, c.st>>>(view(L), hub_rows(L), L.pi, mv, c.topo, c.Jacc, c.state, kind);
-  if (L.n_huge) count_launch();
+    br.side([&] {
+      k_delta_high<Mv><<<(unsigned)std::max<int64_t>(
+                             1, std::min<int64_t>((L.n_hub_chunks + kSpanChunks - 1) / kSpanChunks, (int64_t)c.num_sms * 8)),
+                         kHiThreads, 0, c.st>>>(view(L), hub_rows(L), L.pi, mv, c.topo, c.Jacc, c.state, kind);
+      count_launch();
+    });
+  if (L.n_hi > L.n_huge)
+    br.side([&] {
+      k_delta_mid<Mv><<<mid_grid(c, (const void*)k_delta_mid<Mv>, 0, L.n_hi), kMidThreads, 0, c.st>>>(
+          view(L), L.hi, L.n_hi, L.pi, mv, c.topo, c.Jacc, c.state, kind); count_launch();
+    });
+  k_delta_low<Mv><<<grid_for(c, kThreads, L.n), kThreads, 0, c.st>>>(view(L), L.pi, mv, c.topo, c.Jacc, c.state, kind);
+  count_launch();
+  br.join();
 }
 
 void launch_lp(Ctx& c, int lvl) {
@@ -2394,49 +2352,62 @@ void launch_lp(Ctx& c, int lvl) {
   const int32_t* gsel = mid_tab ? L.huge : nullptr;
   const int32_t ng = mid_tab ? L.n_huge : L.n_hi;
   c.prof_level = lvl;
-  cudaEvent_t ev = c.prof_begin();
+  cudaEvent_t ev = nullptr;
   const LpFilter flt{c.cfg.lp_relax_num, c.cfg.lp_relax_den};
+  Branches br(c, L.n_hi > 0);
+  br.side([&] {
+    if (ng) {
+      const int64_t me = mid_tab ? L.m_huge : L.m_hi;
+      ev = c.prof_begin();
+      if (mid_tab) {
+        const LpHubPolicy pol{L.pi, c.lock, c.pp, c.gain, c.inx, c.topo, glay, flt, c.state};
+        launch_hub_tab(c, L, pol, (size_t)glay.total * sizeof(int32_t));
+      } else {
+        k_lp_gain_high<<<std::max(1, std::min(ng, c.num_sms * 8)), kHiThreads, conn_smem(c), c.st>>>(
+            view(L), L.hi, gsel, ng, L.pi, c.lock, c.pp, c.gain, c.inx, c.topo, glay, flt, c.state); count_launch();
+      }
+      c.prof_end(ev, PK_LP_GAIN_HIGH, 26 * (int64_t)ng + 12 * me);
+    }
+  });
+  br.side([&] {
+    if (mid_tab && L.n_hi > L.n_huge) {
+      const size_t sm = mid_table_smem(glay.total);
+      ev = c.prof_begin();
+      k_lp_gain_mid<<<mid_grid(c, (const void*)k_lp_gain_mid, sm, L.n_hi), kMidThreads, sm, c.st>>>(
+          view(L), L.hi, L.n_hi, L.pi, c.lock, c.pp, c.gain, c.inx, c.topo, glay, flt, c.state); count_launch();
+      c.prof_end(ev, PK_LP_GAIN_MID, 26 * (int64_t)(L.n_hi - L.n_huge) + 12 * (L.m_hi - L.m_huge));
+    }
+  });
+  ev = c.prof_begin();
   k_lp_gain_tile<<<tile_grid(c, (const void*)k_lp_gain_tile, L.n), kTileThreads, 0, c.st>>>(view(L), L.pi, c.lock, c.pp, c.gain, c.inx, c.topo,
                                                                 flt, c.state); count_launch();
   // per vertex: xadj 8, P 4, lock 1, X 1, P' 4, g 8; per entry: adjacency 4, weight 4, gathered P(u) 4
   c.prof_end(ev, PK_LP_GAIN, 26 * (int64_t)(L.n - L.n_hi) + 12 * (L.m - L.m_hi));
-  if (mid_tab && L.n_hi > L.n_huge) {
-    const size_t sm = mid_table_smem(glay.total);
-    ev = c.prof_begin();
-    k_lp_gain_mid<<<mid_grid(c, (const void*)k_lp_gain_mid, sm, L.n_hi), kMidThreads, sm, c.st>>>(
-        view(L), L.hi, L.n_hi, L.pi, c.lock, c.pp, c.gain, c.inx, c.topo, glay, flt, c.state); count_launch();
-    c.prof_end(ev, PK_LP_GAIN_MID, 26 * (int64_t)(L.n_hi - L.n_huge) + 12 * (L.m_hi - L.m_huge));
-  }
-  if (ng) {
-    const int64_t me = mid_tab ? L.m_huge : L.m_hi;
-    ev = c.prof_begin();
-    if (mid_tab) {
-      const LpHubPolicy pol{L.pi, c.lock, c.pp, c.gain, c.inx, c.topo, glay, flt, c.state};
-      launch_hub_tab(c, L, pol, (size_t)glay.total * sizeof(int32_t));
-    } else {
-      k_lp_gain_high<<<std::max(1, std::min(ng, c.num_sms * 8)), kHiThreads, conn_smem(c), c.st>>>(
-          view(L), L.hi, gsel, ng, L.pi, c.lock, c.pp, c.gain, c.inx, c.topo, glay, flt, c.state); count_launch();
+  br.join();
+  Branches ba(c, L.n_hi > 0);
+  ba.side([&] {
+    if (L.n_huge) {
+      const int64_t res = (int64_t)c.num_sms * c.resident_blocks((const void*)k_lp_after_hub, kHiThreads, 0);
+      const int64_t spans = (L.n_hub_chunks + kSpanChunks - 1) / kSpanChunks;
+      k_lp_after_hub<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(spans, res)), kHiThreads, 0, c.st>>>(
+          view(L), hub_rows(L), L.pi, c.pp, c.gain, c.inx, L.hub_acc, c.topo, c.state, c.hub_ctr);
+      count_launch();
+      k_lp_after_hub_finish<<<grid_for(c, kThreads, L.n_huge), kThreads, 0, c.st>>>(hub_rows(L), c.inx, L.hub_acc,
+                                                                                  c.lock, c.state);
+      count_launch();
     }
-    c.prof_end(ev, PK_LP_GAIN_HIGH, 26 * (int64_t)ng + 12 * me);
-  }
+  });
+  ba.side([&] {
+    if (L.n_hi > L.n_huge) {
+      k_lp_after_mid<<<mid_grid(c, (const void*)k_lp_after_mid, 0, L.n_hi), kMidThreads, 0, c.st>>>(
+          view(L), L.hi, L.n_hi, L.pi, c.pp, c.gain, c.inx, c.lock, c.topo, c.state); count_launch();
+    }
+  });
   ev = c.prof_begin();
   k_lp_after_low<<<gl, kThreads, 0, c.st>>>(view(L), L.pi, c.pp, c.gain, c.inx, c.lock, c.topo, c.state); count_launch();
   // the X flag of every vertex (the work on X itself is data dependent)
   c.prof_end(ev, PK_LP_AFTER, (int64_t)(L.n - L.n_hi));
-  if (L.n_hi > L.n_huge) {
-    k_lp_after_mid<<<mid_grid(c, (const void*)k_lp_after_mid, 0, L.n_hi), kMidThreads, 0, c.st>>>(
-        view(L), L.hi, L.n_hi, L.pi, c.pp, c.gain, c.inx, c.lock, c.topo, c.state); count_launch();
-  }
-  if (L.n_huge) {
-    const int64_t res = (int64_t)c.num_sms * c.resident_blocks((const void*)k_lp_after_hub, kHiThreads, 0);
-    const int64_t spans = (L.n_hub_chunks + kSpanChunks - 1) / kSpanChunks;
-    k_lp_after_hub<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(spans, res)), kHiThreads, 0, c.st>>>(
-        view(L), hub_rows(L), L.pi, c.pp, c.gain, c.inx, L.hub_acc, c.topo, c.state, c.hub_ctr);
-    count_launch();
-    k_lp_after_hub_finish<<<grid_for(c, kThreads, L.n_huge), kThreads, 0, c.st>>>(hub_rows(L), c.inx, L.hub_acc,
-                                                                                c.lock, c.state);
-    count_launch();
-  }
+  ba.join();
   launch_delta(c, lvl, LpMoves{c.lock, c.pp}, KIND_LP);
   k_lp_apply<<<grid_for(c, kThreads, L.n), kThreads, 0, c.st>>>(L.n, L.pi, c.pp, c.lock, L.vw, c.W, c.topo.kc,
                                                                  c.state); count_launch();
@@ -2455,28 +2426,34 @@ void launch_rebalance(Ctx& c, int lvl, bool prep_done = false) {
     k_reb_prep<<<1, 1024, 0, c.st>>>(reb_prep_args(c), c.state); count_launch();
   }
   RebArgs a{c.W, c.U, c.counters, c.tab, c.lmax, c.cV, c.k, c.cfg.seed, c.cfg.reb_objective, c.topo};
-  k_reb_select_low<<<grid_for(c, kThreads, n), kThreads, 0, c.st>>>(view(L), L.pi, a, c.dest, bucket,
-                                                                                 c.elig, c.state); count_launch();
+  Branches br(c, L.n_hi > 0);
   if (L.n_hi) {
     const GroupLayout gl = group_layout(c.topo);
     const int32_t words = c.cfg.reb_objective ? gl.total : c.topo.kc;
     const size_t smem = (size_t)words * sizeof(int32_t);
     const bool mid_tab = mid_tables(c);
-    if (mid_tab && L.n_hi > L.n_huge) {
-      const size_t sm = mid_table_smem(words);
-      k_reb_select_mid<<<mid_grid(c, (const void*)k_reb_select_mid, sm, L.n_hi), kMidThreads, sm, c.st>>>(
-          view(L), L.hi, L.n_hi, L.pi, a, c.topo.kc, gl, c.dest, bucket, c.elig, c.state); count_launch();
-    }
     const int32_t ng = mid_tab ? L.n_huge : L.n_hi;
-    if (ng && mid_tab) {
-      const RebHubPolicy pol{L.pi, L.vw, a, gl, c.dest, bucket, c.elig, c.state};
-      launch_hub_tab(c, L, pol, smem);
-    } else if (ng) {
-      k_reb_select_high<<<std::max(1, std::min(ng, c.num_sms * 8)), kHiThreads, smem, c.st>>>(
-          view(L), L.hi, nullptr, ng, L.pi, a, c.topo.kc, gl, c.dest, bucket, c.elig, c.state);
-      count_launch();
-    }
+    if (ng)
+      br.side([&] {
+        if (mid_tab) {
+          const RebHubPolicy pol{L.pi, L.vw, a, gl, c.dest, bucket, c.elig, c.state};
+          launch_hub_tab(c, L, pol, smem);
+        } else {
+          k_reb_select_high<<<std::max(1, std::min(ng, c.num_sms * 8)), kHiThreads, smem, c.st>>>(
+              view(L), L.hi, nullptr, ng, L.pi, a, c.topo.kc, gl, c.dest, bucket, c.elig, c.state);
+          count_launch();
+        }
+      });
+    if (mid_tab && L.n_hi > L.n_huge)
+      br.side([&] {
+        const size_t sm = mid_table_smem(words);
+        k_reb_select_mid<<<mid_grid(c, (const void*)k_reb_select_mid, sm, L.n_hi), kMidThreads, sm, c.st>>>(
+            view(L), L.hi, L.n_hi, L.pi, a, c.topo.kc, gl, c.dest, bucket, c.elig, c.state); count_launch();
+      });
   }
+  k_reb_select_low<<<grid_for(c, kThreads, n), kThreads, 0, c.st>>>(view(L), L.pi, a, c.dest, bucket, c.elig, c.state);
+  count_launch();
+  br.join();
   const unsigned gcut = (unsigned)((c.topo.kc + kCutThreads / 32 - 1) / (kCutThreads / 32));
   k_reb_cut<<<gcut, kCutThreads, 0, c.st>>>(c.W, c.topo.kc, c.lmax, c.tab, c.bcut, c.rem, c.counters, c.state);
   count_launch();
@@ -3904,8 +3881,6 @@ void refine_alloc(Ctx& c) {
   GM_CUDA(cudaMemsetAsync(c.tab, 0, kc * kBuckets * sizeof(int64_t), c.st));
   c.counters = c.mem.make<int64_t>(CNT_N);
   c.Jacc = c.mem.make<int64_t>(2);
-  c.evctr = reinterpret_cast<unsigned int*>(c.mem.make<int64_t>(1));
-  GM_CUDA(cudaMemsetAsync(c.evctr, 0, sizeof(int64_t), c.st));
   c.state = c.mem.make<RefineState>(1);
   c.probe_state = c.mem.make<RefineState>(1);
   GM_CUDA(cudaMemsetAsync(c.probe_state, 0, sizeof(RefineState), c.st));  // kind 0 = KIND_LP
@@ -4000,9 +3975,9 @@ static void refine_stream(Ctx& c, int lvl, int32_t rounds, int64_t* J, int64_t* 
   *c.h_state = s;
   GM_CUDA(cudaMemcpyAsync(c.state, c.h_state, sizeof(RefineState), cudaMemcpyHostToDevice, c.st));
   GM_CUDA(cudaMemsetAsync(c.Jacc, 0, sizeof(int64_t), c.st));
-  const EvalCtl ec0{c.state, c.evctr, c.W, ctl_args(c), 0, 0, 0};
-  const EvalCtl ec1{c.state, c.evctr, c.W, ctl_args(c), 1, 0, 0};
-  launch_eval(c, lvl, &ec0);
+  const CtlArgs ca = ctl_args(c);
+  launch_eval(c, lvl);
+  k_control<<<1, 1024, 0, c.st>>>(c.state, c.Jacc, c.W, ca, 0, 0, 0); count_launch();
   const unsigned gcopy = grid_for(c, kThreads * 4, L.n);
   while (true) {
     GM_CUDA(cudaMemcpyAsync(c.h_state, c.state, sizeof(RefineState), cudaMemcpyDeviceToHost, c.st));
@@ -4013,9 +3988,14 @@ static void refine_stream(Ctx& c, int lvl, int32_t rounds, int64_t* J, int64_t* 
       launch_lp(c, lvl);
     } else {
       launch_rebalance(c, lvl);
-      if (h.kind == KIND_STRONG) launch_rebalance_strong_tail(c, lvl);
+      if (h.kind == KIND_STRONG) {
+        launch_rebalance_strong_tail(c, lvl);
+        launch_eval(c, lvl);
+      }
     }
-    launch_eval(c, lvl, &ec1, h.kind == KIND_STRONG);
+    cudaEvent_t ev = h.kind == KIND_STRONG ? nullptr : c.prof_begin();
+    k_control<<<1, 1024, 0, c.st>>>(c.state, c.Jacc, c.W, ca, 1, 0, 0); count_launch();
+    c.prof_end(ev, PK_EVAL_CTL, 0);
     k_copy_best<<<gcopy, kThreads, 0, c.st>>>(c.state, L.pi, c.pi_best, L.n, IterCounts{0, 0, 0, 0}); count_launch();
     GM_CUDA(cudaGetLastError());
   }
@@ -4038,7 +4018,7 @@ void drop_graph(Level& L) {
 
 // Captures one level's whole Alg. 6 run as a graph: initial J / weights, then
 // WHILE(not done) { decide; IF(LP){Alg. 4}; IF(weak or strong){Alg. 5};
-// IF(strong){strong tail}; J; control; copy best }, then best -> P.
+// IF(strong){strong tail; J}; control; copy best }, then best -> P.
 static void build_refine_graph(Ctx& c, int lvl, int32_t rounds) {
   Level& L = c.lv[lvl];
   drop_graph(L);
@@ -4061,9 +4041,8 @@ static void build_refine_graph(Ctx& c, int lvl, int32_t rounds) {
     k_state_init<<<1, 1, 0, cs>>>(c.state, rounds, lvl); count_launch();
     GM_CUDA(cudaMemsetAsync(c.Jacc, 0, sizeof(int64_t), cs));
     cudaGraphConditionalHandle h_loop = cap_handle(cs, 0);
-    const EvalCtl ec0{c.state, c.evctr, c.W, ca, 0, h_loop, 1};
-    const EvalCtl ec1{c.state, c.evctr, c.W, ca, 1, h_loop, 1};
-    launch_eval(c, lvl, &ec0);
+    launch_eval(c, lvl);
+    k_control<<<1, 1024, 0, cs>>>(c.state, c.Jacc, c.W, ca, 0, h_loop, 1); count_launch();
     cap_cond(c.cap, cs, h_loop, cudaGraphCondTypeWhile, [&](cudaStream_t bs) {
       c.st = bs;
       set_capture_counter(&n_fixed);
@@ -4085,10 +4064,11 @@ static void build_refine_graph(Ctx& c, int lvl, int32_t rounds) {
       cap_cond(c.cap, bs, h_strong, cudaGraphCondTypeIf, [&](cudaStream_t s2) {
         c.st = s2;
         launch_rebalance_strong_tail(c, lvl);
+        launch_eval(c, lvl);
       });
       set_capture_counter(&n_fixed);
       c.st = bs;
-      launch_eval(c, lvl, &ec1);
+      k_control<<<1, 1024, 0, bs>>>(c.state, c.Jacc, c.W, ca, 1, h_loop, 1); count_launch();
       // this node is the iteration's last: all body counts are known now
       const IterCounts ic{(unsigned long long)n_fixed + 1, (unsigned long long)n_lp, (unsigned long long)n_reb,
                           (unsigned long long)n_strong};
@@ -4725,7 +4705,7 @@ double probe_ms(Ctx& c, int lvl) {
   double best = 1e30;
   for (int rep = 0; rep < 2; rep++) {
     GM_CUDA(cudaEventRecord(e0, c.st));
-    launch_eval(c, lvl, nullptr, true);
+    launch_eval(c, lvl);
     if (L.n_hi > L.n_huge) {
       const size_t sm = mid_table_smem(glay.total);
       k_lp_gain_mid<<<mid_grid(c, (const void*)k_lp_gain_mid, sm, L.n_hi), kMidThreads, sm, c.st>>>(
