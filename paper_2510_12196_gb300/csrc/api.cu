@@ -457,13 +457,7 @@ map_status map_set_mapping(map_ctx* ctx, int32_t level, const int32_t* pi) {
   return guarded(ctx, [&](Ctx& c) {
     Level& L = level_at(c, level);
     if (!pi) throw ApiError(MAP_E_INVALID, "pi is NULL");
-    std::vector<int32_t> codes((size_t)L.n);
-    for (int32_t v = 0; v < L.n; v++) {
-      if (pi[v] < 0 || pi[v] >= c.k) throw ApiError(MAP_E_INVALID, "mapping entry out of [0, k)");
-      codes[(size_t)v] = c.code_of_pe[(size_t)pi[v]];
-    }
-    GM_CUDA(cudaMemcpyAsync(L.pi, codes.data(), codes.size() * sizeof(int32_t), cudaMemcpyHostToDevice, c.st));
-    sync(c);
+    upload_mapping(c, pi, L.n, L.pi);
   });
 }
 
@@ -471,9 +465,7 @@ map_status map_get_mapping(map_ctx* ctx, int32_t level, int32_t* pi) {
   return guarded(ctx, [&](Ctx& c) {
     Level& L = level_at(c, level);
     if (!pi) throw ApiError(MAP_E_INVALID, "pi is NULL");
-    GM_CUDA(cudaMemcpyAsync(pi, L.pi, (size_t)L.n * sizeof(int32_t), cudaMemcpyDeviceToHost, c.st));
-    sync(c);
-    for (int32_t v = 0; v < L.n; v++) pi[v] = c.pe_of_code[(size_t)pi[v]];
+    download_mapping(c, L.pi, L.n, pi);
   });
 }
 
@@ -509,13 +501,11 @@ map_status map_get_lp_state(map_ctx* ctx, int32_t level, int32_t* pi_prime, int6
   return guarded(ctx, [&](Ctx& c) {
     Level& L = level_at(c, level);
     const size_t n = (size_t)L.n;
-    if (pi_prime) GM_CUDA(cudaMemcpyAsync(pi_prime, c.pp, n * sizeof(int32_t), cudaMemcpyDeviceToHost, c.st));
+    if (pi_prime) download_mapping(c, c.pp, L.n, pi_prime);
     if (gain) GM_CUDA(cudaMemcpyAsync(gain, c.gain, n * sizeof(int64_t), cudaMemcpyDeviceToHost, c.st));
     if (in_x) GM_CUDA(cudaMemcpyAsync(in_x, c.inx, n, cudaMemcpyDeviceToHost, c.st));
     if (moved) GM_CUDA(cudaMemcpyAsync(moved, c.lock, n, cudaMemcpyDeviceToHost, c.st));
     sync(c);
-    if (pi_prime)
-      for (size_t v = 0; v < n; v++) pi_prime[v] = c.pe_of_code[(size_t)pi_prime[v]];
   });
 }
 
@@ -654,12 +644,7 @@ map_status map_run(map_ctx* ctx, int32_t* out_pi, int64_t* out_J) {
         }
       }
     }
-    if (out_pi) {
-      Level& L = c.lv[0];
-      GM_CUDA(cudaMemcpyAsync(out_pi, L.pi, (size_t)L.n * sizeof(int32_t), cudaMemcpyDeviceToHost, c.st));
-      sync(c);
-      for (int32_t v = 0; v < L.n; v++) out_pi[v] = c.pe_of_code[(size_t)out_pi[v]];
-    }
+    if (out_pi) download_mapping(c, c.lv[0].pi, c.lv[0].n, out_pi);
     if (out_J) *out_J = J;
   });
 }
@@ -670,12 +655,7 @@ map_status map_run_hm(map_ctx* ctx, int32_t workers, int32_t* out_pi, int64_t* o
     hm_run(c, 0, workers ? workers : 8, &c.hm);
     int64_t J = 0, mw = 0;
     objective(c, 0, &J, &mw);
-    if (out_pi) {
-      Level& L = c.lv[0];
-      GM_CUDA(cudaMemcpyAsync(out_pi, L.pi, (size_t)L.n * sizeof(int32_t), cudaMemcpyDeviceToHost, c.st));
-      sync(c);
-      for (int32_t v = 0; v < L.n; v++) out_pi[v] = c.pe_of_code[(size_t)out_pi[v]];
-    }
+    if (out_pi) download_mapping(c, c.lv[0].pi, c.lv[0].n, out_pi);
     if (out_J) *out_J = J;
   });
 }

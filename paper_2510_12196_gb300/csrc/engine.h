@@ -419,6 +419,10 @@ ContractSort contract_sort(Ctx& c, const Level& F, int32_t nc, int bits, int wbi
 // writes the coarse CSR (xadj nc + 1, adj and adjw s.mc entries)
 void contract_rows(Ctx& c, const ContractSort& s, int32_t nc, int64_t* xadj, int32_t* adj, int32_t* adjw);
 
+// mapping.cu: PE ids of the caller <-> PE codes on the device
+void download_mapping(Ctx& c, const int32_t* codes, int32_t n, int32_t* out);
+void upload_mapping(Ctx& c, const int32_t* pi, int32_t n, int32_t* codes);
+
 // match.cu
 int32_t match_level(Ctx& c, int lvl);  // two-hop matching of level lvl into its M; returns n_c
 
