@@ -2,7 +2,7 @@
 //
 // A warp takes 32 consecutive vertices.  The CSR entries of the whole tile
 // form one contiguous range [E0, E1); the warp streams it with coalesced
-// loads, four independent loads per lane in flight, gathers one 32-bit value
+// loads, eight independent loads per lane in flight, gathers one 32-bit value
 // per neighbour (its PE code or cluster label) and stores (value, weight)
 // pairs in shared memory.  Then every lane walks the entries of its own
 // vertex there.  Compared with one sub-warp per vertex, the dependent chain
@@ -73,25 +73,30 @@ __device__ __forceinline__ TileLane stage_tile(const TileGraph& g, int64_t v0, i
   const int64_t span = E1 - t.E0;
   t.staged = span <= kTE;
   if (t.staged) {
-    // every load of the tile is issued before any is used: one round trip
-    // for the adjacency and weights, one for the gathers
-    constexpr int kQ = kTE / 32;
-    int32_t u[kQ];
+    // by parts of 256 entries (a tile of a 3D grid has 192, of a random
+    // geometric graph 384): every load of a part is issued before any is used,
+    // one round trip for the adjacency and weights, one for the gathers (all
+    // 512 slots at once, most of them empty, cost k_lp_gain_tile 76 instead of
+    // 64 us on a 3D grid of 2^21 vertices)
+    constexpr int kQ = 8;
+    for (int j0 = 0; j0 < span; j0 += 32 * kQ) {
+      int32_t u[kQ];
 #pragma unroll
-    for (int q = 0; q < kQ; q++) {
-      const int jj = q * 32 + lane;
-      u[q] = (jj < span) ? g.adj[t.E0 + jj] : 0;
-      if (jj < span) sw[jj] = g.adjw[t.E0 + jj];
-    }
+      for (int q = 0; q < kQ; q++) {
+        const int jj = j0 + q * 32 + lane;
+        u[q] = (jj < span) ? g.adj[t.E0 + jj] : 0;
+        if (jj < span) sw[jj] = g.adjw[t.E0 + jj];
+      }
 #pragma unroll
-    for (int q = 0; q < kQ; q++) {
-      const int jj = q * 32 + lane;
-      if (jj < span) u[q] = gather(u[q]);
-    }
+      for (int q = 0; q < kQ; q++) {
+        const int jj = j0 + q * 32 + lane;
+        if (jj < span) u[q] = gather(u[q]);
+      }
 #pragma unroll
-    for (int q = 0; q < kQ; q++) {
-      const int jj = q * 32 + lane;
-      if (jj < span) sc[jj] = u[q];
+      for (int q = 0; q < kQ; q++) {
+        const int jj = j0 + q * 32 + lane;
+        if (jj < span) sc[jj] = u[q];
+      }
     }
   }
   __syncwarp();
@@ -114,23 +119,25 @@ __device__ __forceinline__ TileLane stage_tile_packed(const TileGraph& g, int64_
   const int64_t span = E1 - t.E0;
   t.staged = span <= kTE;
   if (t.staged) {
-    constexpr int kQ = kTE / 32;
-    int32_t u[kQ], w[kQ];
+    constexpr int kQ = 8;
+    for (int j0 = 0; j0 < span; j0 += 32 * kQ) {
+      int32_t u[kQ], w[kQ];
 #pragma unroll
-    for (int q = 0; q < kQ; q++) {
-      const int jj = q * 32 + lane;
-      u[q] = (jj < span) ? g.adj[t.E0 + jj] : 0;
-      w[q] = (jj < span) ? g.adjw[t.E0 + jj] : 0;
-    }
+      for (int q = 0; q < kQ; q++) {
+        const int jj = j0 + q * 32 + lane;
+        u[q] = (jj < span) ? g.adj[t.E0 + jj] : 0;
+        w[q] = (jj < span) ? g.adjw[t.E0 + jj] : 0;
+      }
 #pragma unroll
-    for (int q = 0; q < kQ; q++) {
-      const int jj = q * 32 + lane;
-      if (jj < span) u[q] = gather(u[q]);
-    }
+      for (int q = 0; q < kQ; q++) {
+        const int jj = j0 + q * 32 + lane;
+        if (jj < span) u[q] = gather(u[q]);
+      }
 #pragma unroll
-    for (int q = 0; q < kQ; q++) {
-      const int jj = q * 32 + lane;
-      if (jj < span) scw[jj] = make_int2(u[q], w[q]);
+      for (int q = 0; q < kQ; q++) {
+        const int jj = j0 + q * 32 + lane;
+        if (jj < span) scw[jj] = make_int2(u[q], w[q]);
+      }
     }
   }
   __syncwarp();
