@@ -1238,17 +1238,12 @@ __global__ void __launch_bounds__(1024) k_reb_prep(RebPrepArgs p, const RefineSt
   reb_prep_body(p, st->kind == KIND_STRONG);
 }
 
-// Graph mode: the start of one Alg. 6 iteration selects the step bodies and,
-// for a rebalancing step, prepares it.
-__global__ void __launch_bounds__(1024) k_decide_prep(const RefineState* s, cudaGraphConditionalHandle h_lp,
-                                                      cudaGraphConditionalHandle h_reb,
-                                                      cudaGraphConditionalHandle h_strong, RebPrepArgs p) {
+// Graph mode: the start of one Alg. 6 iteration tells whether the strong tail
+// runs and, for a rebalancing step, prepares it.
+__global__ void __launch_bounds__(1024) k_decide_prep(const RefineState* s, cudaGraphConditionalHandle h_strong,
+                                                      RebPrepArgs p) {
   const int32_t kind = s->kind;
-  if (threadIdx.x == 0) {
-    cudaGraphSetConditional(h_lp, kind == KIND_LP ? 1u : 0u);
-    cudaGraphSetConditional(h_reb, (kind == KIND_WEAK || kind == KIND_STRONG) ? 1u : 0u);
-    cudaGraphSetConditional(h_strong, kind == KIND_STRONG ? 1u : 0u);
-  }
+  if (threadIdx.x == 0) cudaGraphSetConditional(h_strong, kind == KIND_STRONG ? 1u : 0u);
   if (kind == KIND_WEAK || kind == KIND_STRONG) reb_prep_body(p, kind == KIND_STRONG);
 }
 
@@ -1924,7 +1919,10 @@ __global__ void __launch_bounds__(kSmallThreads) k_reb_resolve(const uint64_t* _
   int32_t* wcnt = vs + 2 * kSmallSort;
   __shared__ int32_t dbase[257];
   __shared__ int64_t sm[33];
-  if (!kind_is(st, (1 << KIND_WEAK) | (1 << KIND_STRONG))) return;
+  if (!kind_is(st, (1 << KIND_WEAK) | (1 << KIND_STRONG))) {
+    if (use_h && threadIdx.x == 0) cudaGraphSetConditional(h_big, 0u);  // (the list is an earlier step's)
+    return;
+  }
   const int64_t n64 = cnt[CNT_ELIG];
   if (use_h && threadIdx.x == 0) cudaGraphSetConditional(h_big, n64 > kSmallSort ? 1u : 0u);
   if (n64 <= 0 || n64 > kSmallSort) return;
@@ -2258,7 +2256,7 @@ __global__ void __launch_bounds__(1024) k_control(RefineState* s, int64_t* Jacc,
 // Kernels run by one graph iteration: the fixed nodes plus the body of the
 // step that ran (the kind is recorded by k_control before it moves on).
 struct IterCounts {
-  unsigned long long fixed, lp, reb, strong;
+  unsigned long long fixed, strong;
 };
 
 __global__ void k_state_init(RefineState* s, int32_t rounds, int32_t level) {
@@ -2271,9 +2269,7 @@ __global__ void k_state_init(RefineState* s, int32_t rounds, int32_t level) {
 __global__ void k_copy_best(RefineState* s, const int32_t* __restrict__ pi, int32_t* __restrict__ best, int32_t n,
                             IterCounts ic) {
   if (ic.fixed && blockIdx.x == 0 && threadIdx.x == 0) {
-    const int32_t k = s->last_kind;
-    s->kernels += ic.fixed + (k == KIND_LP ? ic.lp : 0) + ((k == KIND_WEAK || k == KIND_STRONG) ? ic.reb : 0) +
-                  (k == KIND_STRONG ? ic.strong : 0);
+    s->kernels += ic.fixed + (s->last_kind == KIND_STRONG ? ic.strong : 0);
   }
   if (!s->copy_best) return;
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
@@ -4033,7 +4029,7 @@ static void refine_stream(Ctx& c, int lvl, int32_t rounds, int64_t* J, int64_t* 
     cudaEvent_t ev = h.kind == KIND_STRONG ? nullptr : c.prof_begin();
     k_control<<<1, 1024, 0, c.st>>>(c.state, c.Jacc, c.W, ca, 1, 0, 0); count_launch();
     c.prof_end(ev, PK_EVAL_CTL, 0);
-    k_copy_best<<<gcopy, kThreads, 0, c.st>>>(c.state, L.pi, c.pi_best, L.n, IterCounts{0, 0, 0, 0}); count_launch();
+    k_copy_best<<<gcopy, kThreads, 0, c.st>>>(c.state, L.pi, c.pi_best, L.n, IterCounts{0, 0}); count_launch();
     GM_CUDA(cudaGetLastError());
   }
   GM_CUDA(cudaMemcpyAsync(L.pi, c.pi_best, (size_t)L.n * sizeof(int32_t), cudaMemcpyDeviceToDevice, c.st));
@@ -4054,8 +4050,11 @@ void drop_graph(Level& L) {
 }
 
 // Captures one level's whole Alg. 6 run as a graph: initial J / weights, then
-// WHILE(not done) { decide; IF(LP){Alg. 4}; IF(weak or strong){Alg. 5};
-// IF(strong){strong tail; J}; control; copy best }, then best -> P.
+// WHILE(not done) { prepare; Alg. 4 beside Alg. 5; IF(strong){strong tail; J};
+// control; copy best }, then best -> P.  The kernels of Alg. 4 and of Alg. 5
+// test the step's kind and the inactive ones leave at once, beside the active
+// chain: a conditional node costs 5 us whether its body runs or not, so only
+// the strong tail (whose scans do not test it) is one.
 static void build_refine_graph(Ctx& c, int lvl, int32_t rounds) {
   Level& L = c.lv[lvl];
   drop_graph(L);
@@ -4064,7 +4063,7 @@ static void build_refine_graph(Ctx& c, int lvl, int32_t rounds) {
   cudaStream_t cs = c.cap.s[0];
   const CtlArgs ca = ctl_args(c);
   const unsigned gcopy = grid_for(c, kThreads * 4, L.n);
-  long long root = 0, n_fixed = 0, n_lp = 0, n_reb = 0, n_strong = 0;
+  long long root = 0, n_fixed = 0, n_strong = 0;
   long long* outer = set_capture_counter(&root);
   GM_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeRelaxed));
   c.cap.depth = 0;
@@ -4083,20 +4082,12 @@ static void build_refine_graph(Ctx& c, int lvl, int32_t rounds) {
     cap_cond(c.cap, cs, h_loop, cudaGraphCondTypeWhile, [&](cudaStream_t bs) {
       c.st = bs;
       set_capture_counter(&n_fixed);
-      cudaGraphConditionalHandle h_lp = cap_handle(bs, 0), h_reb = cap_handle(bs, 0), h_strong = cap_handle(bs, 0);
-      // counts of the bodies are known only after they are captured: the
-      // decide node reads them from this iteration's parameters below
-      k_decide_prep<<<1, 1024, 0, bs>>>(c.state, h_lp, h_reb, h_strong, reb_prep_args(c)); count_launch();
-      set_capture_counter(&n_lp);
-      cap_cond(c.cap, bs, h_lp, cudaGraphCondTypeIf, [&](cudaStream_t s2) {
-        c.st = s2;
-        launch_lp(c, lvl);
-      });
-      set_capture_counter(&n_reb);
-      cap_cond(c.cap, bs, h_reb, cudaGraphCondTypeIf, [&](cudaStream_t s2) {
-        c.st = s2;
-        launch_rebalance(c, lvl, /*prep_done=*/true);
-      });
+      cudaGraphConditionalHandle h_strong = cap_handle(bs, 0);
+      k_decide_prep<<<1, 1024, 0, bs>>>(c.state, h_strong, reb_prep_args(c)); count_launch();
+      Branches steps(c, true);
+      steps.side([&] { launch_lp(c, lvl); });
+      launch_rebalance(c, lvl, /*prep_done=*/true);
+      steps.join();
       set_capture_counter(&n_strong);
       cap_cond(c.cap, bs, h_strong, cudaGraphCondTypeIf, [&](cudaStream_t s2) {
         c.st = s2;
@@ -4106,9 +4097,8 @@ static void build_refine_graph(Ctx& c, int lvl, int32_t rounds) {
       set_capture_counter(&n_fixed);
       c.st = bs;
       k_control<<<1, 1024, 0, bs>>>(c.state, c.Jacc, c.W, ca, 1, h_loop, 1); count_launch();
-      // this node is the iteration's last: all body counts are known now
-      const IterCounts ic{(unsigned long long)n_fixed + 1, (unsigned long long)n_lp, (unsigned long long)n_reb,
-                          (unsigned long long)n_strong};
+      // this node is the iteration's last: all counts are known now
+      const IterCounts ic{(unsigned long long)n_fixed + 1, (unsigned long long)n_strong};
       k_copy_best<<<gcopy, kThreads, 0, bs>>>(c.state, L.pi, c.pi_best, L.n, ic); count_launch();
       set_capture_counter(&root);
     });
