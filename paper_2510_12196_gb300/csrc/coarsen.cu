@@ -184,10 +184,11 @@ struct ClusterArgs {
   const ClusterState* cs;  // current iteration
   int32_t level;
   int32_t round;
+  int32_t it = 0;  // copy of cs->it (set by the kernel)
 };
 
 __device__ __forceinline__ bool cluster_active(const ClusterArgs& a, int32_t v, int64_t deg) {
-  return deg > 0 && (int32_t)((h_active(a.seed, a.level, v) >> a.cs->it) & 1ULL) == a.round;
+  return deg > 0 && (int32_t)((h_active(a.seed, a.level, v) >> a.it) & 1ULL) == a.round;
 }
 
 __device__ __forceinline__ void cluster_request(const ClusterArgs& a, int32_t v, int32_t own, int32_t best,
@@ -212,98 +213,104 @@ struct GatherLabel {
 // inside, as on power-law graphs) each sub-warp first copies its vertex's
 // row (at most kLowDeg entries) into its quarter of the warp's buffer.
 static_assert(kTileE / 4 >= kLowDeg, "a sub-warp's quarter of the staging buffer holds one low-degree row");
+template <class Gather>
+__device__ __forceinline__ void cluster_rate_tile(const GraphView& g, const ClusterArgs& a, int64_t tile, int lane,
+                                                  int2* scw, Gather gather, int max_deg) {
+  const int sub = lane >> 3, sl = lane & 7;
+  const TileGraph tg{g.n, g.xadj, g.adj, g.adjw};
+  const TileLane t = stage_tile_packed(tg, tile * kTileV, lane, scw, gather);
+  const int deg = (int)(t.e - t.b);
+  const bool low = t.v < g.n && deg <= max_deg;
+  const bool active = low && cluster_active(a, (int32_t)t.v, deg);
+  int32_t own = active ? a.C[t.v] : -1;
+  if (low && !active) a.req[t.v] = -1;
+  const unsigned work = __ballot_sync(0xffffffffu, active);
+  const int rank = __popc(work & ((1u << lane) - 1u));
+  const int rounds = (__popc(work) + 3) / 4;
+  for (int r = 0; r < rounds; r++) {
+    const int src = tile_worker_ranked(work, rank, r, sub, lane);
+    const int s2 = src < 0 ? 0 : src;
+    const int64_t vb = __shfl_sync(0xffffffffu, t.b, s2);
+    int off = (int)(vb - t.E0);
+    const int dg = (int)(__shfl_sync(0xffffffffu, t.e, s2) - vb);
+    const int32_t ow = __shfl_sync(0xffffffffu, own, s2);
+    if (!t.staged) {  // warp-uniform
+      off = sub * (kTileE / 4);
+      __syncwarp();  // the previous round has read this quarter
+      if (src >= 0)
+        for (int j = sl; j < dg; j += kSubWarp) scw[off + j] = make_int2(gather(g.adj[vb + j]), g.adjw[vb + j]);
+      __syncwarp();
+    }
+    const int2* cw = scw + off;
+    // best (score, tie-hash, label) over this lane's candidates; the hash
+    // of the current best is computed once, on the first tie
+    int32_t bs = 0, bt = -1, so = 0;
+    uint64_t bh = 0;
+    bool bhk = false;
+    if (src >= 0) {
+      for (int j = sl; j < dg; j += kSubWarp) {
+        const int2 xj = cw[j];
+        const int32_t cj = xj.x;
+        so += (cj == ow) ? xj.y : 0;
+        if (cj == ow || cj == bt) continue;
+        int32_t scj = 0;
+#pragma unroll 4
+        for (int l = 0; l < dg; l++) {
+          const int2 x = cw[l];
+          scj += (x.x == cj) ? x.y : 0;
+        }
+        if (bt < 0 || scj > bs) {
+          bs = scj;
+          bt = cj;
+          bhk = false;
+          continue;
+        }
+        if (scj < bs) continue;
+        if (!bhk) {
+          bh = h_tie(a.seed, a.level, bt);
+          bhk = true;
+        }
+        const uint64_t hj = h_tie(a.seed, a.level, cj);
+        if (hj < bh || (hj == bh && cj < bt)) {
+          bt = cj;
+          bh = hj;
+        }
+      }
+    }
+    if (bt >= 0 && !bhk) bh = h_tie(a.seed, a.level, bt);
+#pragma unroll
+    for (int o = kSubWarp / 2; o > 0; o >>= 1) {
+      so += __shfl_xor_sync(0xffffffffu, so, o);
+      const int32_t os = __shfl_xor_sync(0xffffffffu, bs, o);
+      const int32_t ot = __shfl_xor_sync(0xffffffffu, bt, o);
+      const uint64_t oh = __shfl_xor_sync(0xffffffffu, bh, o);
+      if (ot >= 0 && (bt < 0 || os > bs || (os == bs && (oh < bh || (oh == bh && ot < bt))))) {
+        bs = os;
+        bt = ot;
+        bh = oh;
+      }
+    }
+    if (src >= 0 && sl == 0) {
+      const int32_t v = (int32_t)(tile * kTileV + src);
+      // against the own cluster: larger score, then smaller tie-hash, then smaller label
+      bool take = bt >= 0 && bs >= so;
+      if (take && bs == so) {
+        const uint64_t ho = h_tie(a.seed, a.level, ow);
+        take = bh < ho || (bh == ho && bt < ow);
+      }
+      cluster_request(a, v, ow, take ? bt : ow, g.vw[v]);
+    }
+  }
+  __syncwarp();
+}
+
 __global__ void __launch_bounds__(kTileThreads, 9) k_cluster_tile(GraphView g, ClusterArgs a) {
   __shared__ int2 scw[kTileWarps][kTileE];  // (label, weight) per staged entry
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int sub = lane >> 3, sl = lane & 7;
-  const TileGraph tg{g.n, g.xadj, g.adj, g.adjw};
+  a.it = a.cs->it;
   const int64_t ntiles = ((int64_t)g.n + kTileV - 1) / kTileV;
-  for (int64_t tile = (int64_t)blockIdx.x * kTileWarps + warp; tile < ntiles; tile += (int64_t)gridDim.x * kTileWarps) {
-    const TileLane t = stage_tile_packed(tg, tile * kTileV, lane, scw[warp], GatherLabel{a.C});
-    const int deg = (int)(t.e - t.b);
-    const bool low = t.v < g.n && deg <= kLowDeg;
-    const bool active = low && cluster_active(a, (int32_t)t.v, deg);
-    int32_t own = active ? a.C[t.v] : -1;
-    if (low && !active) a.req[t.v] = -1;
-    const unsigned work = __ballot_sync(0xffffffffu, active);
-    const int rank = __popc(work & ((1u << lane) - 1u));
-    const int rounds = (__popc(work) + 3) / 4;
-    for (int r = 0; r < rounds; r++) {
-      const int src = tile_worker_ranked(work, rank, r, sub, lane);
-      const int s2 = src < 0 ? 0 : src;
-      const int64_t vb = __shfl_sync(0xffffffffu, t.b, s2);
-      int off = (int)(vb - t.E0);
-      const int dg = (int)(__shfl_sync(0xffffffffu, t.e, s2) - vb);
-      const int32_t ow = __shfl_sync(0xffffffffu, own, s2);
-      if (!t.staged) {  // warp-uniform
-        off = sub * (kTileE / 4);
-        __syncwarp();  // the previous round has read this quarter
-        if (src >= 0)
-          for (int j = sl; j < dg; j += kSubWarp) scw[warp][off + j] = make_int2(a.C[g.adj[vb + j]], g.adjw[vb + j]);
-        __syncwarp();
-      }
-      const int2* cw = scw[warp] + off;
-      // best (score, tie-hash, label) over this lane's candidates; the hash
-      // of the current best is computed once, on the first tie
-      int32_t bs = 0, bt = -1, so = 0;
-      uint64_t bh = 0;
-      bool bhk = false;
-      if (src >= 0) {
-        for (int j = sl; j < dg; j += kSubWarp) {
-          const int2 xj = cw[j];
-          const int32_t cj = xj.x;
-          so += (cj == ow) ? xj.y : 0;
-          if (cj == ow || cj == bt) continue;
-          int32_t scj = 0;
-#pragma unroll 4
-          for (int l = 0; l < dg; l++) {
-            const int2 x = cw[l];
-            scj += (x.x == cj) ? x.y : 0;
-          }
-          if (bt < 0 || scj > bs) {
-            bs = scj;
-            bt = cj;
-            bhk = false;
-            continue;
-          }
-          if (scj < bs) continue;
-          if (!bhk) {
-            bh = h_tie(a.seed, a.level, bt);
-            bhk = true;
-          }
-          const uint64_t hj = h_tie(a.seed, a.level, cj);
-          if (hj < bh || (hj == bh && cj < bt)) {
-            bt = cj;
-            bh = hj;
-          }
-        }
-      }
-      if (bt >= 0 && !bhk) bh = h_tie(a.seed, a.level, bt);
-#pragma unroll
-      for (int o = kSubWarp / 2; o > 0; o >>= 1) {
-        so += __shfl_xor_sync(0xffffffffu, so, o);
-        const int32_t os = __shfl_xor_sync(0xffffffffu, bs, o);
-        const int32_t ot = __shfl_xor_sync(0xffffffffu, bt, o);
-        const uint64_t oh = __shfl_xor_sync(0xffffffffu, bh, o);
-        if (ot >= 0 && (bt < 0 || os > bs || (os == bs && (oh < bh || (oh == bh && ot < bt))))) {
-          bs = os;
-          bt = ot;
-          bh = oh;
-        }
-      }
-      if (src >= 0 && sl == 0) {
-        const int32_t v = (int32_t)(tile * kTileV + src);
-        // against the own cluster: larger score, then smaller tie-hash, then smaller label
-        bool take = bt >= 0 && bs >= so;
-        if (take && bs == so) {
-          const uint64_t ho = h_tie(a.seed, a.level, ow);
-          take = bh < ho || (bh == ho && bt < ow);
-        }
-        cluster_request(a, v, ow, take ? bt : ow, g.vw[v]);
-      }
-    }
-    __syncwarp();
-  }
+  for (int64_t tile = (int64_t)blockIdx.x * kTileWarps + warp; tile < ntiles; tile += (int64_t)gridDim.x * kTileWarps)
+    cluster_rate_tile(g, a, tile, lane, scw[warp], GatherLabel{a.C}, kLowDeg);
 }
 
 __device__ __forceinline__ uint32_t slot_hash(int32_t t) {
@@ -444,7 +451,7 @@ struct BestScratch {
 using HubScratch = BestScratch<kHiThreads / 32>;
 
 // Whether the labels are still the vertices themselves (the first sub-round of a level).
-__device__ __forceinline__ bool cluster_single(const ClusterArgs& a) { return a.cs->it == 0 && a.round == 0; }
+__device__ __forceinline__ bool cluster_single(const ClusterArgs& a) { return a.it == 0 && a.round == 0; }
 
 __device__ __forceinline__ bool label_before(uint64_t h, int32_t t, uint64_t bh, int32_t bt) {
   return h < bh || (h == bh && t < bt);
@@ -710,6 +717,7 @@ __global__ void __launch_bounds__(kHiThreads, 5) k_cluster_high(GraphView g, Hub
   __shared__ int32_t s_v[kChunkRows];  // -1: nothing for this chunk to do
   __shared__ int32_t s_own[kChunkRows], s_idx[kChunkRows];
   __shared__ int64_t s_rb[kChunkRows], s_re[kChunkRows], s_x0[kChunkRows];
+  a.it = a.cs->it;
   for (uint32_t s = threadIdx.x; s < kSmemSlots; s += blockDim.x) stab[s] = kEmptySlot;
   __syncthreads();
   const bool single = cluster_single(a);
@@ -825,6 +833,7 @@ __global__ void __launch_bounds__(kT) k_cluster_big(GraphView g, HubRows hr, con
   extern __shared__ __align__(16) unsigned long long btab[];  // [big_slots(kT)]
   __shared__ BestScratch<kT / 32> sx;
   __shared__ int64_t s_j;
+  a.it = a.cs->it;
   if (cluster_single(a)) return;  // k_cluster_high rated them
   for (uint32_t s = threadIdx.x; s < big_slots(kT); s += kT) btab[s] = kEmptySlot;
   const RowGroup cta = cta_group();
@@ -855,6 +864,7 @@ __global__ void __launch_bounds__(kHiThreads) k_cluster_giant(HubRows hr, const 
   __shared__ int64_t s_ch;
   __shared__ int32_t s_idx[kChunkRows];  // the chunk's active larger rows (-1: none)
   __shared__ int64_t s_rb[kChunkRows], s_re[kChunkRows];
+  a.it = a.cs->it;
   if (cluster_single(a)) return;  // no tables: k_cluster_high stored the parts
   const int64_t m_hub = hr.pre[hr.n_huge];
   for (int64_t ch = next_chunk(ctr, &s_ch); ch < hr.nchunks; ch = next_chunk(ctr, &s_ch)) {
@@ -900,6 +910,7 @@ __global__ void __launch_bounds__(kHiThreads) k_cluster_giant(HubRows hr, const 
 // slices, then its request.
 __global__ void k_cluster_giant_finish(HubRows hr, const unsigned long long* __restrict__ part, const int32_t* vw,
                                        ClusterArgs a) {
+  a.it = a.cs->it;
   for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < hr.n_huge; r += (int64_t)gridDim.x * blockDim.x) {
     const int64_t rb = hr.pre[r], re = hr.pre[r + 1];
     if (re - rb <= kBigRowDeg) continue;
@@ -952,6 +963,7 @@ __global__ void __launch_bounds__(kMidThreads) k_cluster_mid(GraphView g, const 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int32_t* K = sk[warp];
   int32_t* V = sv[warp];
+  a.it = a.cs->it;
   for (int s = lane; s < kMidSlots; s += 32) {
     K[s] = -1;
     V[s] = 0;
@@ -1058,52 +1070,61 @@ __global__ void k_cluster_classify(int32_t n, const int32_t* __restrict__ req, c
 // does not depend on the append order) and admits each while the target's
 // weight plus the requests up to it stay within the cap.  Longer lists take
 // the multi-CTA path (scan compaction in id order, stable radix sort).
+struct ResolveSmem {
+  uint64_t sk[kSmallThreads];
+  int32_t sv[kSmallThreads];
+  uint64_t ok[kSmallThreads];
+  int32_t ov[kSmallThreads];
+  int64_t ex[kSmallThreads];
+  int64_t sm[33];
+};
+__device__ __forceinline__ void cluster_resolve(const uint64_t* key, const int32_t* val, int n, const int32_t* Wc,
+                                                const int32_t* __restrict__ vw, int64_t wcap, uint8_t* flag,
+                                                ResolveSmem& R) {
+  const int i = threadIdx.x;
+  uint64_t ki = 0;
+  int32_t vi = 0;
+  if (i < n) {
+    ki = key[i];
+    vi = val[i];
+    R.sk[i] = ki;
+    R.sv[i] = vi;
+  }
+  __syncthreads();
+  if (i < n) {
+    int r = 0;
+    for (int j = 0; j < n; j++) {
+      const uint64_t kj = R.sk[j];
+      r += (kj < ki || (kj == ki && R.sv[j] < vi)) ? 1 : 0;
+    }
+    R.ok[r] = ki;
+    R.ov[r] = vi;
+  }
+  __syncthreads();
+  const int64_t c = i < n ? (int64_t)vw[R.ov[i]] : 0;
+  int64_t tot;
+  const int64_t e = block_exclusive_scan(c, R.sm, &tot);
+  R.ex[i] = e;
+  __syncthreads();
+  if (i < n) {
+    const uint32_t t = (uint32_t)(R.ok[i] >> 32);
+    int h = i;
+    while (h > 0 && (uint32_t)(R.ok[h - 1] >> 32) == t) h--;  // first request of the same target
+    flag[R.ov[i]] = ((int64_t)Wc[t] + (e + c - R.ex[h]) <= wcap) ? 1 : 0;
+  }
+}
+
 __global__ void __launch_bounds__(kSmallThreads) k_cluster_resolve(const uint64_t* __restrict__ key,
                                                                    const int32_t* __restrict__ val,
                                                                    const ClusterState* cs,
                                                                    const int32_t* __restrict__ Wc,
                                                                    const int32_t* __restrict__ vw, int64_t wcap,
                                                                    uint8_t* flag, cudaGraphConditionalHandle h_big) {
-  __shared__ uint64_t sk[kSmallThreads];
-  __shared__ int32_t sv[kSmallThreads];
-  __shared__ uint64_t ok[kSmallThreads];
-  __shared__ int32_t ov[kSmallThreads];
-  __shared__ int64_t ex[kSmallThreads];
-  __shared__ int64_t sm[33];
-  const int64_t n64 = cs->ncont;
-  if (threadIdx.x == 0) cudaGraphSetConditional(h_big, n64 > kSmallThreads ? 1u : 0u);
-  if (n64 <= 0 || n64 > kSmallThreads) return;
-  const int n = (int)n64, i = threadIdx.x;
-  uint64_t ki = 0;
-  int32_t vi = 0;
-  if (i < n) {
-    ki = key[i];
-    vi = val[i];
-    sk[i] = ki;
-    sv[i] = vi;
-  }
-  __syncthreads();
-  if (i < n) {
-    int r = 0;
-    for (int j = 0; j < n; j++) {
-      const uint64_t kj = sk[j];
-      r += (kj < ki || (kj == ki && sv[j] < vi)) ? 1 : 0;
-    }
-    ok[r] = ki;
-    ov[r] = vi;
-  }
-  __syncthreads();
-  const int64_t c = i < n ? (int64_t)vw[ov[i]] : 0;
-  int64_t tot;
-  const int64_t e = block_exclusive_scan(c, sm, &tot);
-  ex[i] = e;
-  __syncthreads();
-  if (i < n) {
-    const uint32_t t = (uint32_t)(ok[i] >> 32);
-    int h = i;
-    while (h > 0 && (uint32_t)(ok[h - 1] >> 32) == t) h--;  // first request of the same target
-    flag[ov[i]] = ((int64_t)Wc[t] + (e + c - ex[h]) <= wcap) ? 1 : 0;
-  }
+  __shared__ ResolveSmem R;
+  const int64_t n = cs->ncont;
+  if (threadIdx.x == 0) cudaGraphSetConditional(h_big, n > kSmallThreads ? 1u : 0u);
+  if (n <= 0 || n > kSmallThreads) return;
+  cluster_resolve(key, val, (int)n, Wc, vw, wcap, flag, R);
 }
 
 struct LoadContested {
@@ -1192,6 +1213,157 @@ __global__ void k_cl_end(ClusterState* cs, int32_t n, int32_t iters, cudaGraphCo
   cs->it += 1;
   cs->done = stop ? 1 : 0;
   if (use_h) cudaGraphSetConditional(h, stop ? 0u : 1u);
+}
+
+// The whole clustering loop of a small level in one launch, by one cluster of
+// CTAs: the phases of a sub-round (ratings | classification | moves) are
+// separated by cluster barriers instead of kernel boundaries.  On a level of a
+// few thousand vertices the graph of kernels is all launch gaps (and its
+// capture and instantiation, paid by every new level, cost as much as a run):
+// map of a 16^3 grid 4.3 -> 3.5 ms, hierarchical multisection of an RGG of 2^17
+// vertices (37 maps by 8 threads) 63 -> 38 ms.
+// For levels of at most kClEngMaxN vertices without rows above kClEngRow and
+// with few above kLowDeg (a sub-warp takes each).  Contested requests: up to
+// kSmallThreads are ordered by the first CTA; of longer lists every CTA ranks
+// its share of the entries (by counting) into the second sort buffers, and the
+// first CTA takes the per-target prefixes.
+constexpr int kClEngThreads = 1024;
+constexpr int kClEngMaxN = 1 << 15;
+constexpr int kClEngMaxCluster = 8;  // the portable limit
+constexpr int kClEngRow = kTileE / 4;
+static_assert(kClEngThreads == kSmallThreads, "the resolution takes one request per thread");
+struct PlainLabel {  // labels change inside the launch: plain loads
+  const int32_t* C;
+  __device__ __forceinline__ int32_t operator()(int32_t u) const { return C[u]; }
+};
+struct ClusterEngineArgs {
+  int32_t* C;
+  int32_t* Wc;
+  int32_t* ReqW;
+  uint8_t* flag;
+  uint64_t* key[2];
+  int32_t* val[2];
+  int64_t* P;
+  int64_t* headP;
+  ClusterState* cs;
+  int32_t iters;
+};
+__global__ void __launch_bounds__(kClEngThreads, 1) k_cluster_engine(GraphView g, ClusterArgs a, ClusterEngineArgs e) {
+  extern __shared__ __align__(16) int2 cl_scw[];  // [warps][kTileE]
+  __shared__ ResolveSmem R;
+  cg::cluster_group cl = cg::this_cluster();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const bool lead = cl.block_rank() == 0;
+  const int64_t gt = (int64_t)cl.block_rank() * kClEngThreads + threadIdx.x;
+  const int64_t GT = (int64_t)cl.num_blocks() * kClEngThreads;
+  const int64_t gw = gt >> 5, GW = GT >> 5;
+  const int32_t n = g.n;
+  const int64_t ntiles = ((int64_t)n + kTileV - 1) / kTileV;
+  ClusterState* cs = e.cs;
+  for (int64_t v = gt; v < n; v += GT) {
+    e.C[v] = (int32_t)v;
+    e.Wc[v] = g.vw[v];
+    e.ReqW[v] = 0;
+  }
+  if (lead && threadIdx.x == 0) {
+    cs->moved = 0;
+    cs->moved2 = 0;
+    cs->ncont = 0;
+    cs->kernels = 0;
+  }
+  cl.sync();
+  for (int32_t it = 0; it < e.iters; it++) {
+    a.it = it;
+    int64_t* moved = (it & 1) ? &cs->moved2 : &cs->moved;
+    for (int32_t round = 0; round < 2; round++) {
+      a.round = round;
+      for (int64_t tile = gw; tile < ntiles; tile += GW)
+        cluster_rate_tile(g, a, tile, lane, cl_scw + warp * kTileE, PlainLabel{e.C}, kClEngRow);
+      cl.sync();
+      for (int64_t v = gt; v < n; v += GT) {
+        const int32_t t = a.req[v];
+        uint8_t f = 0;
+        if (t >= 0) f = ((int64_t)e.Wc[t] + e.ReqW[t] <= a.wcap) ? 1 : 2;
+        e.flag[v] = f;
+        if (f == 2) {
+          const unsigned long long i = atomicAdd((unsigned long long*)&cs->ncont, 1ULL);
+          e.key[0][i] = ((uint64_t)(uint32_t)t << 32) | (uint32_t)(h_active(a.seed, a.level, (int32_t)v) >> 32);
+          e.val[0][i] = (int32_t)v;
+        }
+      }
+      cl.sync();
+      const int nc = (int)*(volatile int64_t*)&cs->ncont;
+      if (nc > kSmallThreads) {
+        // rank of every request: the requests before it in (target, hash, id) order
+        for (int64_t b = (int64_t)cl.block_rank() * kClEngThreads; b < nc; b += GT) {  // (block-uniform)
+          const int64_t i = b + threadIdx.x;
+          const uint64_t ki = i < nc ? e.key[0][i] : 0;
+          const int32_t vi = i < nc ? e.val[0][i] : 0;
+          int r = 0;
+          for (int c0 = 0; c0 < nc; c0 += kClEngThreads) {
+            const int m = min(kClEngThreads, nc - c0);
+            __syncthreads();
+            if ((int)threadIdx.x < m) {
+              R.sk[threadIdx.x] = e.key[0][c0 + threadIdx.x];
+              R.sv[threadIdx.x] = e.val[0][c0 + threadIdx.x];
+            }
+            __syncthreads();
+            for (int j = 0; j < m; j++) {
+              const uint64_t kj = R.sk[j];
+              r += (kj < ki || (kj == ki && R.sv[j] < vi)) ? 1 : 0;
+            }
+          }
+          if (i < nc) {
+            e.key[1][r] = ki;
+            e.val[1][r] = vi;
+          }
+        }
+        cl.sync();
+        if (lead) {
+          int64_t carry = 0;
+          for (int b = 0; b < nc; b += kClEngThreads) {
+            const int i = b + (int)threadIdx.x;
+            const int64_t c = i < nc ? (int64_t)g.vw[e.val[1][i]] : 0;
+            int64_t tot;
+            const int64_t x = block_exclusive_scan(c, R.sm, &tot) + carry;
+            if (i < nc) {
+              e.P[i] = x;
+              const uint64_t t = e.key[1][i] >> 32;
+              if (i == 0 || (e.key[1][i - 1] >> 32) != t) e.headP[t] = x;
+            }
+            carry += tot;
+          }
+          __syncthreads();
+          for (int i = threadIdx.x; i < nc; i += kClEngThreads) {
+            const int32_t t = (int32_t)(e.key[1][i] >> 32), v = e.val[1][i];
+            e.flag[v] = ((int64_t)e.Wc[t] + (e.P[i] + g.vw[v] - e.headP[t]) <= a.wcap) ? 1 : 0;
+          }
+        }
+        cl.sync();
+      } else if (nc > 0) {
+        if (lead) cluster_resolve(e.key[0], e.val[0], nc, e.Wc, g.vw, a.wcap, e.flag, R);
+        cl.sync();
+      }
+      if (nc > 0 && lead && threadIdx.x == 0) cs->ncont = 0;  // (every CTA has read it)
+      int32_t mine = 0;
+      for (int64_t v = gt; v < n; v += GT) {
+        const int32_t t = a.req[v];
+        if (t < 0) continue;
+        e.ReqW[t] = 0;
+        if (e.flag[v] != 1) continue;
+        const int32_t cv = g.vw[v];
+        atomicAdd(&e.Wc[e.C[v]], -cv);
+        atomicAdd(&e.Wc[t], cv);
+        e.C[v] = t;
+        mine++;
+      }
+      mine = warp_sum(mine);
+      if (lane == 0 && mine) atomicAdd((unsigned long long*)moved, (unsigned long long)mine);
+      cl.sync();
+    }
+    if (*(volatile int64_t*)moved * 100 < (int64_t)n) break;
+    if (lead && threadIdx.x == 0) *(moved == &cs->moved ? &cs->moved2 : &cs->moved) = 0;  // the next iteration's
+  }
 }
 
 // isolated vertices: chunks of weight <= cap in id order, labelled n + chunk
@@ -1621,7 +1793,7 @@ void launch_subround(Ctx& c, int lvl, int32_t r, int64_t wcap) {
   uint8_t* flag = c.elig;
   int64_t* d_cont = c.counters + 6;
   const int kbits = bits_for(n) + 32;
-  ClusterArgs a{c.C, c.Wc, c.ReqW, c.req, wcap, c.cfg.seed, c.cstate, lvl, r};
+  ClusterArgs a{c.C, c.Wc, c.ReqW, c.req, wcap, c.cfg.seed, c.cstate, lvl, r, 0};
   c.prof_level = lvl;
   cudaEvent_t ev = nullptr;
   Branches br(c, L.n_hi > 0);
@@ -1792,7 +1964,31 @@ int32_t cluster_level(Ctx& c, int lvl) {
   }
   ClusterState* cs = c.cstate;
   bool graph_ran = false;
-  if (c.use_graphs && !c.prof) {
+  if (c.use_graphs && !c.prof && n <= kClEngMaxN && L.max_deg <= kClEngRow && L.m_hi * 16 <= L.m) {
+    static std::atomic<unsigned long long> attr_done{0};  // one bit per device
+    const unsigned long long bit = 1ULL << (c.dev & 63);
+    const size_t smem = (size_t)(kClEngThreads / 32) * kTileE * sizeof(int2);
+    if (!(attr_done.load() & bit)) {
+      GM_CUDA(cudaFuncSetAttribute(k_cluster_engine, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+      attr_done.fetch_or(bit);
+    }
+    const ClusterArgs a{c.C, c.Wc, c.ReqW, c.req, wcap, c.cfg.seed, cs, lvl, 0, 0};
+    const ClusterEngineArgs e{c.C, c.Wc, c.ReqW, c.elig, {c.sort.key[0], c.sort.key[1]}, {c.sort.val[0], c.sort.val[1]},
+                              c.P64, c.headP, cs, c.cfg.cluster_iters};
+    cudaLaunchAttribute attr{};
+    cudaLaunchConfig_t lc{};
+    const unsigned C = (unsigned)std::min(kClEngMaxCluster, (n + kClEngThreads - 1) / kClEngThreads);
+    lc.gridDim = dim3(C);
+    lc.blockDim = dim3(kClEngThreads);
+    lc.dynamicSmemBytes = smem;
+    lc.stream = c.st;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = C;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    lc.attrs = &attr;
+    lc.numAttrs = 1;
+    GM_CUDA(cudaLaunchKernelEx(&lc, k_cluster_engine, view(L), a, e)); count_launch();
+  } else if (c.use_graphs && !c.prof) {
     const int64_t key[8] = {(int64_t)L.n | ((int64_t)L.n_big << 32), L.m, (int64_t)L.n_hi | ((int64_t)L.n_huge << 32), L.hi_slots, wcap,
                             (int64_t)(intptr_t)c.htab, (int64_t)(intptr_t)L.hub_chunk, L.n_hub_chunks};
     bool same = L.cgexec != nullptr;

@@ -60,6 +60,7 @@ struct ClusterState {
   int64_t moved;       // vertices moved in the current iteration
   unsigned long long kernels;  // kernels run by conditional graph bodies
   int64_t ncont;       // contested requests of the current sub-round (appended)
+  int64_t moved2;      // k_cluster_engine: vertices moved in the odd iterations
 };
 
 // Kernel classes timed by the optional CUDA-event profiler.
