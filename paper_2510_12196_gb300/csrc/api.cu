@@ -65,9 +65,7 @@ void keep_pool_memory(int dev) {
   done.fetch_or(bit);
 }
 
-void* DevMem::get(size_t bytes) {
-  if (bytes == 0) bytes = 16;
-  bytes = (bytes + 255) & ~(size_t)255;
+void* DevMem::raw(size_t bytes) {
   void* p = nullptr;
   if (afn && ffn) {
     p = afn(bytes, user, (void*)st);
@@ -80,31 +78,84 @@ void* DevMem::get(size_t bytes) {
                                     cudaGetErrorString(e));
     }
   }
-  blocks.push_back({p, bytes});
   total += bytes;
   peak = std::max(peak, total);
+  return p;
+}
+
+void DevMem::add_slab(size_t bytes) {
+  slabs.reserve(slabs.size() + 1);
+  if (cur_left) free_list.push_back({cur, cur_left, true});
+  cur_left = 0;
+  cur = static_cast<char*>(raw(bytes));
+  slabs.push_back({cur, bytes, false});
+  cur_left = bytes;
+}
+
+void DevMem::reserve(size_t bytes) {
+  if (!afn && bytes <= kSlabReserve) add_slab((bytes + 255) & ~(size_t)255);
+}
+
+void* DevMem::get(size_t bytes) {
+  if (bytes == 0) bytes = 16;
+  bytes = (bytes + 255) & ~(size_t)255;
+  blocks.reserve(blocks.size() + 1);
+  free_list.reserve(slabs.size() + blocks.size() + 2);  // (put does not allocate)
+  const size_t slab = std::min<size_t>(kSlabMax, std::max<size_t>(256 << 10, total / 128));
+  if ((afn && ffn) || (bytes >= slab / 4 && bytes > cur_left)) {
+    void* p = raw(bytes);
+    blocks.push_back({p, bytes, false});
+    return p;
+  }
+  size_t best = free_list.size();  // the smallest free piece that is not much too large
+  for (size_t i = 0; i < free_list.size(); i++)
+    if (free_list[i].bytes >= bytes && free_list[i].bytes <= bytes + bytes / 4 + 4096 &&
+        (best == free_list.size() || free_list[i].bytes < free_list[best].bytes))
+      best = i;
+  if (best < free_list.size()) {
+    const Block b = free_list[best];
+    free_list[best] = free_list.back();
+    free_list.pop_back();
+    blocks.push_back(b);
+    return b.p;
+  }
+  if (bytes > cur_left) add_slab(slab);
+  void* p = cur;
+  cur += bytes;
+  cur_left -= bytes;
+  blocks.push_back({p, bytes, true});
   return p;
 }
 
 void DevMem::put(void* p) {
   for (size_t i = 0; i < blocks.size(); i++) {
     if (blocks[i].p == p) {
-      if (afn && ffn) ffn(p, blocks[i].bytes, user, (void*)st);
-      else cudaFreeAsync(p, st);
-      total -= blocks[i].bytes;
+      const Block b = blocks[i];
       blocks[i] = blocks.back();
       blocks.pop_back();
+      if (b.slab) {
+        free_list.push_back(b);
+        return;
+      }
+      if (afn && ffn) ffn(p, b.bytes, user, (void*)st);
+      else cudaFreeAsync(p, st);
+      total -= b.bytes;
       return;
     }
   }
 }
 
 void DevMem::release_all() {
-  for (auto& b : blocks) {
-    if (afn && ffn) ffn(b.p, b.bytes, user, (void*)st);
-    else cudaFreeAsync(b.p, st);
-  }
+  for (auto* list : {&blocks, &slabs})
+    for (auto& b : *list) {
+      if (b.slab) continue;
+      if (afn && ffn) ffn(b.p, b.bytes, user, (void*)st);
+      else cudaFreeAsync(b.p, st);
+    }
   blocks.clear();
+  slabs.clear();
+  free_list.clear();
+  cur_left = 0;
   total = 0;
 }
 
@@ -340,6 +391,10 @@ map_status map_create(const int64_t* xadj, const int32_t* adjncy, const int32_t*
     if (m > 0 && !adjncy) throw ApiError(MAP_E_INVALID, "adjncy is required when the graph has edges");
     c.n0 = n;
     c.m0 = m;
+    {  // what the calls below allocate (a little more, for the rounding of every buffer)
+      const size_t sn = (size_t)n, sm = (size_t)m, cap = std::max(sn, sm), kc = (size_t)c.topo.kc;
+      c.mem.reserve(40 * cap + cap / 2 + 8 * sm + 98 * sn + 8 * std::max(kc, sn) + 564 * kc + (128 << 10));
+    }
     Level L;
     L.n = n;
     L.m = m;
