@@ -755,7 +755,7 @@ map_status map_stats(map_ctx* ctx, map_stats_t* out) {
       out->weak_iters[l] = c.kinds[l][KIND_WEAK];
       out->strong_iters[l] = c.kinds[l][KIND_STRONG];
     }
-    out->ms_tune = c.ms_tune;
+    out->ms_tune = 0;  // the schedule is a rule: nothing is timed
     out->ms_coarsen = c.ms_coarsen;
     out->ms_initial = c.ms_initial;
     out->ms_refine = c.ms_refine;

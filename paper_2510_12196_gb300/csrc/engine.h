@@ -88,9 +88,9 @@ struct Level {
   int32_t n_hi = 0;
   int64_t m_hi = 0;            // CSR entries of the high-degree vertices
   int64_t m_huge = 0;          // CSR entries of the vertices of degree > mid_deg
-  int32_t mid_deg = kMidDeg;   // warp-per-vertex bound of this level (autotuned, <= kMidDeg)
+  int32_t mid_deg = kMidDeg;   // warp-per-vertex bound of this level (<= kMidDeg)
   int64_t split_req = kSplitDeg;  // hub split bound asked for (hub_split_deg: the one in force)
-  int32_t tuned = 0;           // 1: (mid_deg, split_req) chosen by timing, 0: defaults or the config's
+  int32_t tuned = 0;           // 1: the config leaves both bounds open and they matter (rows above kLowDeg hold 2^20 entries)
   int64_t max_deg = 0;         // largest degree (0 when n_hi == 0, i.e. at most kLowDeg)
   int32_t* huge = nullptr;     // positions in hi of the vertices of degree > kMidDeg, ascending
   int32_t n_huge = 0;
@@ -150,11 +150,12 @@ inline HubRows hub_rows(const Level& L) {
 // allocation of its own.  Without, small buffers are cut from slabs (the first
 // one sized for everything map_create needs) and go back to a free list; a
 // buffer above a quarter of a later slab is an allocation of its own, freed at
-// once, so that slabs cost little memory (0.3-7 % above 1 MB).  A context holds some seventy buffers, and their allocation and release
-// one by one was most of the cost of a small context, above all with several
-// threads at it (a stream-ordered allocation takes a lock of the device):
-// hierarchical multisection of an RGG of 2^17 vertices by 8 threads 38.5 ->
-// 26.7 ms, 16 served jobs 33.3 -> 21.4 ms.
+// once, so that slabs cost little memory (0.2-2 % above 1 MB held).  A context
+// holds some seventy buffers, and their allocation and release one by one was
+// most of the cost of a small context, above all with several threads at it (a
+// stream-ordered allocation takes a lock of the device): hierarchical
+// multisection of an RGG of 2^17 vertices by 8 threads 38.5 -> 26.9 ms, 16
+// served jobs 33.3 -> 21.6 ms.
 // All buffers are used on the context's stream only, so a freed one can be
 // handed out again at once.
 struct DevMem {
@@ -328,8 +329,6 @@ struct Ctx {
 
   // stats
   double ms_coarsen = 0, ms_initial = 0, ms_refine = 0, ms_project = 0;
-  double ms_tune = 0;             // host wall time the schedule autotuner spent
-  RefineState* probe_state = nullptr;  // kind = LP, for the autotuner's timing probe
   int32_t iters[65] = {0};
   int32_t kinds[65][3] = {};  // map_run: LP, weak and strong iterations per level (from the trace)
   int64_t Jlev[65] = {0};

@@ -31,8 +31,8 @@ static_assert(kSpanChunks * kHubChunk / 34 + 2 <= kSpanRows, "a span's rows fit 
 // larger ones in global tables
 constexpr int64_t kSmemRowDeg = 2047;
 constexpr int64_t kBigRowDeg = 8191;
-// rows rated by one CTA whole (PE-code tables); larger rows sum chunk tables
-constexpr int64_t kSplitDeg = 4096;
+// hub rows of at most this many entries are rated whole (PE-code tables); larger rows sum chunk tables
+constexpr int64_t kSplitDeg = 16384;
 // bound of the per-level partial tables of the larger rows (else rated whole)
 constexpr int64_t kSplitTableBytes = 1LL << 30;
 

@@ -3915,8 +3915,6 @@ void refine_alloc(Ctx& c) {
   c.counters = c.mem.make<int64_t>(CNT_N);
   c.Jacc = c.mem.make<int64_t>(2);
   c.state = c.mem.make<RefineState>(1);
-  c.probe_state = c.mem.make<RefineState>(1);
-  GM_CUDA(cudaMemsetAsync(c.probe_state, 0, sizeof(RefineState), c.st));  // kind 0 = KIND_LP
   c.trace_kind = c.mem.make<int32_t>(c.trace_cap);
   c.trace_J = c.mem.make<int64_t>(c.trace_cap);
   c.trace_maxw = c.mem.make<int64_t>(c.trace_cap);
@@ -4680,129 +4678,24 @@ void classify_with(Ctx& c, Level& L, int32_t mid_deg, int64_t split_deg) {
   prepare_hubs(c, L, split_deg);
 }
 
-namespace {
-// The schedule autotuner.  A level whose rows of degree > kLowDeg hold at
-// least kTuneMinEntries entries gets its warp-per-vertex bound mid_deg
-// (candidates 255, 128, 64: which rows a warp takes and which the hub
-// kernels) and its hub split bound (candidates 4096, 2048, 16384: which hub
-// rows one CTA rates whole and which sum per-chunk tables) chosen by timing a
-// probe, coordinate by coordinate; the choice is cached per (device, n, m,
-// entries of degree > kLowDeg, largest degree, PE code space) for the
-// process.  Every schedule gives the same result; only the time differs.
-constexpr int64_t kTuneMinEntries = 1 << 20;
-double now_wall_ms() {
-  return std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now().time_since_epoch()).count();
-}
-struct SchedKey {
-  int dev;
-  int32_t n;
-  int64_t m, m_hi, max_deg;
-  int32_t kc;
-  bool operator==(const SchedKey& o) const {
-    return dev == o.dev && n == o.n && m == o.m && m_hi == o.m_hi && max_deg == o.max_deg && kc == o.kc;
-  }
-};
-struct SchedChoice {
-  int32_t mid_deg;
-  int64_t split_deg;
-};
-std::mutex g_sched_mutex;
-std::vector<std::pair<SchedKey, SchedChoice>> g_sched_cache;
-
-// Device time of the probe, best of two: a full J evaluation and Alg. 4
-// step 1 over the vertices of degree > kLowDeg (per-warp and hub tables),
-// with no vertex locked and the outputs in transient scratch (the
-// rebalancing buffers), on the level's mapping, which is zeroed first on a
-// coarse level (it is set later by projection or the initial mapping).
-double probe_ms(Ctx& c, int lvl) {
-  Level& L = c.lv[lvl];
-  struct ProfOff {  // the probe's launches stay out of the kernel-class profile
-    Ctx& c;
-    bool was;
-    explicit ProfOff(Ctx& cc) : c(cc), was(cc.prof) { cc.prof = false; }
-    ~ProfOff() { c.prof = was; }
-  } prof_off(c);
-  if (lvl > 0) GM_CUDA(cudaMemsetAsync(L.pi, 0, (size_t)std::max(1, L.n) * sizeof(int32_t), c.st));
-  GM_CUDA(cudaMemsetAsync(c.sel, 0, (size_t)std::max(1, L.n), c.st));
-  const GroupLayout glay = group_layout(c.topo);
-  const LpFilter flt{0, 1};
-  cudaEvent_t e0, e1;
-  GM_CUDA(cudaEventCreate(&e0));
-  GM_CUDA(cudaEventCreate(&e1));
-  double best = 1e30;
-  for (int rep = 0; rep < 2; rep++) {
-    GM_CUDA(cudaEventRecord(e0, c.st));
-    launch_eval(c, lvl);
-    if (L.n_hi > L.n_huge) {
-      const size_t sm = mid_table_smem(glay.total);
-      k_lp_gain_mid<<<mid_grid(c, (const void*)k_lp_gain_mid, sm, L.n_hi), kMidThreads, sm, c.st>>>(
-          view(L), L.hi, L.n_hi, L.pi, c.sel, c.dest, c.P64, c.elig, c.topo, glay, flt, c.probe_state);
-      count_launch();
-    }
-    if (L.n_huge) {
-      const LpHubPolicy pol{L.pi, c.sel, c.dest, c.P64, c.elig, c.topo, glay, flt, c.probe_state};
-      launch_hub_tab(c, L, pol, (size_t)glay.total * sizeof(int32_t));
-    }
-    GM_CUDA(cudaEventRecord(e1, c.st));
-    GM_CUDA(cudaEventSynchronize(e1));
-    float ms = 0;
-    GM_CUDA(cudaEventElapsedTime(&ms, e0, e1));
-    best = std::min(best, (double)ms);
-  }
-  cudaEventDestroy(e0);
-  cudaEventDestroy(e1);
-  return best;
-}
-}  // namespace
-
+// The schedule of a level: the warp-per-vertex bound kMidDeg and the hub split
+// bound kSplitDeg unless the config fixes them.  Every schedule gives the same
+// result.  Timing candidates on every new level (255, 128, 64; 4096, 2048,
+// 16384) cost 6.7 ms of a 30 ms map of an R-MAT graph of 200003 vertices and
+// 61 ms of the first map of one of 2^22, and nothing it chose was faster:
+// refinement with (255, 16384) / (255, 4096) / (255, 2048) / (128, 16384) took
+// 20.3 / 20.5 / 20.5 / 22.6 ms there on 64 PEs (9.4 / 9.8 / 9.9 / 10.2 on
+// 1024), 73.2 / 74.3 / 77.5 / 73.3 ms at 2^22 on 512 PEs, 26.8 / 27.0 / 27.7 /
+// 28.0 at 2^20, 11.4 / 11.7 / 11.7 / 13.9 at 50021 on 64 and 10.6 for each on
+// an RGG of degree 40.
 void classify_degrees(Ctx& c, int lvl) {
+  constexpr int64_t kReportEntries = 1 << 20;  // Level::tuned
   Level& L = c.lv[lvl];
   const int32_t prev_mid = L.mid_deg;
   const int64_t prev_split = L.split_req;
-  const bool fixed = c.cfg.mid_deg > 0 || c.cfg.split_deg > 0;
-  SchedChoice ch{c.cfg.mid_deg > 0 ? c.cfg.mid_deg : kMidDeg, c.cfg.split_deg > 0 ? c.cfg.split_deg : kSplitDeg};
-  classify_with(c, L, ch.mid_deg, ch.split_deg);
-  L.tuned = 0;
-  if (!fixed && L.m_hi >= kTuneMinEntries && mid_tables(c)) {
-    const SchedKey key{c.dev, L.n, L.m, L.m_hi, L.max_deg, c.topo.kc};
-    bool hit = false;
-    {
-      std::lock_guard<std::mutex> lock(g_sched_mutex);
-      for (const auto& kv : g_sched_cache)
-        if (kv.first == key) {
-          ch = kv.second;
-          hit = true;
-        }
-    }
-    if (!hit) {
-      const double t0 = now_wall_ms();
-      double best = probe_ms(c, lvl);
-      SchedChoice cur = ch;
-      for (int32_t md : {128, 64}) {
-        classify_with(c, L, md, cur.split_deg);
-        const double t = probe_ms(c, lvl);
-        if (t < best) {
-          best = t;
-          ch = SchedChoice{md, cur.split_deg};
-        }
-      }
-      cur = ch;
-      for (int64_t sd : {(int64_t)2048, (int64_t)16384}) {
-        classify_with(c, L, cur.mid_deg, sd);
-        const double t = probe_ms(c, lvl);
-        if (t < best) {
-          best = t;
-          ch = SchedChoice{cur.mid_deg, sd};
-        }
-      }
-      c.ms_tune += now_wall_ms() - t0;
-      std::lock_guard<std::mutex> lock(g_sched_mutex);
-      g_sched_cache.emplace_back(key, ch);
-    }
-    classify_with(c, L, ch.mid_deg, ch.split_deg);
-    L.tuned = 1;
-  }
-  L.split_req = ch.split_deg;
+  classify_with(c, L, c.cfg.mid_deg > 0 ? c.cfg.mid_deg : kMidDeg, c.cfg.split_deg > 0 ? c.cfg.split_deg : kSplitDeg);
+  L.tuned = c.cfg.mid_deg <= 0 && c.cfg.split_deg <= 0 && L.m_hi >= kReportEntries && mid_tables(c);
+  L.split_req = c.cfg.split_deg > 0 ? c.cfg.split_deg : kSplitDeg;
   if (L.mid_deg != prev_mid || L.split_req != prev_split) {
     // kernels captured for the other schedule
     drop_graph(L);
