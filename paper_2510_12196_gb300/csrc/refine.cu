@@ -549,42 +549,75 @@ __host__ inline GroupLayout group_layout(const Topo& t) {
 
 // Fills conn[0, kc) (already zeroed) with the edge weights of v per neighbour
 // PE and the level group sums after it.  Returns T(P(v)) summed over the block.
+// The threads that fill and read one connectivity table: a CTA or a warp.
+struct CtaRow {
+  static constexpr bool kWarp = false;
+  __device__ __forceinline__ static int tid() { return (int)threadIdx.x; }
+  __device__ __forceinline__ static int size() { return (int)blockDim.x; }
+  __device__ __forceinline__ static void sync() { __syncthreads(); }
+};
+struct WarpRow {
+  static constexpr bool kWarp = true;
+  __device__ __forceinline__ static int tid() { return (int)(threadIdx.x & 31); }
+  __device__ __forceinline__ static int size() { return 32; }
+  __device__ __forceinline__ static void sync() { __syncwarp(); }
+};
+
 // conn of the CSR entries [e0, e1) added into tab[code] (shared memory):
-// four entries per thread at a time, whose adjacency loads and PE gathers
-// are all issued before the first add.
+// several entries per thread at a time (four in a CTA, eight in a warp), whose
+// adjacency loads and PE gathers are all issued before the first add.
+template <class R = CtaRow>
 __device__ __forceinline__ void conn_add(const GraphView& g, int64_t e0, int64_t e1, const int32_t* __restrict__ pi,
                                          int32_t* tab) {
-  constexpr int kB = 4;
-  const int64_t step = blockDim.x;
-  int64_t e = e0 + threadIdx.x;
-  for (; e + (kB - 1) * step < e1; e += kB * step) {
-    int32_t u[kB], w[kB];
+  constexpr int kB = R::kWarp ? 8 : 4;
+  const int64_t step = R::size();
+  int64_t e = e0 + R::tid();
+  if constexpr (R::kWarp) {  // rows of a few hundred entries: the last batch as wide as the others
+    for (; e - R::tid() < e1; e += kB * step) {
+      int32_t u[kB], w[kB];
 #pragma unroll
-    for (int b = 0; b < kB; b++) {
-      u[b] = g.adj[e + b * step];
-      w[b] = g.adjw[e + b * step];
+      for (int b = 0; b < kB; b++) {
+        const bool in = e + b * step < e1;
+        u[b] = in ? g.adj[e + b * step] : -1;
+        w[b] = in ? g.adjw[e + b * step] : 0;
+      }
+#pragma unroll
+      for (int b = 0; b < kB; b++) u[b] = u[b] >= 0 ? pi[u[b]] : -1;
+#pragma unroll
+      for (int b = 0; b < kB; b++)
+        if (u[b] >= 0) atomicAdd(&tab[u[b]], w[b]);
     }
+  } else {
+    for (; e + (kB - 1) * step < e1; e += kB * step) {
+      int32_t u[kB], w[kB];
 #pragma unroll
-    for (int b = 0; b < kB; b++) u[b] = pi[u[b]];
+      for (int b = 0; b < kB; b++) {
+        u[b] = g.adj[e + b * step];
+        w[b] = g.adjw[e + b * step];
+      }
 #pragma unroll
-    for (int b = 0; b < kB; b++) atomicAdd(&tab[u[b]], w[b]);
+      for (int b = 0; b < kB; b++) u[b] = pi[u[b]];
+#pragma unroll
+      for (int b = 0; b < kB; b++) atomicAdd(&tab[u[b]], w[b]);
+    }
+    for (; e < e1; e += step) atomicAdd(&tab[pi[g.adj[e]]], g.adjw[e]);
   }
-  for (; e < e1; e += step) atomicAdd(&tab[pi[g.adj[e]]], g.adjw[e]);
 }
 
 // The level group sums of a complete conn table (layout of GroupLayout).
+template <class R = CtaRow>
 __device__ void conn_groups(const Topo& topo, const GroupLayout& gl, int32_t* tab) {
   for (int i = 1; i <= topo.levels; i++) {
     const int32_t cnt = topo.kc >> topo.s[i];
     const int32_t sh = topo.s[i] - topo.s[i - 1];
     const int32_t* prev = tab + gl.off[i - 1];
     int32_t* cur = tab + gl.off[i];
-    for (int32_t gidx = threadIdx.x; gidx < cnt; gidx += blockDim.x) {
+    for (int32_t gidx = R::tid(); gidx < cnt; gidx += R::size()) {
       int32_t s = 0;
       for (int32_t j = 0; j < (1 << sh); j++) s += prev[(gidx << sh) + j];
       cur[gidx] = s;
     }
-    __syncthreads();
+    R::sync();
   }
 }
 
@@ -610,13 +643,14 @@ __device__ __forceinline__ int64_t conn_T(const int32_t* tab, const Topo& topo, 
 // Alg. 4 step 1 for vertex v (current PE code p) from its complete table
 // (conn over the PE codes and the level group sums): the neighbouring PE
 // q != p of smallest T(q) (lowest code on ties), the filter, the outputs.
-// All threads of the CTA call it; ends with a barrier.
+// All threads of the row call it; ends with their barrier.
+template <class R = CtaRow>
 __device__ __forceinline__ void lp_hub_decide(const int32_t* tab, const Topo& topo, const GroupLayout& gl,
                                               const LpFilter& flt, int32_t v, int32_t p, int32_t* pp, int64_t* gain,
                                               uint8_t* inx, int64_t* sbt, int32_t* sbc) {
   int64_t bt = INT64_MAX;
   int32_t bc = INT32_MAX;
-  for (int32_t q = threadIdx.x; q < topo.kc; q += blockDim.x) {
+  for (int32_t q = R::tid(); q < topo.kc; q += R::size()) {
     if (q == p || tab[q] == 0) continue;
     const int64_t T = conn_T(tab, topo, gl, q);
     if (T < bt || (T == bt && q < bc)) {
@@ -633,13 +667,15 @@ __device__ __forceinline__ void lp_hub_decide(const int32_t* tab, const Topo& to
       bc = oc;
     }
   }
-  if ((threadIdx.x & 31) == 0) {
-    sbt[threadIdx.x >> 5] = bt;
-    sbc[threadIdx.x >> 5] = bc;
+  if constexpr (!R::kWarp) {
+    if ((threadIdx.x & 31) == 0) {
+      sbt[threadIdx.x >> 5] = bt;
+      sbc[threadIdx.x >> 5] = bc;
+    }
+    __syncthreads();
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); w++)
+  if (R::tid() == 0) {
+    for (int w = 1; w < R::size() >> 5; w++)
       if (sbt[w] < bt || (sbt[w] == bt && sbc[w] < bc)) {
         bt = sbt[w];
         bc = sbc[w];
@@ -656,7 +692,7 @@ __device__ __forceinline__ void lp_hub_decide(const int32_t* tab, const Topo& to
       gain[v] = 0;
     }
   }
-  __syncthreads();
+  R::sync();
 }
 
 __global__ void __launch_bounds__(kHiThreads) k_lp_gain_high(GraphView g, const int32_t* __restrict__ hi,
@@ -1526,7 +1562,8 @@ __global__ void __launch_bounds__(kMidThreads) k_reb_select_mid(GraphView g, con
 // table (conn over the PE codes, plus the level group sums for the J gains):
 // the best destination below sigma among the neighbouring blocks (the drawn
 // block of U if none), its loss bucket, and the per-(block, bucket) weight
-// totals.  All threads of the CTA call it; ends with a barrier.
+// totals.  All threads of the row call it; ends with their barrier.
+template <class R = CtaRow>
 __device__ __forceinline__ void reb_hub_decide(const int32_t* tab, const RebArgs& a, int32_t kc, const GroupLayout& gl,
                                                int32_t v, int32_t A, int32_t cv, int32_t* dest, uint8_t* bkt,
                                                uint8_t* elig, const RefineState* st, int64_t* sbb, int32_t* sbc) {
@@ -1535,7 +1572,7 @@ __device__ __forceinline__ void reb_hub_decide(const int32_t* tab, const RebArgs
   // score: conn(v, q), or -T(q) for the J gains; -1 / INT64_MIN: none
   int64_t bconn = a.obj ? INT64_MIN : -1;
   int32_t bc = INT32_MAX;
-  for (int32_t b = threadIdx.x; b < kc; b += blockDim.x) {
+  for (int32_t b = R::tid(); b < kc; b += R::size()) {
     const int32_t x = tab[b];
     if (x == 0 || b == A || a.W[b] > sigma) continue;
     const int64_t sc = a.obj ? -conn_T(tab, a.topo, gl, b) : (int64_t)x;
@@ -1553,13 +1590,15 @@ __device__ __forceinline__ void reb_hub_decide(const int32_t* tab, const RebArgs
       bc = oc;
     }
   }
-  if ((threadIdx.x & 31) == 0) {
-    sbb[threadIdx.x >> 5] = bconn;
-    sbc[threadIdx.x >> 5] = bc;
+  if constexpr (!R::kWarp) {
+    if ((threadIdx.x & 31) == 0) {
+      sbb[threadIdx.x >> 5] = bconn;
+      sbc[threadIdx.x >> 5] = bc;
+    }
+    __syncthreads();
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); w++)
+  if (R::tid() == 0) {
+    for (int w = 1; w < R::size() >> 5; w++)
       if (sbb[w] > bconn || (sbb[w] == bconn && sbc[w] < bc)) {
         bconn = sbb[w];
         bc = sbc[w];
@@ -1583,7 +1622,7 @@ __device__ __forceinline__ void reb_hub_decide(const int32_t* tab, const RebArgs
     }
     elig[v] = ok ? 1 : 0;
   }
-  __syncthreads();
+  R::sync();
 }
 
 __global__ void __launch_bounds__(kHiThreads) k_reb_select_high(GraphView g, const int32_t* __restrict__ hi,
@@ -1619,12 +1658,18 @@ __global__ void __launch_bounds__(kHiThreads) k_reb_select_high(GraphView g, con
 // Connectivity-table kernels over the rows of degree > kMidDeg, spread over
 // CTAs by chunk tickets (the table over the PE codes does not grow with the
 // degree; the work does).  A row of at most split_deg entries is rated whole
-// by the CTA that draws the chunk holding its first entry.  A larger row is
+// by the CTA that draws the chunk holding its first entry: rows of at most
+// kWarpRowDeg entries by one of its warps with a table of its own (mid_tables),
+// with no barrier of the CTA between the phases of a row, larger rows by all.  A row's phases (loads, gathers, table, scan) each wait on
+// the one before, so rows side by side set the pace: 3.0e6 entries (n 33853, 64
+// PEs) 37.7 -> 21.2 us a rebalancing step and 40.3 -> 24.3 us an LP step, 7.9e7
+// entries (R-MAT 2^22 coarsened, 512 PEs) 487 -> 380 us an LP step.  A larger row is
 // rated in two launches: every chunk adds the conn of its entries into the
 // row's global partial table, then one CTA per row reads the table back
 // (emptying it), adds the level group sums and decides.  The policy P gives
 // the table width, whether group sums are needed, which vertices take part
 // and the decision.
+constexpr int32_t kWarpRowDeg = 1023;
 struct LpHubPolicy {  // Alg. 4 step 1
   // skip() clears the lock that want() reads: a barrier between them
   static constexpr bool kWantBarrier = true;
@@ -1650,8 +1695,9 @@ struct LpHubPolicy {  // Alg. 4 step 1
     gain[v] = 0;
     lock[v] = 0;
   }
+  template <class R>
   __device__ void decide(const int32_t* tab, int32_t v, int32_t cv, int64_t* sb, int32_t* sc) const {
-    lp_hub_decide(tab, topo, gl, flt, v, pi[v], pp, gain, inx, sb, sc);
+    lp_hub_decide<R>(tab, topo, gl, flt, v, pi[v], pp, gain, inx, sb, sc);
   }
 };
 struct RebHubPolicy {  // rebalancing selection
@@ -1671,8 +1717,9 @@ struct RebHubPolicy {  // rebalancing selection
   __device__ bool groups() const { return a.obj != 0; }
   __device__ bool want(int32_t v) const { return reb_eligible(a, pi[v], vw[v]); }
   __device__ void skip(int32_t v) const { elig[v] = 0; }
+  template <class R>
   __device__ void decide(const int32_t* tab, int32_t v, int32_t cv, int64_t* sb, int32_t* sc) const {
-    reb_hub_decide(tab, a, a.topo.kc, gl, v, pi[v], cv, dest, bkt, elig, st, sb, sc);
+    reb_hub_decide<R>(tab, a, a.topo.kc, gl, v, pi[v], cv, dest, bkt, elig, st, sb, sc);
   }
 };
 
@@ -1681,7 +1728,8 @@ __global__ void __launch_bounds__(kHiThreads) k_hub_tab(GraphView g, HubRows hr,
                                                         const int32_t* __restrict__ sidx, int32_t* gtab,
                                                         unsigned long long* ctr) {
   static_assert(kHiThreads == kSpanRows, "one thread per row of a span");
-  extern __shared__ int32_t tab[];
+  static_assert(kHiThreads == kMidThreads, "a table per warp");
+  extern __shared__ __align__(16) int32_t tab[];  // a table per warp, the first also the CTA's
   __shared__ int64_t sb[32];
   __shared__ int32_t sc[32];
   __shared__ int64_t s_ch;
@@ -1691,7 +1739,8 @@ __global__ void __launch_bounds__(kHiThreads) k_hub_tab(GraphView g, HubRows hr,
   __shared__ uint8_t s_split[kSpanRows];
   if (!pol.run()) return;
   const int32_t words = pol.words(), kc = pol.topo_kc();
-  for (int32_t b = threadIdx.x; b < words; b += blockDim.x) tab[b] = 0;
+  const int32_t stride = (words + 3) & ~3;  // of the warps' tables
+  for (int32_t b = threadIdx.x; b < kMidWarps * stride; b += blockDim.x) tab[b] = 0;
   __syncthreads();
   const int64_t m_hub = hr.pre[hr.n_huge];
   const int64_t nspans = (hr.nchunks + kSpanChunks - 1) / kSpanChunks;
@@ -1722,16 +1771,34 @@ __global__ void __launch_bounds__(kHiThreads) k_hub_tab(GraphView g, HubRows hr,
       s_split[threadIdx.x] = sp_row;
     }
     const int nrows = __syncthreads_count(row);  // the span's rows are a prefix
+    {
+      const int warp = (int)threadIdx.x >> 5, lane = (int)threadIdx.x & 31;
+      int32_t* wt = tab + warp * stride;
+      for (int i = warp; i < nrows; i += kMidWarps) {
+        const int32_t v = s_v[i];
+        const int64_t deg = s_re[i] - s_rb[i];
+        if (v < 0 || s_split[i] || deg > kWarpRowDeg) continue;
+        const int64_t e0 = g.xadj[v];
+        conn_add<WarpRow>(g, e0, e0 + deg, pol.pi, wt);
+        __syncwarp();
+        if (pol.groups()) conn_groups<WarpRow>(pol.topo_of(), pol.gl, wt);
+        pol.template decide<WarpRow>(wt, v, g.vw[v], sb, sc);
+        for (int32_t b = 4 * lane; b < stride; b += 128) *reinterpret_cast<int4*>(wt + b) = make_int4(0, 0, 0, 0);
+        __syncwarp();
+      }
+      __syncthreads();  // the first table is empty again: the CTA's
+    }
     for (int i = 0; i < nrows; i++) {
       const int32_t v = s_v[i];
       if (v < 0) continue;
       const int64_t rb = s_rb[i], re = s_re[i];
+      if (!s_split[i] && re - rb <= kWarpRowDeg) continue;  // rated by a warp above
       const int64_t x0 = g.xadj[v] - rb;
       if (!s_split[i]) {
         conn_add(g, x0 + rb, x0 + re, pol.pi, tab);
         __syncthreads();
         if (pol.groups()) conn_groups(pol.topo_of(), pol.gl, tab);
-        pol.decide(tab, v, g.vw[v], sb, sc);
+        pol.template decide<CtaRow>(tab, v, g.vw[v], sb, sc);
       } else {
         conn_add(g, x0 + max(rb, cb), x0 + min(re, ce), pol.pi, tab);
         __syncthreads();
@@ -1775,7 +1842,7 @@ __global__ void __launch_bounds__(kHiThreads) k_hub_tab_finish(GraphView g, HubR
     }
     __syncthreads();
     if (pol.groups()) conn_groups(pol.topo_of(), pol.gl, tab);
-    pol.decide(tab, v, g.vw[v], sb, sc);
+    pol.template decide<CtaRow>(tab, v, g.vw[v], sb, sc);
     for (int32_t b = threadIdx.x; b < words; b += blockDim.x) tab[b] = 0;
     __syncthreads();
   }
@@ -2304,14 +2371,17 @@ inline unsigned mid_grid(Ctx& c, const void* fn, size_t smem, int64_t n_hi) {
 inline bool mid_tables(const Ctx& c) { return group_layout(c.topo).total <= kMidTableMax; }
 inline size_t mid_table_smem(int32_t words) { return (size_t)kMidWarps * words * sizeof(int32_t); }
 
+inline size_t hub_tab_smem(size_t table) { return kMidWarps * ((table + 15) & ~(size_t)15); }
+
 // The two launches of a hub table kernel (the second only for rows summed
 // over chunks), each one wave of resident CTAs drawing tickets.
 template <class P>
 void launch_hub_tab(Ctx& c, Level& L, const P& pol, size_t smem) {
   const void* f1 = (const void*)k_hub_tab<P>;
-  const int64_t r1 = (int64_t)c.num_sms * c.resident_blocks(f1, kHiThreads, smem);
+  const size_t smem1 = hub_tab_smem(smem);
+  const int64_t r1 = (int64_t)c.num_sms * c.resident_blocks(f1, kHiThreads, smem1);
   const int64_t spans = (L.n_hub_chunks + kSpanChunks - 1) / kSpanChunks;
-  k_hub_tab<P><<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(spans, r1)), kHiThreads, smem, c.st>>>(
+  k_hub_tab<P><<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(spans, r1)), kHiThreads, smem1, c.st>>>(
       view(L), hub_rows(L), pol, L.hub_split_deg, L.hub_sidx, L.hub_gtab, c.hub_ctr);
   count_launch();
   if (L.n_split) {
@@ -3937,6 +4007,11 @@ void refine_alloc(Ctx& c) {
   }
   const size_t reb_smem = (size_t)(c.cfg.reb_objective ? group_layout(c.topo).total : kc) * sizeof(int32_t);
   if (reb_smem > 48 * 1024) raise_smem((const void*)k_reb_select_high, reb_smem);
+  if (mid_tables(c)) {  // (with their static arrays up to 54 KB)
+    const size_t tab = hub_tab_smem((size_t)group_layout(c.topo).total * sizeof(int32_t));
+    raise_smem((const void*)k_hub_tab<LpHubPolicy>, tab);
+    raise_smem((const void*)k_hub_tab<RebHubPolicy>, tab);
+  }
   if (kc * sizeof(int32_t) > 48 * 1024) raise_smem((const void*)k_block_weights, kc * sizeof(int32_t));
 }
 
