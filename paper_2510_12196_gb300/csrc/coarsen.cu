@@ -1640,102 +1640,175 @@ __global__ void k_project(int32_t n, const int32_t* __restrict__ M, const int32_
 // ---------------------------------------------------------------------------
 // initial mapping: breadth-first order in one CTA, cut into k weight chunks
 // ---------------------------------------------------------------------------
-constexpr int kInitSmemN = 12288;  // coarsest graphs up to this size keep the BFS state in shared memory
+constexpr int kInitSmemN = 12288;  // coarsest graphs up to this size keep the search state in shared memory
+// graphs of more entries with rows this long (hubs: the last levels reread most
+// rows) are searched by the whole GPU: R-MAT of 8192 vertices 0.74 ms here and
+// 0.77 there at 6.4e5 entries, 1.1 and 0.78 at 1.5e6, 1.6 and 0.78 at 2.7e6;
+// without hubs one CTA stays level or ahead (4.9e6 entries of 12288 vertices in
+// equal rows: 0.14 and 0.77 ms)
+constexpr int64_t kInitEntries = 1 << 20;
+constexpr int kInitThreads = 1024;
+constexpr size_t kInitSmem = 224 * 1024;  // with the rows too, where they fit
+inline size_t init_state(int64_t n) { return (size_t)n * 3 * sizeof(int32_t); }
+inline size_t init_rows(int64_t n, int64_t m) { return (size_t)(n + 1 + m) * sizeof(int32_t); }
 
-__global__ void __launch_bounds__(1024) k_initial(GraphView g, int32_t* order, int32_t* claim, int32_t* seen,
-                                                  const int32_t* __restrict__ code_of_pe, int64_t k, int64_t cV,
-                                                  int32_t* pi, uint32_t* err) {
+// Bounded by latency: a search of a mesh's coarsest graph has 30-50 levels of
+// 20-100 vertices.  A frontier vertex is taken by kW lanes together (8 on short
+// rows, 32 otherwise), so that its row costs one round trip, not one per entry,
+// and hub rows spread over a warp; the claims (shared memory) hold the visited
+// marks too (-1).  Per level: claim by the earliest frontier position; count
+// each vertex's children; scan; write them in (position, adjacency) order.  Of
+// the unvisited ids a warp looks at 32 at a time, and vertices without edges are
+// appended without a level of their own.  The rows are staged too where they fit
+// (up to 3700 vertices of degree 8).  One thread per frontier vertex, rereading
+// its row entry by entry, took 250 us for the coarsest graph of an RGG of 2^20
+// vertices (1682 vertices, 9730 entries) and 5.3 ms for that of an R-MAT graph
+// of 50021 (7679, 694466); this takes 90 us and 0.8 ms.
+template <int kW>
+__global__ void __launch_bounds__(kInitThreads) k_initial(GraphView g, int32_t* order, int32_t* claim, int32_t* cnt,
+                                                          const int32_t* __restrict__ code_of_pe, int64_t k, int64_t cV,
+                                                          int32_t* pi, int staged, uint32_t* err) {
   __shared__ int64_t sm[33];
-  __shared__ int32_t s_tail, s_head, s_next;
+  __shared__ int32_t sm32[33], s_tail, s_end;
   extern __shared__ __align__(16) int32_t init_smem[];
   const int32_t n = g.n;
   if (n <= kInitSmemN) {  // same algorithm, state on chip (the launch provides 3 * n words)
     order = init_smem;
     claim = init_smem + n;
-    seen = init_smem + 2 * (size_t)n;
+    cnt = init_smem + 2 * (size_t)n;
   }
-  for (int32_t v = threadIdx.x; v < n; v += blockDim.x) {
-    seen[v] = 0;
-    claim[v] = INT32_MAX;
+  int32_t* sx = init_smem + 3 * (size_t)n;  // staged: the rows' bounds and entries on chip too
+  const int32_t* adj = staged ? sx + n + 1 : g.adj;
+  if (staged) {
+    for (int32_t v = threadIdx.x; v <= n; v += kInitThreads) sx[v] = (int32_t)g.xadj[v];
+    const int32_t m = (int32_t)g.xadj[n];
+#pragma unroll 4
+    for (int32_t e = threadIdx.x; e < m; e += kInitThreads) sx[n + 1 + e] = g.adj[e];
   }
-  if (threadIdx.x == 0) {
-    s_tail = 0;
-    s_head = 0;
-    s_next = 0;
-  }
+  auto row = [&](int32_t v, int32_t& deg) {  // first entry, degree
+    const int64_t b = staged ? sx[v] : g.xadj[v], e = staged ? sx[v + 1] : g.xadj[v + 1];
+    deg = (int32_t)(e - b);
+    return adj + b;
+  };
+  volatile int32_t* vclaim = claim;  // (changed by atomics and other warps between barriers)
+  for (int32_t v = threadIdx.x; v < n; v += kInitThreads) claim[v] = INT32_MAX;
+  const int lane = (int)threadIdx.x & 31, sl = lane % kW;
+  const unsigned group = kW == 32 ? 0xffffffffu : ((1u << kW) - 1u) << (lane - sl);
+  const int32_t g0 = (int32_t)threadIdx.x / kW, ng = kInitThreads / kW;  // lane group, groups of the CTA
+  const unsigned before = (1u << lane) - 1u;
   __syncthreads();
+  int32_t head = 0, tail = 0, next = 0;  // (next: thread 0's warp only)
   int64_t guard = 0;
-  while (true) {
-    const int32_t tail = s_tail;
-    const int32_t head = s_head;
-    if (tail >= n) break;
+  while (tail < n) {
     if (++guard > 2 * (int64_t)n + 4) {  // cannot happen; bounded for safety
       if (threadIdx.x == 0) atomicOr(err, ERR_TIMEOUT);
       break;
     }
-    __syncthreads();
     if (head == tail) {  // next component: lowest unvisited id
-      if (threadIdx.x == 0) {
-        int32_t s = s_next;
-        while (seen[s]) s++;
-        s_next = s + 1;
-        order[tail] = s;
-        seen[s] = 1;
-        s_tail = tail + 1;
+      if (threadIdx.x < 32) {
+        int32_t at = tail;
+        bool root = false;
+        while (at < n && next < n && !root) {
+          const int32_t v = next + lane;
+          const bool open = v < n && vclaim[v] != -1;
+          int32_t deg = 0;
+          if (open) row(v, deg);
+          const bool edges = deg > 0;
+          const unsigned om = __ballot_sync(0xffffffffu, open), em = __ballot_sync(0xffffffffu, edges);
+          // the open vertices up to the first one with edges
+          const unsigned take = em ? om & (em ^ (em - 1u)) : om;
+          if ((take >> lane) & 1u) {
+            order[at + __popc(take & before)] = v;
+            vclaim[v] = -1;
+          }
+          at += __popc(take);
+          root = em != 0;
+          next += em ? __ffs(em) : 32;
+        }
+        if (lane == 0) s_tail = at;
       }
       __syncthreads();
-      continue;
+      const int32_t at = s_tail;
+      __syncthreads();
+      // the last one appended is the component's root; the ones before it have no edges
+      head = at - 1;
+      tail = at;
+      if (tail >= n) break;
     }
     // one level: frontier [head, tail); children claimed by the earliest parent
-    for (int32_t i = head + threadIdx.x; i < tail; i += blockDim.x) {
-      const int32_t v = order[i];
-      for (int64_t e = g.xadj[v]; e < g.xadj[v + 1]; e++) {
-        const int32_t u = g.adj[e];
-        if (!seen[u]) atomicMin(&claim[u], i);
-      }
+    for (int32_t i = head + g0; i < tail; i += ng) {
+      int32_t deg;
+      const int32_t* r = row(order[i], deg);
+#pragma unroll 4
+      for (int32_t j = sl; j < deg; j += kW) atomicMin(&claim[r[j]], i);
     }
     __syncthreads();
-    int64_t carry = 0;
-    for (int32_t base = head; base < tail; base += blockDim.x) {
-      const int32_t i = base + threadIdx.x;
-      int64_t cnt = 0;
-      if (i < tail) {
-        const int32_t v = order[i];
-        for (int64_t e = g.xadj[v]; e < g.xadj[v + 1]; e++) {
-          const int32_t u = g.adj[e];
-          if (!seen[u] && claim[u] == i) cnt++;
+    for (int32_t i = head + g0; i < tail; i += ng) {
+      int32_t deg, x = 0;
+      const int32_t* r = row(order[i], deg);
+#pragma unroll 4
+      for (int32_t j = sl; j < deg; j += kW) x += vclaim[r[j]] == i;
+#pragma unroll
+      for (int o = kW / 2; o > 0; o >>= 1) x += __shfl_xor_sync(group, x, o);
+      if (sl == 0) cnt[i] = x;
+    }
+    __syncthreads();
+    // cnt: the first child's position, -1 for none
+    int32_t end = tail;
+    if (tail - head <= 128) {  // by one warp, behind one barrier instead of four
+      if (threadIdx.x < 32) {
+        for (int32_t base = head; base < tail; base += 32) {
+          const int32_t i = base + lane, x = i < tail ? cnt[i] : 0;
+          int32_t in = x;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            const int32_t y = __shfl_up_sync(0xffffffffu, in, o);
+            if (lane >= o) in += y;
+          }
+          if (i < tail) cnt[i] = x ? end + in - x : -1;
+          end += __shfl_sync(0xffffffffu, in, 31);
+        }
+        if (lane == 0) s_end = end;
+      }
+      __syncthreads();
+      end = s_end;  // (the next write of s_end is two barriers away)
+    } else {
+      for (int32_t base = head; base < tail; base += kInitThreads) {
+        const int32_t i = base + (int32_t)threadIdx.x, x = i < tail ? cnt[i] : 0;
+        int32_t total;
+        const int32_t ex = block_exclusive_scan(x, sm32, &total);
+        if (i < tail) cnt[i] = x ? end + ex : -1;
+        end += total;
+      }
+      __syncthreads();
+    }
+    if (end > tail) {
+      for (int32_t i = head + g0; i < tail; i += ng) {
+        int32_t pos = cnt[i];
+        if (pos < 0) continue;  // (uniform in the group)
+        int32_t deg;
+        const int32_t* r = row(order[i], deg);
+        for (int32_t j0 = 0; j0 < deg; j0 += kW) {
+          const int32_t u = j0 + sl < deg ? r[j0 + sl] : -1;
+          const bool child = u >= 0 && vclaim[u] == i;
+          const unsigned cm = __ballot_sync(group, child) & group;
+          if (child) {
+            order[pos + __popc(cm & before)] = u;
+            vclaim[u] = -1;  // (no other entry of the frontier is claimed by i)
+          }
+          pos += __popc(cm);
         }
       }
-      int64_t total;
-      const int64_t ex = block_exclusive_scan(cnt, sm, &total);
-      if (i < tail && cnt) {
-        int64_t pos = tail + carry + ex;
-        const int32_t v = order[i];
-        for (int64_t e = g.xadj[v]; e < g.xadj[v + 1]; e++) {
-          const int32_t u = g.adj[e];
-          if (!seen[u] && claim[u] == i) order[pos++] = u;
-        }
-      }
-      carry += total;
+      __syncthreads();
     }
-    __syncthreads();
-    for (int64_t j = tail + threadIdx.x; j < tail + carry; j += blockDim.x) {
-      const int32_t u = order[j];
-      seen[u] = 1;
-      claim[u] = INT32_MAX;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      s_head = tail;
-      s_tail = (int32_t)(tail + carry);
-    }
-    __syncthreads();
+    head = tail;
+    tail = end;
   }
   __syncthreads();
   // PE of the vertex whose preceding weight in breadth-first order is s
   int64_t carry = 0;
-  for (int32_t base = 0; base < n; base += blockDim.x) {
-    const int32_t i = base + threadIdx.x;
+  for (int32_t base = 0; base < n; base += kInitThreads) {
+    const int32_t i = base + (int32_t)threadIdx.x;
     const int64_t cv = (i < n) ? g.vw[order[i]] : 0;
     int64_t total;
     const int64_t ex = block_exclusive_scan(cv, sm, &total);
@@ -2257,16 +2330,21 @@ void initial_map(Ctx& c) {
     hm_run(c, (int)c.lv.size() - 1, 8, &c.hm_init);
     return;
   }
-  if (L.n > kInitSmemN && initial_map_large(c)) return;
-  const size_t smem = L.n <= kInitSmemN ? (size_t)3 * L.n * sizeof(int32_t) : 0;
+  const bool many = L.m > kInitEntries && L.max_deg > L.n / 4;
+  if ((L.n > kInitSmemN || many) && initial_map_large(c)) return;
+  const size_t rows = init_rows(L.n, L.m);
+  const int staged = L.n <= kInitSmemN && L.m < INT32_MAX && init_state(L.n) + rows <= kInitSmem;
+  const size_t smem = L.n <= kInitSmemN ? init_state(L.n) + (staged ? rows : 0) : 0;
   static std::atomic<unsigned long long> attr_done{0};  // one bit per device
   const unsigned long long bit = 1ULL << (c.dev & 63);
   if (!(attr_done.load() & bit)) {
-    GM_CUDA(cudaFuncSetAttribute(k_initial, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(3 * kInitSmemN * sizeof(int32_t))));
+    for (auto* fn : {k_initial<8>, k_initial<32>})
+      GM_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kInitSmem));
     attr_done.fetch_or(bit);
   }
-  k_initial<<<1, 1024, smem, c.st>>>(view(L), c.C, c.req, c.Wc, c.d_code_of_pe, c.k, c.cV, L.pi, c.errword); count_launch();
+  auto* fn = L.m <= 16 * (int64_t)L.n ? k_initial<8> : k_initial<32>;
+  fn<<<1, kInitThreads, smem, c.st>>>(view(L), c.C, c.req, c.Wc, c.d_code_of_pe, c.k, c.cV, L.pi, staged, c.errword);
+  count_launch();
   GM_CUDA(cudaGetLastError());
   check_err(c);
 }
