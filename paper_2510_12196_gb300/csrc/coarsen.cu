@@ -25,6 +25,7 @@
 #include "engine.h"
 #include "tile.cuh"
 #include "mid.cuh"
+#include "gridbar.cuh"
 
 namespace gm {
 
@@ -1106,6 +1107,7 @@ __global__ void k_cluster_classify(int32_t n, const int32_t* __restrict__ req, c
 // the multi-CTA path (scan compaction in id order, stable radix sort).
 struct ResolveSmem {
   uint64_t sk[kSmallThreads];
+  int32_t sw[kSmallThreads];
   int32_t sv[kSmallThreads];
   uint64_t ok[kSmallThreads];
   int32_t ov[kSmallThreads];
@@ -1258,11 +1260,13 @@ __global__ void k_cl_end(ClusterState* cs, int32_t n, int32_t iters, cudaGraphCo
 // vertices (37 maps by 8 threads) 63 -> 38 ms.
 // For levels of at most kClEngMaxN vertices without rows above kClEngRow and
 // with few above kLowDeg (a sub-warp takes each).  Contested requests: up to
-// kSmallThreads are ordered by the first CTA; of longer lists every CTA ranks
-// its share of the entries (by counting) into the second sort buffers, and the
-// first CTA takes the per-target prefixes.
+// kSmallThreads are ordered by the first CTA; of longer lists all CTAs compare
+// every request with every other (45 us for 1.6e4 over 152 SMs, where a sort of
+// any length costs 100 us); above kClEngRequests the launch gives up.
 constexpr int kClEngThreads = 1024;
 constexpr int kClEngMaxN = 1 << 15;
+constexpr int kClGridMaxN = 1 << 17;
+constexpr int kClEngRequests = 1 << 14;
 constexpr int kClEngMaxCluster = 8;  // the portable limit
 constexpr int kClEngRow = kTileE / 4;
 static_assert(kClEngThreads == kSmallThreads, "the resolution takes one request per thread");
@@ -1275,22 +1279,21 @@ struct ClusterEngineArgs {
   int32_t* Wc;
   int32_t* ReqW;
   uint8_t* flag;
-  uint64_t* key[2];
-  int32_t* val[2];
+  uint64_t* key;  // contested requests: (target, tie-hash), vertex, weight of those before
+  int32_t* val;
   int64_t* P;
-  int64_t* headP;
   ClusterState* cs;
   int32_t iters;
 };
-__global__ void __launch_bounds__(kClEngThreads, 1) k_cluster_engine(GraphView g, ClusterArgs a, ClusterEngineArgs e) {
-  extern __shared__ __align__(16) int2 cl_scw[];  // [warps][kTileE]
-  __shared__ ResolveSmem R;
-  cg::cluster_group cl = cg::this_cluster();
+template <class Sync>
+__device__ __forceinline__ void cluster_engine_run(const GraphView& g, ClusterArgs a, const ClusterEngineArgs& e,
+                                                   int2* cl_scw, ResolveSmem& R, int rank, int nblocks,
+                                                   const Sync& cl) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const bool lead = cl.block_rank() == 0;
-  const int64_t gt = (int64_t)cl.block_rank() * kClEngThreads + threadIdx.x;
-  const int64_t GT = (int64_t)cl.num_blocks() * kClEngThreads;
-  const int64_t gw = gt >> 5, GW = GT >> 5;
+  const bool lead = rank == 0;
+  const int64_t gt = (int64_t)rank * kClEngThreads + threadIdx.x;
+  const int64_t GT = (int64_t)nblocks * kClEngThreads;
+  const int64_t gw = (int64_t)warp * nblocks + rank, GW = GT >> 5;  // (tiles over all CTAs first)
   const int32_t n = g.n;
   const int64_t ntiles = ((int64_t)n + kTileV - 1) / kTileV;
   ClusterState* cs = e.cs;
@@ -1321,61 +1324,53 @@ __global__ void __launch_bounds__(kClEngThreads, 1) k_cluster_engine(GraphView g
         e.flag[v] = f;
         if (f == 2) {
           const unsigned long long i = atomicAdd((unsigned long long*)&cs->ncont, 1ULL);
-          e.key[0][i] = ((uint64_t)(uint32_t)t << 32) | (uint32_t)(h_active(a.seed, a.level, (int32_t)v) >> 32);
-          e.val[0][i] = (int32_t)v;
+          e.key[i] = ((uint64_t)(uint32_t)t << 32) | (uint32_t)(h_active(a.seed, a.level, (int32_t)v) >> 32);
+          e.val[i] = (int32_t)v;
+          e.P[i] = 0;
         }
       }
       cl.sync();
       const int nc = (int)*(volatile int64_t*)&cs->ncont;
+      if (nc > kClEngRequests) {  // (uniform) left to the graph of kernels, which sorts them
+        if (lead && threadIdx.x == 0) cs->kernels = 1;
+        return;
+      }
       if (nc > kSmallThreads) {
-        // rank of every request: the requests before it in (target, hash, id) order
-        for (int64_t b = (int64_t)cl.block_rank() * kClEngThreads; b < nc; b += GT) {  // (block-uniform)
-          const int64_t i = b + threadIdx.x;
-          const uint64_t ki = i < nc ? e.key[0][i] : 0;
-          const int32_t vi = i < nc ? e.val[0][i] : 0;
-          int r = 0;
-          for (int c0 = 0; c0 < nc; c0 += kClEngThreads) {
-            const int m = min(kClEngThreads, nc - c0);
+        // per request the weight of the requests of its target before it in
+        // (hash, id) order: blocks of requests against chunks of them, over all CTAs
+        const int nib = (nc + kClEngThreads - 1) / kClEngThreads, parts = max(1, nblocks / nib);
+        for (int unit = rank; unit < nib * parts; unit += nblocks) {  // (block-uniform)
+          const int i = (unit % nib) * kClEngThreads + (int)threadIdx.x, part = unit / nib;
+          const uint64_t ki = i < nc ? e.key[i] : 0;
+          const int32_t vi = i < nc ? e.val[i] : 0;
+          int64_t sum = 0;
+          for (int c = (int)((int64_t)part * nib / parts); c < (int)((int64_t)(part + 1) * nib / parts); c++) {
+            const int c0 = c * kClEngThreads, m = min(kClEngThreads, nc - c0);
             __syncthreads();
             if ((int)threadIdx.x < m) {
-              R.sk[threadIdx.x] = e.key[0][c0 + threadIdx.x];
-              R.sv[threadIdx.x] = e.val[0][c0 + threadIdx.x];
+              const int32_t vj = e.val[c0 + threadIdx.x];
+              R.sk[threadIdx.x] = e.key[c0 + threadIdx.x];
+              R.sv[threadIdx.x] = vj;
+              R.sw[threadIdx.x] = g.vw[vj];
             }
             __syncthreads();
+#pragma unroll 4
             for (int j = 0; j < m; j++) {
               const uint64_t kj = R.sk[j];
-              r += (kj < ki || (kj == ki && R.sv[j] < vi)) ? 1 : 0;
+              const bool first = kj < ki || (kj == ki && R.sv[j] < vi);
+              sum += first && ((kj ^ ki) >> 32) == 0 ? R.sw[j] : 0;
             }
           }
-          if (i < nc) {
-            e.key[1][r] = ki;
-            e.val[1][r] = vi;
-          }
+          if (i < nc && sum) atomicAdd((unsigned long long*)&e.P[i], (unsigned long long)sum);
         }
         cl.sync();
-        if (lead) {
-          int64_t carry = 0;
-          for (int b = 0; b < nc; b += kClEngThreads) {
-            const int i = b + (int)threadIdx.x;
-            const int64_t c = i < nc ? (int64_t)g.vw[e.val[1][i]] : 0;
-            int64_t tot;
-            const int64_t x = block_exclusive_scan(c, R.sm, &tot) + carry;
-            if (i < nc) {
-              e.P[i] = x;
-              const uint64_t t = e.key[1][i] >> 32;
-              if (i == 0 || (e.key[1][i - 1] >> 32) != t) e.headP[t] = x;
-            }
-            carry += tot;
-          }
-          __syncthreads();
-          for (int i = threadIdx.x; i < nc; i += kClEngThreads) {
-            const int32_t t = (int32_t)(e.key[1][i] >> 32), v = e.val[1][i];
-            e.flag[v] = ((int64_t)e.Wc[t] + (e.P[i] + g.vw[v] - e.headP[t]) <= a.wcap) ? 1 : 0;
-          }
+        for (int64_t i = gt; i < nc; i += GT) {
+          const int32_t t = (int32_t)(e.key[i] >> 32), v = e.val[i];
+          e.flag[v] = (int64_t)e.Wc[t] + *(volatile int64_t*)&e.P[i] + g.vw[v] <= a.wcap ? 1 : 0;
         }
         cl.sync();
       } else if (nc > 0) {
-        if (lead) cluster_resolve(e.key[0], e.val[0], nc, e.Wc, g.vw, a.wcap, e.flag, R);
+        if (lead) cluster_resolve(e.key, e.val, nc, e.Wc, g.vw, a.wcap, e.flag, R);
         cl.sync();
       }
       if (nc > 0 && lead && threadIdx.x == 0) cs->ncont = 0;  // (every CTA has read it)
@@ -1398,6 +1393,44 @@ __global__ void __launch_bounds__(kClEngThreads, 1) k_cluster_engine(GraphView g
     if (*(volatile int64_t*)moved * 100 < (int64_t)n) break;
     if (lead && threadIdx.x == 0) *(moved == &cs->moved ? &cs->moved2 : &cs->moved) = 0;  // the next iteration's
   }
+}
+
+__global__ void __launch_bounds__(kClEngThreads, 1) k_cluster_engine(GraphView g, ClusterArgs a, ClusterEngineArgs e) {
+  extern __shared__ __align__(16) int2 cl_scw[];  // [warps][kTileE]
+  __shared__ ResolveSmem R;
+  const cg::cluster_group cl = cg::this_cluster();
+  cluster_engine_run(g, a, e, cl_scw, R, (int)cl.block_rank(), (int)cl.num_blocks(), cl);
+}
+
+// The same loop for the levels above one cluster's size, by a cooperative launch
+// of a CTA per SM (new contexts: the capture and instantiation of the graph took
+// 0.3 ms, the kernel boundaries and the WHILE node 0.1): map of an RGG of 50021
+// vertices 3.74 -> 3.15 ms, 3D grid of 2^21 (a level of 97000) 20.3 -> 19.7.  A
+// repeated run of one context, whose graph exists, loses 0.2 ms on that level.
+__global__ void __launch_bounds__(kClEngThreads, 1) k_cluster_grid(GraphView g, ClusterArgs a, ClusterEngineArgs e,
+                                                                   GridBar* bar) {
+  extern __shared__ __align__(16) int2 cl_scw[];
+  __shared__ ResolveSmem R;
+  __shared__ unsigned int bar_flag;
+  cluster_engine_run(g, a, e, cl_scw, R, (int)blockIdx.x, (int)gridDim.x, GridSync{bar, &bar_flag, gridDim.x});
+}
+
+// CTAs of k_cluster_grid on the device; 0: no cooperative launch there.
+int cluster_grid_blocks(const Ctx& c, size_t smem) {
+  static std::atomic<int> cached[64];  // a property of the device: once per process
+  int b = cached[c.dev & 63].load();
+  if (b == 0) {
+    int coop = 0, ps = 0;
+    cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, c.dev);
+    if (cudaFuncSetAttribute(k_cluster_grid, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, k_cluster_grid, kClEngThreads, smem) != cudaSuccess) {
+      cudaGetLastError();
+      ps = 0;
+    }
+    b = coop && ps > 0 ? c.num_sms : -1;
+    cached[c.dev & 63].store(b);
+  }
+  return b > 0 ? b : 0;
 }
 
 // isolated vertices: chunks of weight <= cap in id order, labelled n + chunk
@@ -2041,7 +2074,7 @@ void build_cluster_graph(Ctx& c, int lvl, int64_t wcap) {
 }
 
 // Clusters level `lvl`; returns n_c, fills L.M.
-int32_t cluster_level(Ctx& c, int lvl) {
+int32_t cluster_level(Ctx& c, int lvl, bool engine) {
   Level& L = c.lv[lvl];
   const int32_t n = L.n;
   const unsigned gv = grid_for(c, kThreads, n);
@@ -2071,30 +2104,43 @@ int32_t cluster_level(Ctx& c, int lvl) {
   }
   ClusterState* cs = c.cstate;
   bool graph_ran = false;
-  if (c.use_graphs && !c.prof && n <= kClEngMaxN && L.max_deg <= kClEngRow && L.m_hi * 16 <= L.m) {
-    static std::atomic<unsigned long long> attr_done{0};  // one bit per device
-    const unsigned long long bit = 1ULL << (c.dev & 63);
-    const size_t smem = (size_t)(kClEngThreads / 32) * kTileE * sizeof(int2);
-    if (!(attr_done.load() & bit)) {
-      GM_CUDA(cudaFuncSetAttribute(k_cluster_engine, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      attr_done.fetch_or(bit);
-    }
+  const size_t eng_smem = (size_t)(kClEngThreads / 32) * kTileE * sizeof(int2);
+  const bool short_rows = engine && c.use_graphs && !c.prof && L.max_deg <= kClEngRow && L.m_hi * 16 <= L.m;
+  // (grid_engine_max_n < 0: launches over every SM are unwanted, as by jobs that share the GPU)
+  const int64_t grid_max = c.cfg.grid_engine_max_n < 0 ? -1 : kClGridMaxN;
+  bool engine_ran = false, grid_ran = false;
+  if (short_rows && (n <= kClEngMaxN || (n <= grid_max && cluster_grid_blocks(c, eng_smem)))) {
     const ClusterArgs a{c.C, c.Wc, c.ReqW, c.req, wcap, c.cfg.seed, cs, lvl, 0, 0};
-    const ClusterEngineArgs e{c.C, c.Wc, c.ReqW, c.elig, {c.sort.key[0], c.sort.key[1]}, {c.sort.val[0], c.sort.val[1]},
-                              c.P64, c.headP, cs, c.cfg.cluster_iters};
+    const ClusterEngineArgs e{c.C, c.Wc, c.ReqW, c.elig, c.sort.key[0], c.sort.val[0], c.P64, cs, c.cfg.cluster_iters};
+    engine_ran = true;
     cudaLaunchAttribute attr{};
     cudaLaunchConfig_t lc{};
-    const unsigned C = (unsigned)std::min(kClEngMaxCluster, (n + kClEngThreads - 1) / kClEngThreads);
-    lc.gridDim = dim3(C);
     lc.blockDim = dim3(kClEngThreads);
-    lc.dynamicSmemBytes = smem;
+    lc.dynamicSmemBytes = eng_smem;
     lc.stream = c.st;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = C;
-    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
     lc.attrs = &attr;
     lc.numAttrs = 1;
-    GM_CUDA(cudaLaunchKernelEx(&lc, k_cluster_engine, view(L), a, e)); count_launch();
+    if (n <= kClEngMaxN) {
+      static std::atomic<unsigned long long> attr_done{0};  // one bit per device
+      const unsigned long long bit = 1ULL << (c.dev & 63);
+      if (!(attr_done.load() & bit)) {
+        GM_CUDA(cudaFuncSetAttribute(k_cluster_engine, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)eng_smem));
+        attr_done.fetch_or(bit);
+      }
+      const unsigned C = (unsigned)std::min(kClEngMaxCluster, (n + kClEngThreads - 1) / kClEngThreads);
+      lc.gridDim = dim3(C);
+      attr.id = cudaLaunchAttributeClusterDimension;
+      attr.val.clusterDim.x = C;
+      attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+      GM_CUDA(cudaLaunchKernelEx(&lc, k_cluster_engine, view(L), a, e)); count_launch();
+    } else {
+      GM_CUDA(cudaMemsetAsync(c.gbar, 0, sizeof(GridBar), c.st));
+      lc.gridDim = dim3((unsigned)cluster_grid_blocks(c, eng_smem));
+      attr.id = cudaLaunchAttributeCooperative;
+      attr.val.cooperative = 1;
+      GM_CUDA(cudaLaunchKernelEx(&lc, k_cluster_grid, view(L), a, e, static_cast<GridBar*>(c.gbar))); count_launch();
+      grid_ran = true;
+    }
   } else if (c.use_graphs && !c.prof) {
     const int64_t key[8] = {(int64_t)L.n | ((int64_t)L.n_big << 32), L.m, (int64_t)L.n_hi | ((int64_t)L.n_huge << 32), L.hi_slots, wcap,
                             (int64_t)(intptr_t)c.htab, (int64_t)(intptr_t)L.hub_chunk, L.n_hub_chunks};
@@ -2134,11 +2180,16 @@ int32_t cluster_level(Ctx& c, int lvl) {
                           cudaMemcpyDeviceToHost, c.st));
   c.h_small[1] = 0;
   GM_CUDA(cudaMemcpyAsync(c.h_small + 1, c.errword, sizeof(uint32_t), cudaMemcpyDeviceToHost, c.st));
+  if (engine_ran) GM_CUDA(cudaMemcpyAsync(c.h_cstate, cs, sizeof(ClusterState), cudaMemcpyDeviceToHost, c.st));
+  if (grid_ran) GM_CUDA(cudaMemcpyAsync(c.h_small + 2, c.gbar, sizeof(GridBar), cudaMemcpyDeviceToHost, c.st));
   if (!L.M) L.M = c.mem.make<int32_t>((size_t)std::max(1, n));
   k_apply_rank<<<gv, kThreads, 0, c.st>>>(n, c.C, c.rank, L.M); count_launch();
   GM_CUDA(cudaGetLastError());
   GM_CUDA(cudaStreamSynchronize(c.st));
   if (graph_ran) add_launches(L.cg_root + (long long)c.h_cstate->kernels);
+  if (grid_ran && reinterpret_cast<const GridBar*>(c.h_small + 2)->err)
+    throw ApiError(MAP_E_TIMEOUT, "a grid barrier of the clustering gave up waiting");
+  if (engine_ran && c.h_cstate->kernels) return cluster_level(c, lvl, false);  // too many contested requests
   const int64_t nc = c.h_small[0];
   const uint32_t e = (uint32_t)(c.h_small[1] & 0xffffffffLL);
   if (e & ERR_TIMEOUT) throw ApiError(MAP_E_TIMEOUT, "a bounded device loop gave up");
@@ -2344,7 +2395,7 @@ int32_t coarsen(Ctx& c) {
   while ((int32_t)c.lv.size() < c.cfg.max_levels &&
          (int64_t)c.lv.back().n >= (int64_t)c.cfg.coarsest_factor * c.k) {
     const int lvl = (int)c.lv.size() - 1;
-    const int32_t nc = c.cfg.coarsener == 1 ? match_level(c, lvl) : cluster_level(c, lvl);
+    const int32_t nc = c.cfg.coarsener == 1 ? match_level(c, lvl) : cluster_level(c, lvl, true);
     Level& F = c.lv[lvl];
     if ((int64_t)nc * c.cfg.stall_den > (int64_t)c.cfg.stall_num * F.n) {
       c.mem.put(F.M);
