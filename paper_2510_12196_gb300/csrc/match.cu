@@ -21,6 +21,7 @@
 #include <string>
 
 #include "engine.h"
+#include "gridbar.cuh"
 
 namespace gm {
 namespace {
@@ -83,24 +84,24 @@ __device__ __forceinline__ void pref_offer(Pref& b, uint64_t ww, uint64_t c, int
   if (hu < b.h || (hu == b.h && u < b.u)) b = Pref{ww, c, hu, u, true};
 }
 
-__global__ void __launch_bounds__(kMThreads) k_match_prefer(MatchGraph g, const int32_t* __restrict__ mate,
-                                                             int64_t lmax, uint64_t seed, int32_t level,
-                                                             int32_t* __restrict__ pref) {
+// Preferences of the vertices by nsw sub-warps; `first` is the caller's.
+// Mate: the partners behind a load that suits the kernel.
+template <class Mate>
+__device__ __forceinline__ void match_prefer(const MatchGraph& g, const Mate& mate, int64_t lmax, uint64_t seed,
+                                             int32_t level, int32_t* pref, int64_t first, int64_t nsw) {
   const int sl = threadIdx.x & (kSubWarp - 1);
-  const int64_t nsw = ((int64_t)gridDim.x * blockDim.x) / kSubWarp;
   // the whole warp iterates together (the shuffles below take every lane)
-  const int64_t first = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kSubWarp;
   const int64_t wfirst = first - (first % (32 / kSubWarp));
   for (int64_t w0 = wfirst; w0 < g.n; w0 += nsw) {
     const int64_t v0 = w0 + (first - wfirst);
-    const bool free_v = v0 < g.n && mate[v0] < 0;
+    const bool free_v = v0 < g.n && mate((int32_t)v0) < 0;
     const int32_t v = (int32_t)v0;
     Pref b{0, 0, 0, -1, false};
     if (free_v) {
       const int64_t cv = g.vw[v];
       for (int64_t x = g.xadj[v] + sl; x < g.xadj[v + 1]; x += kSubWarp) {
         const int32_t u = g.adj[x];
-        if (mate[u] >= 0) continue;
+        if (mate(u) >= 0) continue;
         const int64_t cu = g.vw[u];
         if (cv + cu > lmax) continue;
         const uint64_t w = (uint64_t)g.adjw[x];
@@ -125,6 +126,23 @@ __global__ void __launch_bounds__(kMThreads) k_match_prefer(MatchGraph g, const 
     }
     if (sl == 0 && v0 < g.n) pref[v] = free_v ? b.u : -1;
   }
+}
+
+struct ConstMate {
+  const int32_t* __restrict__ p;
+  __device__ __forceinline__ int32_t operator()(int32_t v) const { return p[v]; }
+};
+struct PlainMate {  // the partners change inside the launch
+  const int32_t* p;
+  __device__ __forceinline__ int32_t operator()(int32_t v) const { return p[v]; }
+};
+
+__global__ void __launch_bounds__(kMThreads) k_match_prefer(MatchGraph g, const int32_t* __restrict__ mate,
+                                                             int64_t lmax, uint64_t seed, int32_t level,
+                                                             int32_t* __restrict__ pref) {
+  match_prefer(g, ConstMate{mate}, lmax, seed, level, pref,
+               ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / kSubWarp,
+               ((int64_t)gridDim.x * blockDim.x) / kSubWarp);
 }
 
 // warp-aggregated addition to a device counter
@@ -300,6 +318,64 @@ __global__ void k_mt_stage_end(MatchState* s, unsigned long long body_kernels) {
   s->kernels += body_kernels;
 }
 
+// All heavy-edge rounds of a level in one cooperative launch.  A new context
+// used to capture and instantiate a graph for every level of the matching,
+// 0.3 ms each, for rounds of two kernels of a few microseconds: map of an RGG of
+// 2^18 vertices by matching (eight levels) 12.7 -> 9.3 ms, 9.0 -> 8.5 on a kept
+// context whose graphs exist.  (The two-hop stages follow as launches, one read
+// of the count each; most levels need none.)
+constexpr int kMRoundThreads = 1024;
+constexpr int kMRoundMaxN = 1 << 18;
+constexpr int kMRoundShared = 16;  // CTAs at most where launches over every SM are unwanted
+__global__ void __launch_bounds__(kMRoundThreads, 1) k_match_rounds(MatchGraph g, int32_t* mate, int32_t* pref,
+                                                                    int64_t lmax, uint64_t seed, int32_t level,
+                                                                    int32_t rounds, MatchState* s, GridBar* bar) {
+  __shared__ unsigned int bar_flag;
+  const GridSync grid{bar, &bar_flag, gridDim.x};
+  const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, GT = (int64_t)gridDim.x * blockDim.x;
+  const bool lead = gt == 0;
+  for (int64_t v = gt; v < g.n; v += GT) mate[v] = -1;
+  if (lead) {
+    s->matched = 0;
+    s->now = 0;
+    s->got = 0;
+    s->round = 0;
+    s->kernels = 0;
+  }
+  grid.sync();
+  for (int32_t r = 0; r < rounds; r++) {
+    match_prefer(g, PlainMate{mate}, lmax, seed, level, pref, gt / kSubWarp, GT / kSubWarp);
+    grid.sync();
+    int64_t* now = (r & 1) ? &s->got : &s->now;
+    int64_t mine = 0;
+    for (int64_t v = gt; v < g.n; v += GT) {
+      const int32_t u = pref[v];
+      if (u >= 0 && pref[u] == (int32_t)v) {
+        mate[v] = u;
+        mine++;
+      }
+    }
+    count_add(now, mine);
+    grid.sync();
+    const int64_t x = *(volatile int64_t*)now;
+    if (lead) {
+      s->matched += x;
+      *(now == &s->now ? &s->got : &s->now) = 0;  // the next round's; all have read the last one's
+    }
+    if (x == 0) break;
+  }
+}
+
+// CTAs of k_match_rounds for a level of n vertices; 0: the graph of kernels.
+int match_round_blocks(const Ctx& c, int32_t n) {
+  if (n > kMRoundMaxN) return 0;
+  const int want = (int)std::min<int64_t>(c.num_sms, ((int64_t)n * kSubWarp + kMRoundThreads - 1) / kMRoundThreads);
+  if (c.cfg.grid_engine_max_n < 0 && want > kMRoundShared) return 0;
+  int coop = 0;
+  cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, c.dev);
+  return coop ? std::max(1, want) : 0;
+}
+
 unsigned mgrid(const Ctx& c, int64_t items_per_block, int64_t n) {
   int64_t g = (n + items_per_block - 1) / items_per_block;
   const int64_t cap = (int64_t)c.num_sms * 8;
@@ -431,7 +507,8 @@ int32_t match_level(Ctx& c, int lvl) {
   const int32_t n = L.n;
   MatchState* s = state_of(c);
   if (!L.M) L.M = c.mem.make<int32_t>((size_t)std::max(1, n));
-  if (c.use_graphs && !c.prof) {
+  const int blocks = c.use_graphs && !c.prof ? match_round_blocks(c, n) : 0;
+  if (c.use_graphs && !c.prof && !blocks) {
     // the graph writes L.M, which a stalled level gives back, so its address is part of the key
     const int64_t key[6] = {(int64_t)n, L.m, c.lmax, (int64_t)c.cfg.match_rounds, -1, (int64_t)(intptr_t)L.M};
     bool same = L.cgexec != nullptr;
@@ -453,6 +530,33 @@ int32_t match_level(Ctx& c, int lvl) {
     GM_CUDA(cudaStreamSynchronize(c.st));
     return c.h_small[0];
   };
+  if (blocks) {
+    GM_CUDA(cudaMemsetAsync(c.gbar, 0, sizeof(GridBar), c.st));
+    cudaLaunchAttribute attr{};
+    cudaLaunchConfig_t lc{};
+    lc.gridDim = dim3((unsigned)blocks);
+    lc.blockDim = dim3(kMRoundThreads);
+    lc.stream = c.st;
+    attr.id = cudaLaunchAttributeCooperative;
+    attr.val.cooperative = 1;
+    lc.attrs = &attr;
+    lc.numAttrs = 1;
+    GM_CUDA(cudaLaunchKernelEx(&lc, k_match_rounds, mview(L), c.C, c.req, c.lmax, c.cfg.seed, (int32_t)lvl,
+                               c.cfg.match_rounds, s, static_cast<GridBar*>(c.gbar))); count_launch();
+    GM_CUDA(cudaMemcpyAsync(c.h_small + 2, c.gbar, sizeof(GridBar), cudaMemcpyDeviceToHost, c.st));
+    int64_t matched = read(&s->matched);
+    if (reinterpret_cast<const GridBar*>(c.h_small + 2)->err)
+      throw ApiError(MAP_E_TIMEOUT, "a grid barrier of the matching gave up waiting");
+    for (int stage = 1; stage <= 4 && 4 * matched <= 3 * (int64_t)n; stage++) {
+      k_mt_stage_begin<<<1, 1, 0, c.st>>>(s, n, 0, 0); count_launch();
+      emit_stage(c, lvl, stage, c.st, nullptr);
+      k_mt_stage_end<<<1, 1, 0, c.st>>>(s, 0); count_launch();
+      matched = read(&s->matched);
+    }
+    emit_number(c, lvl, c.st);
+    GM_CUDA(cudaGetLastError());
+    return (int32_t)read(&s->nc);
+  }
   GM_CUDA(cudaMemsetAsync(c.C, 0xFF, (size_t)std::max(1, n) * sizeof(int32_t), c.st));
   k_mt_init<<<1, 1, 0, c.st>>>(s, c.cfg.match_rounds, 0, 0); count_launch();
   for (int32_t r = 0; r < c.cfg.match_rounds; r++) {
