@@ -96,7 +96,8 @@ typedef struct {
                             more than 1/16 of their entries in rows of degree > 32 left to the graph of kernels);
                             -1: never */
   int32_t grid_engine_max_n; /* larger levels with at most this many vertices (same condition) run the same
-                            engine over all SMs (cooperative launch); 0: library default (262144); -1: never */
+                            engine over all SMs (cooperative launch); 0: library default (262144, as above);
+                            -1: never, and no cooperative launch for the clustering either */
   int32_t coarsener;     /* 0: label-propagation clustering (default); 1: two-hop matching (heavy-edge rounds
                             with the rating w^2 / (c(u) c(v)), then leaf, twin, relative and isolated pairing
                             while at most 75% of the vertices are matched) */
@@ -378,7 +379,7 @@ GPUMAP_API map_status map_selftest_barrier_timeout(void* stream);
  * level, rounds) on the same context, whatever the schedule.
  *
  * The schedule (CTAs per job and staged CSR entries per warp tile) is picked
- * by timing every candidate on the batch itself during the first launch (the
+ * by timing candidates on the batch itself during the first launch (the
  * jobs' mappings are saved and restored around the trials) and cached per
  * batch shape for the rest of the process; autotune = 0 takes `cluster` and
  * `tile_entries` instead (0: a size-based default).

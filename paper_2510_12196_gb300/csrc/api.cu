@@ -365,8 +365,8 @@ map_status map_create(const int64_t* xadj, const int32_t* adjncy, const int32_t*
     if (c.cfg.reb_objective < 0 || c.cfg.reb_objective > 1)
       throw ApiError(MAP_E_INVALID, "reb_objective must be 0 or 1");
     if (c.cfg.mid_deg != 0 && (c.cfg.mid_deg <= kLowDeg || c.cfg.mid_deg > kMidDeg))
-      throw ApiError(MAP_E_INVALID, "mid_deg must be 0 (autotuned) or in 33..255");
-    if (c.cfg.split_deg < 0) throw ApiError(MAP_E_INVALID, "split_deg must be 0 (autotuned) or positive");
+      throw ApiError(MAP_E_INVALID, "mid_deg must be 0 (default) or in 33..255");
+    if (c.cfg.split_deg < 0) throw ApiError(MAP_E_INVALID, "split_deg must be 0 (default) or positive");
     c.st = (cudaStream_t)stream;
     GM_CUDA(cudaGetDevice(&c.dev));
     sort_init();

@@ -18,8 +18,8 @@
 // digit counts are kept per block, not per tile, and a block's writes to a
 // digit follow one another.  What bounds it is HBM traffic: 8 + 4 (M from L2)
 // + 8 bytes in k_ct_gen, 16 per scatter, 8 per count, 16 to number and write.
-// R-MAT 2^22, 128 M entries to 84 M, and two more levels of 84 and 80 M: 3.3 ms a
-// level (k_ct_gen 0.58, two scatters 1.79, counts 0.17 + 0.12, k_ct_apply 0.53),
+// R-MAT 2^22, 128 M entries to 84 M, and two more levels of 84 and 80 M: 3.2 ms a
+// level (k_ct_gen 0.58, two scatters 1.66, counts 0.17 + 0.12, k_ct_apply 0.53),
 // where keys (source, target) with separate weights, five or six 8-bit passes
 // with per-tile digit counts and three scans took 11 ms.
 #include <algorithm>

@@ -366,7 +366,7 @@ KERNEL_CLASSES = {0: "lp_gain", 1: "lp_after", 2: "eval_J", 3: "cluster", 4: "ra
 # the kernel each profiled class times
 KERNEL_OF_CLASS = {"lp_gain": "k_lp_gain_tile", "lp_after": "k_lp_after_low", "eval_J": "k_eval_tile",
                    "cluster": "k_cluster_tile", "radix_sort": "radix-sort passes (k_sort_hist + k_sort_scatter)",
-                   "eval_J_close": "k_eval_tile (controller only)", "match_prefer": "k_match_prefer",
+                   "eval_J_close": "k_control", "match_prefer": "k_match_prefer",
                    "cluster_mid": "k_cluster_mid", "cluster_high": "k_cluster_high", "eval_J_mid": "k_eval_mid",
                    "eval_J_high": "k_eval_high", "lp_gain_mid": "k_lp_gain_mid", "lp_gain_high": "k_lp_gain_high"}
 
