@@ -218,6 +218,7 @@ int radix_sort_pairs(SortBufs& b, int64_t max_n, const int64_t* d_n, int bits, c
                      unsigned long long* kcount) {
   if (max_n <= 0 || bits <= 0) return 0;
   const int passes = (bits + 7) / 8;
+  const long long per_pass = 2 + scan_launches(256 * sort_tiles(max_n));
   const int out = passes & 1;  // buffer holding the result after `passes` swaps
   sort_init();
   if (!d_n) {
@@ -236,13 +237,13 @@ int radix_sort_pairs(SortBufs& b, int64_t max_n, const int64_t* d_n, int bits, c
   if (max_n <= kSmallSort) return out;
   if (cap && cap->on()) {
     cudaGraphConditionalHandle h = cap_handle(st, 0);
-    k_sort_gate<<<1, 1, 0, st>>>(d_n, h, kcount, (unsigned long long)passes * 5); count_launch();
+    k_sort_gate<<<1, 1, 0, st>>>(d_n, h, kcount, (unsigned long long)(passes * per_pass)); count_launch();
     long long body = 0;
     long long* outer = set_capture_counter(&body);
     cap_cond(*cap, st, h, cudaGraphCondTypeIf,
              [&](cudaStream_t bs) { sort_passes(b, max_n, d_n, bits, kSmallSort, bs); });
     set_capture_counter(outer);
-    if (body != (long long)passes * 5) throw std::runtime_error("radix_sort_pairs: unexpected pass kernel count");
+    if (body != passes * per_pass) throw std::runtime_error("radix_sort_pairs: unexpected pass kernel count");
   } else {
     sort_passes(b, max_n, d_n, bits, kSmallSort, st);
   }
