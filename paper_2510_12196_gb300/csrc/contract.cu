@@ -26,6 +26,7 @@
 #include <atomic>
 
 #include "engine.h"
+#include "search.h"
 
 namespace gm {
 namespace {
@@ -86,16 +87,10 @@ __global__ void k_ct_copy(const int64_t* src, int64_t* dst) { *dst = *src; }
 
 // Largest i in [0, n) with a[i] <= x (a[0] <= x); all kGenThreads threads call it.
 __device__ __forceinline__ int64_t find_row(const int64_t* __restrict__ a, int64_t n, int64_t x) {
-  int64_t lo = 0, len = n;
-  while (len > 1) {
-    const int64_t step = (len + kGenThreads - 1) / kGenThreads;
+  return last_by_probes(n, kGenThreads, [&](int64_t lo, int64_t len, int64_t step) {
     const int64_t at = (int64_t)threadIdx.x * step;
-    const int cnt = __syncthreads_count(at < len && a[lo + at] <= x);
-    const int64_t skip = cnt > 0 ? (cnt - 1) * step : 0;
-    lo += skip;
-    len = min(step, len - skip);
-  }
-  return lo;
+    return __syncthreads_count(at < len && a[lo + at] <= x);
+  });
 }
 
 // The words of the stream, in coarse source order.  A tile's rows are looked

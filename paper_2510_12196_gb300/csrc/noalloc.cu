@@ -25,6 +25,7 @@
 #include <string>
 
 #include "engine.h"
+#include "search.h"
 
 namespace gm {
 namespace {
@@ -88,19 +89,11 @@ constexpr int kNaCodes = 2048;
 
 // Largest v in [0, n) with xadj[v] <= e, -1 if none; all threads call it.
 __device__ __forceinline__ int32_t na_row_of(const int64_t* __restrict__ xadj, int32_t n, int64_t e) {
-  int32_t lo = 0, len = n;
-  bool first = true;
-  while (len > 1 || first) {
-    const int32_t step = (len + kNaThreads - 1) / kNaThreads;
+  if (xadj[0] > e) return -1;
+  return (int32_t)last_by_probes(n, kNaThreads, [&](int64_t lo, int64_t len, int64_t step) {
     const int64_t at = (int64_t)threadIdx.x * step;
-    const int cnt = __syncthreads_count(at < len && xadj[lo + at] <= e);
-    if (first && cnt == 0) return -1;
-    first = false;
-    const int32_t skip = cnt > 0 ? (cnt - 1) * step : 0;
-    lo += skip;
-    len = min(step, len - skip);
-  }
-  return lo;
+    return __syncthreads_count(at < len && xadj[lo + at] <= e);
+  });
 }
 
 __device__ __forceinline__ void na_load8(const int32_t* __restrict__ a, int64_t e, int cnt, bool vec,
@@ -194,13 +187,7 @@ __global__ void __launch_bounds__(kNaThreads, 5) k_na_eval(int32_t n, const int6
         return p >= 0 && p < t.k ? code_of(p) : -1;
       };
       auto search = [&](int32_t from, int x) {  // largest row i >= from with row_start(i) <= x
-        int32_t l = from, h = nr;
-        while (h - l > 1) {
-          const int32_t mid = (l + h) >> 1;
-          if (row_start(mid) <= x) l = mid;
-          else h = mid;
-        }
-        return l;
+        return last_by_bisection(from, nr, [&](int32_t i) { return row_start(i) <= x; });
       };
       const int64_t base = row_start(0);  // after the tile's start only when xadj[0] > 0
       int32_t i = search(0, first), cv = -1;
