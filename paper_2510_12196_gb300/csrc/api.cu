@@ -65,7 +65,7 @@ void keep_pool_memory(int dev) {
   done.fetch_or(bit);
 }
 
-void* DevMem::raw(size_t bytes) {
+void* DevMem::obtain(size_t bytes) {
   void* p = nullptr;
   if (afn && ffn) {
     p = afn(bytes, user, (void*)st);
@@ -78,85 +78,12 @@ void* DevMem::raw(size_t bytes) {
                                     cudaGetErrorString(e));
     }
   }
-  total += bytes;
-  peak = std::max(peak, total);
   return p;
 }
 
-void DevMem::add_slab(size_t bytes) {
-  slabs.reserve(slabs.size() + 1);
-  if (cur_left) free_list.push_back({cur, cur_left, true});
-  cur_left = 0;
-  cur = static_cast<char*>(raw(bytes));
-  slabs.push_back({cur, bytes, false});
-  cur_left = bytes;
-}
-
-void DevMem::reserve(size_t bytes) {
-  if (!afn && bytes <= kSlabReserve) add_slab((bytes + 255) & ~(size_t)255);
-}
-
-void* DevMem::get(size_t bytes) {
-  if (bytes == 0) bytes = 16;
-  bytes = (bytes + 255) & ~(size_t)255;
-  blocks.reserve(blocks.size() + 1);
-  free_list.reserve(slabs.size() + blocks.size() + 2);  // (put does not allocate)
-  const size_t slab = std::min<size_t>(kSlabMax, std::max<size_t>(256 << 10, total / 128));
-  if ((afn && ffn) || (bytes >= slab / 4 && bytes > cur_left)) {
-    void* p = raw(bytes);
-    blocks.push_back({p, bytes, false});
-    return p;
-  }
-  size_t best = free_list.size();  // the smallest free piece that is not much too large
-  for (size_t i = 0; i < free_list.size(); i++)
-    if (free_list[i].bytes >= bytes && free_list[i].bytes <= bytes + bytes / 4 + 4096 &&
-        (best == free_list.size() || free_list[i].bytes < free_list[best].bytes))
-      best = i;
-  if (best < free_list.size()) {
-    const Block b = free_list[best];
-    free_list[best] = free_list.back();
-    free_list.pop_back();
-    blocks.push_back(b);
-    return b.p;
-  }
-  if (bytes > cur_left) add_slab(slab);
-  void* p = cur;
-  cur += bytes;
-  cur_left -= bytes;
-  blocks.push_back({p, bytes, true});
-  return p;
-}
-
-void DevMem::put(void* p) {
-  for (size_t i = 0; i < blocks.size(); i++) {
-    if (blocks[i].p == p) {
-      const Block b = blocks[i];
-      blocks[i] = blocks.back();
-      blocks.pop_back();
-      if (b.slab) {
-        free_list.push_back(b);
-        return;
-      }
-      if (afn && ffn) ffn(p, b.bytes, user, (void*)st);
-      else cudaFreeAsync(p, st);
-      total -= b.bytes;
-      return;
-    }
-  }
-}
-
-void DevMem::release_all() {
-  for (auto* list : {&blocks, &slabs})
-    for (auto& b : *list) {
-      if (b.slab) continue;
-      if (afn && ffn) ffn(b.p, b.bytes, user, (void*)st);
-      else cudaFreeAsync(b.p, st);
-    }
-  blocks.clear();
-  slabs.clear();
-  free_list.clear();
-  cur_left = 0;
-  total = 0;
+void DevMem::raw_free(void* p, size_t bytes) noexcept {
+  if (afn && ffn) ffn(p, bytes, user, (void*)st);
+  else cudaFreeAsync(p, st);
 }
 
 cudaEvent_t Ctx::prof_begin() {

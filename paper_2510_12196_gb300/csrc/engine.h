@@ -10,6 +10,7 @@
 
 #include "../../include/gpumap.h"
 #include "common.cuh"
+#include "devmem.h"
 #include "prim.cuh"
 #include "mid.cuh"
 
@@ -145,48 +146,6 @@ struct HubRows {
 inline HubRows hub_rows(const Level& L) {
   return HubRows{L.hi, L.huge, L.n_huge, L.hub_pre, L.hub_chunk, L.n_hub_chunks};
 }
-
-// Device memory of one context.  With the caller's allocator every buffer is an
-// allocation of its own.  Without, small buffers are cut from slabs (the first
-// one sized for everything map_create needs) and go back to a free list; a
-// buffer above a quarter of a later slab is an allocation of its own, freed at
-// once, so that slabs cost little memory (0.2-2 % above 1 MB held).  A context
-// holds some seventy buffers, and their allocation and release one by one was
-// most of the cost of a small context, above all with several threads at it (a
-// stream-ordered allocation takes a lock of the device): hierarchical
-// multisection of an RGG of 2^17 vertices by 8 threads 38.5 -> 26.9 ms, 16
-// served jobs 33.3 -> 21.6 ms.
-// All buffers are used on the context's stream only, so a freed one can be
-// handed out again at once.
-struct DevMem {
-  static constexpr size_t kSlabMax = 1 << 20;       // a later slab: 1/128 of what is held, up to this
-  static constexpr size_t kSlabReserve = 64 << 20;  // a first slab of at most this size
-  map_alloc_fn afn = nullptr;
-  map_free_fn ffn = nullptr;
-  void* user = nullptr;
-  cudaStream_t st = nullptr;
-  struct Block {
-    void* p;
-    size_t bytes;
-    bool slab;  // cut from a slab
-  };
-  std::vector<Block> blocks;            // handed out
-  std::vector<Block> slabs, free_list;  // slabs, and the pieces given back
-  char* cur = nullptr;                  // rest of the newest slab
-  size_t cur_left = 0;
-  void* raw(size_t bytes);
-  void add_slab(size_t bytes);
-  void reserve(size_t bytes);  // the first slab
-  size_t total = 0;
-  size_t peak = 0;  // largest `total` so far
-  void* get(size_t bytes);
-  void put(void* p);
-  void release_all();
-  template <class T>
-  T* make(size_t count) {
-    return static_cast<T*>(get(count * sizeof(T)));
-  }
-};
 
 // statistics of the last hierarchical multisection run (hm.cu)
 struct HmStats {
