@@ -199,8 +199,8 @@ GPUMAP_API map_status map_block_weights(map_ctx* ctx, int32_t level, int64_t* ou
 GPUMAP_API map_status map_lp_step(map_ctx* ctx, int32_t level, int32_t* out_moved);
 
 /* The per-vertex results of the last map_lp_step on `level` (host arrays of
- * n_level entries, any may be NULL): target PE P'(v) (P(v) outside X),
- * gain g(v) (0 outside X), membership in X, and the lock (= moved) flags. */
+ * n_level entries, any may be NULL): target PE P'(v) (P(v) outside X; -1
+ * before the first step), gain g(v) (0 outside X), membership in X, and the lock (= moved) flags. */
 GPUMAP_API map_status map_get_lp_state(map_ctx* ctx, int32_t level, int32_t* pi_prime, int64_t* gain,
                             uint8_t* in_x, uint8_t* moved);
 

@@ -16,7 +16,7 @@ constexpr int32_t kHostConvert = 8192;  // mappings up to this size: a host loop
 __global__ void k_ids_of_codes(int32_t n, const int32_t* __restrict__ code, const int32_t* __restrict__ pe_of_code,
                                int32_t kc, int32_t* __restrict__ id) {
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t x = code[v];  // (targets that no step has set yet hold anything)
+    const int32_t x = code[v];
     id[v] = x >= 0 && x < kc ? pe_of_code[x] : -1;
   }
 }
@@ -36,7 +36,8 @@ unsigned grid(const Ctx& c, int64_t n) {
 
 }  // namespace
 
-// Reads n codes back as PE ids (synchronises).
+// Reads n codes back as PE ids, -1 where there is none: targets that no step
+// has set yet are -1 (synchronises).
 void download_mapping(Ctx& c, const int32_t* codes, int32_t n, int32_t* out) {
   const bool same = c.k == c.topo.kc;  // every code is a PE, and codes ascend with the ids
   const bool host = !same && n <= kHostConvert;
@@ -49,7 +50,10 @@ void download_mapping(Ctx& c, const int32_t* codes, int32_t n, int32_t* out) {
   GM_CUDA(cudaMemcpyAsync(out, codes, (size_t)n * sizeof(int32_t), cudaMemcpyDeviceToHost, c.st));
   GM_CUDA(cudaStreamSynchronize(c.st));
   if (host)
-    for (int32_t v = 0; v < n; v++) out[v] = c.pe_of_code[(size_t)out[v]];
+    for (int32_t v = 0; v < n; v++) {
+      const int32_t x = out[v];
+      out[v] = x >= 0 && x < c.topo.kc ? c.pe_of_code[(size_t)x] : -1;
+    }
 }
 
 // Sets n codes from PE ids; MAP_E_INVALID, and the codes unchanged, when an id

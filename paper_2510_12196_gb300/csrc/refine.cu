@@ -3938,6 +3938,7 @@ void refine_alloc(Ctx& c) {
   c.trace_maxw = c.mem.make<int64_t>(c.trace_cap);
   GM_CUDA(cudaMemsetAsync(c.Jacc, 0, sizeof(int64_t), c.st));
   GM_CUDA(cudaMemsetAsync(c.lock, 0, n, c.st));
+  GM_CUDA(cudaMemsetAsync(c.pp, 0xFF, n * sizeof(int32_t), c.st));  // no targets yet (map_get_lp_state)
   GM_CUDA(cudaMemsetAsync(c.counters, 0, CNT_N * sizeof(int64_t), c.st));
   GM_CUDA(cudaMemsetAsync(c.state, 0, sizeof(RefineState), c.st));
   static_assert(sizeof(RefineState) <= kPinnedBlock, "pinned block too small");
