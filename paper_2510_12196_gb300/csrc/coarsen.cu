@@ -2142,13 +2142,21 @@ int32_t cluster_level(Ctx& c, int lvl, bool engine) {
       grid_ran = true;
     }
   } else if (c.use_graphs && !c.prof) {
-    const int64_t key[8] = {(int64_t)L.n | ((int64_t)L.n_big << 32), L.m, (int64_t)L.n_hi | ((int64_t)L.n_huge << 32), L.hi_slots, wcap,
-                            (int64_t)(intptr_t)c.htab, (int64_t)(intptr_t)L.hub_chunk, L.n_hub_chunks};
+    // what the captured launches depend on (the longest row decides which hub kernels there are)
+    const int64_t key[Level::kCgKey] = {(int64_t)L.n | ((int64_t)L.n_big << 32),
+                                        L.m,
+                                        (int64_t)L.n_hi | ((int64_t)L.n_huge << 32),
+                                        L.hi_slots,
+                                        wcap,
+                                        (int64_t)(intptr_t)c.htab,
+                                        (int64_t)(intptr_t)L.hub_chunk,
+                                        L.n_hub_chunks,
+                                        L.max_deg};
     bool same = L.cgexec != nullptr;
-    for (int i = 0; i < 8 && same; i++) same = L.cg_key[i] == key[i];
+    for (int i = 0; i < Level::kCgKey && same; i++) same = L.cg_key[i] == key[i];
     if (!same) {
       build_cluster_graph(c, lvl, wcap);
-      for (int i = 0; i < 8; i++) L.cg_key[i] = key[i];
+      for (int i = 0; i < Level::kCgKey; i++) L.cg_key[i] = key[i];
     }
     GM_CUDA(cudaGraphLaunch(L.cgexec, c.st));
     // read back with the cluster count below (kernel accounting only)

@@ -130,7 +130,8 @@ struct Level {
   long long g_root = 0;  // kernel nodes outside the conditional bodies
   // instantiated clustering graph of this level and its key
   cudaGraphExec_t cgexec = nullptr;
-  int64_t cg_key[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  static constexpr int kCgKey = 9;
+  int64_t cg_key[kCgKey] = {};
   long long cg_root = 0;
 };
 
