@@ -367,6 +367,13 @@ GPUMAP_API map_status map_objective_noalloc(const int64_t* xadj, const int32_t* 
  * error.  The text is in map_last_error(NULL). */
 GPUMAP_API map_status map_selftest_barrier_timeout(void* stream);
 
+/* Self-test of the coarsening without its cooperative launches (none in the
+ * paper).  The next `launches` of them on this context wait for one block more
+ * than there are, so that their barriers give up after about a second, as they
+ * would where the GPU is taken away for that long; the coarsening then runs as
+ * a graph of kernels, with the same result.  0: none (the default). */
+GPUMAP_API map_status map_selftest_coarsen_timeout(map_ctx* ctx, int32_t launches);
+
 /* ------------------------------------------------------------------------
  * Batched refinement.  The paper refines one graph at a time; it has no
  * batched mode.  Here many contexts (graphs of uneven size, each with its own

@@ -730,6 +730,13 @@ map_status map_profile_read(map_ctx* ctx, int32_t which, int32_t level, int64_t*
 
 long long map_launch_count(void) { return gm::launch_count(); }
 
+map_status map_selftest_coarsen_timeout(map_ctx* ctx, int32_t launches) {
+  return guarded(ctx, [&](Ctx& c) {
+    if (launches < 0) throw ApiError(MAP_E_INVALID, "launches must be >= 0");
+    c.lost_arrivals = launches;
+  });
+}
+
 map_status map_selftest_barrier_timeout(void* stream) {
   last_create_error().clear();
   try {

@@ -1408,11 +1408,11 @@ __global__ void __launch_bounds__(kClEngThreads, 1) k_cluster_engine(GraphView g
 // vertices 3.74 -> 3.15 ms, 3D grid of 2^21 (a level of 97000) 20.3 -> 19.7.  A
 // repeated run of one context, whose graph exists, loses 0.2 ms on that level.
 __global__ void __launch_bounds__(kClEngThreads, 1) k_cluster_grid(GraphView g, ClusterArgs a, ClusterEngineArgs e,
-                                                                   GridBar* bar) {
+                                                                   GridBar* bar, unsigned arrivals) {
   extern __shared__ __align__(16) int2 cl_scw[];
   __shared__ ResolveSmem R;
   __shared__ unsigned int bar_flag;
-  cluster_engine_run(g, a, e, cl_scw, R, (int)blockIdx.x, (int)gridDim.x, GridSync{bar, &bar_flag, gridDim.x});
+  cluster_engine_run(g, a, e, cl_scw, R, (int)blockIdx.x, (int)gridDim.x, GridSync{bar, &bar_flag, arrivals});
 }
 
 // CTAs of k_cluster_grid on the device; 0: no cooperative launch there.
@@ -2138,7 +2138,8 @@ int32_t cluster_level(Ctx& c, int lvl, bool engine) {
       lc.gridDim = dim3((unsigned)cluster_grid_blocks(c, eng_smem));
       attr.id = cudaLaunchAttributeCooperative;
       attr.val.cooperative = 1;
-      GM_CUDA(cudaLaunchKernelEx(&lc, k_cluster_grid, view(L), a, e, static_cast<GridBar*>(c.gbar))); count_launch();
+      GM_CUDA(cudaLaunchKernelEx(&lc, k_cluster_grid, view(L), a, e, static_cast<GridBar*>(c.gbar),
+                                 bar_arrivals(c, lc.gridDim.x))); count_launch();
       grid_ran = true;
     }
   } else if (c.use_graphs && !c.prof) {
@@ -2195,8 +2196,8 @@ int32_t cluster_level(Ctx& c, int lvl, bool engine) {
   GM_CUDA(cudaGetLastError());
   GM_CUDA(cudaStreamSynchronize(c.st));
   if (graph_ran) add_launches(L.cg_root + (long long)c.h_cstate->kernels);
-  if (grid_ran && reinterpret_cast<const GridBar*>(c.h_small + 2)->err)
-    throw ApiError(MAP_E_TIMEOUT, "a grid barrier of the clustering gave up waiting");
+  // a barrier gave up waiting (its time runs on while other users of the GPU have it): the graph, which waits for none
+  if (grid_ran && reinterpret_cast<const GridBar*>(c.h_small + 2)->err) return cluster_level(c, lvl, false);
   if (engine_ran && c.h_cstate->kernels) return cluster_level(c, lvl, false);  // too many contested requests
   const int64_t nc = c.h_small[0];
   const uint32_t e = (uint32_t)(c.h_small[1] & 0xffffffffLL);

@@ -229,6 +229,7 @@ struct Ctx {
   // bumped by every coarsening (coarse level buffers may be freed and
   // reallocated): a batch built on this context refuses to launch after it
   uint64_t level_gen = 0;
+  int32_t lost_arrivals = 0;  // map_selftest_coarsen_timeout: launches that are still to give up
 
   // sort / scan scratch
   SortBufs sort;
@@ -378,6 +379,14 @@ class Branches {
     if (!tails.empty()) set(tails);
   }
 };
+
+// Arrivals that release the barriers of a cooperative launch of the coarsening (one that never comes where
+// map_selftest_coarsen_timeout asked for it).
+inline unsigned bar_arrivals(Ctx& c, unsigned blocks) {
+  if (c.lost_arrivals <= 0) return blocks;
+  c.lost_arrivals--;
+  return blocks + 1;
+}
 
 // initial.cu: breadth-first initial mapping of a large coarsest graph over the whole GPU; false when
 // its component labelling did not settle within its round limit (the caller then runs the one-CTA kernel)

@@ -97,6 +97,7 @@ _SIGS = {
     "map_launch_count": (C.c_longlong, []),
     "map_objective_noalloc": (C.c_int, [_P, _P, _P, _P, C.c_int32, _P, _P, _P, C.c_int32, _P, _P]),
     "map_selftest_barrier_timeout": (C.c_int, [_P]),
+    "map_selftest_coarsen_timeout": (C.c_int, [_P, C.c_int32]),
     "map_batch_opts_default": (None, [_P]),
     "map_batch_create": (C.c_int, [_P, C.c_int32, _P, _P, _P]),
     "map_batch_launch": (C.c_int, [_P]),
@@ -404,6 +405,11 @@ def map_objective_noalloc(xadj, adjncy, adjwgt, vwgt, n: int, pi, hier, dist, ou
 def map_selftest_barrier_timeout(stream=None) -> int:
     """Status of the bounded grid-barrier self-test (MAP_E_TIMEOUT = 5 is the pass)."""
     return int(lib().map_selftest_barrier_timeout(_stream_handle(stream)))
+
+
+def map_selftest_coarsen_timeout(ctx, launches: int) -> None:
+    """Lets the next ``launches`` cooperative launches of the context's coarsening give up (see include/gpumap.h)."""
+    _check(ctx, lib().map_selftest_coarsen_timeout(ctx, launches), "map_selftest_coarsen_timeout")
 
 
 class MapBatchOpts(C.Structure):
