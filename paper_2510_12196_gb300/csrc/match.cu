@@ -329,9 +329,10 @@ constexpr int kMRoundMaxN = 1 << 18;
 constexpr int kMRoundShared = 16;  // CTAs at most where launches over every SM are unwanted
 __global__ void __launch_bounds__(kMRoundThreads, 1) k_match_rounds(MatchGraph g, int32_t* mate, int32_t* pref,
                                                                     int64_t lmax, uint64_t seed, int32_t level,
-                                                                    int32_t rounds, MatchState* s, GridBar* bar) {
+                                                                    int32_t rounds, MatchState* s, GridBar* bar,
+                                                                    unsigned arrivals) {
   __shared__ unsigned int bar_flag;
-  const GridSync grid{bar, &bar_flag, gridDim.x};
+  const GridSync grid{bar, &bar_flag, arrivals};
   const int64_t gt = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, GT = (int64_t)gridDim.x * blockDim.x;
   const bool lead = gt == 0;
   for (int64_t v = gt; v < g.n; v += GT) mate[v] = -1;
@@ -501,13 +502,14 @@ void build_match_graph(Ctx& c, int lvl) {
 
 // Matches level lvl and writes its map to the next level into L.M; returns
 // n_c.  Uses the clustering scratch (labels as partners, requests as
-// preferences, the rank array) and the sort buffers.
-int32_t match_level(Ctx& c, int lvl) {
+// preferences, the rank array) and the sort buffers.  one_launch: the rounds of
+// a small level may run in one cooperative launch.
+int32_t match_level(Ctx& c, int lvl, bool one_launch) {
   Level& L = c.lv[lvl];
   const int32_t n = L.n;
   MatchState* s = state_of(c);
   if (!L.M) L.M = c.mem.make<int32_t>((size_t)std::max(1, n));
-  const int blocks = c.use_graphs && !c.prof ? match_round_blocks(c, n) : 0;
+  const int blocks = one_launch && c.use_graphs && !c.prof ? match_round_blocks(c, n) : 0;
   if (c.use_graphs && !c.prof && !blocks) {
     // the graph writes L.M, which a stalled level gives back, so its address is part of the key
     const int64_t key[6] = {(int64_t)n, L.m, c.lmax, (int64_t)c.cfg.match_rounds, -1, (int64_t)(intptr_t)L.M};
@@ -542,11 +544,12 @@ int32_t match_level(Ctx& c, int lvl) {
     lc.attrs = &attr;
     lc.numAttrs = 1;
     GM_CUDA(cudaLaunchKernelEx(&lc, k_match_rounds, mview(L), c.C, c.req, c.lmax, c.cfg.seed, (int32_t)lvl,
-                               c.cfg.match_rounds, s, static_cast<GridBar*>(c.gbar))); count_launch();
+                               c.cfg.match_rounds, s, static_cast<GridBar*>(c.gbar),
+                               bar_arrivals(c, (unsigned)blocks))); count_launch();
     GM_CUDA(cudaMemcpyAsync(c.h_small + 2, c.gbar, sizeof(GridBar), cudaMemcpyDeviceToHost, c.st));
     int64_t matched = read(&s->matched);
-    if (reinterpret_cast<const GridBar*>(c.h_small + 2)->err)
-      throw ApiError(MAP_E_TIMEOUT, "a grid barrier of the matching gave up waiting");
+    // a barrier gave up waiting: the graph, which waits for no other block
+    if (reinterpret_cast<const GridBar*>(c.h_small + 2)->err) return match_level(c, lvl, false);
     for (int stage = 1; stage <= 4 && 4 * matched <= 3 * (int64_t)n; stage++) {
       k_mt_stage_begin<<<1, 1, 0, c.st>>>(s, n, 0, 0); count_launch();
       emit_stage(c, lvl, stage, c.st, nullptr);

@@ -39,3 +39,9 @@ def _same(a, b):
 def test_clustering(name):
     g = GRAPHS[name]()
     _same(_run(g, 1), _run(g, 0))
+
+
+@pytest.mark.parametrize("name", GRAPHS)
+def test_matching(name):
+    g = GRAPHS[name]()
+    _same(_run(g, 2, coarsener=1), _run(g, 0, coarsener=1))
