@@ -1107,7 +1107,6 @@ __global__ void k_cluster_classify(int32_t n, const int32_t* __restrict__ req, c
 // the multi-CTA path (scan compaction in id order, stable radix sort).
 struct ResolveSmem {
   uint64_t sk[kSmallThreads];
-  int32_t sw[kSmallThreads];
   int32_t sv[kSmallThreads];
   uint64_t ok[kSmallThreads];
   int32_t ov[kSmallThreads];
@@ -1259,17 +1258,21 @@ __global__ void k_cl_end(ClusterState* cs, int32_t n, int32_t iters, cudaGraphCo
 // map of a 16^3 grid 4.3 -> 3.5 ms, hierarchical multisection of an RGG of 2^17
 // vertices (37 maps by 8 threads) 63 -> 38 ms.
 // For levels of at most kClEngMaxN vertices without rows above kClEngRow and
-// with few above kLowDeg (a sub-warp takes each).  Contested requests: up to
-// kSmallThreads are ordered by the first CTA; of longer lists all CTAs compare
-// every request with every other (45 us for 1.6e4 over 152 SMs, where a sort of
-// any length costs 100 us); above kClEngRequests the launch gives up.
+// with few above kLowDeg (a sub-warp takes each).  The contested requests are
+// chained by target, and each follows its target's chain to sum the weights of
+// the requests before it in (hash, id) order: chains are as long as a cluster
+// has neighbours that want in, a handful where the caps are tight and most
+// requests contested, however many there are in all (every request compared
+// with every other took 1 ms a sub-round of 1.6e4 on one cluster: coarsening of a
+// 3D grid of 32768 vertices on 4096 PEs 3.3 ms, now 0.56, the graph of kernels
+// 0.71; of an RGG of 131072 on 4096 PEs 1.6, 0.67 and 1.76).  With a chain of
+// kClEngChain requests or more the launch gives up: the graph sorts them.
 constexpr int kClEngThreads = 1024;
 constexpr int kClEngMaxN = 1 << 15;
 constexpr int kClGridMaxN = 1 << 17;
-constexpr int kClEngRequests = 1 << 14;
+constexpr int kClEngChain = 512;
 constexpr int kClEngMaxCluster = 8;  // the portable limit
 constexpr int kClEngRow = kTileE / 4;
-static_assert(kClEngThreads == kSmallThreads, "the resolution takes one request per thread");
 struct PlainLabel {  // labels change inside the launch: plain loads
   const int32_t* C;
   __device__ __forceinline__ int32_t operator()(int32_t u) const { return C[u]; }
@@ -1279,16 +1282,18 @@ struct ClusterEngineArgs {
   int32_t* Wc;
   int32_t* ReqW;
   uint8_t* flag;
-  uint64_t* key;  // contested requests: (target, tie-hash), vertex, weight of those before
-  int32_t* val;
-  int64_t* P;
+  int32_t* head;  // per target the contested request chained last (-1: none)
+  int32_t* next;  // per contested request the one chained before it
   ClusterState* cs;
   int32_t iters;
 };
+// The place of a contested request among those of its target.
+__device__ __forceinline__ uint32_t contest_hash(const ClusterArgs& a, int32_t v) {
+  return (uint32_t)(h_active(a.seed, a.level, v) >> 32);
+}
 template <class Sync>
 __device__ __forceinline__ void cluster_engine_run(const GraphView& g, ClusterArgs a, const ClusterEngineArgs& e,
-                                                   int2* cl_scw, ResolveSmem& R, int rank, int nblocks,
-                                                   const Sync& cl) {
+                                                   int2* cl_scw, int rank, int nblocks, const Sync& cl) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool lead = rank == 0;
   const int64_t gt = (int64_t)rank * kClEngThreads + threadIdx.x;
@@ -1301,6 +1306,7 @@ __device__ __forceinline__ void cluster_engine_run(const GraphView& g, ClusterAr
     e.C[v] = (int32_t)v;
     e.Wc[v] = g.vw[v];
     e.ReqW[v] = 0;
+    e.head[v] = -1;
   }
   if (lead && threadIdx.x == 0) {
     cs->moved = 0;
@@ -1317,68 +1323,44 @@ __device__ __forceinline__ void cluster_engine_run(const GraphView& g, ClusterAr
       for (int64_t tile = gw; tile < ntiles; tile += GW)
         cluster_rate_tile(g, a, tile, lane, cl_scw + warp * kTileE, PlainLabel{e.C}, kClEngRow);
       cl.sync();
+      bool mine2 = false;
       for (int64_t v = gt; v < n; v += GT) {
         const int32_t t = a.req[v];
         uint8_t f = 0;
         if (t >= 0) f = ((int64_t)e.Wc[t] + e.ReqW[t] <= a.wcap) ? 1 : 2;
         e.flag[v] = f;
         if (f == 2) {
-          const unsigned long long i = atomicAdd((unsigned long long*)&cs->ncont, 1ULL);
-          e.key[i] = ((uint64_t)(uint32_t)t << 32) | (uint32_t)(h_active(a.seed, a.level, (int32_t)v) >> 32);
-          e.val[i] = (int32_t)v;
-          e.P[i] = 0;
+          e.next[v] = atomicExch(&e.head[t], (int32_t)v);
+          mine2 = true;
         }
       }
+      if (__syncthreads_or(mine2) && threadIdx.x == 0) *(volatile int64_t*)&cs->ncont = 1;
       cl.sync();
-      const int nc = (int)*(volatile int64_t*)&cs->ncont;
-      if (nc > kClEngRequests) {  // (uniform) left to the graph of kernels, which sorts them
-        if (lead && threadIdx.x == 0) cs->kernels = 1;
-        return;
-      }
-      if (nc > kSmallThreads) {
-        // per request the weight of the requests of its target before it in
-        // (hash, id) order: blocks of requests against chunks of them, over all CTAs
-        const int nib = (nc + kClEngThreads - 1) / kClEngThreads, parts = max(1, nblocks / nib);
-        for (int unit = rank; unit < nib * parts; unit += nblocks) {  // (block-uniform)
-          const int i = (unit % nib) * kClEngThreads + (int)threadIdx.x, part = unit / nib;
-          const uint64_t ki = i < nc ? e.key[i] : 0;
-          const int32_t vi = i < nc ? e.val[i] : 0;
-          int64_t sum = 0;
-          for (int c = (int)((int64_t)part * nib / parts); c < (int)((int64_t)(part + 1) * nib / parts); c++) {
-            const int c0 = c * kClEngThreads, m = min(kClEngThreads, nc - c0);
-            __syncthreads();
-            if ((int)threadIdx.x < m) {
-              const int32_t vj = e.val[c0 + threadIdx.x];
-              R.sk[threadIdx.x] = e.key[c0 + threadIdx.x];
-              R.sv[threadIdx.x] = vj;
-              R.sw[threadIdx.x] = g.vw[vj];
-            }
-            __syncthreads();
-#pragma unroll 4
-            for (int j = 0; j < m; j++) {
-              const uint64_t kj = R.sk[j];
-              const bool first = kj < ki || (kj == ki && R.sv[j] < vi);
-              sum += first && ((kj ^ ki) >> 32) == 0 ? R.sw[j] : 0;
-            }
+      const bool contested = *(volatile int64_t*)&cs->ncont != 0;
+      if (contested) {
+        for (int64_t v = gt; v < n; v += GT) {
+          if (e.flag[v] != 2) continue;
+          const int32_t t = a.req[v];
+          const uint32_t hv = contest_hash(a, (int32_t)v);
+          int64_t before = 0;
+          int32_t u = e.head[t], len = 0;
+          for (; u >= 0 && len < kClEngChain; u = e.next[u], len++) {
+            const uint32_t hu = contest_hash(a, u);
+            if (hu < hv || (hu == hv && u < (int32_t)v)) before += g.vw[u];
           }
-          if (i < nc && sum) atomicAdd((unsigned long long*)&e.P[i], (unsigned long long)sum);
+          if (u >= 0) *(volatile unsigned long long*)&cs->kernels = 1;
+          e.flag[v] = (int64_t)e.Wc[t] + before + g.vw[v] <= a.wcap ? 1 : 0;
         }
         cl.sync();
-        for (int64_t i = gt; i < nc; i += GT) {
-          const int32_t t = (int32_t)(e.key[i] >> 32), v = e.val[i];
-          e.flag[v] = (int64_t)e.Wc[t] + *(volatile int64_t*)&e.P[i] + g.vw[v] <= a.wcap ? 1 : 0;
-        }
-        cl.sync();
-      } else if (nc > 0) {
-        if (lead) cluster_resolve(e.key, e.val, nc, e.Wc, g.vw, a.wcap, e.flag, R);
-        cl.sync();
+        if (*(volatile unsigned long long*)&cs->kernels) return;  // (uniform) left to the graph of kernels, which sorts
+        if (lead && threadIdx.x == 0) cs->ncont = 0;              // (every CTA has read it)
       }
-      if (nc > 0 && lead && threadIdx.x == 0) cs->ncont = 0;  // (every CTA has read it)
       int32_t mine = 0;
       for (int64_t v = gt; v < n; v += GT) {
         const int32_t t = a.req[v];
         if (t < 0) continue;
         e.ReqW[t] = 0;
+        if (contested) e.head[t] = -1;
         if (e.flag[v] != 1) continue;
         const int32_t cv = g.vw[v];
         atomicAdd(&e.Wc[e.C[v]], -cv);
@@ -1397,9 +1379,8 @@ __device__ __forceinline__ void cluster_engine_run(const GraphView& g, ClusterAr
 
 __global__ void __launch_bounds__(kClEngThreads, 1) k_cluster_engine(GraphView g, ClusterArgs a, ClusterEngineArgs e) {
   extern __shared__ __align__(16) int2 cl_scw[];  // [warps][kTileE]
-  __shared__ ResolveSmem R;
   const cg::cluster_group cl = cg::this_cluster();
-  cluster_engine_run(g, a, e, cl_scw, R, (int)cl.block_rank(), (int)cl.num_blocks(), cl);
+  cluster_engine_run(g, a, e, cl_scw, (int)cl.block_rank(), (int)cl.num_blocks(), cl);
 }
 
 // The same loop for the levels above one cluster's size, by a cooperative launch
@@ -1410,9 +1391,8 @@ __global__ void __launch_bounds__(kClEngThreads, 1) k_cluster_engine(GraphView g
 __global__ void __launch_bounds__(kClEngThreads, 1) k_cluster_grid(GraphView g, ClusterArgs a, ClusterEngineArgs e,
                                                                    GridBar* bar, unsigned arrivals) {
   extern __shared__ __align__(16) int2 cl_scw[];
-  __shared__ ResolveSmem R;
   __shared__ unsigned int bar_flag;
-  cluster_engine_run(g, a, e, cl_scw, R, (int)blockIdx.x, (int)gridDim.x, GridSync{bar, &bar_flag, arrivals});
+  cluster_engine_run(g, a, e, cl_scw, (int)blockIdx.x, (int)gridDim.x, GridSync{bar, &bar_flag, arrivals});
 }
 
 // CTAs of k_cluster_grid on the device; 0: no cooperative launch there.
@@ -2111,7 +2091,8 @@ int32_t cluster_level(Ctx& c, int lvl, bool engine) {
   bool engine_ran = false, grid_ran = false;
   if (short_rows && (n <= kClEngMaxN || (n <= grid_max && cluster_grid_blocks(c, eng_smem)))) {
     const ClusterArgs a{c.C, c.Wc, c.ReqW, c.req, wcap, c.cfg.seed, cs, lvl, 0, 0};
-    const ClusterEngineArgs e{c.C, c.Wc, c.ReqW, c.elig, c.sort.key[0], c.sort.val[0], c.P64, cs, c.cfg.cluster_iters};
+    const ClusterEngineArgs e{c.C, c.Wc, c.ReqW, c.elig, reinterpret_cast<int32_t*>(c.sort.key[0]), c.sort.val[0],
+                              cs, c.cfg.cluster_iters};
     engine_ran = true;
     cudaLaunchAttribute attr{};
     cudaLaunchConfig_t lc{};
@@ -2198,7 +2179,7 @@ int32_t cluster_level(Ctx& c, int lvl, bool engine) {
   if (graph_ran) add_launches(L.cg_root + (long long)c.h_cstate->kernels);
   // a barrier gave up waiting (its time runs on while other users of the GPU have it): the graph, which waits for none
   if (grid_ran && reinterpret_cast<const GridBar*>(c.h_small + 2)->err) return cluster_level(c, lvl, false);
-  if (engine_ran && c.h_cstate->kernels) return cluster_level(c, lvl, false);  // too many contested requests
+  if (engine_ran && c.h_cstate->kernels) return cluster_level(c, lvl, false);  // a chain of contested requests too long
   const int64_t nc = c.h_small[0];
   const uint32_t e = (uint32_t)(c.h_small[1] & 0xffffffffLL);
   if (e & ERR_TIMEOUT) throw ApiError(MAP_E_TIMEOUT, "a bounded device loop gave up");
