@@ -2054,7 +2054,7 @@ void build_cluster_graph(Ctx& c, int lvl, int64_t wcap) {
 }
 
 // Clusters level `lvl`; returns n_c, fills L.M.
-int32_t cluster_level(Ctx& c, int lvl, bool engine) {
+int32_t cluster_level(Ctx& c, int lvl) {
   Level& L = c.lv[lvl];
   const int32_t n = L.n;
   const unsigned gv = grid_for(c, kThreads, n);
@@ -2085,7 +2085,7 @@ int32_t cluster_level(Ctx& c, int lvl, bool engine) {
   ClusterState* cs = c.cstate;
   bool graph_ran = false;
   const size_t eng_smem = (size_t)(kClEngThreads / 32) * kTileE * sizeof(int2);
-  const bool short_rows = engine && c.use_graphs && !c.prof && L.max_deg <= kClEngRow && L.m_hi * 16 <= L.m;
+  const bool short_rows = !L.no_one_launch && c.use_graphs && !c.prof && L.max_deg <= kClEngRow && L.m_hi * 16 <= L.m;
   // (grid_engine_max_n < 0: launches over every SM are unwanted, as by jobs that share the GPU)
   const int64_t grid_max = c.cfg.grid_engine_max_n < 0 ? -1 : kClGridMaxN;
   bool engine_ran = false, grid_ran = false;
@@ -2177,9 +2177,12 @@ int32_t cluster_level(Ctx& c, int lvl, bool engine) {
   GM_CUDA(cudaGetLastError());
   GM_CUDA(cudaStreamSynchronize(c.st));
   if (graph_ran) add_launches(L.cg_root + (long long)c.h_cstate->kernels);
-  // a barrier gave up waiting (its time runs on while other users of the GPU have it): the graph, which waits for none
-  if (grid_ran && reinterpret_cast<const GridBar*>(c.h_small + 2)->err) return cluster_level(c, lvl, false);
-  if (engine_ran && c.h_cstate->kernels) return cluster_level(c, lvl, false);  // a chain of contested requests too long
+  // a barrier gave up waiting (its time runs on while other users of the GPU have it), or a chain of contested
+  // requests was too long: the graph, also in this level's later runs
+  if (engine_ran && (c.h_cstate->kernels || (grid_ran && reinterpret_cast<const GridBar*>(c.h_small + 2)->err))) {
+    L.no_one_launch = true;
+    return cluster_level(c, lvl);
+  }
   const int64_t nc = c.h_small[0];
   const uint32_t e = (uint32_t)(c.h_small[1] & 0xffffffffLL);
   if (e & ERR_TIMEOUT) throw ApiError(MAP_E_TIMEOUT, "a bounded device loop gave up");
@@ -2385,7 +2388,7 @@ int32_t coarsen(Ctx& c) {
   while ((int32_t)c.lv.size() < c.cfg.max_levels &&
          (int64_t)c.lv.back().n >= (int64_t)c.cfg.coarsest_factor * c.k) {
     const int lvl = (int)c.lv.size() - 1;
-    const int32_t nc = c.cfg.coarsener == 1 ? match_level(c, lvl, true) : cluster_level(c, lvl, true);
+    const int32_t nc = c.cfg.coarsener == 1 ? match_level(c, lvl) : cluster_level(c, lvl);
     Level& F = c.lv[lvl];
     if ((int64_t)nc * c.cfg.stall_den > (int64_t)c.cfg.stall_num * F.n) {
       c.mem.put(F.M);

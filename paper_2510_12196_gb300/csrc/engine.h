@@ -128,6 +128,7 @@ struct Level {
   int32_t g_nhi = -1;
   int32_t g_nhuge = -1;
   long long g_root = 0;  // kernel nodes outside the conditional bodies
+  bool no_one_launch = false;  // the coarsening of this level in one launch gave up once: its later runs take the graph
   // instantiated clustering graph of this level and its key
   cudaGraphExec_t cgexec = nullptr;
   static constexpr int kCgKey = 9;
@@ -413,7 +414,7 @@ void download_mapping(Ctx& c, const int32_t* codes, int32_t n, int32_t* out);
 void upload_mapping(Ctx& c, const int32_t* pi, int32_t n, int32_t* codes);
 
 // match.cu
-int32_t match_level(Ctx& c, int lvl, bool one_launch);  // two-hop matching of level lvl into its M; returns n_c
+int32_t match_level(Ctx& c, int lvl);  // two-hop matching of level lvl into its M; returns n_c
 
 // hm.cu: hierarchical multisection of level lvl's graph into its pi (codes)
 void hm_run(Ctx& c, int lvl, int32_t workers, HmStats* st);

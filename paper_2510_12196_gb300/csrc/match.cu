@@ -502,14 +502,13 @@ void build_match_graph(Ctx& c, int lvl) {
 
 // Matches level lvl and writes its map to the next level into L.M; returns
 // n_c.  Uses the clustering scratch (labels as partners, requests as
-// preferences, the rank array) and the sort buffers.  one_launch: the rounds of
-// a small level may run in one cooperative launch.
-int32_t match_level(Ctx& c, int lvl, bool one_launch) {
+// preferences, the rank array) and the sort buffers.
+int32_t match_level(Ctx& c, int lvl) {
   Level& L = c.lv[lvl];
   const int32_t n = L.n;
   MatchState* s = state_of(c);
   if (!L.M) L.M = c.mem.make<int32_t>((size_t)std::max(1, n));
-  const int blocks = one_launch && c.use_graphs && !c.prof ? match_round_blocks(c, n) : 0;
+  const int blocks = !L.no_one_launch && c.use_graphs && !c.prof ? match_round_blocks(c, n) : 0;
   if (c.use_graphs && !c.prof && !blocks) {
     // the graph writes L.M, which a stalled level gives back, so its address is part of the key
     const int64_t key[6] = {(int64_t)n, L.m, c.lmax, (int64_t)c.cfg.match_rounds, -1, (int64_t)(intptr_t)L.M};
@@ -548,8 +547,11 @@ int32_t match_level(Ctx& c, int lvl, bool one_launch) {
                                bar_arrivals(c, (unsigned)blocks))); count_launch();
     GM_CUDA(cudaMemcpyAsync(c.h_small + 2, c.gbar, sizeof(GridBar), cudaMemcpyDeviceToHost, c.st));
     int64_t matched = read(&s->matched);
-    // a barrier gave up waiting: the graph, which waits for no other block
-    if (reinterpret_cast<const GridBar*>(c.h_small + 2)->err) return match_level(c, lvl, false);
+    // a barrier gave up waiting: the graph, which waits for no other block, also in this level's later runs
+    if (reinterpret_cast<const GridBar*>(c.h_small + 2)->err) {
+      L.no_one_launch = true;
+      return match_level(c, lvl);
+    }
     for (int stage = 1; stage <= 4 && 4 * matched <= 3 * (int64_t)n; stage++) {
       k_mt_stage_begin<<<1, 1, 0, c.st>>>(s, n, 0, 0); count_launch();
       emit_stage(c, lvl, stage, c.st, nullptr);

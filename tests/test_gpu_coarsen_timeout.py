@@ -1,6 +1,8 @@
 """A coarsening whose cooperative launches give up waiting (a barrier that one
 arrival never reaches, about a second each) goes on as a graph of kernels with
 the same levels and the same mapping, and the context keeps working."""
+import time
+
 import numpy as np
 import pytest
 
@@ -33,6 +35,23 @@ def _run(g, launches, **over):
 def _same(a, b):
     for (na, ja, pa), (nb, jb, pb) in zip(a, b):
         assert list(na) == list(nb) and ja == jb and np.array_equal(pa, pb)
+
+
+@pytest.mark.parametrize("coarsener", [0, 1])
+def test_later_runs_do_not_wait_again(coarsener):
+    """The level that gave up takes the graph in the next run, which asks for no further launch there."""
+    g = GRAPHS["rgg"]()
+    ctx = make_ctx(g, (4, 8), (1, 10), coarsener=coarsener)
+    try:
+        G.map_selftest_coarsen_timeout(ctx, 100)
+        times = []
+        for _ in range(2):
+            t0 = time.perf_counter()
+            G.map_coarsen(ctx)
+            times.append(time.perf_counter() - t0)
+    finally:
+        G.map_destroy(ctx)
+    assert times[0] > 0.9 and times[1] < 0.5
 
 
 @pytest.mark.parametrize("name", GRAPHS)
