@@ -1262,10 +1262,10 @@ __global__ void k_cl_end(ClusterState* cs, int32_t n, int32_t iters, cudaGraphCo
 // chained by target, and each follows its target's chain to sum the weights of
 // the requests before it in (hash, id) order: chains are as long as a cluster
 // has neighbours that want in, a handful where the caps are tight and most
-// requests contested, however many there are in all (every request compared
-// with every other took 1 ms a sub-round of 1.6e4 on one cluster: coarsening of a
-// 3D grid of 32768 vertices on 4096 PEs 3.3 ms, now 0.56, the graph of kernels
-// 0.71; of an RGG of 131072 on 4096 PEs 1.6, 0.67 and 1.76).  With a chain of
+// requests contested, however many there are in all (coarsening of a 3D grid of
+// 32768 vertices on 4096 PEs: 0.56 ms, with every request compared with every
+// other 3.3, as a graph of kernels 0.71; of an RGG of 131072 on 4096 PEs 0.67, 1.6
+// and 1.76).  With a chain of
 // kClEngChain requests or more the launch gives up: the graph sorts them.
 constexpr int kClEngThreads = 1024;
 constexpr int kClEngMaxN = 1 << 15;

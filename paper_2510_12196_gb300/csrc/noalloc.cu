@@ -68,17 +68,18 @@ __global__ void k_na_clear(NoAllocScratch* s, Topo t, Hier h) {
 }
 
 // J and block weights.  The CSR entries are split evenly whatever the degrees:
-// a block takes consecutive tiles of kNaTile entries, finds the row of its
-// first entry by one 256-way search of xadj, reads the starts and PEs of a
-// tile's rows into shared memory while the tile's entries and their PEs are in
-// flight, and each thread follows the rows of its own kNaItems consecutive
-// entries.  The pass streams 8 bytes an entry and gathers 4 from L2.  One 8-lane sub-warp per row (as before)
-// left the hubs of a power-law graph to eight lanes, and one global atomic
-// per vertex for the block weights queued on k words: R-MAT 2^20, k = 512:
-// 5.59 ms before, 0.27 ms now (0.94 TB/s of the 8-byte stream; the gathers
-// of the PEs from L2 bound it).
-// The weights of a code space of at most kNaCodes are summed per block in
-// shared memory first (16 KB; larger spaces spread their global atomics).
+// a block takes consecutive tiles of kNaTile entries and finds the row of its
+// first entry by one 256-way search of xadj.  The rows that start in a tile set
+// a bit at their first entry and store their PE there, and an entry takes its
+// row's PE from the last bit at or before it.  A warp's entries are 32
+// consecutive ones at a time, so that their neighbours' PEs, near one another
+// where the ids have locality, come in few cache lines.  The pass streams 8
+// bytes an entry and gathers 4.  RGG of 2^20 vertices, 12.6e6 entries: 64-85 us
+// whatever the mapping and the code space (eight consecutive entries per thread
+// 87-135 us; eight lanes per row 81-610 us, R-MAT 2^20 5.5 ms).
+// The weights are summed by warp and PE first, then in the block's shared
+// memory where it has more vertices than there are PE codes (at most kNaCodes),
+// else straight into the global sums.
 // Mapping entries or neighbours outside their range are skipped, and only
 // entries of [0, xadj[n]) are read, so that a malformed xadj cannot make the
 // pass read outside the adjacency arrays.  The last block to finish writes
@@ -86,6 +87,8 @@ __global__ void k_na_clear(NoAllocScratch* s, Topo t, Hier h) {
 constexpr int kNaItems = 8;
 constexpr int kNaTile = kNaThreads * kNaItems;
 constexpr int kNaCodes = 2048;
+constexpr int kNaShare = 8;
+constexpr int64_t kNaVertices = 1024;  // vertices per block at least (blocks past the last one sum no weights)
 
 // Largest v in [0, n) with xadj[v] <= e, -1 if none; all threads call it.
 __device__ __forceinline__ int32_t na_row_of(const int64_t* __restrict__ xadj, int32_t n, int64_t e) {
@@ -96,125 +99,146 @@ __device__ __forceinline__ int32_t na_row_of(const int64_t* __restrict__ xadj, i
   });
 }
 
-__device__ __forceinline__ void na_load8(const int32_t* __restrict__ a, int64_t e, int cnt, bool vec,
-                                         int32_t (&x)[kNaItems]) {
-  static_assert(kNaItems == 8, "two 16-byte loads");
-  if (vec && cnt == kNaItems) {
-    const int4 p = *reinterpret_cast<const int4*>(a + e), q = *reinterpret_cast<const int4*>(a + e + 4);
-    x[0] = p.x; x[1] = p.y; x[2] = p.z; x[3] = p.w;
-    x[4] = q.x; x[5] = q.y; x[6] = q.z; x[7] = q.w;
-  } else {
-#pragma unroll
-    for (int j = 0; j < kNaItems; j++) x[j] = j < cnt ? a[e + j] : 0;
-  }
-}
+// The rows of a tile, two tiles in turn.
+struct NaRows {
+  uint32_t heads[2][kNaTile / 32];  // entries that start a row
+  int16_t code[2][kNaTile];         // and its PE code (-1: PE id out of range)
+  int16_t carry[2];                 // code of the row that the tile's first entries go on with
+  int16_t last[kNaTile / 32];       // last start before each 32 entries (-1: none)
+};
 
 // plain: the PE ids are their own codes (every a_i a power of two)
 __global__ void __launch_bounds__(kNaThreads, 5) k_na_eval(int32_t n, const int64_t* __restrict__ xadj,
-                                                        const int32_t* __restrict__ adj,
-                                                        const int32_t* __restrict__ adjw,
-                                                        const int32_t* __restrict__ vw,
-                                                        const int32_t* __restrict__ pi, NoAllocScratch* s, Topo t,
-                                                        int plain, int64_t* out) {
+                                                           const int32_t* __restrict__ adj,
+                                                           const int32_t* __restrict__ adjw,
+                                                           const int32_t* __restrict__ vw,
+                                                           const int32_t* __restrict__ pi, NoAllocScratch* s, Topo t,
+                                                           int plain, int64_t* out) {
   extern __shared__ __align__(16) unsigned char na_dyn[];
   unsigned long long* sW = reinterpret_cast<unsigned long long*>(na_dyn);  // [kc] when kc <= kNaCodes
-  const bool local = t.kc <= kNaCodes;
-  uint16_t* scode = reinterpret_cast<uint16_t*>(na_dyn + (local ? (size_t)t.kc * 8 : 0));  // [k] unless plain
+  const bool fits = t.kc <= kNaCodes;
+  uint16_t* scode = reinterpret_cast<uint16_t*>(na_dyn + (fits ? (size_t)t.kc * 8 : 0));  // [k] unless plain
   __shared__ int32_t sdist[32];
   __shared__ int64_t sm[33];
-  // the rows of the tile: starts relative to its first entry, PE codes (-1: PE id out of range)
-  __shared__ int32_t start[kNaTile + 1];
-  __shared__ int16_t rcode[kNaTile + 1];
+  __shared__ NaRows R;
   __shared__ unsigned int last;
+  static_assert(kNaTile / 32 == 64, "a warp scans the words of a tile, two per lane");
+  const int lane = (int)threadIdx.x & 31;
+  // consecutive vertices per block
+  const int64_t per = max(kNaVertices, ((int64_t)n + gridDim.x - 1) / gridDim.x);
+  const int64_t va = min((int64_t)n, blockIdx.x * per), vb = min((int64_t)n, va + per);
+  const bool local = fits && per >= t.kc && va < vb;
   load_sdist(sdist, t);
+  if (threadIdx.x < 2 * (kNaTile / 32)) R.heads[threadIdx.x / (kNaTile / 32)][threadIdx.x % (kNaTile / 32)] = 0;
   if (local)
     for (int b = threadIdx.x; b < t.kc; b += kNaThreads) sW[b] = 0;
   if (!plain)
     for (int p = threadIdx.x; p < t.k; p += kNaThreads) scode[p] = (uint16_t)s->code[p];
   __syncthreads();
   auto code_of = [&](int32_t p) { return plain ? p : (int32_t)scode[p]; };
+  auto code_or_none = [&](int32_t p) { return p >= 0 && p < t.k ? code_of(p) : -1; };
+  auto add_weight = [&](int32_t c, int64_t x) {
+    atomicAdd(local ? &sW[c] : (unsigned long long*)&s->W[c], (unsigned long long)x);
+  };
 
-  for (int64_t v = (int64_t)blockIdx.x * kNaThreads + threadIdx.x; v < n; v += (int64_t)gridDim.x * kNaThreads) {
-    const int32_t p = pi[v];
-    if (p < 0 || p >= t.k) continue;
-    atomicAdd(local ? &sW[code_of(p)] : (unsigned long long*)&s->W[code_of(p)], (unsigned long long)(int64_t)vw[v]);
+  for (int64_t v0 = va + (threadIdx.x - lane); v0 < vb; v0 += kNaThreads) {  // (warp-uniform)
+    const int64_t v = v0 + lane;
+    const int32_t c = v < vb ? code_or_none(pi[v]) : -1;
+    const int32_t x = c >= 0 ? vw[v] : 0;
+    unsigned left = __ballot_sync(0xffffffffu, c >= 0);
+    // a PE of kNaShare or more of the warp's vertices at once (their single updates would queue on one word)
+    while (left) {
+      const int src = __ffs(left) - 1;
+      const int32_t cs = __shfl_sync(0xffffffffu, c, src);
+      const unsigned same = __ballot_sync(0xffffffffu, c == cs) & left;
+      if (__popc(same) < kNaShare) break;
+      const int32_t y = c == cs ? x : 0;
+      // 32 values of 32 bits: the sums of their halves fit
+      const int64_t lo = (int64_t)__reduce_add_sync(0xffffffffu, (unsigned)y & 0xffffu);
+      const int64_t hi = (int64_t)__reduce_add_sync(0xffffffffu, y >> 16);
+      if (lane == src) add_weight(c, hi * 65536 + lo);
+      left &= ~same;
+    }
+    if ((left >> lane) & 1u) add_weight(c, x);
   }
 
   const int64_t m = xadj[n];
-  const bool vec = (((uintptr_t)adj | (uintptr_t)adjw) & 15) == 0;
   int64_t acc = 0;
   const int64_t tiles = (m + kNaTile - 1) / kNaTile;
   const int64_t t0 = tiles * blockIdx.x / gridDim.x, t1 = tiles * (blockIdx.x + 1) / gridDim.x;
   // the row of the block's first entry (row 0 for entries before the first row)
   int32_t lo = t0 < t1 ? max(na_row_of(xadj, n, t0 * kNaTile), 0) : 0;
+  const int first = ((int)threadIdx.x - lane) * kNaItems + lane;  // this thread's entries: first + 32 j
   for (int64_t tile = t0; tile < t1; tile++) {
+    const int cur = (int)(tile & 1);
     const int64_t e0 = tile * kNaTile, e1 = min(e0 + kNaTile, m);
-    const int first = (int)threadIdx.x * kNaItems;
-    const int cnt = (int)max((int64_t)0, min((int64_t)kNaItems, e1 - e0 - first));
-    // the entries and their PEs, in flight while the row starts are found
+    const int span = (int)(e1 - e0);
     int32_t u[kNaItems], w[kNaItems];
-    na_load8(adj, e0 + first, cnt, vec, u);
-    if (adjw) {
-      na_load8(adjw, e0 + first, cnt, vec, w);
-    } else {
 #pragma unroll
-      for (int j = 0; j < kNaItems; j++) w[j] = 1;
+    for (int j = 0; j < kNaItems; j++) {
+      const int x = first + 32 * j;
+      u[j] = x < span ? adj[e0 + x] : -1;
+      w[j] = x < span ? (adjw ? adjw[e0 + x] : 1) : 0;
     }
-#pragma unroll
-    for (int j = 0; j < kNaItems; j++) u[j] = (j < cnt && u[j] >= 0 && u[j] < n) ? pi[u[j]] : -1;
-    // start[i] = start of row lo + i, up to the first row that starts at or after e1 (or row n)
-    int32_t nr = 0;  // rows lo .. lo + nr - 1 start before e1
+    // the rows lo .. lo + nr - 1 start before e1
+    int32_t nr = 0;
     bool staged = false;
     while (!staged && nr < kNaTile) {
       const int32_t r = nr + (int32_t)threadIdx.x;
       const int64_t at = (int64_t)lo + r;
-      const int64_t x = at <= n ? xadj[at] - e0 : (int64_t)kNaTile;
-      start[r] = (int32_t)max((int64_t)-1, min(x, (int64_t)kNaTile));
-      const int32_t p = at < n ? pi[at] : -1;
-      rcode[r] = (int16_t)(p >= 0 && p < t.k ? code_of(p) : -1);
-      const int c = __syncthreads_count(at < n && (r == 0 || x < e1 - e0));
-      nr += c;
-      staged = c < kNaThreads;
-    }
-    if (!staged) {  // long runs of empty rows: searched in global memory
-      nr = max(na_row_of(xadj, n, e1 - 1) - lo + 1, 1);
-    }
-    if (cnt > 0) {
-      auto row_start = [&](int32_t i) -> int64_t { return staged ? (int64_t)start[i] : xadj[lo + i] - e0; };
-      auto row_code = [&](int32_t i) -> int32_t {
-        if (staged) return rcode[i];
-        const int32_t p = pi[lo + i];
-        return p >= 0 && p < t.k ? code_of(p) : -1;
-      };
-      auto search = [&](int32_t from, int x) {  // largest row i >= from with row_start(i) <= x
-        return last_by_bisection(from, nr, [&](int32_t i) { return row_start(i) <= x; });
-      };
-      const int64_t base = row_start(0);  // after the tile's start only when xadj[0] > 0
-      int32_t i = search(0, first), cv = -1;
-      int64_t end = row_start(i + 1);
-      bool fresh = true;  // row i's PE code is still to be read
+      const bool is_row = at < n;
+      const int64_t b = is_row ? xadj[at] - e0 : span, e = is_row ? xadj[at + 1] - e0 : span;
+      const int32_t p = is_row ? pi[at] : -1;
+      if (nr == 0) {  // the neighbours' PEs, in flight with the rows
 #pragma unroll
-      for (int j = 0; j < kNaItems; j++) {
-        const int x = first + j;
-        if (j >= cnt || x < base) continue;
-        if (x >= end && i + 1 < nr) {
-          i++;
-          end = row_start(i + 1);
-          if (x >= end) {  // empty rows between
-            i = search(i, x);
-            end = row_start(i + 1);
-          }
-          fresh = true;
-        }
-        if (fresh) {
-          cv = row_code(i);
-          fresh = false;
-        }
-        if (cv >= 0 && u[j] >= 0 && u[j] < t.k) acc += (int64_t)w[j] * dcode(sdist, cv, code_of(u[j]));
+        for (int j = 0; j < kNaItems; j++) u[j] = u[j] >= 0 && u[j] < n ? pi[u[j]] : -1;
       }
+      const int16_t c = (int16_t)code_or_none(p);
+      if (r == 0) R.carry[cur] = b <= 0 ? c : (int16_t)-1;
+      if (is_row && b >= 0 && b < span && e > b) {
+        R.code[cur][b] = c;
+        atomicOr(&R.heads[cur][b >> 5], 1u << (b & 31));
+      }
+      const int got = __syncthreads_count(is_row && (r == 0 || b < span));
+      nr += got;
+      staged = got < kNaThreads;
     }
-    lo += nr - 1;     // the last row of this tile may go on in the next
-    __syncthreads();  // the row starts are rewritten
+    if (!staged) nr = max(na_row_of(xadj, n, e1 - 1) - lo + 1, 1);  // long runs of empty rows: searched below
+    if (threadIdx.x < 32) {
+      const uint32_t a = R.heads[cur][lane], b = R.heads[cur][32 + lane];
+      int x = a ? 32 * lane + 31 - __clz(a) : -1, y = b ? 32 * (32 + lane) + 31 - __clz(b) : -1;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int p = __shfl_up_sync(0xffffffffu, x, o), q = __shfl_up_sync(0xffffffffu, y, o);
+        if (lane >= o) {
+          x = max(x, p);
+          y = max(y, q);
+        }
+      }
+      const int all = __shfl_sync(0xffffffffu, x, 31);
+      const int px = __shfl_up_sync(0xffffffffu, x, 1), py = __shfl_up_sync(0xffffffffu, y, 1);
+      R.last[lane] = (int16_t)(lane ? px : -1);
+      R.last[32 + lane] = (int16_t)max(all, lane ? py : -1);
+    } else if (threadIdx.x < 32 + kNaTile / 32) {
+      R.heads[cur ^ 1][threadIdx.x - 32] = 0;  // the next tile's (every thread is done with the last one)
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kNaItems; j++) {
+      const int x = first + 32 * j;
+      if (x >= span || u[j] < 0 || u[j] >= t.k) continue;
+      int32_t cv;
+      if (staged) {
+        const uint32_t word = R.heads[cur][x >> 5] & (0xffffffffu >> (31 - lane));
+        const int pos = word ? (x & ~31) + 31 - __clz(word) : R.last[x >> 5];
+        cv = pos >= 0 ? R.code[cur][pos] : R.carry[cur];
+      } else {
+        const int32_t i = last_by_bisection(0, nr, [&](int32_t r) { return xadj[lo + r] - e0 <= x; });
+        cv = xadj[lo + i] - e0 <= x ? code_or_none(pi[lo + i]) : -1;
+      }
+      if (cv >= 0) acc += (int64_t)w[j] * dcode(sdist, cv, code_of(u[j]));
+    }
+    lo += nr - 1;  // the last row of this tile may go on in the next
   }
   acc = block_sum(acc, sm);
   if (threadIdx.x == 0 && acc) atomicAdd(&s->J, (unsigned long long)acc);
