@@ -1909,7 +1909,6 @@ void launch_subround(Ctx& c, int lvl, int32_t r, int64_t wcap) {
   Level& L = c.lv[lvl];
   const int32_t n = L.n;
   const unsigned gv = grid_for(c, kThreads, n);
-  const unsigned gl = grid_for(c, kThreads / kSubWarp, n);
   uint8_t* flag = c.elig;
   int64_t* d_cont = c.counters + 6;
   const int kbits = bits_for(n) + 32;
@@ -2058,7 +2057,6 @@ int32_t cluster_level(Ctx& c, int lvl) {
   Level& L = c.lv[lvl];
   const int32_t n = L.n;
   const unsigned gv = grid_for(c, kThreads, n);
-  const unsigned gl = grid_for(c, kThreads / kSubWarp, n);
   int64_t wcap = c.lmax / c.cfg.cluster_cap_div;
   if (wcap < L.max_vw) wcap = L.max_vw;
   if (wcap < 1) wcap = 1;

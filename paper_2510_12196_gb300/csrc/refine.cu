@@ -148,13 +148,10 @@ __global__ void __launch_bounds__(kTileThreads, kTileMinBlocks) k_eval_tile(Grap
   if (threadIdx.x == 0 && acc) atomicAdd((unsigned long long*)Jacc, (unsigned long long)acc);
 }
 
-// The high-degree kernels below come in two forms: one warp per vertex of
-// degree <= kMidDeg (`_mid`, over the whole list hi[] of degree > kLowDeg,
-// skipping the larger ones) and one CTA per vertex (`_high`, over the
-// positions `sel` in hi[], or all of hi[] when sel is null).
-__device__ __forceinline__ int32_t hi_vertex(const int32_t* hi, const int32_t* sel, int32_t j) {
-  return hi[sel ? sel[j] : j];
-}
+// The high-degree kernels below: one warp per vertex of degree <= kMidDeg
+// (`_mid`, over the whole list hi[] of degree > kLowDeg, skipping the larger
+// ones), and for the larger ones chunks of their entries; where a code space
+// is too large for the per-warp tables, one CTA per vertex of hi[] (`_high`).
 
 // J contribution of the vertices of degree in (kLowDeg, kMidDeg], one warp per vertex.
 __global__ void __launch_bounds__(kMidThreads) k_eval_mid(GraphView g, const int32_t* __restrict__ hi, int32_t n_hi,
@@ -548,8 +545,6 @@ __host__ inline GroupLayout group_layout(const Topo& t) {
   return gl;
 }
 
-// Fills conn[0, kc) (already zeroed) with the edge weights of v per neighbour
-// PE and the level group sums after it.  Returns T(P(v)) summed over the block.
 // The threads that fill and read one connectivity table: a CTA or a warp.
 struct CtaRow {
   static constexpr bool kWarp = false;
@@ -622,6 +617,8 @@ __device__ void conn_groups(const Topo& topo, const GroupLayout& gl, int32_t* ta
   }
 }
 
+// Fills tab[0, kc) (already zeroed) with the edge weights of v per neighbour PE
+// and the level group sums after it; all threads of the CTA call it.
 __device__ void conn_build(const GraphView& g, int32_t v, const int32_t* __restrict__ pi, const Topo& topo,
                            const GroupLayout& gl, int32_t* tab) {
   conn_add(g, g.xadj[v], g.xadj[v + 1], pi, tab);
@@ -697,16 +694,16 @@ __device__ __forceinline__ void lp_hub_decide(const int32_t* tab, const Topo& to
 }
 
 __global__ void __launch_bounds__(kHiThreads) k_lp_gain_high(GraphView g, const int32_t* __restrict__ hi,
-                                                             const int32_t* __restrict__ sel, int32_t n_sel,
-                                                             const int32_t* __restrict__ pi, uint8_t* lock,
-                                                             int32_t* pp, int64_t* gain, uint8_t* inx, Topo topo,
-                                                             GroupLayout gl, LpFilter flt, const RefineState* st) {
+                                                             int32_t n_hi, const int32_t* __restrict__ pi,
+                                                             uint8_t* lock, int32_t* pp, int64_t* gain, uint8_t* inx,
+                                                             Topo topo, GroupLayout gl, LpFilter flt,
+                                                             const RefineState* st) {
   extern __shared__ int32_t tab[];
   __shared__ int64_t sbt[32];
   __shared__ int32_t sbc[32];
   if (!kind_is(st, 1 << KIND_LP)) return;
-  for (int32_t i = blockIdx.x; i < n_sel; i += gridDim.x) {
-    const int32_t v = hi_vertex(hi, sel, i);
+  for (int32_t i = blockIdx.x; i < n_hi; i += gridDim.x) {
+    const int32_t v = hi[i];
     const int32_t p = pi[v];
     if (lock[v]) {
       __syncthreads();
@@ -1627,16 +1624,15 @@ __device__ __forceinline__ void reb_hub_decide(const int32_t* tab, const RebArgs
 }
 
 __global__ void __launch_bounds__(kHiThreads) k_reb_select_high(GraphView g, const int32_t* __restrict__ hi,
-                                                                const int32_t* __restrict__ sel, int32_t n_sel,
-                                                                const int32_t* __restrict__ pi, RebArgs a, int32_t kc,
-                                                                GroupLayout gl, int32_t* dest, uint8_t* bkt,
-                                                                uint8_t* elig, const RefineState* st) {
+                                                                int32_t n_hi, const int32_t* __restrict__ pi,
+                                                                RebArgs a, int32_t kc, GroupLayout gl, int32_t* dest,
+                                                                uint8_t* bkt, uint8_t* elig, const RefineState* st) {
   extern __shared__ int32_t tab[];  // conn per PE code (and the level group sums for the J gains)
   __shared__ int64_t sbb[32];
   __shared__ int32_t sbc[32];
   if (!kind_is(st, (1 << KIND_WEAK) | (1 << KIND_STRONG))) return;
-  for (int32_t i = blockIdx.x; i < n_sel; i += gridDim.x) {
-    const int32_t v = hi_vertex(hi, sel, i);
+  for (int32_t i = blockIdx.x; i < n_hi; i += gridDim.x) {
+    const int32_t v = hi[i];
     const int32_t A = pi[v];
     if (!reb_eligible(a, A, g.vw[v])) {
       if (threadIdx.x == 0) elig[v] = 0;
@@ -1661,10 +1657,11 @@ __global__ void __launch_bounds__(kHiThreads) k_reb_select_high(GraphView g, con
 // degree; the work does).  A row of at most split_deg entries is rated whole
 // by the CTA that draws the chunk holding its first entry: rows of at most
 // kWarpRowDeg entries by one of its warps with a table of its own (mid_tables),
-// with no barrier of the CTA between the phases of a row, larger rows by all.  A row's phases (loads, gathers, table, scan) each wait on
-// the one before, so rows side by side set the pace: 3.0e6 entries (n 33853, 64
-// PEs) 37.7 -> 21.2 us a rebalancing step and 40.3 -> 24.3 us an LP step, 7.9e7
-// entries (R-MAT 2^22 coarsened, 512 PEs) 487 -> 380 us an LP step.  A larger row is
+// with no barrier of the CTA between the phases of a row, larger rows by all.
+// A row's phases (loads, gathers, table, scan) each wait on the one before, so
+// rows side by side set the pace: 3.0e6 entries (n 33853, 64 PEs) 37.7 -> 21.2
+// us a rebalancing step and 40.3 -> 24.3 us an LP step, 7.9e7 entries (R-MAT
+// 2^22 coarsened, 512 PEs) 487 -> 380 us an LP step.  A larger row is
 // rated in two launches: every chunk adds the conn of its entries into the
 // row's global partial table, then one CTA per row reads the table back
 // (emptying it), adds the level group sums and decides.  The policy P gives
@@ -2450,8 +2447,7 @@ void launch_lp(Ctx& c, int lvl) {
   const unsigned gl = grid_for(c, kThreads, L.n);
   const bool mid_tab = mid_tables(c);
   const GroupLayout glay = group_layout(c.topo);
-  // vertices of degree > kLowDeg left to the CTA-per-vertex kernels
-  const int32_t* gsel = mid_tab ? L.huge : nullptr;
+  // vertices of degree > kLowDeg left to the hub kernels, or to a CTA each
   const int32_t ng = mid_tab ? L.n_huge : L.n_hi;
   c.prof_level = lvl;
   cudaEvent_t ev = nullptr;
@@ -2466,7 +2462,7 @@ void launch_lp(Ctx& c, int lvl) {
         launch_hub_tab(c, L, pol, (size_t)glay.total * sizeof(int32_t));
       } else {
         k_lp_gain_high<<<std::max(1, std::min(ng, c.num_sms * 8)), kHiThreads, conn_smem(c), c.st>>>(
-            view(L), L.hi, gsel, ng, L.pi, c.lock, c.pp, c.gain, c.inx, c.topo, glay, flt, c.state); count_launch();
+            view(L), L.hi, ng, L.pi, c.lock, c.pp, c.gain, c.inx, c.topo, glay, flt, c.state); count_launch();
       }
       c.prof_end(ev, PK_LP_GAIN_HIGH, 26 * (int64_t)ng + 12 * me);
     }
@@ -2542,7 +2538,7 @@ void launch_rebalance(Ctx& c, int lvl, bool prep_done = false) {
           launch_hub_tab(c, L, pol, smem);
         } else {
           k_reb_select_high<<<std::max(1, std::min(ng, c.num_sms * 8)), kHiThreads, smem, c.st>>>(
-              view(L), L.hi, nullptr, ng, L.pi, a, c.topo.kc, gl, c.dest, bucket, c.elig, c.state);
+              view(L), L.hi, ng, L.pi, a, c.topo.kc, gl, c.dest, bucket, c.elig, c.state);
           count_launch();
         }
       });
