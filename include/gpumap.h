@@ -93,7 +93,8 @@ typedef struct {
                             engine on one thread-block cluster (rows of degree > 128 by whole CTAs; a level
                             with such a row needs a PE code space whose connectivity table, conn per code
                             plus the level group sums, fits in 96 KiB); 0: library default (32768, levels with
-                            more than 1/16 of their entries in rows of degree > 32 left to the graph of kernels);
+                            more than 1/16 of their entries in rows of degree > 32, unless these are a few
+                            long ones, left to the graph of kernels);
                             -1: never */
   int32_t grid_engine_max_n; /* larger levels with at most this many vertices (same condition) run the same
                             engine over all SMs (cooperative launch); 0: library default (262144, as above);

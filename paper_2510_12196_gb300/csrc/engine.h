@@ -89,6 +89,8 @@ struct Level {
   int32_t n_hi = 0;
   int64_t m_hi = 0;            // CSR entries of the high-degree vertices
   int64_t m_huge = 0;          // CSR entries of the vertices of degree > mid_deg
+  int64_t m_lane = 0;          // CSR entries of the rows above kLowDeg that a sub-warp of the fused engine takes
+  int32_t n_long = 0;          // rows that its CTAs take
   int32_t mid_deg = kMidDeg;   // warp-per-vertex bound of this level (<= kMidDeg)
   int64_t split_req = kSplitDeg;  // hub split bound asked for (hub_split_deg: the one in force)
   int32_t tuned = 0;           // 1: the config leaves both bounds open and they matter (rows above kLowDeg hold 2^20 entries)
@@ -221,7 +223,7 @@ struct Ctx {
   RefineState* h_state = nullptr;  // pinned mirror
   int64_t* h_small = nullptr;      // pinned, a few values read back together
   void* h_tables = nullptr;        // pinned staging of small PE code tables
-  int64_t* d_stats = nullptr;      // device, per-level statistics (5 values)
+  int64_t* d_stats = nullptr;      // device, per-level statistics (7 values)
   int32_t* trace_kind = nullptr;
   int64_t* trace_J = nullptr;
   int64_t* trace_maxw = nullptr;

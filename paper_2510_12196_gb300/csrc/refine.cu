@@ -3942,7 +3942,7 @@ void refine_alloc(Ctx& c) {
   if (!c.h_small) c.h_small = static_cast<int64_t*>(pinned_get(8 * sizeof(int64_t)));
   c.gbar = c.mem.make<GridBar>(1);
   GM_CUDA(cudaMemsetAsync(c.gbar, 0, sizeof(GridBar), c.st));
-  c.d_stats = c.mem.make<int64_t>(5);
+  c.d_stats = c.mem.make<int64_t>(7);
   const size_t smem = conn_smem(c);
   if (smem > 48 * 1024) raise_smem((const void*)k_lp_gain_high, smem);
   static std::atomic<unsigned long long> resolve_done{0};  // one bit per device
@@ -4185,24 +4185,35 @@ static bool engine_rows_fit(const Ctx& c, const Level& L) {
 // most 4 %: 17-63 against 43-94; random geometric graph of degree 40, 90 %:
 // 107 against 101; R-MAT with 770 to 200 k vertices, 67-98 %: 370-1900
 // against 109-284.  Hence one entry in 16.
+// Except levels whose long rows are few: a CTA takes a row above kEngLaneDeg in
+// about 4 us and 3 us per 1000 entries, less than the graph's launch gaps where a
+// CTA has at most kEngFewRows of them (rows between, by single sub-warps, cost
+// much more: none but one short one).  Engine against graph, us per iteration:
+// stars of 40 / 1000 / 8000 vertices 32 / 38 / 57 against 44 / 59 / 82 (30000:
+// 155 against 97); random geometric graphs of degree 8 with rows of 400 entries,
+// 2 / 4 / 8 on 1000 vertices (one CTA) 29 / 39 / 61 against 40 / 42 / 50, 16 on 4000
+// (four CTAs) 43 against 48; 4 rows of 8000 on 12000 45 against 56, of 16000 on
+// 30000 57 against 55; 16 rows of 100 on 1000 113 against 41.
 // A limit set in the config (`asked`) is followed as it stands, and a server's
 // jobs keep the cluster engine, in which its batcher runs them together, for
 // levels of up to kEngServedEntries entries (14 R-MAT requests of 2000 to 50000
 // vertices at once: 276 ms with all of them in the batcher, 130 ms with none).
 constexpr int64_t kEngServedEntries = 1 << 17;
-static bool engine_slower(const Ctx& c, const Level& L, int32_t asked) {
-  return asked == 0 && L.m_hi * 16 > L.m && (!c.sink || L.m > kEngServedEntries);
+constexpr int32_t kEngFewRows = 4;
+constexpr int64_t kEngFewDeg = 8192;
+static bool engine_slower(const Ctx& c, const Level& L, int32_t asked, int ctas) {
+  const bool few = L.m_lane <= 2 * kLowDeg && L.n_long <= kEngFewRows * ctas && L.max_deg <= kEngFewDeg;
+  return asked == 0 && L.m_hi * 16 > L.m && !few && (!c.sink || L.m > kEngServedEntries);
 }
 
 // Cluster size of the fused engine for a level (0: not used).
 static int engine_cluster(Ctx& c, const Level& L) {
   const int64_t lim = c.cfg.engine_max_n > 0 ? c.cfg.engine_max_n : (c.cfg.engine_max_n < 0 ? -1 : kEngMaxN);
-  if (engine_slower(c, L, c.cfg.engine_max_n)) return 0;
   if (!c.use_graphs || c.prof || L.n > lim || !engine_rows_fit(c, L)) return 0;
   int C = (L.n + 1023) / 1024;  // about one vertex per thread
   if (C < 1) C = 1;
   if (C > c.eng_max_cluster) C = c.eng_max_cluster;
-  return C;
+  return engine_slower(c, L, c.cfg.engine_max_n, C) ? 0 : C;
 }
 
 using EngineKernel = void (*)(const EngineJob*, int32_t, unsigned int*);
@@ -4370,7 +4381,7 @@ static void refine_engine(Ctx& c, int lvl, int32_t rounds, int C, int64_t* J, in
 static bool engine_grid_ok(Ctx& c, const Level& L) {
   const int64_t lim =
       c.cfg.grid_engine_max_n > 0 ? c.cfg.grid_engine_max_n : (c.cfg.grid_engine_max_n < 0 ? -1 : (1 << 18));
-  if (engine_slower(c, L, c.cfg.grid_engine_max_n)) return false;
+  if (engine_slower(c, L, c.cfg.grid_engine_max_n, c.num_sms)) return false;
   if (!c.use_graphs || c.prof || L.n > lim || !engine_rows_fit(c, L)) return false;
   static std::atomic<int> cached[64];  // a property of the device: once per process
   if (c.eng_grid_blocks == 0) c.eng_grid_blocks = cached[c.dev & 63].load();
@@ -4498,11 +4509,13 @@ struct StoreHigh {
 
 __global__ void k_level_stats(int32_t n, const int64_t* __restrict__ xadj, const int32_t* __restrict__ vw,
                               int32_t mid_deg, unsigned long long* out) {
-  unsigned long long mhi = 0, mdeg = 0, mvw = 0, mhuge = 0;
+  unsigned long long mhi = 0, mdeg = 0, mvw = 0, mhuge = 0, mlane = 0, nlong = 0;
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
     const unsigned long long d = (unsigned long long)(xadj[v + 1] - xadj[v]);
     if (d > (unsigned long long)kLowDeg) mhi += d;
     if (d > (unsigned long long)mid_deg) mhuge += d;
+    if (d > (unsigned long long)kEngLaneDeg) nlong++;
+    else if (d > (unsigned long long)kLowDeg) mlane += d;
     mdeg = d > mdeg ? d : mdeg;
     const unsigned long long w = (unsigned long long)vw[v];
     mvw = w > mvw ? w : mvw;
@@ -4511,6 +4524,8 @@ __global__ void k_level_stats(int32_t n, const int64_t* __restrict__ xadj, const
   for (int o = 16; o > 0; o >>= 1) {
     mhi += __shfl_xor_sync(0xffffffffu, mhi, o);
     mhuge += __shfl_xor_sync(0xffffffffu, mhuge, o);
+    mlane += __shfl_xor_sync(0xffffffffu, mlane, o);
+    nlong += __shfl_xor_sync(0xffffffffu, nlong, o);
     const unsigned long long y = __shfl_xor_sync(0xffffffffu, mdeg, o);
     mdeg = y > mdeg ? y : mdeg;
     const unsigned long long z = __shfl_xor_sync(0xffffffffu, mvw, o);
@@ -4521,6 +4536,8 @@ __global__ void k_level_stats(int32_t n, const int64_t* __restrict__ xadj, const
     if (mdeg) atomicMax(&out[1], mdeg);
     if (mvw) atomicMax(&out[2], mvw);
     if (mhuge) atomicAdd(&out[3], mhuge);
+    if (mlane) atomicAdd(&out[5], mlane);
+    if (nlong) atomicAdd(&out[6], nlong);
   }
 }
 __global__ void k_max_weight(int64_t m, const int32_t* __restrict__ w, int* out) {
@@ -4673,11 +4690,10 @@ void classify_with(Ctx& c, Level& L, int32_t mid_deg, int64_t split_deg) {
   L.mid_deg = mid_deg;
   scan(LoadHigh{L.xadj, mid_deg}, StoreHigh{L.hi, L.huge}, L.n, nullptr, c.scan, c.st);
   unsigned long long* st = reinterpret_cast<unsigned long long*>(c.d_stats);
-  GM_CUDA(cudaMemsetAsync(st, 0, 4 * sizeof(int64_t), c.st));
+  GM_CUDA(cudaMemsetAsync(st, 0, 7 * sizeof(int64_t), c.st));
   const int64_t blocks = std::min<int64_t>(((int64_t)L.n + 255) / 256, (int64_t)c.num_sms * 8);
   k_level_stats<<<(unsigned)std::max<int64_t>(1, blocks), 256, 0, c.st>>>(L.n, L.xadj, L.vw, mid_deg, st);
   count_launch();
-  GM_CUDA(cudaMemsetAsync(c.d_stats + 4, 0, sizeof(int64_t), c.st));
   const bool new_level = L.max_w == 0 && L.m > 0;  // the largest edge weight, once per level
   if (new_level) {
     k_max_weight<<<grid_for(c, 256 * 8, L.m), 256, 0, c.st>>>(L.m, L.adjw, reinterpret_cast<int*>(c.d_stats + 4));
@@ -4686,7 +4702,7 @@ void classify_with(Ctx& c, Level& L, int32_t mid_deg, int64_t split_deg) {
   // count of high-degree vertices and the statistics, one synchronisation
   GM_CUDA(cudaMemcpyAsync(c.h_small, c.scan.tile_sums + std::max<int64_t>(1, scan_tiles(L.n)), sizeof(int64_t),
                           cudaMemcpyDeviceToHost, c.st));
-  GM_CUDA(cudaMemcpyAsync(c.h_small + 1, st, 5 * sizeof(int64_t), cudaMemcpyDeviceToHost, c.st));
+  GM_CUDA(cudaMemcpyAsync(c.h_small + 1, st, 7 * sizeof(int64_t), cudaMemcpyDeviceToHost, c.st));
   GM_CUDA(cudaStreamSynchronize(c.st));
   if (new_level) L.max_w = (int32_t)c.h_small[5];
   L.n_hi = (int32_t)(c.h_small[0] & 0xffffffffLL);
@@ -4695,6 +4711,8 @@ void classify_with(Ctx& c, Level& L, int32_t mid_deg, int64_t split_deg) {
   L.max_deg = c.h_small[2];
   L.max_vw = (int32_t)c.h_small[3];
   L.m_huge = c.h_small[4];
+  L.m_lane = c.h_small[6];
+  L.n_long = (int32_t)c.h_small[7];
   prepare_hubs(c, L, split_deg);
 }
 
