@@ -284,8 +284,8 @@ def _code_only(src):
 def kernel_hash(kernel="k_eval_tile"):
     """Hash of the code (comments left out) of one kernel: its definition
     (launch bounds and body, from refine.cu, coarsen.cu or match.cu, with the
-    function that does its work where that is a shared one), the row helper, the tile-staging functions of tile.cuh that it calls, and
-    common.cuh."""
+    function that does its work where that is a shared one), the row helper,
+    the tile-staging functions of tile.cuh that it calls, and common.cuh."""
     import re
     csrc = os.path.join(ROOT, "paper_2510_12196_gb300", "csrc")
     text = "".join(open(os.path.join(csrc, f)).read() for f in ("refine.cu", "coarsen.cu", "match.cu"))
@@ -547,8 +547,7 @@ def run_ours(args, ws, rank, local):
                                                                          st.strong_iters[i]] for i in range(levels)],
                                         "schedule": {"mid_deg": [st.mid_deg[i] for i in range(levels)],
                                                      "split_deg": [st.split_deg[i] for i in range(levels)],
-                                                     "autotuned": [st.tuned[i] for i in range(levels)],
-                                                     "tune_ms": st.ms_tune}},
+                                                     "by_rule": [st.tuned[i] for i in range(levels)]}},
                                     args.coarsener, args.initial, variant_settings(args)),
                 "edge_rounds_per_s": job_throughput(er * args.steps, ws, total_ms / 1000.0),
                 "J": Js[0], "e2e": e2e, "roofline": roof, "refine_round": refine_round, "cpu_baseline": cpu,
@@ -677,7 +676,7 @@ def run_probe(args, local):
     ctx = G.map_create(g.xadj, g.adj, g.adjw, g.vw, g.n, t.hier, t.dist, t.eps, cfg)
     J = G.map_run(ctx)
     st0 = G.map_stats(ctx)
-    sched0 = {"mid_deg": st0.mid_deg[0], "split_deg": st0.split_deg[0], "autotuned": st0.tuned[0]}
+    sched0 = {"mid_deg": st0.mid_deg[0], "split_deg": st0.split_deg[0], "by_rule": st0.tuned[0]}
     torch.cuda.synchronize()
     torch.cuda.nvtx.range_push("probe_coarsen")
     G.map_coarsen(ctx)

@@ -62,7 +62,7 @@ typedef enum {
 /* Optional device allocator: alloc returns device memory usable on `stream`
  * (NULL on failure); free releases it.  Used for every device buffer of a
  * context when both are set, else cudaMallocAsync / cudaFreeAsync are used;
- * then the device's default memory pool keeps up to 8 GiB of freed memory
+ * then the device's default memory pool keeps up to 32 GiB of freed memory
  * for reuse (its release threshold, set once per process and device). */
 typedef void* (*map_alloc_fn)(size_t bytes, void* user, void* stream);
 typedef void (*map_free_fn)(void* ptr, size_t bytes, void* user, void* stream);
@@ -134,9 +134,10 @@ typedef struct {
   double ms_refine_level[65]; /* host wall time of Alg. 6 on each level (map_run; ends with a synchronisation) */
   int32_t mid_deg[65];     /* per-vertex split in force on each level (map_config.mid_deg) */
   int32_t split_deg[65];   /* hub split bound in force on each level (INT32_MAX: every hub row rated whole) */
-  int32_t tuned[65];       /* 1: the config leaves the schedule open and the level is large enough for it to
-                              matter (rows of degree > 32 hold at least 2^20 entries); else 0 */
-  double ms_tune;          /* host wall time spent timing schedules: 0 (none is timed) */
+  int32_t tuned[65];       /* 1: the schedule is the library's rule and the level is large enough for it to
+                              matter (rows of degree > 32 hold at least 2^20 entries); else 0.  No schedule
+                              is timed */
+  double ms_tune;          /* always 0 (host wall time spent timing schedules) */
   int32_t lp_iters[65];    /* of iters[]: label-propagation, weak and strong rebalancing iterations per */
   int32_t weak_iters[65];  /* level (map_run; counted over the first 4096 iterations of a level) */
   int32_t strong_iters[65];
