@@ -4194,16 +4194,16 @@ static bool engine_rows_fit(const Ctx& c, const Level& L) {
 // 2 / 4 / 8 on 1000 vertices (one CTA) 29 / 39 / 61 against 40 / 42 / 50, 16 on 4000
 // (four CTAs) 43 against 48; 4 rows of 8000 on 12000 45 against 56, of 16000 on
 // 30000 57 against 55; 16 rows of 100 on 1000 113 against 41.
-// A limit set in the config (`asked`) is followed as it stands, and a server's
-// jobs keep the cluster engine, in which its batcher runs them together, for
-// levels of up to kEngServedEntries entries (14 R-MAT requests of 2000 to 50000
-// vertices at once: 276 ms with all of them in the batcher, 130 ms with none).
-constexpr int64_t kEngServedEntries = 1 << 17;
+// A limit set in the config (`asked`) is followed as it stands.  A server's jobs
+// go by the same rule, at every size (ms for a burst of requests on 8 slots, with
+// their levels up to 2^17 entries in the server's batcher against none: 32 complete
+// graphs of 100 vertices 123 against 23, 32 R-MAT of 256 / 1024 22.6 / 118 against
+// 22.3 / 75, 16 of 8192 262 against 92).
 constexpr int32_t kEngFewRows = 4;
 constexpr int64_t kEngFewDeg = 8192;
-static bool engine_slower(const Ctx& c, const Level& L, int32_t asked, int ctas) {
+static bool engine_slower(const Level& L, int32_t asked, int ctas) {
   const bool few = L.m_lane <= 2 * kLowDeg && L.n_long <= kEngFewRows * ctas && L.max_deg <= kEngFewDeg;
-  return asked == 0 && L.m_hi * 16 > L.m && !few && (!c.sink || L.m > kEngServedEntries);
+  return asked == 0 && L.m_hi * 16 > L.m && !few;
 }
 
 // Cluster size of the fused engine for a level (0: not used).
@@ -4213,7 +4213,7 @@ static int engine_cluster(Ctx& c, const Level& L) {
   int C = (L.n + 1023) / 1024;  // about one vertex per thread
   if (C < 1) C = 1;
   if (C > c.eng_max_cluster) C = c.eng_max_cluster;
-  return engine_slower(c, L, c.cfg.engine_max_n, C) ? 0 : C;
+  return engine_slower(L, c.cfg.engine_max_n, C) ? 0 : C;
 }
 
 using EngineKernel = void (*)(const EngineJob*, int32_t, unsigned int*);
@@ -4381,7 +4381,7 @@ static void refine_engine(Ctx& c, int lvl, int32_t rounds, int C, int64_t* J, in
 static bool engine_grid_ok(Ctx& c, const Level& L) {
   const int64_t lim =
       c.cfg.grid_engine_max_n > 0 ? c.cfg.grid_engine_max_n : (c.cfg.grid_engine_max_n < 0 ? -1 : (1 << 18));
-  if (engine_slower(c, L, c.cfg.grid_engine_max_n, c.num_sms)) return false;
+  if (engine_slower(L, c.cfg.grid_engine_max_n, c.num_sms)) return false;
   if (!c.use_graphs || c.prof || L.n > lim || !engine_rows_fit(c, L)) return false;
   static std::atomic<int> cached[64];  // a property of the device: once per process
   if (c.eng_grid_blocks == 0) c.eng_grid_blocks = cached[c.dev & 63].load();
