@@ -946,7 +946,8 @@ __global__ void __launch_bounds__(kHiThreads) k_cluster_giant(HubRows hr, const 
 __global__ void k_cluster_giant_finish(HubRows hr, const unsigned long long* __restrict__ part, const int32_t* vw,
                                        ClusterArgs a) {
   a.it = a.cs->it;
-  for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < hr.n_huge; r += (int64_t)gridDim.x * blockDim.x) {
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < hr.n_huge; r += step) {
     const int64_t rb = hr.pre[r], re = hr.pre[r + 1];
     if (re - rb <= kBigRowDeg) continue;
     const int32_t v = hr.hi[hr.huge[r]];
@@ -1929,8 +1930,9 @@ void launch_subround(Ctx& c, int lvl, int32_t r, int64_t wcap) {
       k_cluster_high<<<gh, kHiThreads, 0, c.st>>>(view(L), hr, L.hi_off, c.htab, L.hub_part, a, c.hub_ctr, c.errword);
       count_launch();
       if (L.n_big) {
-        k_cluster_big<512><<<(unsigned)std::min(L.n_big, 3 * c.num_sms), 512, big_slots(512) * sizeof(unsigned long long),
-                             c.st>>>(view(L), hr, L.hub_big, L.n_big, a, c.hub_ctr, c.errword); count_launch();
+        k_cluster_big<512><<<(unsigned)std::min(L.n_big, 3 * c.num_sms), 512,
+                             big_slots(512) * sizeof(unsigned long long), c.st>>>(
+            view(L), hr, L.hub_big, L.n_big, a, c.hub_ctr, c.errword); count_launch();
         if (L.max_deg >= kRowPer * 512) {
           k_cluster_big<1024><<<(unsigned)std::min(L.n_big, c.num_sms), 1024,
                                 big_slots(1024) * sizeof(unsigned long long), c.st>>>(
@@ -1939,8 +1941,8 @@ void launch_subround(Ctx& c, int lvl, int32_t r, int64_t wcap) {
       }
       if (L.max_deg > kBigRowDeg) {
         const int64_t res2 = (int64_t)c.num_sms * c.resident_blocks((const void*)k_cluster_giant, kHiThreads, 0);
-        k_cluster_giant<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(L.n_hub_chunks, res2)), kHiThreads, 0, c.st>>>(
-            hr, L.hi_off, c.htab, L.hub_part, a, c.hub_ctr); count_launch();
+        const unsigned gg = (unsigned)std::max<int64_t>(1, std::min<int64_t>(L.n_hub_chunks, res2));
+        k_cluster_giant<<<gg, kHiThreads, 0, c.st>>>(hr, L.hi_off, c.htab, L.hub_part, a, c.hub_ctr); count_launch();
         k_cluster_giant_finish<<<grid_for(c, kThreads, L.n_huge), kThreads, 0, c.st>>>(hr, L.hub_part, L.vw, a);
         count_launch();
       }

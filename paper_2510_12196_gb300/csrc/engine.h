@@ -93,7 +93,7 @@ struct Level {
   int32_t n_long = 0;          // rows that its CTAs take
   int32_t mid_deg = kMidDeg;   // warp-per-vertex bound of this level (<= kMidDeg)
   int64_t split_req = kSplitDeg;  // hub split bound asked for (hub_split_deg: the one in force)
-  int32_t tuned = 0;           // 1: the config leaves both bounds open and they matter (rows above kLowDeg hold 2^20 entries)
+  int32_t tuned = 0;           // 1: both bounds are the rule's, and they matter (rows above kLowDeg hold 2^20 entries)
   int64_t max_deg = 0;         // largest degree (0 when n_hi == 0, i.e. at most kLowDeg)
   int32_t* huge = nullptr;     // positions in hi of the vertices of degree > kMidDeg, ascending
   int32_t n_huge = 0;

@@ -22,7 +22,8 @@ __global__ void k_ids_of_codes(int32_t n, const int32_t* __restrict__ code, cons
 }
 
 // In place; *bad is set when an id lies outside [0, k).
-__global__ void k_codes_of_ids(int32_t n, int32_t* pi, const int32_t* __restrict__ code_of_pe, int32_t k, int32_t* bad) {
+__global__ void k_codes_of_ids(int32_t n, int32_t* pi, const int32_t* __restrict__ code_of_pe, int32_t k,
+                               int32_t* bad) {
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
     const int32_t p = pi[v];
     if (p < 0 || p >= k) *bad = 1;

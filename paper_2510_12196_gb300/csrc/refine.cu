@@ -411,8 +411,9 @@ struct PlainRowLoader {  // neighbour PEs through plain loads (the mapping chang
 };
 
 template <class Load, class Out>
-__device__ __forceinline__ void tile_gain_queue(unsigned work, const TileLane& t, int32_t p, int32_t* sc, int32_t* sw, int cap, Load load,
-                                                const int32_t* sdist, int lane, bool own, Out out) {
+__device__ __forceinline__ void tile_gain_queue(unsigned work, const TileLane& t, int32_t p, int32_t* sc, int32_t* sw,
+                                                int cap, Load load, const int32_t* sdist, int lane, bool own,
+                                                Out out) {
   const int sub = lane >> 3, sl = lane & 7;
   const int rounds = (__popc(work) + 3) / 4;
   for (int r = 0; r < rounds; r++) {
@@ -1024,7 +1025,8 @@ struct WeakMoves {  // weak rebalancing: M = eligible and selected, target the d
   const uint8_t* sel;
   const int32_t* dest;
   __device__ __forceinline__ bool moved(int64_t v) const { return elig[v] && sel[v]; }
-  __device__ __forceinline__ uint32_t flags(int64_t v, int per, int64_t n) const {  // both 0 or 1 in the kernels that call it
+  // (both are 0 or 1 in the kernels that call it)
+  __device__ __forceinline__ uint32_t flags(int64_t v, int per, int64_t n) const {
     const uint32_t e = load_flags(elig, v, per, n);
     return e ? e & load_flags(sel, v, per, n) : 0;
   }
@@ -1938,7 +1940,8 @@ __global__ void __launch_bounds__(kCutThreads) k_reb_cut(const int64_t* __restri
   if (A >= kc || W[A] <= lmax) return;  // only overloaded blocks have eligible vertices
   const int64_t E = W[A] - lmax;
   int64_t before;
-  const int cut = warp_first_above(tab + (int64_t)A * kBuckets, true, E, lane, before);  // the table is zero between steps
+  // (the table is zero between steps)
+  const int cut = warp_first_above(tab + (int64_t)A * kBuckets, true, E, lane, before);
   if (lane == 0) {
     bcut[A] = cut;
     rem[A] = cut < kBuckets ? E - before : 0;
@@ -2507,8 +2510,8 @@ void launch_lp(Ctx& c, int lvl) {
   c.prof_end(ev, PK_LP_AFTER, (int64_t)(L.n - L.n_hi));
   ba.join();
   launch_delta(c, lvl, LpMoves{c.lock, c.pp}, KIND_LP);
-  k_lp_apply<<<apply_grid(c, L.n, per), kApplyThreads, 0, c.st>>>(L.n, L.pi, c.pp, c.lock, L.vw, c.W, c.topo.kc, c.state,
-                                                                  per); count_launch();
+  k_lp_apply<<<apply_grid(c, L.n, per), kApplyThreads, 0, c.st>>>(L.n, L.pi, c.pp, c.lock, L.vw, c.W, c.topo.kc,
+                                                                  c.state, per); count_launch();
 }
 
 RebPrepArgs reb_prep_args(const Ctx& c) {
@@ -2588,7 +2591,8 @@ void launch_rebalance(Ctx& c, int lvl, bool prep_done = false) {
   }
   const WeakMoves mv{c.elig, selected, c.dest};
   launch_delta(c, lvl, mv, KIND_WEAK);
-  k_reb_apply_sel<<<apply_grid(c, L.n, per), kApplyThreads, 0, c.st>>>(L.n, mv, L.pi, L.vw, c.W, c.topo.kc, c.state, per);
+  k_reb_apply_sel<<<apply_grid(c, L.n, per), kApplyThreads, 0, c.st>>>(L.n, mv, L.pi, L.vw, c.W, c.topo.kc, c.state,
+                                                                       per);
   count_launch();
 }
 
@@ -2936,7 +2940,8 @@ struct PlainGather {  // neighbour PEs through plain loads (the mapping changes 
 // of the lane's vertex (0 for a row of more than kEngLaneDeg entries).
 template <int kTE>
 __device__ __forceinline__ TileLane eng_stage(const EngineJob& J, const int32_t* pi, const TileGraph& tg,
-                                              int64_t tile, int lane, int32_t* sc, int32_t* sw, const int32_t* sdist, int64_t& Tp) {
+                                              int64_t tile, int lane, int32_t* sc, int32_t* sw,
+                                              const int32_t* sdist, int64_t& Tp) {
   const TileLane t = stage_tile<kTE>(tg, tile * kTileV, lane, sc, sw, PlainGather{pi});
   Tp = 0;
   if (t.v < tg.n && !eng_heavy(J, t.e - t.b)) {
