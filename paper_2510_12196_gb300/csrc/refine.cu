@@ -865,20 +865,20 @@ __global__ void __launch_bounds__(kThreads) k_lp_after_low(GraphView g, const in
                                                            const int32_t* __restrict__ pp,
                                                            const int64_t* __restrict__ gain,
                                                            const uint8_t* __restrict__ inx, uint8_t* lock, Topo topo,
-                                                           const RefineState* st) {
+                                                           const RefineState* st, int vpw) {
   __shared__ int32_t sdist[32];
   if (!kind_is(st, 1 << KIND_LP)) return;
   load_sdist(sdist, topo);
   __syncthreads();
-  // 32 vertices per warp: one lane reads a vertex's flag, then the candidates
-  // are served four at a time by 8-lane sub-warps (most vertices are none; a
-  // sub-warp per vertex spent its time on their flags: 28 us on a 3D grid of
-  // 2^21 vertices, 17 us so)
+  // vpw vertices per warp (flag_group): one lane reads a vertex's flag, then the
+  // candidates are served four at a time by 8-lane sub-warps (most vertices of a
+  // large level are none; a sub-warp per vertex spent its time on their flags:
+  // 28 us on a 3D grid of 2^21 vertices, 17 us so)
   const int lane = threadIdx.x & 31, sub = lane / kSubWarp, sl = lane & (kSubWarp - 1);
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t base = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; base < g.n; base += nwarps * 32) {
+  for (int64_t base = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * vpw; base < g.n; base += nwarps * vpw) {
     const int64_t vl = base + lane;
-    const unsigned work = __ballot_sync(0xffffffffu, vl < g.n && inx[vl]);
+    const unsigned work = __ballot_sync(0xffffffffu, lane < vpw && vl < g.n && inx[vl]);
     const int rounds = (__popc(work) + 3) / 4;
     for (int r = 0; r < rounds; r++) {
       const int src = tile_worker(work, r, sub);
@@ -1047,7 +1047,7 @@ __device__ __forceinline__ int64_t delta_entry(const Mv& mv, const int32_t* pi, 
 // time by the 8-lane sub-warps of the warp (as k_lp_after_low)
 template <class Mv>
 __global__ void __launch_bounds__(kThreads) k_delta_low(GraphView g, const int32_t* __restrict__ pi, Mv mv, Topo topo,
-                                                        int64_t* Jacc, const RefineState* st, int kind) {
+                                                        int64_t* Jacc, const RefineState* st, int kind, int vpw) {
   __shared__ int32_t sdist[32];
   __shared__ int64_t sm[33];
   if (st->kind != kind) return;
@@ -1056,9 +1056,9 @@ __global__ void __launch_bounds__(kThreads) k_delta_low(GraphView g, const int32
   const int lane = threadIdx.x & 31, sub = lane / kSubWarp, sl = lane & (kSubWarp - 1);
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   int64_t acc = 0;
-  for (int64_t base = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; base < g.n; base += nwarps * 32) {
+  for (int64_t base = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * vpw; base < g.n; base += nwarps * vpw) {
     const int64_t vl = base + lane;
-    const unsigned work = __ballot_sync(0xffffffffu, vl < g.n && mv.moved(vl));
+    const unsigned work = __ballot_sync(0xffffffffu, lane < vpw && vl < g.n && mv.moved(vl));
     const int rounds = (__popc(work) + 3) / 4;
     for (int r = 0; r < rounds; r++) {
       const int src = tile_worker(work, r, sub);
@@ -2355,6 +2355,18 @@ inline unsigned grid_for(const Ctx& c, int64_t items_per_block, int64_t n) {
   return (unsigned)g;
 }
 
+// Vertices per warp of the kernels that look for flagged vertices and serve
+// each with a sub-warp: as few as the resident warps allow, since the flagged
+// ones of a warp are served one after another (32 vertices per warp on a grid of
+// 2^14 under a random mapping, where every vertex is flagged, cost a
+// label-propagation step 12 us).
+inline int flag_group(const Ctx& c, int64_t n) {
+  const int64_t warps = (int64_t)c.num_sms * 8 * (kThreads / 32);
+  int vpw = 32 / kSubWarp;
+  while (vpw < 32 && n > vpw * warps) vpw *= 2;
+  return vpw;
+}
+
 size_t conn_smem(const Ctx& c) { return (size_t)group_layout(c.topo).total * sizeof(int32_t); }
 
 // Grid of a mid-degree kernel (one warp per vertex of the high-degree list).
@@ -2439,7 +2451,9 @@ void launch_delta(Ctx& c, int lvl, Mv mv, int kind) {
       k_delta_mid<Mv><<<mid_grid(c, (const void*)k_delta_mid<Mv>, 0, L.n_hi), kMidThreads, 0, c.st>>>(
           view(L), L.hi, L.n_hi, L.pi, mv, c.topo, c.Jacc, c.state, kind); count_launch();
     });
-  k_delta_low<Mv><<<grid_for(c, kThreads, L.n), kThreads, 0, c.st>>>(view(L), L.pi, mv, c.topo, c.Jacc, c.state, kind);
+  const int vpw = flag_group(c, L.n);
+  k_delta_low<Mv><<<grid_for(c, kThreads / 32 * vpw, L.n), kThreads, 0, c.st>>>(view(L), L.pi, mv, c.topo, c.Jacc,
+                                                                                c.state, kind, vpw);
   count_launch();
   br.join();
 }
@@ -2447,7 +2461,7 @@ void launch_delta(Ctx& c, int lvl, Mv mv, int kind) {
 void launch_lp(Ctx& c, int lvl) {
   Level& L = c.lv[lvl];
   const int per = flags_per_lane(L.n);
-  const unsigned gl = grid_for(c, kThreads, L.n);
+  const int vpw = flag_group(c, L.n);
   const bool mid_tab = mid_tables(c);
   const GroupLayout glay = group_layout(c.topo);
   // vertices of degree > kLowDeg left to the hub kernels, or to a CTA each
@@ -2505,7 +2519,9 @@ void launch_lp(Ctx& c, int lvl) {
     }
   });
   ev = c.prof_begin();
-  k_lp_after_low<<<gl, kThreads, 0, c.st>>>(view(L), L.pi, c.pp, c.gain, c.inx, c.lock, c.topo, c.state); count_launch();
+  k_lp_after_low<<<grid_for(c, kThreads / 32 * vpw, L.n), kThreads, 0, c.st>>>(view(L), L.pi, c.pp, c.gain, c.inx,
+                                                                               c.lock, c.topo, c.state, vpw);
+  count_launch();
   // the X flag of every vertex (the work on X itself is data dependent)
   c.prof_end(ev, PK_LP_AFTER, (int64_t)(L.n - L.n_hi));
   ba.join();
