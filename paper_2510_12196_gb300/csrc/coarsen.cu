@@ -1266,13 +1266,19 @@ __global__ void k_cl_end(ClusterState* cs, int32_t n, int32_t iters, cudaGraphCo
 // requests contested, however many there are in all (coarsening of a 3D grid of
 // 32768 vertices on 4096 PEs: 0.56 ms, with every request compared with every
 // other 3.3, as a graph of kernels 0.71; of an RGG of 131072 on 4096 PEs 0.67, 1.6
-// and 1.76).  With a chain of
-// kClEngChain requests or more the launch gives up: the graph sorts them.
+// and 1.76).  With a chain of kClEngChain requests or more the launch gives up:
+// the graph sorts them.
+// A cluster of 16 CTAs, not 8: coarsening of an RGG of 9000 / 32000 vertices 0.67 /
+// 1.17 ms against 0.75 / 1.44 (as graphs of kernels that exist 0.91 / 1.40, 1.3 /
+// 2.0 in a new context).  Levels between 2^13 and 2^15 vertices by a launch over
+// all SMs instead: about the same in one context (RGG of 20000 / 32000 2 % / 4 %
+// faster), but 12000 vertices each in eight threads' contexts 7.1 ms against 4.7
+// with clusters, which run side by side.
 constexpr int kClEngThreads = 1024;
 constexpr int kClEngMaxN = 1 << 15;
 constexpr int kClGridMaxN = 1 << 17;
 constexpr int kClEngChain = 512;
-constexpr int kClEngMaxCluster = 8;  // the portable limit
+constexpr int kClEngMaxCluster = 16;  // 8 (the portable limit) where the device holds none of 16
 constexpr int kClEngRow = kTileE / 4;
 struct PlainLabel {  // labels change inside the launch: plain loads
   const int32_t* C;
@@ -1387,13 +1393,45 @@ __global__ void __launch_bounds__(kClEngThreads, 1) k_cluster_engine(GraphView g
 // The same loop for the levels above one cluster's size, by a cooperative launch
 // of a CTA per SM (new contexts: the capture and instantiation of the graph took
 // 0.3 ms, the kernel boundaries and the WHILE node 0.1): map of an RGG of 50021
-// vertices 3.74 -> 3.15 ms, 3D grid of 2^21 (a level of 97000) 20.3 -> 19.7.  A
-// repeated run of one context, whose graph exists, loses 0.2 ms on that level.
+// vertices 3.74 -> 3.15 ms, 3D grid of 2^21 (a level of 97000) 20.3 -> 19.7.
+// The line at kClGridMaxN, as a launch against a graph (coarsening, ms, new context
+// / its later runs): RGG of 131000 1.42 / 1.43 against 1.79 / 1.46, of 200000 1.58 /
+// 1.57 against 1.82 / 1.55, of 520000 2.41 / 2.41 against 2.75 / 2.45, 3D grid of
+// 125000 1.27 / 1.27 against 2.42 / 2.08, of 216000 1.55 / 1.54 against 2.28 / 1.99.
+// Above it new contexts would gain too; later runs, and contexts side by side, do
+// not everywhere, and the line stays where both do.
 __global__ void __launch_bounds__(kClEngThreads, 1) k_cluster_grid(GraphView g, ClusterArgs a, ClusterEngineArgs e,
                                                                    GridBar* bar, unsigned arrivals) {
   extern __shared__ __align__(16) int2 cl_scw[];
   __shared__ unsigned int bar_flag;
   cluster_engine_run(g, a, e, cl_scw, (int)blockIdx.x, (int)gridDim.x, GridSync{bar, &bar_flag, arrivals});
+}
+
+// CTAs of a cluster of k_cluster_engine at most on the device; sets the kernel's attributes.
+int cluster_engine_max(const Ctx& c, size_t smem) {
+  static std::atomic<int> cached[64];  // a property of the device: once per process
+  int v = cached[c.dev & 63].load();
+  if (v) return v;
+  GM_CUDA(cudaFuncSetAttribute(k_cluster_engine, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = kClEngMaxCluster;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cudaLaunchConfig_t lc{};
+  lc.gridDim = dim3(kClEngMaxCluster);
+  lc.blockDim = dim3(kClEngThreads);
+  lc.dynamicSmemBytes = smem;
+  lc.attrs = &attr;
+  lc.numAttrs = 1;
+  int clusters = 0;
+  if (cudaFuncSetAttribute(k_cluster_engine, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&clusters, k_cluster_engine, &lc) != cudaSuccess) {
+    cudaGetLastError();
+    clusters = 0;
+  }
+  v = clusters > 0 ? kClEngMaxCluster : 8;
+  cached[c.dev & 63].store(v);
+  return v;
 }
 
 // CTAs of k_cluster_grid on the device; 0: no cooperative launch there.
@@ -2102,13 +2140,8 @@ int32_t cluster_level(Ctx& c, int lvl) {
     lc.attrs = &attr;
     lc.numAttrs = 1;
     if (n <= kClEngMaxN) {
-      static std::atomic<unsigned long long> attr_done{0};  // one bit per device
-      const unsigned long long bit = 1ULL << (c.dev & 63);
-      if (!(attr_done.load() & bit)) {
-        GM_CUDA(cudaFuncSetAttribute(k_cluster_engine, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)eng_smem));
-        attr_done.fetch_or(bit);
-      }
-      const unsigned C = (unsigned)std::min(kClEngMaxCluster, (n + kClEngThreads - 1) / kClEngThreads);
+      const unsigned C =
+          (unsigned)std::min(cluster_engine_max(c, eng_smem), (n + kClEngThreads - 1) / kClEngThreads);
       lc.gridDim = dim3(C);
       attr.id = cudaLaunchAttributeClusterDimension;
       attr.val.clusterDim.x = C;
