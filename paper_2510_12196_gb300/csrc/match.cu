@@ -324,6 +324,10 @@ __global__ void k_mt_stage_end(MatchState* s, unsigned long long body_kernels) {
 // 2^18 vertices by matching (eight levels) 12.7 -> 9.3 ms, 9.0 -> 8.5 on a kept
 // context whose graphs exist.  (The two-hop stages follow as launches, one read
 // of the count each; most levels need none.)
+// The line at kMRoundMaxN, as launches against graphs (coarsening, ms, new context
+// / its later runs): RGG of 131000 2.2 / 2.1 against 4.2 / 2.5, of 260000 2.8 / 2.7
+// against 5.3 / 3.2, of 520000 3.8 / 3.8 against 4.6 / 4.0, of 10^6 5.1 / 5.1 against
+// 6.3 / 5.3: it gains above the line too, ever less, and the line has not been moved.
 constexpr int kMRoundThreads = 1024;
 constexpr int kMRoundMaxN = 1 << 18;
 constexpr int kMRoundShared = 16;  // CTAs at most where launches over every SM are unwanted
