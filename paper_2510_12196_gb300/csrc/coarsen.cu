@@ -367,8 +367,9 @@ __device__ __forceinline__ uint32_t slot_hash(int32_t t) {
 //    reset touch those slots only, not the table: k_cluster_high takes the
 //    rows up to kSmemRowDeg, k_cluster_big the others.  Scanning the tables
 //    instead, with the rows above 2047 entries in global tables, took 1.13 ms a
-//    sub-round of R-MAT 2^22 (k_cluster_high 0.83, k_cluster_giant 0.29), this
-//    0.82 (0.53 + k_cluster_big 0.17 + k_cluster_giant 0.12).
+//    sub-round of R-MAT 2^22 (mean over its levels; k_cluster_high 0.83,
+//    k_cluster_giant 0.29), this 0.88 (0.52 + k_cluster_big 0.22 + k_cluster_giant
+//    and its finish 0.15).
 //  * larger rows: their entries, flattened in huge[] order, are cut into
 //    chunks of kHubChunk entries that the CTAs of one wave take in turn, the
 //    table in global memory.  A second launch reads the table back in the

@@ -75,8 +75,9 @@ __global__ void k_na_clear(NoAllocScratch* s, Topo t, Hier h) {
 // consecutive ones at a time, so that their neighbours' PEs, near one another
 // where the ids have locality, come in few cache lines.  The pass streams 8
 // bytes an entry and gathers 4.  RGG of 2^20 vertices, 12.6e6 entries: 64-85 us
-// whatever the mapping and the code space (eight consecutive entries per thread
-// 87-135 us; eight lanes per row 81-610 us, R-MAT 2^20 5.5 ms).
+// whatever the mapping and the code space, R-MAT 2^20 of 31e6 entries 183 us (eight
+// consecutive entries per thread 87-135 and 268 us; eight lanes per row 81-614 us
+// and 5.5 ms).
 // The weights are summed by warp and PE first, then in the block's shared
 // memory where it has more vertices than there are PE codes (at most kNaCodes),
 // else straight into the global sums.
