@@ -88,7 +88,6 @@ __global__ void k_na_clear(NoAllocScratch* s, Topo t, Hier h) {
 constexpr int kNaItems = 8;
 constexpr int kNaTile = kNaThreads * kNaItems;
 constexpr int kNaCodes = 2048;
-constexpr int kNaShare = 8;
 constexpr int64_t kNaVertices = 1024;  // vertices per block at least (blocks past the last one sum no weights)
 
 // Largest v in [0, n) with xadj[v] <= e, -1 if none; all threads call it.
@@ -145,22 +144,7 @@ __global__ void __launch_bounds__(kNaThreads, 5) k_na_eval(int32_t n, const int6
   for (int64_t v0 = va + (threadIdx.x - lane); v0 < vb; v0 += kNaThreads) {  // (warp-uniform)
     const int64_t v = v0 + lane;
     const int32_t c = v < vb ? code_or_none(pi[v]) : -1;
-    const int32_t x = c >= 0 ? vw[v] : 0;
-    unsigned left = __ballot_sync(0xffffffffu, c >= 0);
-    // a PE of kNaShare or more of the warp's vertices at once (their single updates would queue on one word)
-    while (left) {
-      const int src = __ffs(left) - 1;
-      const int32_t cs = __shfl_sync(0xffffffffu, c, src);
-      const unsigned same = __ballot_sync(0xffffffffu, c == cs) & left;
-      if (__popc(same) < kNaShare) break;
-      const int32_t y = c == cs ? x : 0;
-      // 32 values of 32 bits: the sums of their halves fit
-      const int64_t lo = (int64_t)__reduce_add_sync(0xffffffffu, (unsigned)y & 0xffffu);
-      const int64_t hi = (int64_t)__reduce_add_sync(0xffffffffu, y >> 16);
-      if (lane == src) add_weight(c, hi * 65536 + lo);
-      left &= ~same;
-    }
-    if ((left >> lane) & 1u) add_weight(c, x);
+    warp_add(c, c >= 0 ? vw[v] : 0, add_weight);
   }
 
   const int64_t m = xadj[n];

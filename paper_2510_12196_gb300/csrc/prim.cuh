@@ -55,6 +55,29 @@ __device__ T block_sum(T v, T* sm /* >= 32 */) {
   return r;
 }
 
+// add(slot, x) for every lane of the warp with slot >= 0, all lanes calling it:
+// a slot of kWarpShare or more lanes (by the first of them) once with their
+// sum, since single updates of one word queue; the others lane by lane.
+constexpr int kWarpShare = 8;
+template <class Add>
+__device__ __forceinline__ void warp_add(int32_t slot, int32_t x, Add add) {
+  const int lane = threadIdx.x & 31;
+  unsigned left = __ballot_sync(0xffffffffu, slot >= 0);
+  while (left) {
+    const int src = __ffs(left) - 1;
+    const int32_t s = __shfl_sync(0xffffffffu, slot, src);
+    const unsigned same = __ballot_sync(0xffffffffu, slot == s);
+    if (__popc(same) < kWarpShare) break;
+    const int32_t y = slot == s ? x : 0;
+    // 32 values of 32 bits: the sums of their halves fit
+    const int64_t lo = (int64_t)__reduce_add_sync(0xffffffffu, (unsigned)y & 0xffffu);
+    const int64_t hi = (int64_t)__reduce_add_sync(0xffffffffu, y >> 16);
+    if (lane == src) add(s, hi * 65536 + lo);
+    left &= ~same;
+  }
+  if ((left >> lane) & 1u) add(slot, (int64_t)x);
+}
+
 // Exclusive block scan of one value per thread; returns the exclusive prefix
 // and writes the block total to *total.
 template <class T>

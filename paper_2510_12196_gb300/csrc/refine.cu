@@ -1158,7 +1158,10 @@ __global__ void __launch_bounds__(kHiThreads) k_delta_high(GraphView g, HubRows 
 // most kApplyCodes codes each CTA sums its changes in shared memory and adds
 // the non-zero ones to W at the end: movers crowd into a few blocks (a hub's
 // neighbourhood moves together on power-law graphs), and one global atomic per
-// mover on the same few words serialises.
+// mover on the same few words serialises.  So do those in shared memory, and a
+// warp's movers from or to one block are summed first (a 2D grid of 10^6 vertices
+// leaving one PE: k_reb_apply_sel 299 -> 10 us; half a star of 2^19 following its
+// hub: k_lp_apply 185 -> 15).
 constexpr int32_t kApplyCodes = 4096;
 struct BlockDelta {
   long long* dW;  // shared, kApplyCodes
@@ -1169,13 +1172,16 @@ struct BlockDelta {
       for (int32_t b = threadIdx.x; b < kc; b += blockDim.x) dW[b] = 0;
   }
   __device__ __forceinline__ void move(int32_t p, int32_t q, int64_t c) {
-    if (local) {
-      atomicAdd((unsigned long long*)&dW[p], (unsigned long long)(-c));
-      atomicAdd((unsigned long long*)&dW[q], (unsigned long long)c);
-    } else {
-      atomicAdd((unsigned long long*)&W[p], (unsigned long long)(-c));
-      atomicAdd((unsigned long long*)&W[q], (unsigned long long)c);
-    }
+    add(p, -c);
+    add(q, c);
+  }
+  __device__ __forceinline__ void add(int32_t b, int64_t c) {
+    atomicAdd(local ? (unsigned long long*)&dW[b] : (unsigned long long*)&W[b], (unsigned long long)c);
+  }
+  // one mover per lane (p, q < 0: none); all lanes of the warp call it
+  __device__ __forceinline__ void move_warp(int32_t p, int32_t q, int32_t c) {
+    warp_add(p, -c, [&](int32_t b, int64_t x) { add(b, x); });
+    warp_add(q, c, [&](int32_t b, int64_t x) { add(b, x); });
   }
   // after a barrier
   __device__ __forceinline__ void flush(int32_t kc) {
@@ -1207,14 +1213,23 @@ __global__ void __launch_bounds__(kApplyThreads) k_lp_apply(int32_t n, int32_t* 
   if (threadIdx.x == 0) cnt = 0;
   __syncthreads();
   int32_t mine = 0;
-  for (int64_t v0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * per; v0 < n;
+  const int64_t lane0 = (threadIdx.x & 31) * per;  // (v0 - lane0 is the same in a warp)
+  for (int64_t v0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * per; v0 - lane0 < n;
        v0 += (int64_t)gridDim.x * blockDim.x * per) {
-    for (uint32_t f = load_flags(lock, v0, per, n); f; f &= f - 1) {  // (flags are 0 or 1)
-      const int64_t v = v0 + (__ffs(f) - 1) / 8;
-      const int32_t p = pi[v], q = pp[v];
-      pi[v] = q;
-      bd.move(p, q, vw[v]);
-      mine++;
+    const uint32_t f = load_flags(lock, v0, per, n);  // (flags are 0 or 1)
+    for (int j = 0; j < per; j++) {
+      const bool on = (f >> (8 * j)) & 1u;
+      if (!__any_sync(0xffffffffu, on)) continue;
+      const int64_t v = v0 + j;
+      int32_t p = -1, q = -1, c = 0;
+      if (on) {
+        p = pi[v];
+        q = pp[v];
+        c = vw[v];
+        pi[v] = q;
+        mine++;
+      }
+      bd.move_warp(p, q, c);
     }
   }
   if (mine) atomicAdd(&cnt, mine);
@@ -2039,7 +2054,8 @@ __global__ void __launch_bounds__(kSmallThreads) k_reb_resolve(const uint64_t* _
 // the weight of the digits below (k_cut_digit).  The totals use the (block,
 // bucket) table, which is zero between steps.  Nine small launches (25 us on a
 // 3D grid of 2^21 vertices, where the sort of the list by (block, id) and the
-// prefix over it took 100 us); the single-CTA sort (k_reb_resolve) stays for
+// prefix over it took 100 us; 10^6 vertices leaving one PE 0.1 ms, with an update
+// of the totals per vertex 0.65); the single-CTA sort (k_reb_resolve) stays for
 // lists of at most 4096.
 constexpr int kCutDigit = 6;
 static_assert((1 << kCutDigit) == kBuckets, "the digit totals use the bucket table");
@@ -2048,11 +2064,18 @@ __global__ void k_cut_sums(const uint64_t* __restrict__ key, const int32_t* __re
                            const int64_t* __restrict__ prefix, const int32_t* __restrict__ vw, int64_t* tab) {
   const int64_t n = cnt[CNT_ELIG];
   if (n <= kSmallSort) return;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t A = (int32_t)(key[i] >> idbits), v = val[i];
-    if (!first && (v >> (shift + kCutDigit)) != prefix[A]) continue;
-    atomicAdd((unsigned long long*)&tab[(int64_t)A * kBuckets + ((v >> shift) & (kBuckets - 1))],
-              (unsigned long long)(int64_t)vw[v]);
+  const int lane = threadIdx.x & 31;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i - lane < n; i += (int64_t)gridDim.x * blockDim.x) {
+    int32_t slot = -1, c = 0;
+    if (i < n) {
+      const int32_t A = (int32_t)(key[i] >> idbits), v = val[i];
+      if (first || (v >> (shift + kCutDigit)) == prefix[A]) {
+        slot = A * kBuckets + ((v >> shift) & (kBuckets - 1));
+        c = vw[v];
+      }
+    }
+    // (neighbouring ids share their upper digits)
+    warp_add(slot, c, [&](int32_t at, int64_t x) { atomicAdd((unsigned long long*)&tab[at], (unsigned long long)x); });
   }
 }
 __global__ void __launch_bounds__(kCutThreads) k_cut_digit(const int64_t* __restrict__ W, int32_t kc, int64_t lmax,
@@ -2093,14 +2116,23 @@ __global__ void __launch_bounds__(kApplyThreads) k_reb_apply_sel(int32_t n, Weak
   bd.init(kc);
   __syncthreads();
   int32_t mine = 0;
-  for (int64_t v0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * per; v0 < n;
+  const int64_t lane0 = (threadIdx.x & 31) * per;  // (v0 - lane0 is the same in a warp)
+  for (int64_t v0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) * per; v0 - lane0 < n;
        v0 += (int64_t)gridDim.x * blockDim.x * per) {
-    for (uint32_t f = mv.flags(v0, per, n); f; f &= f - 1) {  // (flags are 0 or 1)
-      const int64_t v = v0 + (__ffs(f) - 1) / 8;
-      const int32_t p = pi[v], q = mv.target(v);
-      pi[v] = q;
-      bd.move(p, q, vw[v]);
-      mine++;
+    const uint32_t f = mv.flags(v0, per, n);  // (flags are 0 or 1)
+    for (int j = 0; j < per; j++) {
+      const bool on = (f >> (8 * j)) & 1u;
+      if (!__any_sync(0xffffffffu, on)) continue;
+      const int64_t v = v0 + j;
+      int32_t p = -1, q = -1, c = 0;
+      if (on) {
+        p = pi[v];
+        q = mv.target(v);
+        c = vw[v];
+        pi[v] = q;
+        mine++;
+      }
+      bd.move_warp(p, q, c);
     }
   }
   __syncthreads();
