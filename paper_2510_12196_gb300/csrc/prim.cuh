@@ -164,8 +164,10 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_apply(Load load, Store st
 // three kernels above and the gaps between them are most of a small scan's time
 // (a coarse level runs five to seven): map of a 16^3 grid 3.23 -> 3.15 ms,
 // hierarchical multisection of an RGG of 2^17 vertices 25.9 -> 24.7 ms.  16 items a
-// thread: with 32 the coarsening of 3000 to 60000 vertices took 5-16 % longer (the
-// registers), with 8 it was level within 2 % (by matching up to 4 % longer).
+// thread: 16384 items of 8 bytes take 6.8 us, the three launches 9.1 and the gaps
+// between them (18 us with a thread's items next to one another, a line each).
+// With 32 a thread the coarsening of 3000 to 60000 vertices took 5-16 % longer
+// (the registers), with 8 it was level within 2 % (by matching up to 4 % longer).
 constexpr int kScanOneItems = 16;
 constexpr int64_t kScanOne = 1024 * kScanOneItems;
 template <class Load, class Store>
@@ -173,20 +175,29 @@ __global__ void __launch_bounds__(1024) k_scan_one(Load load, Store store, int64
                                                    int64_t* total_out) {
   __shared__ int64_t sm[33];
   const int n = (int)load_count(d_n, max_n);
-  const int per = (n + 1023) / 1024, first = (int)threadIdx.x * per;  // at most kScanOneItems each
+  const int per = (n + 1023) / 1024;  // items per lane, at most kScanOneItems
+  // a warp's items are consecutive, a lane's 32 apart (loads and stores of whole lines)
+  const int lane = (int)threadIdx.x & 31, first = ((int)threadIdx.x - lane) * per + lane;
   int64_t vals[kScanOneItems];
   int64_t local = 0;
 #pragma unroll
   for (int j = 0; j < kScanOneItems; j++) {
-    vals[j] = j < per && first + j < n ? load(first + j) : 0;
+    vals[j] = j < per && first + 32 * j < n ? load(first + 32 * j) : 0;
     local += vals[j];
   }
   int64_t total;
-  int64_t run = block_exclusive_scan(local, sm, &total);
+  int64_t run = __shfl_sync(0xffffffffu, block_exclusive_scan(local, sm, &total), 0);
 #pragma unroll
   for (int j = 0; j < kScanOneItems; j++) {
-    if (j < per && first + j < n) store(first + j, run, vals[j]);
-    run += vals[j];
+    if (j >= per) break;  // (uniform)
+    int64_t x = vals[j];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (first + 32 * j < n) store(first + 32 * j, run + x - vals[j], vals[j]);
+    run += __shfl_sync(0xffffffffu, x, 31);
   }
   if (threadIdx.x == 0) *total_out = total;
 }
