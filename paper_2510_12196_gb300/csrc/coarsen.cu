@@ -506,6 +506,27 @@ __device__ __forceinline__ void warp_first_label(uint64_t& bh, int32_t& bt) {
   }
 }
 
+// Entries of one warp with the same label, when kWarpShare or more have it (the
+// first entry's, then the next), become one entry of their summed weight, the
+// others none (t = -1): where a few large clusters hold most of a row, its entries
+// would queue on their slots, with compare-and-swap loops on chip (bipartite graph
+// of 200 rows of 3900 entries on 2 PEs: k_cluster_big 107 -> 46 us a sub-round).
+__device__ __forceinline__ void warp_combine(int32_t& t, int32_t& w) {
+  const int lane = threadIdx.x & 31;
+  unsigned left = __ballot_sync(0xffffffffu, t >= 0);
+  while (left) {
+    const int src = __ffs(left) - 1;
+    const int32_t s = __shfl_sync(0xffffffffu, t, src);
+    const bool mine = t == s;
+    const unsigned same = __ballot_sync(0xffffffffu, mine);
+    if (__popc(same) < kWarpShare) return;
+    const int32_t sum = (int32_t)__reduce_add_sync(0xffffffffu, mine ? (unsigned)w : 0u);  // (weights sum below 2^31)
+    if (lane == src) w = sum;
+    else if (mine) t = -1;
+    left &= ~same;
+  }
+}
+
 // Rates one row of deg <= kRowPer * gr.size entries from CSR position e0 in
 // the shared-memory table T (empty before and after) and returns the best
 // label to the group's thread 0; all threads of group gr call it, ends with
@@ -538,6 +559,8 @@ __device__ __forceinline__ int32_t rate_row(const GraphView& g, const ClusterArg
     }
 #pragma unroll
     for (int b = 0; b < kHubBatch; b++) t[b] = t[b] >= 0 ? a.C[t[b]] : -1;
+#pragma unroll
+    for (int b = 0; b < kHubBatch; b++) warp_combine(t[b], w[b]);
 #pragma unroll
     for (int b = 0; b < kHubBatch; b++) {
       h[b] = slot_hash(t[b]) & mask;
