@@ -511,6 +511,9 @@ __device__ __forceinline__ void warp_first_label(uint64_t& bh, int32_t& bt) {
 // others none (t = -1): where a few large clusters hold most of a row, its entries
 // would queue on their slots, with compare-and-swap loops on chip (bipartite graph
 // of 200 rows of 3900 entries on 2 PEs: k_cluster_big 107 -> 46 us a sub-round).
+// For the rows of k_cluster_big only: on those of k_cluster_high it gained less
+// there (39 -> 31 us on R-MAT 2^18, 2 PEs) than it cost where labels are distinct
+// (517 -> 543 us on R-MAT 2^22, 512 PEs).
 __device__ __forceinline__ void warp_combine(int32_t& t, int32_t& w) {
   const int lane = threadIdx.x & 31;
   unsigned left = __ballot_sync(0xffffffffu, t >= 0);
@@ -531,7 +534,7 @@ __device__ __forceinline__ void warp_combine(int32_t& t, int32_t& w) {
 // the shared-memory table T (empty before and after) and returns the best
 // label to the group's thread 0; all threads of group gr call it, ends with
 // the group's barrier.
-template <int kWarps>
+template <bool kCombine, int kWarps>
 __device__ __forceinline__ int32_t rate_row(const GraphView& g, const ClusterArgs& a, int64_t e0, int32_t deg,
                                             int32_t own, unsigned long long* T, uint32_t mask,
                                             BestScratch<kWarps>& sx, const RowGroup& gr, uint32_t* err) {
@@ -560,7 +563,8 @@ __device__ __forceinline__ int32_t rate_row(const GraphView& g, const ClusterArg
 #pragma unroll
     for (int b = 0; b < kHubBatch; b++) t[b] = t[b] >= 0 ? a.C[t[b]] : -1;
 #pragma unroll
-    for (int b = 0; b < kHubBatch; b++) warp_combine(t[b], w[b]);
+    for (int b = 0; b < kHubBatch; b++)
+      if constexpr (kCombine) warp_combine(t[b], w[b]);
 #pragma unroll
     for (int b = 0; b < kHubBatch; b++) {
       h[b] = slot_hash(t[b]) & mask;
@@ -833,7 +837,7 @@ __global__ void __launch_bounds__(kHiThreads, 5) k_cluster_high(GraphView g, Hub
         } else {
           uint32_t size = 64;
           while (size < 2 * (uint32_t)(deg + 1)) size <<= 1;
-          best = rate_row(g, a, e0, (int32_t)deg, own, gtab, size - 1, sx, gr, err);
+          best = rate_row<false>(g, a, e0, (int32_t)deg, own, gtab, size - 1, sx, gr, err);
         }
         if (gr.tid == 0) cluster_request(a, v, own, best, g.vw[v]);
       }
@@ -864,7 +868,7 @@ __global__ void __launch_bounds__(kHiThreads, 5) k_cluster_high(GraphView g, Hub
       if (deg <= kSmemRowDeg) {
         uint32_t size = 64;
         while (size < 2 * (uint32_t)(deg + 1)) size <<= 1;
-        const int32_t best = rate_row(g, a, x0 + rb, (int32_t)deg, own, stab, size - 1, sx, cta, err);
+        const int32_t best = rate_row<false>(g, a, x0 + rb, (int32_t)deg, own, stab, size - 1, sx, cta, err);
         if (threadIdx.x == 0) cluster_request(a, v, own, best, g.vw[v]);
         continue;
       }
@@ -905,7 +909,7 @@ __global__ void __launch_bounds__(kT) k_cluster_big(GraphView g, HubRows hr, con
     uint32_t size = 64;
     while (size < 2 * (uint32_t)(deg + 1)) size <<= 1;
     const int32_t own = a.C[v];
-    const int32_t best = rate_row(g, a, g.xadj[v], deg, own, btab, size - 1, sx, cta, err);
+    const int32_t best = rate_row<true>(g, a, g.xadj[v], deg, own, btab, size - 1, sx, cta, err);
     if (threadIdx.x == 0) cluster_request(a, v, own, best, g.vw[v]);
   }
   leave_chunks(ctr);
